@@ -39,6 +39,24 @@ def test_ensemble_against_oracle(oracle64, M, nq, K, E, power):
     assert (sc == o_sc).all()
 
 
+# unions at and beyond the first launch's table (1,024 slots), the larger table (8,192 slots) and the sort behind it; one
+# place per list; the longest list kept as bytes and the first that is sorted; blocks of 32 models with a remainder of one
+@pytest.mark.parametrize("M,nq,K,E", [(33, 7, 31, 1024), (11, 150, 94, 100_000), (85, 3, 96, 1_000_000), (90, 3, 100, 1_000_000), (160, 2, 102, 1 << 30),
+                                      (40, 9, 1, 12), (4, 5, 254, 300), (4, 5, 255, 300), (65, 40, 2, 5)])
+@pytest.mark.parametrize("power", [-0.5, 1.0])
+def test_ensemble_union_sizes(oracle64, M, nq, K, E, power):
+    rng = np.random.default_rng(M + K)
+    pick = (lambda: rng.permutation(E)[:K]) if E <= 300 else (lambda: rng.integers(0, E, K))
+    lists = np.stack([np.stack([pick() for _ in range(nq)]) for _ in range(M)]).astype(np.int32)
+    if K > 2:
+        lists[0, 0, 1] = lists[0, 0, 0]                 # an entity twice in one list: both places count
+        lists[:, 1, :] = -1                             # a query nobody answered
+    ids, sc = _gpu_ensemble(lists, power, 10)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, power, 10)
+    assert (ids == o_ids).all()
+    assert (sc == o_sc).all()
+
+
 def test_ensemble_fewer_candidates_than_places_and_limits(oracle64):
     import torch
     import paper_2211_12281_b200 as K
