@@ -42,10 +42,8 @@ __device__ __forceinline__ bool ens_before(double sa, int32_t ia, double sb, int
 
 // ------------------------------------------------------------------------------------------
 // Hash form.  Shared memory per slot: entity id, fp64 sum, MB position bytes, one entry of the list of
-// occupied slots.  The cell words of a slot lie `slots` words apart, so the slots a warp touches (random,
-// one model) spread over the banks.  Cost per query: about 28 instructions per list entry (load, hash,
-// probe, one atomic add) and about 4 per (entity, model); 85 x top-100 lists, 15,000 queries, unions of 300
-// entities, against the sort's 105 passes over 16,384 keys: see the launch below for the times.
+// occupied slots.  The cell words of a slot lie `slots` words apart, so that the slots a warp touches
+// (random, one model) spread over the banks.
 // Returns false (all threads) if the union does not fit or a list names an entity twice.
 // ------------------------------------------------------------------------------------------
 template <int MB>
@@ -97,23 +95,26 @@ __device__ bool ens_hash_query(const EnsParams& p, const int q, const int log2_s
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (id[u] < 0) continue;                                        // unused places of a list hold -1
-                const int e = e0 + u * nthr + tid;
-                uint32_t h = (uint32_t)id[u] * 0x9E3779B1u >> (32 - log2_slots);
-                bool ok = false;
-                for (int probe = 0; probe < slots; ++probe) {
-                    int32_t k = *reinterpret_cast<volatile int32_t*>(key + h);
-                    if (k == -1) {
-                        k = atomicCAS(key + h, -1, id[u]);
-                        if (k == -1) { used[atomicAdd(&n_used, 1)] = (uint16_t)h; k = id[u]; }
+                // the warp probes together: left to themselves, the lanes that need one probe more run the rest of the body on their own
+                const int e = e0 + u * nthr + tid, want = id[u];
+                uint32_t h = (uint32_t)want * 0x9E3779B1u >> (32 - log2_slots);
+                int32_t k = want < 0 ? want : *reinterpret_cast<volatile int32_t*>(key + h);       // (unused places of a list hold -1)
+                bool need = k != want;
+                for (int probe = 0; probe < slots && __any_sync(0xffffffffu, need); ++probe) {
+                    if (need && k == -1) {
+                        k = atomicCAS(key + h, -1, want);
+                        if (k == -1) { used[atomicAdd(&n_used, 1)] = (uint16_t)h; k = want; }
                     }
-                    if (k == id[u]) { ok = true; break; }
-                    if ((probe & 15) == 15 && *reinterpret_cast<volatile int*>(&bad)) break;
-                    h = (h + 1) & (uint32_t)(slots - 1);
+                    need = need && k != want;
+                    if (need) {
+                        h = (h + 1) & (uint32_t)(slots - 1);
+                        k = *reinterpret_cast<volatile int32_t*>(key + h);
+                        need = k != want;
+                    }
+                    if ((probe & 15) == 15 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bad))) break;
                 }
                 const uint32_t sh = (uint32_t)(ml[u] & 3) * 8u;
-                if (ok) ok = (atomicAdd(&cell[(ml[u] >> 2) * slots + h], (uint32_t)(e - ml[u] * p.K + 1) << sh) >> sh & 0xffu) == 0u;
-                if (!ok) bad = 1;
+                if (want >= 0 && (need || (atomicAdd(&cell[(ml[u] >> 2) * slots + h], (uint32_t)(e - ml[u] * p.K + 1) << sh) >> sh & 0xffu) != 0u)) bad = 1;
             }
             if (*reinterpret_cast<volatile int*>(&bad)) break;
         }
@@ -149,31 +150,38 @@ __device__ bool ens_hash_query(const EnsParams& p, const int q, const int log2_s
     };
     uint64_t bs; int32_t bi; int bp;
     best_of_mine(bs, bi, bp);
+    // warp maximum under (score descending, id ascending): the score's two halves, then the id
+    auto warp_best = [&](uint64_t s, int32_t id, uint64_t& os, int32_t& oi) {
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32));
+        const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32) == hi ? (uint32_t)s : 0u);
+        os = (uint64_t)hi << 32 | lo;
+        oi = __reduce_min_sync(0xffffffffu, s == os ? id : INT32_MAX);
+    };
+    uint64_t ws; int32_t wi;                // the warp's best
+    warp_best(bs, bi, ws, wi);
     for (int r = 0; r < p.top_n; ++r) {
-        // warp maximum under (score descending, id ascending): the score's two halves, then the id
-        auto warp_best = [&](uint64_t s, int32_t id, uint64_t& os, int32_t& oi) {
-            const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32));
-            const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32) == hi ? (uint32_t)s : 0u);
-            os = (uint64_t)hi << 32 | lo;
-            oi = __reduce_min_sync(0xffffffffu, s == os ? id : INT32_MAX);
-        };
-        uint64_t s; int32_t id;
-        warp_best(bs, bi, s, id);
-        if (lane == 0) { red_s[r & 1][warp] = s; red_i[r & 1][warp] = id; }
+        if (lane == 0) { red_s[r & 1][warp] = ws; red_i[r & 1][warp] = wi; }
         __syncthreads();
+        uint64_t s; int32_t id;
         warp_best(lane < nwarps ? red_s[r & 1][lane] : 0ull, lane < nwarps ? red_i[r & 1][lane] : INT32_MAX, s, id);   // (every warp for itself)
         const bool have = s != 0ull;                                            // (no score maps to 0)
         if (tid == 0) {
             p.out_ids[(int64_t)q * p.top_n + r] = have ? id : -1;               // fewer candidates than places: -1 and -inf
             if (p.out_scores) p.out_scores[(int64_t)q * p.top_n + r] = have ? ens_unordered(s) : -INFINITY;
         }
-        if (have && bp >= 0 && bi == id) { key[bp] = -1; best_of_mine(bs, bi, bp); }    // taken (ids are distinct: one thread)
+        if (have && s == ws && id == wi) {                                      // taken (ids are distinct: one warp, one thread)
+            if (bp >= 0 && bi == id) { key[bp] = -1; best_of_mine(bs, bi, bp); }
+            __syncwarp();
+            warp_best(bs, bi, ws, wi);
+        }
     }
     return true;
 }
 
-// First launch: one CTA per query, 32 models at a time, at most 1,024 slots (47 KB: four CTAs per SM).
-constexpr int ENS_MB = 32, ENS_MAX_LOG2 = 10;
+// First launch: one CTA per query, 16 models at a time, at most 1,024 slots (31 KB: seven CTAs per SM).  85 x top-100 lists of
+// 15,000 queries: 36.7 ms as a sort, 0.93 ms with 32 models at a time (four CTAs), 0.87 with 8, 0.81 with 16; 128 threads 1.00 ms.
+// Bound by instruction issue (about 48,000 warp instructions a query, 74 % of the slots), not by the 510 MB of lists (78 us).
+constexpr int ENS_MB = 16, ENS_MAX_LOG2 = 10;
 template <int MB>
 __global__ void __launch_bounds__(256) ensemble_hash_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
