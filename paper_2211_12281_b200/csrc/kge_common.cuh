@@ -242,7 +242,7 @@ int encoder_make_maps(kge_handle* h);
 int launch_encoder_forward(kge_handle* h, const int32_t* heads, const int32_t* tails, const int32_t* negs, cudaStream_t s);
 int launch_encoder_backward(kge_handle* h, uint64_t step, float lr, cudaStream_t s);
 int launch_cast_bf16(kge_handle* h, const float* src, uint16_t* dst, int64_t count, cudaStream_t s);
-int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, cudaStream_t s);
+int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, int first, cudaStream_t s);
 int dedup_tiles(int n);     // sort tiles of a list of n ids
 // On-device graph preprocessing and table initialisation (kge_graph.cu).
 size_t graph_hist_words(int64_t num_triples);

@@ -12,7 +12,6 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
-#include <vector>
 
 #include <cuda_bf16.h>
 
@@ -38,7 +37,11 @@ struct InferParams {
     const float* ext_q;            // [nq, d] finished query vectors, or NULL: build them from qh, qr
     const float* ext_ftrue;        // [nq] scores of the true tails, or NULL: score them here
     int raw_beat;                  // out_ranks receives the shard's count of entities ordered before the true tail, not 1 + count
-    Workspace w;
+    const uint16_t* Eb;            // tensor-core arithmetic: the bf16 copy of the table (the true tail is scored from it), or NULL
+    int first;                     // first chunk: nothing is filtered, the scores go to the candidate lists in entity order
+    int last;                      // last chunk: its selection writes the outputs
+    int32_t* out_ids; float* out_scores; int32_t* out_ranks;
+    Workspace w;                   // status[1]: a candidate list overflowed (nothing further of this call runs), status[6]: entities done
 };
 
 // One canonical accumulation step over the 4 floats of a slice.
@@ -155,27 +158,89 @@ __device__ __forceinline__ float score_seq(const InferParams& p, const float* qv
     }
 }
 
-__global__ void query_setup_kernel(InferParams p) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per query (one thread per query read every row element by element: 105 us for 128 queries of width 256, 51 us
+// for 15,000 of width 128).  The lanes fetch the rows and form what is independent per coordinate; a sum whose order is
+// canonical runs on one lane, over rows in shared memory.
+constexpr int SETUP_WARPS = 4;
+__global__ void __launch_bounds__(32 * SETUP_WARPS) query_setup_kernel(InferParams p) {
+    __shared__ __align__(16) float rows[SETUP_WARPS][3][kMaxDim];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = blockIdx.x * SETUP_WARPS + warp;
+    allow_dependents();
+    if (blockIdx.x == 0 && threadIdx.x == 0) { p.w.status[1] = 0; p.w.status[6] = 0; }
     if (q >= p.nq) return;
     const int d = p.d;
+    const bool th = p.score == KGE_TRANSH;
+    float *qv = rows[warp][0], *wh = rows[warp][1], *tv = rows[warp][2];
     const int64_t rid = checked_id(p.qr[q], p.R, p.w.status);
-    float* qv = p.w.iq + (int64_t)q * d;
-    float* wh = p.score == KGE_TRANSH ? p.w.iwhat + (int64_t)q * d : nullptr;
-    if (p.ext_q) {   // sharded: the query vector was built by the shard that holds the head
-        for (int k = 0; k < d; ++k) qv[k] = p.ext_q[(int64_t)q * d + k];
-        if (wh) unit_normal_seq(p, rid, wh);
-    } else {
-        build_query_seq(p, p.ent + checked_id(p.qh[q], p.E, p.w.status) * d, rid, qv, wh);
+    if (th) {
+        const float* wrow = p.relw + rid * d;
+        for (int k = lane; k < d; k += 32) wh[k] = wrow[k];
+        __syncwarp();
+        float s = 0.f;
+        if (lane == 0) for (int k = 0; k < d; ++k) s = __fmaf_rn(wh[k], wh[k], s);
+        const float den = fmaxf(__fsqrt_rn(__shfl_sync(0xffffffffu, s, 0)), 1e-12f);
+        for (int k = lane; k < d; k += 32) wh[k] = __fdiv_rn(wh[k], den);
+        __syncwarp();
     }
-    if (p.ext_ftrue) p.w.iftrue[q] = p.ext_ftrue[q];
-    else if (p.tt) p.w.iftrue[q] = score_seq(p, qv, wh, p.ent + checked_id(p.tt[q], p.E, p.w.status) * d);
-    for (int j = 0; j < p.k; ++j) {
+    if (p.ext_q) {   // sharded: the query vector was built by the shard that holds the head
+        for (int k = lane; k < d; k += 32) qv[k] = p.ext_q[(int64_t)q * d + k];
+    } else {
+        const float* h = p.ent + checked_id(p.qh[q], p.E, p.w.status) * d;
+        if (p.score == KGE_TRANSE || p.score == KGE_DISTMULT) {
+            const float* r = p.rel + rid * d;
+            for (int k = lane; k < d; k += 32) qv[k] = p.score == KGE_TRANSE ? __fadd_rn(h[k], r[k]) : __fmul_rn(r[k], h[k]);
+        } else if (p.score == KGE_COMPLEX) {
+            const float* r = p.rel + rid * d;
+            for (int k = 2 * lane; k < d; k += 64) {
+                qv[k] = __fmaf_rn(r[k], h[k], -__fmul_rn(r[k + 1], h[k + 1]));
+                qv[k + 1] = __fmaf_rn(r[k], h[k + 1], __fmul_rn(r[k + 1], h[k]));
+            }
+        } else if (p.score == KGE_ROTATE) {
+            const float* ph = p.rel + rid * (d / 2);
+            for (int k = 2 * lane; k < d; k += 64) {
+                const float cs = cosf(ph[k / 2]), sn = sinf(ph[k / 2]);
+                qv[k] = __fmaf_rn(h[k], cs, -__fmul_rn(h[k + 1], sn));
+                qv[k + 1] = __fmaf_rn(h[k], sn, __fmul_rn(h[k + 1], cs));
+            }
+        } else {  // TransH
+            const float* r = p.rel + rid * d;
+            for (int k = lane; k < d; k += 32) tv[k] = h[k];
+            __syncwarp();
+            float a = 0.f;
+            if (lane == 0) for (int k = 0; k < d; ++k) a = __fmaf_rn(wh[k], tv[k], a);
+            a = __shfl_sync(0xffffffffu, a, 0);
+            for (int k = lane; k < d; k += 32) qv[k] = __fadd_rn(__fmaf_rn(-a, wh[k], tv[k]), r[k]);
+        }
+    }
+    __syncwarp();
+    for (int k = lane; k < d; k += 32) {
+        p.w.iq[(int64_t)q * d + k] = qv[k];
+        if (th) p.w.iwhat[(int64_t)q * d + k] = wh[k];
+        if (p.Eb) p.w.iqb[(int64_t)q * d + k] = __bfloat16_as_ushort(__float2bfloat16_rn(qv[k]));
+    }
+    if (p.ext_ftrue) {
+        if (lane == 0) p.w.iftrue[q] = p.ext_ftrue[q];
+    } else if (p.tt) {
+        const int64_t tid = checked_id(p.tt[q], p.E, p.w.status);
+        if (p.Eb) {   // the arithmetic of the tensor-core path: operands rounded to bf16, fp32 accumulation
+            const uint16_t* t = p.Eb + tid * d;
+            for (int k = lane; k < d; k += 32) { tv[k] = __uint_as_float((uint32_t)t[k] << 16); qv[k] = __bfloat162float(__float2bfloat16_rn(qv[k])); }
+        } else {
+            const float* t = p.ent + tid * d;
+            for (int k = lane; k < d; k += 32) tv[k] = t[k];
+        }
+        __syncwarp();
+        if (lane == 0) p.w.iftrue[q] = score_seq(p, qv, wh, tv);
+    }
+    for (int j = lane; j < p.k; j += 32) {
         p.w.top_score[(int64_t)q * p.k + j] = -INFINITY;
         p.w.top_id[(int64_t)q * p.k + j] = INT_MAX;
     }
-    p.w.thr[q] = -INFINITY; p.w.thr_id[q] = INT_MAX;
-    p.w.cand_cnt[q] = 0; p.w.beat_tmp[q] = 0; p.w.beat[q] = 0;
+    if (lane == 0) {
+        p.w.thr[q] = -INFINITY; p.w.thr_id[q] = INT_MAX;
+        p.w.cand_cnt[q] = 0; p.w.beat_tmp[q] = 0; p.w.beat[q] = 0;
+    }
 }
 
 constexpr int IQ = 64, IE = 64, IKC = 32, ILD = IKC + 4;
@@ -222,6 +287,7 @@ __device__ __forceinline__ void score_tile_epilogue(const InferParams& p, const 
                                                     const float4* cuts = nullptr) {
     const int64_t g0 = e0 + p.id_base;                  // the id the caller knows the tile's first entity by
     const bool whole = e0 + IE <= p.e_hi;
+    const bool first = p.first != 0;
     int beat_all = 0;                                   // four rows' counts, one byte each (at most 4 per thread, 64 per row)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -289,7 +355,8 @@ __device__ __forceinline__ void score_tile_epilogue(const InferParams& p, const 
                 const float f = canon_finish(KIND, acc[i][j]);
                 const int32_t ge = (int32_t)(e + p.id_base);
                 if (p.tt && ordered_before(f, ge, ft, tt)) ++beat;
-                if (ordered_before(f, ge, thr, thr_id)) append(f, ge);
+                if (first) p.w.cand_score[(int64_t)q * kCandCap + (e - p.e_lo)] = f;
+                else if (ordered_before(f, ge, thr, thr_id)) append(f, ge);
             }
         }
         beat_all |= beat << (8 * i);
@@ -328,6 +395,10 @@ __global__ void __launch_bounds__(256) score_tile_kernel(InferParams p) {
     const float4* Tg = reinterpret_cast<const float4*>(p.ent);
 
     __shared__ float4 cuts[IQ];
+    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
+    grid_dependency_wait();
+    allow_dependents();
+    if (tid == 0) skip = p.w.status[1];
     if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barriers of the loop below)
     float acc[4][4], u[4][4];
 #pragma unroll
@@ -354,6 +425,7 @@ __global__ void __launch_bounds__(256) score_tile_kernel(InferParams p) {
                 if (TH) *reinterpret_cast<float4*>(&Ws[row * ILD + c4 * 4]) = wv;
             }
             __syncthreads();
+            if (skip) return;
 #pragma unroll
             for (int kk = 0; kk < IKC; kk += 4) {
                 float4 qv[4], tv[4], wv[4];
@@ -384,62 +456,48 @@ __global__ void __launch_bounds__(256) score_tile_kernel(InferParams p) {
 }
 
 // ------------------------------------------------------------------------------------------
-// score tile, kinds that are a function of (q, t) alone: the same 64 x 64 tile and the same
-// operation order (one accumulator per pair, coordinates ascending), but the 64 query rows and
-// 64 entity rows arrive by one asynchronous bulk copy per row into padded shared-memory rows (up
-// to 128 coordinates per stage, two stages for longer rows), so a CTA waits once per stage instead
-// of loading and synchronising every 32 coordinates.
+// score tile, kinds that are a function of (q, t) alone, rows of fewer than 32 floats: the same 64 x 64 tile
+// and the same operation order (one accumulator per pair, coordinates ascending), but the 64 query
+// rows and 64 entity rows arrive by one asynchronous bulk copy per row into padded shared-memory
+// rows, so a CTA waits once instead of loading and synchronising every 32 coordinates.
 // ------------------------------------------------------------------------------------------
-constexpr int IKT = 128;
-__host__ __device__ inline int infer_tma_kc(int d) { return d < IKT ? d : IKT; }
-__host__ __device__ inline int infer_tma_stages(int d) { return d > IKT ? 2 : 1; }
-inline size_t infer_tma_smem(int d) {
-    return (size_t)infer_tma_stages(d) * (IQ + IE) * (infer_tma_kc(d) + 4) * sizeof(float) + 2 * sizeof(uint64_t);
-}
+constexpr int ITENSOR_MIN_D = 32;          // rows from here on are staged by tensor copies (below)
+inline size_t infer_tma_smem(int d) { return (size_t)(IQ + IE) * (d + 4) * sizeof(float) + sizeof(uint64_t); }
 
-// KC: the stage length when known at compile time (rows of at least IKT floats; shared-memory
-// addresses of the inner loop are then constants off one base per operand), 0: shorter rows.
-template <int KIND, int KC>
+template <int KIND>
 __global__ void __launch_bounds__(256) score_tile_tma_kernel(InferParams p) {
     extern __shared__ __align__(128) unsigned char smraw[];
-    constexpr int ROWS = IQ + IE;        // rows [0, IQ) of a stage hold queries, the rest entities
-    const int kc = KC ? KC : infer_tma_kc(p.d), ld = kc + 4, nstage = infer_tma_stages(p.d);
-    const int nchunk = (p.d + kc - 1) / kc;
+    constexpr int ROWS = IQ + IE;        // rows [0, IQ) hold queries, the rest entities
+    const int ld = p.d + 4;
     float* base = reinterpret_cast<float*>(smraw);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smraw + (size_t)nstage * ROWS * ld * sizeof(float));
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + (size_t)ROWS * ld * sizeof(float));
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int qt = blockIdx.x % p.q_tiles;
     const int64_t et = blockIdx.x / p.q_tiles;
     const int q0 = qt * IQ;
     const int64_t e0 = p.e_lo + et * IE;
 
-    if (tid == 0) {
-        for (int st = 0; st < nstage; ++st) mbar_init(&bars[st], ROWS);
-        mbar_init_fence();
-    }
+    if (tid == 0) { mbar_init(bar, ROWS); mbar_init_fence(); }
     __syncthreads();
-
-    auto issue = [&](int chunk, int stage) {     // thread r < ROWS owns row r of the stage
-        if (tid >= ROWS) return;
+    grid_dependency_wait();
+    allow_dependents();
+    if (tid < ROWS) {                            // thread r owns row r
         const bool isq = tid < IQ;
         const int64_t g = isq ? q0 + tid : e0 + (tid - IQ);
         const bool in = isq ? g < p.nq : g < p.e_hi;
-        float* dst = base + ((size_t)stage * ROWS + tid) * ld;
-        const int k0 = chunk * kc, len = min(kc, p.d - k0);
+        float* dst = base + (size_t)tid * ld;
         if (in) {
-            const float* src = (isq ? p.w.iq : p.ent) + g * p.d + k0;
-            mbar_arrive_expect_tx(&bars[stage], (uint32_t)len * 4u);
-            bulk_g2s(dst, src, (uint32_t)len * 4u, &bars[stage]);
+            mbar_arrive_expect_tx(bar, (uint32_t)p.d * 4u);
+            bulk_g2s(dst, (isq ? p.w.iq : p.ent) + g * p.d, (uint32_t)p.d * 4u, bar);
         } else {
-            if (chunk < nstage)   // rows outside the problem stay zero for the whole kernel
-                for (int k = 0; k < kc; k += 4) *reinterpret_cast<float4*>(dst + k) = make_float4(0.f, 0.f, 0.f, 0.f);
-            mbar_arrive(&bars[stage]);
+            for (int k = 0; k < p.d; k += 4) *reinterpret_cast<float4*>(dst + k) = make_float4(0.f, 0.f, 0.f, 0.f);
+            mbar_arrive(bar);
         }
-    };
-    issue(0, 0);
-    if (nstage > 1 && nchunk > 1) issue(1, 1);
+    }
     __shared__ float4 cuts[IQ];
-    if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barrier that follows the first wait)
+    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
+    if (tid == 128) skip = p.w.status[1];
+    if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barrier that follows the wait)
 
     float acc[4][4];
 #pragma unroll
@@ -447,55 +505,81 @@ __global__ void __launch_bounds__(256) score_tile_tma_kernel(InferParams p) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 
-    for (int chunk = 0; chunk < nchunk; ++chunk) {
-        const int stage = chunk % nstage;
-        const bool ok = mbar_wait_bounded(&bars[stage], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
-        if (!__syncthreads_and(ok)) {
-            if (tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
-            // give copies still in flight a bounded chance to land before shared memory is released
-            for (int st = 0; st < nstage; ++st) (void)mbar_wait_bounded(&bars[st], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
-            return;
-        }
-        const float* Qs = base + (size_t)stage * ROWS * ld;
-        const float* Ts = Qs + IQ * ld;
-        const int len = min(kc, p.d - chunk * kc);
+    const bool ok = mbar_wait_bounded(bar, 0u, p.wait_limit);
+    if (!__syncthreads_and(ok)) {
+        if (tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
+        // give copies still in flight a bounded chance to land before shared memory is released
+        (void)mbar_wait_bounded(bar, 0u, p.wait_limit);
+        return;
+    }
+    if (skip) return;
+    const float* Qs = base;
+    const float* Ts = Qs + IQ * ld;
 #pragma unroll 2
-        for (int kk = 0; kk < len; kk += 4) {
-            float4 qv[4], tv[4];
+    for (int kk = 0; kk < p.d; kk += 4) {
+        float4 qv[4], tv[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                qv[i] = *reinterpret_cast<const float4*>(&Qs[(ty + 16 * i) * ld + kk]);
-                tv[i] = *reinterpret_cast<const float4*>(&Ts[(tx + 16 * i) * ld + kk]);
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) canon_update<KIND>(acc[i][j], qv[i], tv[j]);
+        for (int i = 0; i < 4; ++i) {
+            qv[i] = *reinterpret_cast<const float4*>(&Qs[(ty + 16 * i) * ld + kk]);
+            tv[i] = *reinterpret_cast<const float4*>(&Ts[(tx + 16 * i) * ld + kk]);
         }
-        if (chunk + nstage < nchunk) {
-            __syncthreads();             // every thread is done reading this stage
-            issue(chunk + nstage, stage);
-        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) canon_update<KIND>(acc[i][j], qv[i], tv[j]);
     }
     score_tile_epilogue<KIND>(p, acc, q0, e0, tx, ty, cuts);
 }
 
 // ------------------------------------------------------------------------------------------
-// The same score tile for rows of at least 128 floats, staged by the TMA engine's tensor copies:
-// eight copies per stage (four 64-row x 32-float boxes of the queries, four of the entities, 128-byte
-// swizzle) issued by one thread, instead of one bulk copy per row issued lane by lane (128 per
-// tile, about 5 % of the kernel's instructions).  A box holds a row's 32 floats as eight 16-byte
-// units, unit u of row r at position u ^ (r & 7): a thread's rows all share r & 7, so its eight
-// unit offsets are computed once and every 128-bit read is base + constant + one of them, without
-// bank conflicts.  What a box covers beyond the matrix reads as zero, and adding the term of a
-// zero pair leaves every accumulator as it is, so ragged rows keep the canonical order and value.
+// The same score tile for rows of at least 32 floats, staged by the TMA engine's tensor copies: four
+// copies per stage of 64 coordinates (two 64-row x 32-float boxes of the queries, two of the entities,
+// 128-byte swizzle) issued by one thread.  A box holds a row's 32 floats as eight 16-byte units, unit
+// u of row r at position u ^ (r & 7): a thread's rows all share r & 7, so its eight unit offsets are
+// computed once and every 128-bit read is base + constant + one of them, without bank conflicts.
+// Two stages of 32 KB whatever the row length, so that three CTAs share an SM: with stages of 128
+// coordinates, rows of more than 128 floats left one CTA per SM (0.67 of the instruction rate).
+//
+// Bound: the FMA pipe (L1: one subtraction and one addition per element).  The differences of two
+// coordinates are one packed subtraction (the same rounding, one issue slot for two): a packed
+// instruction holds the pipe for two cycles and adds no arithmetic rate, but leaves issue slots for
+// the shared-memory reads, which otherwise take 8 of every 136.
 // ------------------------------------------------------------------------------------------
-constexpr int ITB_BOX_BYTES = 64 * 128, ITB_CHUNK_BYTES = 4 * ITB_BOX_BYTES, ITB_STAGE_BYTES = 2 * ITB_CHUNK_BYTES;
-inline size_t infer_tensor_smem(int d) { return 1024 + (size_t)infer_tma_stages(d) * ITB_STAGE_BYTES + 2 * sizeof(uint64_t); }
+constexpr int ITB_KC = 64;
+constexpr int ITB_BOX_BYTES = 64 * 128, ITB_CHUNK_BYTES = 2 * ITB_BOX_BYTES, ITB_STAGE_BYTES = 2 * ITB_CHUNK_BYTES;
+__host__ __device__ inline int infer_tensor_stages(int d) { return d > ITB_KC ? 2 : 1; }
+inline size_t infer_tensor_smem(int d) { return 1024 + (size_t)infer_tensor_stages(d) * ITB_STAGE_BYTES + 2 * sizeof(uint64_t); }
 __device__ __forceinline__ void tile_load_2d(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(dst)), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
+}
+
+// Two differences in one instruction, each rounded as a single subtraction would be.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    uint64_t x, y, d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
+}
+// canon_update with the subtractions of neighbouring coordinates packed.
+template <int KIND>
+__device__ __forceinline__ void canon_update_packed(float& acc, float4 q, float4 t) {
+    if (KIND == KIND_DOT) { canon_update<KIND>(acc, q, t); return; }
+    const float2 a = sub2(make_float2(q.x, q.y), make_float2(t.x, t.y)), b = sub2(make_float2(q.z, q.w), make_float2(t.z, t.w));
+    if (KIND == KIND_L1) {
+        acc = __fadd_rn(acc, fabsf(a.x)); acc = __fadd_rn(acc, fabsf(a.y));
+        acc = __fadd_rn(acc, fabsf(b.x)); acc = __fadd_rn(acc, fabsf(b.y));
+    } else if (KIND == KIND_L2) {
+        acc = __fmaf_rn(a.x, a.x, acc); acc = __fmaf_rn(a.y, a.y, acc);
+        acc = __fmaf_rn(b.x, b.x, acc); acc = __fmaf_rn(b.y, b.y, acc);
+    } else {  // KIND_CL1
+        acc = __fadd_rn(acc, __fsqrt_rn(__fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y))));
+        acc = __fadd_rn(acc, __fsqrt_rn(__fmaf_rn(b.x, b.x, __fmul_rn(b.y, b.y))));
+    }
 }
 
 template <int KIND>
@@ -503,8 +587,8 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
                                                                    InferParams p) {
     extern __shared__ unsigned char smraw_t[];
     unsigned char* base = smraw_t + ((1024u - (smem_u32(smraw_t) & 1023u)) & 1023u);       // swizzled boxes want 1024-byte alignment
-    const int nstage = infer_tma_stages(p.d);
-    const int nchunk = (p.d + IKT - 1) / IKT;
+    const int nstage = infer_tensor_stages(p.d);
+    const int nchunk = (p.d + ITB_KC - 1) / ITB_KC;
     uint64_t* bars = reinterpret_cast<uint64_t*>(base + (size_t)nstage * ITB_STAGE_BYTES);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int qt = blockIdx.x % p.q_tiles;
@@ -517,19 +601,26 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
         mbar_init_fence();
     }
     __syncthreads();
-    auto issue = [&](int chunk, int stage) {
+    grid_dependency_wait();
+    allow_dependents();
+    auto issue = [&](int chunk, int stage) {     // (a box that begins beyond the row is left out)
         if (tid != 0) return;
         unsigned char* qs = base + (size_t)stage * ITB_STAGE_BYTES;
-        mbar_arrive_expect_tx(&bars[stage], (uint32_t)ITB_STAGE_BYTES);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            tile_load_2d(qs + b * ITB_BOX_BYTES, &tmQ, chunk * IKT + 32 * b, q0, &bars[stage]);
-            tile_load_2d(qs + ITB_CHUNK_BYTES + b * ITB_BOX_BYTES, &tmE, chunk * IKT + 32 * b, (int)e0, &bars[stage]);
+        const int x = chunk * ITB_KC;
+        const bool two = x + 32 < p.d;
+        mbar_arrive_expect_tx(&bars[stage], (uint32_t)(two ? ITB_STAGE_BYTES : ITB_STAGE_BYTES / 2));
+        tile_load_2d(qs, &tmQ, x, q0, &bars[stage]);
+        tile_load_2d(qs + ITB_CHUNK_BYTES, &tmE, x, (int)e0, &bars[stage]);
+        if (two) {
+            tile_load_2d(qs + ITB_BOX_BYTES, &tmQ, x + 32, q0, &bars[stage]);
+            tile_load_2d(qs + ITB_CHUNK_BYTES + ITB_BOX_BYTES, &tmE, x + 32, (int)e0, &bars[stage]);
         }
     };
     issue(0, 0);
-    if (nstage > 1 && nchunk > 1) issue(1, 1);
+    if (nchunk > 1) issue(1, 1);
     __shared__ float4 cuts[IQ];
+    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
+    if (tid == 128) skip = p.w.status[1];
     if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barrier that follows the first wait)
 
     float acc[4][4];
@@ -544,31 +635,36 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
     for (int chunk = 0; chunk < nchunk; ++chunk) {
         const int stage = chunk % nstage;
         const bool ok = mbar_wait_bounded(&bars[stage], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
-        if (!__syncthreads_and(ok)) {
-            if (tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
-            for (int st = 0; st < nstage; ++st) (void)mbar_wait_bounded(&bars[st], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
+        const bool all = __syncthreads_and(ok);
+        if (!all || skip) {
+            if (!all && tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
+            for (int st = 0; st < min(nstage, nchunk); ++st) (void)mbar_wait_bounded(&bars[st], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
             return;
         }
         const unsigned char* qrow = base + (size_t)stage * ITB_STAGE_BYTES + ty * 128;
         const unsigned char* trow = base + (size_t)stage * ITB_STAGE_BYTES + ITB_CHUNK_BYTES + tx * 128;
-        const int nbox = (min(IKT, p.d - chunk * IKT) + 31) / 32;
-#pragma unroll 1
-        for (int b = 0; b < nbox; ++b) {
-            const unsigned char* qb = qrow + b * ITB_BOX_BYTES;
-            const unsigned char* tb = trow + b * ITB_BOX_BYTES;
+        const int len = min(ITB_KC, p.d - chunk * ITB_KC);
+        auto unit = [&](const unsigned char* qb, const unsigned char* tb) {      // four coordinates of the 4 x 4 pairs
+            float4 qv[4], tv[4];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                float4 qv[4], tv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    qv[i] = *reinterpret_cast<const float4*>(qb + i * (16 * 128) + qoff[u]);
-                    tv[i] = *reinterpret_cast<const float4*>(tb + i * (16 * 128) + toff[u]);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) canon_update<KIND>(acc[i][j], qv[i], tv[j]);
+            for (int i = 0; i < 4; ++i) {
+                qv[i] = *reinterpret_cast<const float4*>(qb + i * (16 * 128));
+                tv[i] = *reinterpret_cast<const float4*>(tb + i * (16 * 128));
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) canon_update_packed<KIND>(acc[i][j], qv[i], tv[j]);
+        };
+#pragma unroll 1
+        for (int b = 0; b < len / 32; ++b) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) unit(qrow + b * ITB_BOX_BYTES + qoff[u], trow + b * ITB_BOX_BYTES + toff[u]);
+        }
+        if (len % 32 != 0) {             // the row ends inside a box
+            const int at = (len / 32) * ITB_BOX_BYTES;
+#pragma unroll 1
+            for (int u = 0; u < (len % 32) / 4; ++u) unit(qrow + at + ((u ^ (ty & 7)) << 4), trow + at + ((u ^ (tx & 7)) << 4));
         }
         if (chunk + nstage < nchunk) {
             __syncthreads();             // every thread is done reading this stage
@@ -585,81 +681,126 @@ cudaError_t launch_score_tile_tensor(const kge_handle* h, const InferParams& p, 
         return cudaFuncSetAttribute(score_tile_tensor_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)infer_tensor_smem(kMaxDim));
     });
     if (e != cudaSuccess) return e;
-    score_tile_tensor_kernel<KIND><<<grid, 256, infer_tensor_smem(p.d), s>>>(*reinterpret_cast<const CUtensorMap*>(h->tm_iq32),
-                                                                            *reinterpret_cast<const CUtensorMap*>(h->tm_ent32), p);
-    return cudaSuccess;
+    return launch_dependent(score_tile_tensor_kernel<KIND>, dim3(grid), dim3(256), infer_tensor_smem(p.d), s,
+                            *reinterpret_cast<const CUtensorMap*>(h->tm_iq32), *reinterpret_cast<const CUtensorMap*>(h->tm_ent32), p);
 }
 
 template <int KIND>
 cudaError_t launch_score_tile_tma(const InferParams& p, unsigned grid, cudaStream_t s) {
-    static DeviceOnce configured;
-    const cudaError_t e = once_per_device(configured, [] {
-        const cudaError_t e0 = cudaFuncSetAttribute(score_tile_tma_kernel<KIND, IKT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)infer_tma_smem(kMaxDim));
-        return e0 != cudaSuccess ? e0 : cudaFuncSetAttribute(score_tile_tma_kernel<KIND, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)infer_tma_smem(IKT));
-    });
-    if (e != cudaSuccess) return e;
-    if (p.d >= IKT) score_tile_tma_kernel<KIND, IKT><<<grid, 256, infer_tma_smem(p.d), s>>>(p);
-    else score_tile_tma_kernel<KIND, 0><<<grid, 256, infer_tma_smem(p.d), s>>>(p);
-    return cudaSuccess;
+    return launch_dependent(score_tile_tma_kernel<KIND>, dim3(grid), dim3(256), infer_tma_smem(p.d), s, p);
 }
 
 // ------------------------------------------------------------------------------------------
 // select: one CTA per query merges the running top-k with this chunk's candidates by a
 // bitonic sort in shared memory under (score descending, id ascending), commits the chunk's
-// rank count and resets the candidate list.
+// rank count and resets the candidate list; after the last chunk it writes the outputs.
+//
+// A long list (the first chunk's 1,024 unfiltered scores) is cut down first: each of the 128 threads
+// takes the best of its share, and the k-th best of those 128 is a lower bound of the k-th best of
+// all, so only what reaches it is sorted (k = 10: some 13 of 1,024 instead of a sort of 2,048 places,
+// 1,435 us for 15,000 queries).  Up to 64 entries are sorted by one warp without CTA-wide barriers.
 // ------------------------------------------------------------------------------------------
 constexpr int SEL_THREADS = 128;
 constexpr int SEL_MAX = 2 * kCandCap;   // k <= kCandCap plus at most kCandCap candidates
+constexpr int SEL_CUT_MIN = 192;        // candidates from which the cut pays
 
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(InferParams p) {
     __shared__ float ss[SEL_MAX];
     __shared__ int32_t si[SEL_MAX];
+    __shared__ __align__(16) float best[SEL_THREADS];
+    __shared__ float cut_sm;
+    __shared__ int kept;
     const int q = blockIdx.x, tid = threadIdx.x;
-    const int cnt = min(p.w.cand_cnt[q], kCandCap);
-    const int total = p.k + cnt;
-    int n2 = 1;
-    while (n2 < total) n2 <<= 1;
-    for (int i = tid; i < n2; i += SEL_THREADS) {
-        float s = -INFINITY; int32_t id = INT_MAX;
-        if (i < p.k) { s = p.w.top_score[(int64_t)q * p.k + i]; id = p.w.top_id[(int64_t)q * p.k + i]; }
-        else if (i < total) { s = p.w.cand_score[(int64_t)q * kCandCap + i - p.k]; id = p.w.cand_id[(int64_t)q * kCandCap + i - p.k]; }
-        ss[i] = s; si[i] = id;
-    }
-    __syncthreads();
-    for (int size = 2; size <= n2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < n2 / 2; t += SEL_THREADS) {
-                const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
-                const bool up = (lo & size) == 0;   // "up" blocks end with the best element first
-                const float a = ss[lo], b = ss[hi]; const int32_t ia = si[lo], ib = si[hi];
-                const bool b_first = ordered_before(b, ib, a, ia);
-                if (b_first == up) { ss[lo] = b; si[lo] = ib; ss[hi] = a; si[hi] = ia; }
-            }
-            __syncthreads();
+    grid_dependency_wait();
+    allow_dependents();
+    if (p.w.status[1]) return;              // (nothing in flight writes it)
+    const int cnt = p.first ? (int)(p.e_hi - p.e_lo) : min(p.w.cand_cnt[q], kCandCap);
+    const float* cs = p.w.cand_score + (int64_t)q * kCandCap;
+    const int32_t* ci = p.w.cand_id + (int64_t)q * kCandCap;
+    const int32_t first_id = (int32_t)(p.e_lo + p.id_base);
+    auto candidate = [&](int i, float& s, int32_t& id) {
+        s = cs[i];
+        id = p.first ? first_id + i : ci[i];
+        // never candidates: what is not a number and, in the tensor-core arithmetic, -inf
+        if (p.first && (!(s == s) || (p.Eb && s == -INFINITY))) { s = -INFINITY; id = INT_MAX; }
+    };
+    const int run = p.first ? 0 : p.k;      // before the first chunk the running list is empty
+    int total = run + cnt;
+    const bool cut = cnt >= SEL_CUT_MIN && p.k <= SEL_THREADS;
+    for (int i = tid; i < run; i += SEL_THREADS) { ss[i] = p.w.top_score[(int64_t)q * p.k + i]; si[i] = p.w.top_id[(int64_t)q * p.k + i]; }
+    if (cut) {
+        constexpr int PER = kCandCap / SEL_THREADS;
+        float v[PER]; int32_t id[PER];
+        float b = -INFINITY;
+        if (tid == 0) { kept = 0; cut_sm = -INFINITY; }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            v[i] = -INFINITY; id[i] = INT_MAX;
+            if (tid + i * SEL_THREADS < cnt) candidate(tid + i * SEL_THREADS, v[i], id[i]);
+            b = fmaxf(b, v[i]);
         }
+        best[tid] = b;
+        __syncthreads();
+        int rank = 0;                       // threads whose best comes before mine
+#pragma unroll 8
+        for (int j = 0; j < SEL_THREADS; j += 4) {
+            const float4 o = *reinterpret_cast<const float4*>(&best[j]);
+            rank += (o.x > b || (o.x == b && j < tid)) + (o.y > b || (o.y == b && j + 1 < tid)) + (o.z > b || (o.z == b && j + 2 < tid)) + (o.w > b || (o.w == b && j + 3 < tid));
+        }
+        if (rank == p.k - 1) cut_sm = b;
+        __syncthreads();
+        const float c = cut_sm;
+#pragma unroll
+        for (int i = 0; i < PER; ++i)
+            if (tid + i * SEL_THREADS < cnt && v[i] >= c) { const int at = run + atomicAdd(&kept, 1); ss[at] = v[i]; si[at] = id[i]; }
+        __syncthreads();
+        total = run + kept;
+    } else {
+        for (int i = tid; i < cnt; i += SEL_THREADS) { float s; int32_t id; candidate(i, s, id); ss[run + i] = s; si[run + i] = id; }
+    }
+    int n2 = 1;
+    while (n2 < total || n2 < p.k) n2 <<= 1;
+    for (int i = total + tid; i < n2; i += SEL_THREADS) { ss[i] = -INFINITY; si[i] = INT_MAX; }
+    __syncthreads();
+    auto exchange = [&](int t, int size, int stride) {
+        const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
+        const bool up = (lo & size) == 0;   // "up" blocks end with the best element first
+        const float a = ss[lo], b = ss[hi]; const int32_t ia = si[lo], ib = si[hi];
+        const bool b_first = ordered_before(b, ib, a, ia);
+        if (b_first == up) { ss[lo] = b; si[lo] = ib; ss[hi] = a; si[hi] = ia; }
+    };
+    if (n2 <= 64) {
+        if (tid < 32) {
+            for (int size = 2; size <= n2; size <<= 1)
+                for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                    if (tid < n2 / 2) exchange(tid, size, stride);
+                    __syncwarp();
+                }
+        }
+        __syncthreads();
+    } else {
+        for (int size = 2; size <= n2; size <<= 1)
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                for (int t = tid; t < n2 / 2; t += SEL_THREADS) exchange(t, size, stride);
+                __syncthreads();
+            }
     }
     for (int i = tid; i < p.k; i += SEL_THREADS) {
         p.w.top_score[(int64_t)q * p.k + i] = ss[i];
         p.w.top_id[(int64_t)q * p.k + i] = si[i];
+        if (p.last && p.out_ids) {
+            p.out_ids[(int64_t)q * p.k + i] = si[i] == INT_MAX ? -1 : si[i];
+            p.out_scores[(int64_t)q * p.k + i] = ss[i];
+        }
     }
     if (tid == 0) {
         p.w.thr[q] = ss[p.k - 1]; p.w.thr_id[q] = si[p.k - 1];
-        p.w.beat[q] += p.w.beat_tmp[q];
+        const int beat = p.w.beat[q] + p.w.beat_tmp[q];
+        p.w.beat[q] = beat;
         p.w.beat_tmp[q] = 0; p.w.cand_cnt[q] = 0;
+        if (q == 0) p.w.status[6] = (int32_t)p.e_hi;
+        if (p.last && p.out_ranks) p.out_ranks[q] = (p.raw_beat ? 0 : 1) + beat;      // (may be the array of the chunk's counts)
     }
-}
-
-// Tensor-core inference: the true tail's score in the arithmetic of that path (operands rounded
-// to bf16, fp32 accumulation), one thread per query.
-__global__ void ftrue_bf16_kernel(InferParams p) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= p.nq || !p.tt) return;
-    const uint16_t* qb = p.w.iqb + (int64_t)q * p.d;
-    const uint16_t* tb = p.w.Eb + checked_id(p.tt[q], p.E, p.w.status) * p.d;
-    float acc = 0.f;
-    for (int k = 0; k < p.d; ++k)
-        acc = __fmaf_rn(__uint_as_float((uint32_t)qb[k] << 16), __uint_as_float((uint32_t)tb[k] << 16), acc);
-    p.w.iftrue[q] = acc;
 }
 
 // ---- sharded inference: the pieces that need rows of one shard only ----
@@ -740,22 +881,10 @@ __global__ void reset_chunk_kernel(InferParams p) {
     if (q == 0) p.w.status[1] = 0;
 }
 
-__global__ void finish_kernel(InferParams p, int32_t* out_ids, float* out_scores, int32_t* out_ranks) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= p.nq) return;
-    if (out_ids)
-        for (int j = 0; j < p.k; ++j) {
-            const int32_t id = p.w.top_id[(int64_t)q * p.k + j];
-            out_ids[(int64_t)q * p.k + j] = id == INT_MAX ? -1 : id;
-            out_scores[(int64_t)q * p.k + j] = p.w.top_score[(int64_t)q * p.k + j];
-        }
-    if (out_ranks) out_ranks[q] = (p.raw_beat ? 0 : 1) + p.w.beat[q];
-}
-
 cudaError_t launch_score_tiles(const kge_handle* h, const InferParams& p, cudaStream_t s) {
     const int64_t e_tiles = (p.e_hi - p.e_lo + IE - 1) / IE;
     const unsigned grid = (unsigned)(e_tiles * p.q_tiles);
-    if (h->tiles32_ready && p.d >= IKT) {      // rows of at least 128 floats: tiles staged by tensor copies
+    if (h->tiles32_ready && p.d >= ITENSOR_MIN_D) {      // tiles staged by tensor copies
         switch (p.kind) {
             case KIND_L1: return launch_score_tile_tensor<KIND_L1>(h, p, grid, s);
             case KIND_L2: return launch_score_tile_tensor<KIND_L2>(h, p, grid, s);
@@ -769,10 +898,9 @@ cudaError_t launch_score_tiles(const kge_handle* h, const InferParams& p, cudaSt
         case KIND_L2: return launch_score_tile_tma<KIND_L2>(p, grid, s);
         case KIND_CL1: return launch_score_tile_tma<KIND_CL1>(p, grid, s);
         case KIND_DOT: return launch_score_tile_tma<KIND_DOT>(p, grid, s);
-        case KIND_TH_L1: score_tile_kernel<KIND_TH_L1><<<grid, 256, 0, s>>>(p); break;
-        default: score_tile_kernel<KIND_TH_L2><<<grid, 256, 0, s>>>(p); break;
+        case KIND_TH_L1: return launch_dependent(score_tile_kernel<KIND_TH_L1>, dim3(grid), dim3(256), 0, s, p);
+        default: return launch_dependent(score_tile_kernel<KIND_TH_L2>, dim3(grid), dim3(256), 0, s, p);
     }
-    return cudaSuccess;
 }
 
 }  // namespace
@@ -790,6 +918,8 @@ InferParams infer_params(kge_handle* h, const int32_t* qh, const int32_t* qr, in
     p.id_base = 0; p.ext_q = nullptr; p.ext_ftrue = nullptr; p.raw_beat = 0;
     p.w = h->ws;
     p.e_lo = 0; p.e_hi = 0;
+    p.Eb = nullptr; p.first = 0; p.last = 0;
+    p.out_ids = nullptr; p.out_scores = nullptr; p.out_ranks = nullptr;
     return p;
 }
 }  // namespace
@@ -830,67 +960,66 @@ int run_score_all_topk(kge_handle* h, const int32_t* qh, const int32_t* qr, int3
     InferParams p = infer_params(h, qh, qr, nq, k, true_tails);
     if (shard) { p.id_base = shard->ent_base; p.ext_q = shard->qvec; p.ext_ftrue = shard->ftrue; p.raw_beat = 1; }
     const int qblocks = (nq + 127) / 128;
-    query_setup_kernel<<<qblocks, 128, 0, s>>>(p);
-    KGE_LAUNCH_CHECK(h);
-    KGE_CUDA_CHECK(h, cudaMemsetAsync(h->ws.status + 1, 0, 4, s));
     const bool tc = h->ws.Eb != nullptr;    // dot-product model with the tensor-core score block
-    if (tc) {
-        int rc = launch_cast_bf16(h, h->ws.iq, h->ws.iqb, (int64_t)nq * c.dim, s);
-        if (rc == KGE_OK && !h->eb_valid) {     // the bf16 copy of the table is kept until the table changes
-            rc = launch_cast_bf16(h, h->ent, h->ws.Eb, c.num_entities * c.dim, s);
-            if (rc == KGE_OK) h->eb_valid = true;
-        }
+    if (tc && !h->eb_valid) {               // the bf16 copy of the table is kept until the table changes
+        const int rc = launch_cast_bf16(h, h->ent, h->ws.Eb, c.num_entities * c.dim, s);
         if (rc != KGE_OK) return rc;
-        if (!p.ext_ftrue) {
-            ftrue_bf16_kernel<<<qblocks, 128, 0, s>>>(p);
-            KGE_LAUNCH_CHECK(h);
-        }
+        h->eb_valid = true;
     }
-    if (!tc && !h->tiles32_ready && c.dim >= IKT && h->kind != KIND_TH_L1 && h->kind != KIND_TH_L2) {
+    if (tc) p.Eb = h->ws.Eb;
+    p.out_ids = out_ids; p.out_scores = out_scores; p.out_ranks = out_ranks;
+    query_setup_kernel<<<(nq + SETUP_WARPS - 1) / SETUP_WARPS, 32 * SETUP_WARPS, 0, s>>>(p);
+    KGE_LAUNCH_CHECK(h);
+    if (!tc && !h->tiles32_ready && c.dim >= ITENSOR_MIN_D && h->kind != KIND_TH_L1 && h->kind != KIND_TH_L2) {
         // tensor maps of the fp32 query vectors and of the entity table (host-side encoding, nothing allocated)
         int rc = tc_make_f32_tile_map(h, h->tm_iq32, h->ws.iq, h->max_queries, c.dim);
         if (rc == KGE_OK) rc = tc_make_f32_tile_map(h, h->tm_ent32, h->ent, c.num_entities, c.dim);
         if (rc != KGE_OK) return rc;
         h->tiles32_ready = true;
     }
-    auto score_chunk = [&](const InferParams& ip) -> int {
-        if (tc) return launch_tc_infer_chunk(h, nq, ip.e_lo, ip.e_hi, true_tails, ip.id_base, s);
-        KGE_CUDA_CHECK(h, launch_score_tiles(h, ip, s));
-        KGE_LAUNCH_CHECK(h);
-        return KGE_OK;
-    };
 
-    // Chunk i covers as many entities as all chunks before it (the first: one candidate
-    // list's worth, since nothing is filtered yet), capped so a launch stays bounded.
+    // The first chunk is one candidate list's worth, since nothing is filtered yet; a later one covers `grow` times what all
+    // chunks before it did, so that about grow x k entities per query beat the threshold (at most a quarter of a list at the
+    // usual k), capped so that a launch stays bounded.  Twice as long a chunk each time was 14 chunks for 8 M entities at
+    // some 50 us of selection, start-up and drain each; four times as long is 7.
+    //
+    // The chunks are queued without waiting for one another.  A list that fills up (scores rising along the table) sets
+    // status[1]: what is queued behind does nothing, status[6] says how far the call has come, and the chunk is redone in
+    // shorter pieces (pieces of one list's worth cannot overflow).
     const int64_t max_chunk = std::max<int64_t>(kCandCap, std::min<int64_t>((int64_t)1 << 22, (int64_t)0x7fffffff / p.q_tiles * IE / 2));
+    const int64_t grow = std::max(1, std::min(4, 256 / k));
+    int64_t piece = max_chunk, piece_until = 0;      // entities below piece_until go in chunks of at most `piece`
+    auto chunk_len = [&](int64_t lo) {
+        const int64_t len = std::min(std::max<int64_t>(lo * grow, kCandCap), lo < piece_until ? piece : max_chunk);
+        return std::min(len, p.E - lo);
+    };
     int64_t lo = 0;
     while (lo < p.E) {
-        const int64_t len = std::min<int64_t>(std::min<int64_t>(std::max<int64_t>(lo, kCandCap), max_chunk), p.E - lo);
-        p.e_lo = lo; p.e_hi = lo + len;
-        { const int rc = score_chunk(p); if (rc != KGE_OK) return rc; }
-        int32_t overflow = 0;
-        KGE_CUDA_CHECK(h, cudaMemcpyAsync(&overflow, h->ws.status + 1, 4, cudaMemcpyDeviceToHost, s));
-        KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
-        if (!overflow) {
-            select_kernel<<<nq, SEL_THREADS, 0, s>>>(p);
-            KGE_LAUNCH_CHECK(h);
-        } else {
-            // A list filled up (scores rising along the table): redo the chunk in pieces that
-            // cannot overflow, selecting after each.
-            reset_chunk_kernel<<<qblocks, 128, 0, s>>>(p);
-            KGE_LAUNCH_CHECK(h);
-            for (int64_t sub = lo; sub < lo + len; sub += kCandCap) {
-                p.e_lo = sub; p.e_hi = std::min<int64_t>(sub + kCandCap, lo + len);
-                { const int rc = score_chunk(p); if (rc != KGE_OK) return rc; }
-                select_kernel<<<nq, SEL_THREADS, 0, s>>>(p);
+        for (int64_t at = lo; at < p.E;) {
+            p.e_lo = at; p.e_hi = at + chunk_len(at);
+            p.first = at == 0; p.last = p.e_hi == p.E;
+            if (tc) {
+                const int rc = launch_tc_infer_chunk(h, nq, p.e_lo, p.e_hi, true_tails, p.id_base, p.first, s);
+                if (rc != KGE_OK) return rc;
+            } else {
+                KGE_CUDA_CHECK(h, launch_score_tiles(h, p, s));
                 KGE_LAUNCH_CHECK(h);
             }
+            KGE_CUDA_CHECK(h, launch_dependent(select_kernel, dim3(nq), dim3(SEL_THREADS), 0, s, p));
+            KGE_LAUNCH_CHECK(h);
+            at = p.e_hi;
         }
-        lo += len;
+        int32_t flags[6];
+        KGE_CUDA_CHECK(h, cudaMemcpyAsync(flags, h->ws.status + 1, sizeof(flags), cudaMemcpyDeviceToHost, s));
+        KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
+        if (!flags[0]) break;
+        lo = flags[5];
+        const int64_t len = chunk_len(lo);
+        piece_until = std::max(piece_until, lo + len);
+        piece = std::max<int64_t>(kCandCap, (len / 8 + kCandCap - 1) / kCandCap * kCandCap);
+        reset_chunk_kernel<<<qblocks, 128, 0, s>>>(p);
+        KGE_LAUNCH_CHECK(h);
     }
-    finish_kernel<<<qblocks, 128, 0, s>>>(p, out_ids, out_scores, out_ranks);
-    KGE_LAUNCH_CHECK(h);
-    KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
     return KGE_OK;
 }
 

@@ -82,7 +82,8 @@ struct TcGemmParams {
     int32_t *cand_cnt, *beat_tmp;         // [M] candidates appended in this chunk; entities ordered before the true tail
     float* cand_score; int32_t* cand_id;  // [M, cand_cap]
     int cand_cap;
-    int32_t* overflow;                    // set when a candidate list is full
+    int32_t* overflow;                    // set when a candidate list is full: the call's later launches do nothing
+    int first;                            // first chunk: nothing is filtered, the scores go to the candidate lists in entity order
     int beat_rows;                        // rows whose rank counts are gathered in shared memory first (0: global atomics)
     int resident_b;                       // EPI_TOPK: the column tile has a buffer of its own and the ring holds row tiles only
 };
@@ -444,6 +445,14 @@ __device__ __forceinline__ void tc_epilogue_topk(const TcGemmParams& p, const Tc
                 }
             }
         }
+        if (p.first) {         // (a chunk starts at a multiple of 32 columns: whole 128-byte pieces of the row's list)
+            if (rin) {
+                float4* dst = reinterpret_cast<float4*>(p.cand_score + (int64_t)row * p.cand_cap + ncol);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            }
+            return;
+        }
         // candidates: anything ordered before the current k-th best
         float vm[4];           // a tree of three-input maxima, not a chain of 31
 #pragma unroll
@@ -475,7 +484,7 @@ __device__ __forceinline__ void tc_epilogue_topk(const TcGemmParams& p, const Tc
                     p.cand_score[(int64_t)row_s * p.cand_cap + slot] = f;
                     p.cand_id[(int64_t)row_s * p.cand_cap + slot] = e;
                 } else {
-                    *p.overflow = 1;   // the host redoes this chunk in pieces that cannot overflow
+                    *p.overflow = 1;   // the host redoes this chunk in shorter pieces
                 }
             }
         }
@@ -591,16 +600,19 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     uint64_t* b_free = b_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(b_free + 1);
     volatile uint32_t* stop = tmem_slot + 1;     // set by a warp whose wait ran out
+    volatile int* cta_items = reinterpret_cast<volatile int*>(tmem_slot + 2);
     int32_t* beat_sm = reinterpret_cast<int32_t*>(base + (size_t)TC_STAGES * TC_STAGE_BYTES + 256);   // [beat_rows], EPI_TOPK
     if ((EPI & 3) == EPI_TOPK)
         for (int i = threadIdx.x; i < p.beat_rows; i += TC_THREADS) beat_sm[i] = 0;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int per_cta = (p.items + gridDim.x - 1) / gridDim.x;
-    const int item_begin = blockIdx.x * per_cta, item_end = min(p.items, item_begin + per_cta);
+    const int item_begin = blockIdx.x * per_cta;
     const int kb_total = (p.K + TC_BK - 1) / TC_BK;
 
     if (threadIdx.x == 0) {
+        // full-entity scoring after a list overflowed: no items (one thread's reading: the flag may change while this launch runs)
+        *cta_items = (EPI & 3) == EPI_TOPK && *reinterpret_cast<volatile int32_t*>(p.overflow) ? 0 : per_cta;
         for (int s = 0; s < TC_RING_MAX; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         mbar_init(b_full, 1); mbar_init(b_free, 1);
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], GW); }
@@ -615,6 +627,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    const int item_end = min(p.items, item_begin + *cta_items);
 
     // Full-entity scoring with rows of at most 128 coordinates: the column (entity) tile of the
     // current run of items sits in a buffer of its own (2 x 32 KB) and the rest of the stage memory
@@ -1525,7 +1538,7 @@ int launch_cast_bf16(kge_handle* h, const float* src, uint16_t* dst, int64_t cou
 
 // One chunk of full-entity scoring on tensor cores: the bf16 query vectors against the bf16
 // rows [e_lo, e_hi) of the entity table, survivors appended to the candidate lists.
-int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, cudaStream_t s) {
+int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, int first, cudaStream_t s) {
     const Workspace& w = h->ws;
     TcGemmParams p{};
     p.M = nq; p.N = (int)(e_hi - e_lo); p.K = h->cfg.dim;
@@ -1538,7 +1551,7 @@ int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, con
     p.m_fastest = 1; p.n_base = e_lo; p.id_base = id_base;
     p.thr = w.thr; p.thr_id = w.thr_id; p.ftrue = w.iftrue; p.tt = true_tails;
     p.cand_cnt = w.cand_cnt; p.beat_tmp = w.beat_tmp; p.cand_score = w.cand_score; p.cand_id = w.cand_id;
-    p.cand_cap = kCandCap; p.overflow = w.status + 1;
+    p.cand_cap = kCandCap; p.overflow = w.status + 1; p.first = first;
     p.beat_rows = std::min(nq, TC_BEAT_ROWS_MAX);   // the other rows count with global atomics
     p.resident_b = p.kb_per_split <= 2 ? 1 : 0;     // the column tile's two slices fit beside an eight-stage ring of row-tile slices
     // (the table's tensor map covers all rows; the kernel offsets its row coordinate by n_base)

@@ -160,3 +160,42 @@ def test_rising_scores_take_the_overflow_path(oracle32):
     o_ids, _, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, None, qh, qr, K, true_tails=tt)
     assert (ids == o_ids).all() and (ranks == o_ranks).all()
     assert (ids[0] == np.arange(E - 1, E - 1 - K, -1)).all()
+
+
+@pytest.mark.parametrize("d", [28, 32, 36, 64, 68, 96, 132, 196, 260])
+@pytest.mark.parametrize("score,p,K", [("transe", 1, 10), ("transe", 2, 100), ("distmult", 1, 129)])
+def test_row_widths_at_the_edges_of_a_staged_box(oracle32, score, p, d, K):
+    """Rows that end at, before and after the 32-float boxes and 64-float stages of the score tile; lists of up to 128 places
+    (cut down before they are sorted) and one more; 65 queries (a second tile of one row), 2,500 entities in three chunks."""
+    import kge_synth
+    E, R, nq = 2500, 5, 65
+    prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=p, B=4, N=4, P=1, graph_seed=31)
+    prob.ent[2400] = prob.ent[17]; prob.ent[1000] = prob.ent[17]
+    qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=31)
+    tt[0] = qh[0]; tt[1] = 2400; qh[2] = 17
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, None, qh, qr, K, true_tails=tt)
+    assert (ids == o_ids).all() and (ranks == o_ranks).all()
+    assert (sc == o_sc).all()
+
+
+@pytest.mark.parametrize("score,tc,d", [("distmult", False, 32), ("distmult", True, 64), ("distmult", False, 16)])
+@pytest.mark.parametrize("lo,hi", [(3000, 9000), (1024, 30000)])
+@pytest.mark.parametrize("K", [1, 40])
+def test_scores_that_rise_along_a_stretch(oracle32, score, tc, d, lo, hi, K):
+    """A list that fills up in the middle of the table: the chunk is redone in pieces (of several sizes in the longer
+    stretch) while the chunks queued behind it wait.  Values with eight significant bits: exact in every arithmetic, with
+    ties decided by the id."""
+    E = 40_000
+    prob = Problem(E=E, R=2, T=50, d=d, score=score, B=4, N=4, P=1, graph_seed=13, tc=tc)
+    prob.ent[:] = 0.0
+    prob.ent[:, 0] = 0.25
+    prob.ent[lo:hi, 0] = 0.5 + np.floor(np.arange(hi - lo) * 127.0 / (hi - lo)) / 256.0
+    prob.rel[:] = 1.0
+    gpu = GpuSide(prob, max_queries=70, topk=K, load_graph=False)
+    rng = np.random.default_rng(5)
+    qh, qr, tt = rng.integers(0, E, 66), rng.integers(0, 2, 66), rng.integers(0, E, 66)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, None, qh, qr, K, true_tails=tt)
+    assert (ids == o_ids).all() and (ranks == o_ranks).all() and (sc == o_sc).all()
