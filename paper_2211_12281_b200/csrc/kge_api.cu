@@ -100,7 +100,7 @@ size_t layout(const kge_handle* h, char* base, int64_t T, int32_t maxq, int32_t 
         w.Mb = cv.take<uint16_t>(2 * d * F);
         w.proj = cv.take<float>((2 * B + N) * d);
         w.Gslot = cv.take<uint16_t>((2 * B + N) * d);
-        w.dMpart = cv.take<float>((size_t)2 * h->split_m * d * F);
+        w.dMpart = cv.take<float>((size_t)(h->split_mh + h->split_mt) * d * F);
     }
     const bool tc = c.prec == KGE_PREC_BF16_TC;
     w.Qb = tc ? cv.take<uint16_t>(B * d) : nullptr;
@@ -289,10 +289,12 @@ int kge_create(const kge_config* cfg, kge_handle** out) {
         const int kb = 2 * ((std::min(c.batch, c.num_neg) + 63) / 64);
         h->th_gsplit = std::max(1, std::min(std::min(h->num_sms / tiles, kb / 8), 4));
     }
-    h->split_m = 1;
+    h->split_mh = h->split_mt = 1;
     h->features_bound = false;
-    if (c.feat_dim > 0)   // dM = dE^T . F: [d, F] over the batch's slots, split over the slots so that every SM has a tile
-        h->split_m = pick_split_tc(c.dim, c.feat_dim, c.batch, h->num_sms);
+    if (c.feat_dim > 0) {   // dM = dE^T . F: [d, F] over the role's slots, split over the slots so that every SM has a tile
+        h->split_mh = pick_split_tc(c.dim, c.feat_dim, c.batch, h->num_sms);
+        h->split_mt = pick_split_tc(c.dim, c.feat_dim, c.batch + c.num_neg, h->num_sms);
+    }
     *out = h;
     return KGE_OK;
 }
@@ -538,8 +540,8 @@ int kge_train_step(kge_handle* h, uint64_t step, float lr, const int32_t* heads,
         // triple bucket and the bucket's cumulative weights fit its shared memory.
         const kge_config& c = h->cfg;
         const int buckets = c.head_part < 0 ? c.num_parts * c.num_parts : c.num_parts;
-        // (with an encoder the ids must exist before the gather: the features of the batch are projected first)
-        fused = fork && (c.batch / buckets) % 8 == 0 && c.num_relations + 1 <= 4096 && c.feat_dim == 0;
+        // (with an encoder the features of the batch are projected first: its first kernel draws the batch the same way)
+        fused = fork && (c.batch / buckets) % 8 == 0 && c.num_relations + 1 <= 4096;
         if (!fused) {
             rc = launch_sample(h, step, w.heads, w.rels, w.tails, w.negs, s);
             if (rc != KGE_OK) return rc;
@@ -548,15 +550,28 @@ int kge_train_step(kge_handle* h, uint64_t step, float lr, const int32_t* heads,
     }
     if (h->cfg.feat_dim > 0) {
         if (!h->features_bound) return KGE_ERR_NOT_READY;
-        if ((rc = launch_encoder_forward(h, heads, tails, negs, s)) != KGE_OK) return rc;
+        if ((rc = launch_encoder_forward(h, heads, tails, negs, fused, step, s)) != KGE_OK) return rc;
+        fused = false;
     }
     rc = launch_forward_backward(h, heads, rels, tails, negs, loss_out, s, fork ? h->side[1] : nullptr,
                                  fork ? h->side[0] : nullptr, fused, step);
     if (rc != KGE_OK) return rc;
     // with side streams the id sort has been joined before the chain kernel
     if (!fork && (rc = launch_dedup(h, heads, rels, tails, negs, s)) != KGE_OK) return rc;
+    // the matrices' gradients and steps need the gradient rows only: they run beside the update of the rows
+    cudaStream_t se = fork ? h->side[1] : s;
+    if (h->cfg.feat_dim > 0 && fork) {
+        KGE_CUDA_CHECK(h, cudaEventRecord(h->ev_loss, s));
+        KGE_CUDA_CHECK(h, cudaStreamWaitEvent(se, h->ev_loss, 0));
+    }
     rc = launch_update(h, step, lr, s);
-    if (rc == KGE_OK && h->cfg.feat_dim > 0) rc = launch_encoder_backward(h, step, lr, s);
+    if (rc == KGE_OK && h->cfg.feat_dim > 0) {
+        rc = launch_encoder_backward(h, step, lr, se);
+        if (fork) {
+            KGE_CUDA_CHECK(h, cudaEventRecord(h->ev_t, se));
+            KGE_CUDA_CHECK(h, cudaStreamWaitEvent(s, h->ev_t, 0));
+        }
+    }
     h->eb_valid = false;          // the entity table has moved on: tensor-core inference must refresh its bf16 copy
     if (rc != KGE_OK) return rc;
     return h->prof.on ? stage_collect(h, s) : KGE_OK;

@@ -54,8 +54,8 @@ struct Workspace {
     uint16_t *Fb;                          // [2B+N, F] bf16 features of the batch's slots [heads | tails | negs]
     uint16_t *Mb;                          // [2][d, F] bf16 copies of M_H, M_T
     float *proj;                           // [2B+N, d] M e_F of every slot (added to the gathered rows)
-    uint16_t *Gslot;                       // [2B+N, d] bf16 copy of the slots' gradient rows
-    float *dMpart;                         // [2][splits][d, F] partial gradients of M_H, M_T
+    uint16_t *Gslot;                       // [2B+N, d] bf16 copy of the slots' gradient rows (written with them)
+    float *dMpart;                         // [split_mh + split_mt][d, F] partial gradients of M_H, M_T
     float *reg_s3;                         // [2B+N] sum of |e_k|^3 of the gathered rows [heads | tails | negs] (L3 regulariser), or NULL
     uint16_t *Qb, *Tb;                     // [B,d], [N,d] bf16 copies of Q and Tneg (tensor-core scoring)
     uint16_t *Gb;                          // bf16 [B,ldN] dL/dF (ldN = N rounded up to 8)
@@ -143,7 +143,7 @@ struct kge_handle {
     alignas(64) unsigned char tm_fh[128], tm_ft[128], tm_mh[128], tm_mt[128], tm_gh64[128], tm_gt64[128], tm_fh64[128], tm_ft64[128];
     const uint16_t* feat;   // [E, F] bf16 text features (fixed)
     float *MH, *MT, *MH_state, *MT_state;   // [d, F] projection matrices and their optimiser state
-    int split_m;            // K splits of the two dM contractions
+    int split_mh, split_mt; // K splits of the two dM contractions (heads; tails and negatives)
     bool features_bound;
     bool streams_ready;
     cudaStream_t side[2];
@@ -233,13 +233,14 @@ int launch_th_contract_gemm(kge_handle* h, cudaStream_t s);
 int launch_tc_forward(kge_handle* h, cudaStream_t s);
 int launch_tc_gemm_terms(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int tstride, float* C,
                          int64_t ldc, cudaStream_t s);
-int launch_tc_gemm_nt(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int K, float* C, int64_t ldc,
-                      cudaStream_t s);
-int launch_tc_gemm_tn(kge_handle* h, const unsigned char* tmA64, const unsigned char* tmB64, int M, int N, int K, int split, float* C,
-                      int64_t ldc, cudaStream_t s);
+int launch_tc_dual_nt(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1, const unsigned char* tmB1,
+                      int M0, int M1, int N, int K, float* C0, float* C1, cudaStream_t s);
+int launch_tc_dual_tn(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1, const unsigned char* tmB1,
+                      int M, int N, int K0, int K1, int split0, int split1, float* C0, float* C1, cudaStream_t s);
 // Feature-projection encoder (kge_encoder.cu): M e_F of the batch's slots before the gather; dM and the dense step after the backward.
 int encoder_make_maps(kge_handle* h);
-int launch_encoder_forward(kge_handle* h, const int32_t* heads, const int32_t* tails, const int32_t* negs, cudaStream_t s);
+// (with `fused_sample` the first kernel draws the batch of `step` itself and leaves the ids in the workspace, as launch_forward_backward's does)
+int launch_encoder_forward(kge_handle* h, const int32_t* heads, const int32_t* tails, const int32_t* negs, bool fused_sample, uint64_t step, cudaStream_t s);
 int launch_encoder_backward(kge_handle* h, uint64_t step, float lr, cudaStream_t s);
 int launch_cast_bf16(kge_handle* h, const float* src, uint16_t* dst, int64_t count, cudaStream_t s);
 int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, int first, cudaStream_t s);

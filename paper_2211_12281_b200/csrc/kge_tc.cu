@@ -834,7 +834,10 @@ struct DualProb {
 // coefficients against one [x1 | x2] operand).  A stage then holds both segments' A tiles beside the one B tile and both
 // are multiplied into the accumulator, so a B slice is fetched once instead of once per segment (a third fewer operand
 // bytes per flop); K runs over one segment's slices.  Three stages instead of four fit.
-template <int BN, bool PAIR = false>
+// FORM: how the operands of both problems are read.  DUAL_STEP: as above.  DUAL_NT: A and B K-major (the encoder's two
+// projections).  DUAL_TN: A and B MN-major (the encoder's two matrix gradients).
+enum { DUAL_STEP = 0, DUAL_NT = 1, DUAL_TN = 2 };
+template <int BN, bool PAIR = false, int FORM = DUAL_STEP>
 __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kernel(const __grid_constant__ CUtensorMap tmA0,
                                                                                     const __grid_constant__ CUtensorMap tmB0,
                                                                                     const __grid_constant__ CUtensorMap tmA1,
@@ -878,6 +881,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (FORM != DUAL_STEP) { grid_dependency_wait(); allow_dependents(); }
 
     if (warp == 0) {
         if (lane == 0) {
@@ -899,7 +903,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
 #pragma unroll
                     for (int half = 0; half < (PAIR ? 2 : 1); ++half) {       // PAIR: both segments' A tiles of this slice
                         unsigned char* da = sa + half * TC_A_BYTES;
-                        if (which) {      // dL/dF with the contraction index as rows: two boxes of 64 output rows
+                        if (FORM == DUAL_TN || (FORM == DUAL_STEP && which)) {      // the contraction index as rows: two boxes of 64 output rows
 #pragma unroll
                             for (int g = 0; g < TC_BM / 64; ++g)
                                 tma_load_2d(da + g * TC_MN_GROUP_BYTES, ta, it.m0 + 64 * g + (PAIR ? half : seg) * q.a_seg_x, kseg, &full[s]);
@@ -907,14 +911,19 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                             tma_load_2d(da, ta, k0 + half * q.seg_kb * TC_BK, it.m0, &full[s]);
                         }
                     }
+                    if (FORM == DUAL_NT) {
 #pragma unroll
-                    for (int g = 0; g < BN / 64; ++g) tma_load_2d(sa + A_BYTES + g * TC_MN_GROUP_BYTES, tb, it.n0 + 64 * g, kseg, &full[s]);
+                        for (int g = 0; g < BN / 128; ++g) tma_load_2d(sa + A_BYTES + g * (128 * TC_BK * 2), tb, kseg, it.n0 + 128 * g, &full[s]);
+                    } else {
+#pragma unroll
+                        for (int g = 0; g < BN / 64; ++g) tma_load_2d(sa + A_BYTES + g * TC_MN_GROUP_BYTES, tb, it.n0 + 64 * g, kseg, &full[s]);
+                    }
                 }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc_k = umma_idesc_bf16(TC_BM, BN, false, true), idesc_mn = umma_idesc_bf16(TC_BM, BN, true, true);
+            constexpr uint32_t idesc_k = umma_idesc_bf16(TC_BM, BN, false, FORM != DUAL_NT), idesc_mn = umma_idesc_bf16(TC_BM, BN, true, true);
             int ring = 0;
             bool ok = true;
             for (int item = blockIdx.x, local = 0; item < total && ok && !*stop; item += gridDim.x, ++local) {
@@ -936,9 +945,10 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
 #pragma unroll
                         for (int k = 0; k < TC_BK / 16; ++k) {
                             const uint32_t aa = sa + half * TC_A_BYTES;
-                            const uint64_t ad = which ? umma_desc_mn_sw128(aa + k * 2048) : umma_desc_k_sw128(aa + k * 32);
-                            const uint64_t bd = umma_desc_mn_sw128(sa + A_BYTES + k * 2048);
-                            umma_bf16(tmem_acc, ad, bd, which ? idesc_mn : idesc_k, (kb | k | half) != 0);
+                            const bool a_mn = FORM == DUAL_TN || (FORM == DUAL_STEP && which);
+                            const uint64_t ad = a_mn ? umma_desc_mn_sw128(aa + k * 2048) : umma_desc_k_sw128(aa + k * 32);
+                            const uint64_t bd = FORM == DUAL_NT ? umma_desc_k_sw128(sa + A_BYTES + k * 32) : umma_desc_mn_sw128(sa + A_BYTES + k * 2048);
+                            umma_bf16(tmem_acc, ad, bd, a_mn ? idesc_mn : idesc_k, (kb | k | half) != 0);
                         }
                     }
                     umma_commit(&empty[s]);
@@ -1360,27 +1370,6 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
 }
 
 namespace {
-// One backward contraction C[M, N] (+ K splits) with the tile width that fits the row width.
-template <bool A_MN>
-int launch_tc_bwd_gemm(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int K, int split,
-                       float* C, int64_t ldc, cudaStream_t s) {
-    TcGemmParams p{};
-    p.M = M; p.N = N; p.K = K;
-    const int kb = (K + TC_BK - 1) / TC_BK;
-    p.kb_per_split = (kb + split - 1) / split;
-    p.C = C; p.ldc = ldc; p.split_stride = (int64_t)M * ldc;
-    p.status = h->ws.status; p.wait_limit = h->wait_limit;
-    p.bn = tc_backward_tile_cols(N);
-    p.tiles_m = (M + TC_BM - 1) / TC_BM; p.tiles_n = (N + p.bn - 1) / p.bn;
-    p.items = p.tiles_m * p.tiles_n * ((kb + p.kb_per_split - 1) / p.kb_per_split);
-    if (p.bn == 256) KGE_CUDA_CHECK(h, (launch_gemm_inst<EPI_STORE, 256, A_MN, true>(tmA, tmB, p, h->num_sms, s)));
-    else KGE_CUDA_CHECK(h, (launch_gemm_inst<EPI_STORE, 128, A_MN, true>(tmA, tmB, p, h->num_sms, s)));
-    KGE_LAUNCH_CHECK(h);
-    return KGE_OK;
-}
-}  // namespace
-
-namespace {
 DualProb dual_prob(int M, int N, int K, int split, float* C, int64_t ldc, int bn) {
     DualProb q{};
     q.M = M; q.N = N;
@@ -1392,41 +1381,47 @@ DualProb dual_prob(int M, int N, int K, int split, float* C, int64_t ldc, int bn
     q.seg_kb = q.kb_total; q.a_seg_x = 0; q.fold = 0; q.fold_stride = 0;
     return q;
 }
-template <int BN, bool PAIR = false>
+template <int BN, bool PAIR = false, int FORM = DUAL_STEP>
 cudaError_t launch_gemm_dual(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1,
                              const unsigned char* tmB1, const DualProb& q0, const DualProb& q1, cudaStream_t s) {
     constexpr size_t smem = (PAIR ? 1024 + (size_t)3 * (tc_stage_bytes(BN) + TC_A_BYTES) + 256 : tc_smem_bytes(BN)) +
                             (size_t)TC_EPI_WARPS * TC_STORE_STAGE_BYTES;      // + the epilogue warps' store staging
     static DeviceOnce configured;
     const cudaError_t e = once_per_device(configured, [] {
-        return cudaFuncSetAttribute(tc_gemm_dual_kernel<BN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaFuncSetAttribute(tc_gemm_dual_kernel<BN, PAIR, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     // as few CTAs as give the same number of rounds: SMs left over serve the id sort that runs beside this launch
     const int total = q0.items + q1.items;
     const int rounds = (total + h->num_sms - 1) / h->num_sms;
     const int grid = (total + rounds - 1) / rounds;
-    tc_gemm_dual_kernel<BN, PAIR><<<grid, 32 * (2 + TC_EPI_WARPS), smem, s>>>(
+    if (FORM != DUAL_STEP)
+        return launch_dependent(tc_gemm_dual_kernel<BN, PAIR, FORM>, dim3(grid), dim3(32 * (2 + TC_EPI_WARPS)), smem, s,
+                                *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
+                                *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
+    tc_gemm_dual_kernel<BN, PAIR, FORM><<<grid, 32 * (2 + TC_EPI_WARPS), smem, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
         *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
     return cudaSuccess;
 }
 }  // namespace
 
-// Plain contractions for the feature-projection encoder, on the same kernel.
-//   C[M, N] = A[M, K] . B[N, K]^T   (both operands K-major: tensor maps with 128-row boxes)
-int launch_tc_gemm_nt(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int K, float* C, int64_t ldc,
-                      cudaStream_t s) {
-    TcGemmParams p{};
-    p.M = M; p.N = N; p.K = K;
-    p.kb_per_split = (K + TC_BK - 1) / TC_BK;
-    p.C = C; p.ldc = ldc; p.split_stride = 0;
-    p.status = h->ws.status; p.wait_limit = h->wait_limit;
-    // 256-column tiles halve the operand bytes fetched per output once there are enough of them for every SM
-    p.bn = (N >= 1024 && (int64_t)((M + TC_BM - 1) / TC_BM) * ((N + 255) / 256) >= h->num_sms) ? 256 : TC_BN;
-    p.tiles_m = (M + TC_BM - 1) / TC_BM; p.tiles_n = (N + p.bn - 1) / p.bn; p.items = p.tiles_m * p.tiles_n;
-    if (p.bn == 256) KGE_CUDA_CHECK(h, (launch_gemm_inst<EPI_STORE, 256>(tmA, tmB, p, h->num_sms, s)));
-    else KGE_CUDA_CHECK(h, (launch_gemm_inst<EPI_STORE, 128>(tmA, tmB, p, h->num_sms, s)));
+// The feature-projection encoder's contractions, both roles in one launch.
+//   C0[M0, N] = A0[M0, K] . B0[N, K]^T and C1[M1, N] = A1[M1, K] . B1[N, K]^T   (K-major: tensor maps with 128-row boxes)
+int launch_tc_dual_nt(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1, const unsigned char* tmB1,
+                      int M0, int M1, int N, int K, float* C0, float* C1, cudaStream_t s) {
+    const DualProb q0 = dual_prob(M0, N, K, 1, C0, N, 128), q1 = dual_prob(M1, N, K, 1, C1, N, 128);
+    KGE_CUDA_CHECK(h, (launch_gemm_dual<128, false, DUAL_NT>(h, tmA0, tmB0, tmA1, tmB1, q0, q1, s)));
+    KGE_LAUNCH_CHECK(h);
+    return KGE_OK;
+}
+//   C0[split0][M, N] = A0[K0, M]^T . B0[K0, N] over K slices of each split, and C1 likewise (MN-major: 64-row boxes)
+int launch_tc_dual_tn(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1, const unsigned char* tmB1,
+                      int M, int N, int K0, int K1, int split0, int split1, float* C0, float* C1, cudaStream_t s) {
+    const int bn = tc_backward_tile_cols(N);
+    const DualProb q0 = dual_prob(M, N, K0, split0, C0, N, bn), q1 = dual_prob(M, N, K1, split1, C1, N, bn);
+    KGE_CUDA_CHECK(h, bn == 256 ? (launch_gemm_dual<256, false, DUAL_TN>(h, tmA0, tmB0, tmA1, tmB1, q0, q1, s))
+                                : (launch_gemm_dual<128, false, DUAL_TN>(h, tmA0, tmB0, tmA1, tmB1, q0, q1, s)));
     KGE_LAUNCH_CHECK(h);
     return KGE_OK;
 }
@@ -1447,12 +1442,6 @@ int launch_tc_gemm_terms(kge_handle* h, const unsigned char* tmA, const unsigned
     KGE_LAUNCH_CHECK(h);
     return KGE_OK;
 }
-//   C[split][M, N] = A[K, M]^T . B[K, N] over K slices of each split (both operands MN-major: 64-row boxes)
-int launch_tc_gemm_tn(kge_handle* h, const unsigned char* tmA64, const unsigned char* tmB64, int M, int N, int K, int split, float* C,
-                      int64_t ldc, cudaStream_t s) {
-    return launch_tc_bwd_gemm<true>(h, tmA64, tmB64, M, N, K, split, C, ldc, s);
-}
-
 bool tc_negatives_direct(const kge_handle* h) {
     // (with the regulariser on, the chain kernel still has a term to add to every negative's row)
     return h->cfg.prec == KGE_PREC_BF16_TC && h->kind == KIND_DOT && h->split_t == 1 && !(h->cfg.reg_lambda > 0.f);

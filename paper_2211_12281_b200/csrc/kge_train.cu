@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
     extern __shared__ uint64_t bucket_wcum[];   // fused sampling: cumulative weights of this CTA's bucket
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    grid_dependency_wait();
     allow_dependents();   // the score kernel may set up its shared memory while this one runs
     int64_t bucket_base = 0;
     if (p.fused_sample) {
@@ -994,7 +995,11 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp >= p.B + (p.neg_direct ? 0 : p.N)) return;
     const int d4 = p.d4;
-    float4* gent = reinterpret_cast<float4*>(p.w.grad_ent);
+    // gradient row of a slot; with an encoder its bf16 copy too (an operand of the matrices' gradients)
+    auto put = [&](int slot, int c, float4 g) {
+        reinterpret_cast<float4*>(p.w.grad_ent)[(int64_t)slot * d4 + c] = g;
+        if (p.w.Gslot) reinterpret_cast<uint2*>(p.w.Gslot)[(int64_t)slot * d4 + c] = pack_bf16x4(g);
+    };
     if (warp >= p.B) {
         const int n = warp - p.B;
         const float4* part = reinterpret_cast<const float4*>(p.w.dTpart);
@@ -1010,7 +1015,7 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
                 s = make_float4(s.x - cs * t.x, s.y - cs * t.y, s.z - cs * t.z, s.w - cs * t.w);
             }
             if (p.w.reg_s3) s = f4add(s, f4reg(creg, reinterpret_cast<const float4*>(p.w.Tneg)[(int64_t)n * d4 + c]));
-            gent[(int64_t)(2 * p.B + n) * d4 + c] = s;
+            put(2 * p.B + n, c, s);
         }
         return;
     }
@@ -1045,8 +1050,6 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
         }
         dq[i] = s; dt[i] = f4zero();
     }
-    float4* gh = gent + (int64_t)b * d4;
-    float4* gt = gent + (int64_t)(p.B + b) * d4;
     // L3 regulariser: its gradient joins the head's and the positive tail's rows where they are stored
     const float creg_h = p.w.reg_s3 ? reg_coef(p.reg_lambda, p.reg_form, p.w.reg_s3[b]) : 0.f;
     const float creg_t = p.w.reg_s3 ? reg_coef(p.reg_lambda, p.reg_form, p.w.reg_s3[p.B + b]) : 0.f;
@@ -1106,8 +1109,8 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
         for (int i = 0; i < kMaxChunks; ++i) {
             const int c = lane + 32 * i;
             if (c >= d4) continue;
-            gh[c] = f4add(f4fma(-wdq, wh[i], dq[i]), f4reg(creg_h, h[i]));
-            gt[c] = f4add(dt[i], f4reg(creg_t, t[i]));
+            put(b, c, f4add(f4fma(-wdq, wh[i], dq[i]), f4reg(creg_h, h[i])));
+            put(p.B + b, c, f4add(dt[i], f4reg(creg_t, t[i])));
             gr[c] = dq[i];
             gw[c] = clamped ? f4scale(inv, dwh[i]) : f4scale(inv, f4fma(-wdw, wh[i], dwh[i]));
         }
@@ -1148,9 +1151,9 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
             const float2 ph = th[c];
             float s0, c0, s1, c1;
             sincosf(ph.x, &s0, &c0); sincosf(ph.y, &s1, &c1);
-            gh[c] = f4add(make_float4(dq[i].x * c0 + dq[i].y * s0, -dq[i].x * s0 + dq[i].y * c0,
-                                      dq[i].z * c1 + dq[i].w * s1, -dq[i].z * s1 + dq[i].w * c1), f4reg(creg_h, h[i]));
-            gt[c] = f4add(dt[i], f4reg(creg_t, t[i]));
+            put(b, c, f4add(make_float4(dq[i].x * c0 + dq[i].y * s0, -dq[i].x * s0 + dq[i].y * c0,
+                                      dq[i].z * c1 + dq[i].w * s1, -dq[i].z * s1 + dq[i].w * c1), f4reg(creg_h, h[i])));
+            put(p.B + b, c, f4add(dt[i], f4reg(creg_t, t[i])));
             gr[c] = make_float2(-dq[i].x * q[i].y + dq[i].y * q[i].x, -dq[i].z * q[i].w + dq[i].w * q[i].z);
         }
         return;
@@ -1161,17 +1164,17 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     for (int i = 0; i < kMaxChunks; ++i) {
         const int c = lane + 32 * i;
         if (c >= d4) continue;
-        gt[c] = f4add(dt[i], f4reg(creg_t, t[i]));
+        put(p.B + b, c, f4add(dt[i], f4reg(creg_t, t[i])));
         const float4 rg = f4reg(creg_h, h[i]);
         if (p.score == KGE_TRANSE) {
-            gh[c] = f4add(dq[i], rg); gr[c] = dq[i];
+            put(b, c, f4add(dq[i], rg)); gr[c] = dq[i];
         } else if (p.score == KGE_DISTMULT) {
             const float4 r = rrow[c];
-            gh[c] = f4add(f4mul(dq[i], r), rg); gr[c] = f4mul(dq[i], h[i]);
+            put(b, c, f4add(f4mul(dq[i], r), rg)); gr[c] = f4mul(dq[i], h[i]);
         } else {  // ComplEx: q = r * h
             const float4 r = rrow[c];
-            gh[c] = f4add(make_float4(dq[i].x * r.x + dq[i].y * r.y, -dq[i].x * r.y + dq[i].y * r.x,
-                                      dq[i].z * r.z + dq[i].w * r.w, -dq[i].z * r.w + dq[i].w * r.z), rg);
+            put(b, c, f4add(make_float4(dq[i].x * r.x + dq[i].y * r.y, -dq[i].x * r.y + dq[i].y * r.x,
+                                      dq[i].z * r.z + dq[i].w * r.w, -dq[i].z * r.w + dq[i].w * r.z), rg));
             gr[c] = make_float4(dq[i].x * h[i].x + dq[i].y * h[i].y, -dq[i].x * h[i].y + dq[i].y * h[i].x,
                                 dq[i].z * h[i].z + dq[i].w * h[i].w, -dq[i].z * h[i].w + dq[i].w * h[i].z);
         }
@@ -1260,9 +1263,9 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     {
         const int grid = (row_warps * 32 + 255) / 256;
         const size_t smem = fused_sample ? (size_t)(c.num_relations + 1) * 8 : 0;
-        if (nch == 1) build_kernel<1><<<grid, 256, smem, s>>>(p);
-        else if (nch == 2) build_kernel<2><<<grid, 256, smem, s>>>(p);
-        else build_kernel<4><<<grid, 256, smem, s>>>(p);
+        if (nch == 1) KGE_CUDA_CHECK(h, launch_dependent(build_kernel<1>, dim3(grid), dim3(256), smem, s, p));
+        else if (nch == 2) KGE_CUDA_CHECK(h, launch_dependent(build_kernel<2>, dim3(grid), dim3(256), smem, s, p));
+        else KGE_CUDA_CHECK(h, launch_dependent(build_kernel<4>, dim3(grid), dim3(256), smem, s, p));
     }
     stage_end(h, ST_BUILD, s);
     KGE_LAUNCH_CHECK(h);

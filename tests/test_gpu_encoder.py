@@ -96,3 +96,32 @@ def test_encoder_handle_refuses_what_it_does_not_offer():
     with pytest.raises(K.KgeError) as e:
         gpu.kge.score_all_topk(z, z, 2, None, t.zeros((4, 2), dtype=t.int32, device=z.device), t.zeros((4, 2), device=z.device))
     assert e.value.code == -5
+
+
+# a batch the first kernel draws itself (16 slots per bucket), one it cannot (25), rows longer than one round of the copy; more
+# slots than one K split of the matrices' gradients; a row-wise state; bf16 scores whose negatives' rows come from a contraction
+@pytest.mark.parametrize("B,N,F,d,opt,tc", [(64, 96, 64, 8, "sgd", False), (100, 64, 1088, 40, "adam", False), (256, 1024, 768, 136, "adagrad", False),
+                                            (128, 640, 128, 64, "sgd", True)])
+def test_encoder_step_that_draws_its_batch(oracle64, B, N, F, d, opt, tc):
+    """A step that samples inside against the same step on the ids kge_sample_batch gives: bit for bit."""
+    import torch
+    sides = []
+    for own in (True, False):
+        prob = Problem(E=3000, R=7, T=20000, d=d, score="distmult", loss="softmax", opt=opt, B=B, N=N, P=2, lr=0.02, graph_seed=23, tc=tc)
+        prob.kw.update(feat_dim=F, feat_shared=0)
+        gpu = GpuSide(prob)
+        dev = gpu.ent.device
+        gen = torch.Generator(device=dev); gen.manual_seed(3)
+        feat = torch.randn((prob.E, F), generator=gen, device=dev).mul_(F ** -0.5).to(torch.bfloat16)
+        mats = [torch.randn((d, F), generator=gen, device=dev).mul_(0.3) for _ in range(2)]
+        shape = {"sgd": None, "adam": (d, 2 * F), "adagrad": (d,)}[opt]
+        states = [None if shape is None else torch.zeros(shape, device=dev) for _ in range(2)]
+        gpu.kge.bind_features(feat, *mats, *states)
+        loss = torch.zeros(1, device=dev)
+        for step in range(3):
+            ids = () if own else [gpu.dev_i32(a) for a in gpu.sample(step)]
+            gpu.kge.train_step(step, prob.lr, *ids, loss_out=loss)
+        assert gpu.kge.get_status() == 0
+        sides.append([gpu.ent, gpu.rel, loss, *mats] + [s for s in states if s is not None])
+    for a, b in zip(*sides):
+        assert torch.isfinite(a).all() and torch.equal(a, b)
