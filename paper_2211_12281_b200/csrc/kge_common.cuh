@@ -230,6 +230,10 @@ int launch_th_forward(kge_handle* h, cudaStream_t s);
 int launch_th_backward(kge_handle* h, cudaStream_t sq, cudaStream_t st);
 int th_contract_slabs(const kge_handle* h);          // partial slabs the tensor-core contractions add per side (0 when off)
 int launch_th_contract_gemm(kge_handle* h, cudaStream_t s);
+// Backward of the distance kinds, both sides in one pass (kge_pair_backward.cu).
+bool pair_backward_serves(const kge_handle* h);
+void pair_backward_split(int B, int N, int d4, int num_sms, int* split_q, int* split_t);
+int launch_pair_backward(kge_handle* h, cudaStream_t s);
 int launch_tc_forward(kge_handle* h, cudaStream_t s);
 int launch_tc_gemm_terms(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int tstride, float* C,
                          int64_t ldc, cudaStream_t s);
@@ -333,6 +337,17 @@ __device__ __forceinline__ bool mbar_wait_idle(uint64_t* bar, uint32_t parity, i
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+// Two differences in one instruction, each rounded as a single subtraction would be.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    uint64_t x, y, d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
 }
 
 // Programmatic dependent launch.  A kernel started with launch_dependent() may become resident

@@ -555,16 +555,6 @@ __device__ __forceinline__ void tile_load_2d(void* dst, const CUtensorMap* tm, i
         ::"r"(smem_u32(dst)), "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
 
-// Two differences in one instruction, each rounded as a single subtraction would be.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-    uint64_t x, y, d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
-    return r;
-}
 // canon_update with the subtractions of neighbouring coordinates packed.
 template <int KIND>
 __device__ __forceinline__ void canon_update_packed(float& acc, float4 q, float4 t) {

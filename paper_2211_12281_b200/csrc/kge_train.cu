@@ -271,17 +271,17 @@ template <int KIND>
 __device__ __forceinline__ void pair_update(float& acc, float4 q, float4 t) {
     if (KIND == KIND_DOT) {
         acc = fmaf(q.x, t.x, acc); acc = fmaf(q.y, t.y, acc); acc = fmaf(q.z, t.z, acc); acc = fmaf(q.w, t.w, acc);
-    } else if (KIND == KIND_L1) {
-        acc += fabsf(q.x - t.x); acc += fabsf(q.y - t.y); acc += fabsf(q.z - t.z); acc += fabsf(q.w - t.w);
+        return;
+    }
+    // two differences per instruction: the pipe takes as long, the issue slot serves the shared-memory reads
+    const float2 a = sub2(make_float2(q.x, q.y), make_float2(t.x, t.y)), b = sub2(make_float2(q.z, q.w), make_float2(t.z, t.w));
+    if (KIND == KIND_L1) {
+        acc += fabsf(a.x); acc += fabsf(a.y); acc += fabsf(b.x); acc += fabsf(b.y);
     } else if (KIND == KIND_L2) {
-        float x;
-        x = q.x - t.x; acc = fmaf(x, x, acc); x = q.y - t.y; acc = fmaf(x, x, acc);
-        x = q.z - t.z; acc = fmaf(x, x, acc); x = q.w - t.w; acc = fmaf(x, x, acc);
+        acc = fmaf(a.x, a.x, acc); acc = fmaf(a.y, a.y, acc); acc = fmaf(b.x, b.x, acc); acc = fmaf(b.y, b.y, acc);
     } else {  // KIND_CL1: one special-function square root per complex component (relative error 2^-22)
-        float xr = q.x - t.x, xi = q.y - t.y;
-        acc += approx_sqrt(fmaf(xr, xr, xi * xi));
-        xr = q.z - t.z; xi = q.w - t.w;
-        acc += approx_sqrt(fmaf(xr, xr, xi * xi));
+        acc += approx_sqrt(fmaf(a.x, a.x, a.y * a.y));
+        acc += approx_sqrt(fmaf(b.x, b.x, b.y * b.y));
     }
 }
 
@@ -289,9 +289,10 @@ __device__ __forceinline__ void pair_update(float& acc, float4 q, float4 t) {
 // block, kinds that are a function of (q, t) alone: 32 x 64 pairs per CTA, 4 x 4 per thread.
 // The 32 query rows and 64 negative rows of the tile are brought into shared memory by one
 // asynchronous bulk copy per row (padded rows, so the 128-bit reads below are conflict-free),
-// up to 128 floats of the embedding axis per stage, two stages when the rows are longer.
+// up to 64 floats of the embedding axis per stage, two stages when the rows are longer (52 KB whatever the
+// width: with 128-float stages, rows of more than 128 floats left two CTAs per SM instead of four).
 // ------------------------------------------------------------------------------------------
-constexpr int FKC = 128;
+constexpr int FKC = 64;
 constexpr int FTQ = 32;                  // query rows per tile
 constexpr int FTHREADS = FTQ * 4;        // 4 x 4 pairs per thread, 64 negative columns per tile
 
@@ -1040,7 +1041,7 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
         }
         float4 s = f4zero();
         if (in) s = sum_splits(reinterpret_cast<const float4*>(p.w.dQpart) + (int64_t)b * d4 + c, (int64_t)p.B * d4, p.split_q);
-        if (p.kind == KIND_L1 && in) {   // the splits hold P; dQ = (row sum of dL/dF) - 2 P
+        if (p.kind == KIND_L1 && in) {         // the splits hold P; dQ = (row sum of dL/dF) - 2 P
             const float rs = p.w.Grow[b];
             s = make_float4(rs - 2.f * s.x, rs - 2.f * s.y, rs - 2.f * s.z, rs - 2.f * s.w);
         }
@@ -1215,9 +1216,10 @@ cudaError_t launch_accum_tma_inst(const AccArgs& aq, const AccArgs& at, cudaStre
 
 template <int KIND>
 cudaError_t launch_accum_tma_kind(const AccArgs& aq, const AccArgs& at, cudaStream_t s) {
-    if (aq.d4 <= 32) return launch_accum_tma_inst<KIND, 1>(aq, at, s);
-    if (aq.d4 <= 64) return launch_accum_tma_inst<KIND, 2>(aq, at, s);
-    return launch_accum_tma_inst<KIND, 4>(aq, at, s);
+    // (distance kinds come here with rows of less than 32 floats only, see pair_backward_serves)
+    if (KIND != KIND_DOT || aq.d4 <= 32) return launch_accum_tma_inst<KIND, 1>(aq, at, s);
+    if (aq.d4 <= 64) return launch_accum_tma_inst<KIND == KIND_DOT ? KIND : KIND_DOT, 2>(aq, at, s);
+    return launch_accum_tma_inst<KIND == KIND_DOT ? KIND : KIND_DOT, 4>(aq, at, s);
 }
 
 // dQ and dT of the pair kinds whose operands are plain rows, in one launch.
@@ -1331,11 +1333,16 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     at.own = p.w.Tneg; at.oth = p.w.Q; at.own_rows = p.N; at.oth_rows = p.B; at.split = p.split_t;
     at.out = p.w.dTpart; at.out2 = nullptr; at.csum = p.w.Cpart;
     if (p.kind != KIND_TH_L1 && p.kind != KIND_TH_L2) {
-        // the two accumulations are independent: one launch holds both
         stage_begin(h, ST_ACCUM_Q, s);
-        KGE_CUDA_CHECK(h, launch_accum_tma(p.kind, aq, at, s));
+        if (pair_backward_serves(h)) {
+            const int rc = launch_pair_backward(h, s);
+            if (rc != KGE_OK) return rc;
+        } else {
+            // the two accumulations are independent: one launch holds both
+            KGE_CUDA_CHECK(h, launch_accum_tma(p.kind, aq, at, s));
+            KGE_LAUNCH_CHECK(h);
+        }
         stage_end(h, ST_ACCUM_Q, s);
-        KGE_LAUNCH_CHECK(h);
     } else {
         // TransH: two launches, concurrent when there is a side stream
         if (side) {

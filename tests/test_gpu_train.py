@@ -482,3 +482,22 @@ def test_out_of_range_id_sets_status_and_does_not_fault(oracle64):
     assert gpu.kge.get_status() == -8      # KGE_ERR_ID_RANGE, reported once, then cleared
     assert gpu.kge.get_status() == 0
     assert np.isfinite(gpu.tables()[0]).all()
+
+
+# one-pass backward of the distance kinds: row widths that fill the thread block, leave a remainder, end at a chunk-size change
+# (64 / 65 float4) and the widest; fewer queries than one thread's rows; row and column ranges with ragged ends; several row
+# tiles per row range
+@pytest.mark.parametrize("d,B,N", [(28, 40, 60), (32, 4, 20), (36, 68, 132), (124, 100, 52), (132, 132, 300), (200, 600, 1500), (256, 72, 1028),
+                                   (260, 12, 36), (512, 52, 100), (128, 4096, 512), (64, 1300, 2052)])
+@pytest.mark.parametrize("score,p", [("transe", 1), ("transe", 2), ("rotate", 1)])
+def test_one_pass_backward_shapes(oracle64, score, p, d, B, N):
+    prob = Problem(E=3000, R=7, T=20000, d=d, score=score, p_norm=p, B=B, N=N, P=2, gamma=4.0, adv_temp=0.5, lr=0.05, graph_seed=29)
+    if score == "rotate":
+        # the direction of a complex residual x is known to 2^-22 (|q| + |t|) / |x| only, without a bound as x goes to 0 (N(0, 1/d)
+        # rows put one positive pair at |x| = 1e-3, 2e-5 beyond the tolerance): parts in [0.1, 0.2] and phases within 0.5 of pi keep |x| > 0.2
+        rng = np.random.default_rng(29)
+        prob.ent[:] = rng.uniform(0.1, 0.2, prob.ent.shape)
+        prob.rel[:] = np.pi + rng.uniform(-0.5, 0.5, prob.rel.shape)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0))
