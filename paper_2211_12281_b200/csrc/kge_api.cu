@@ -253,6 +253,7 @@ int kge_create(const kge_config* cfg, kge_handle** out) {
     h->kw = h->cfg.score == KGE_ROTATE ? c.dim / 2 : c.dim;
     h->bound = h->graph_loaded = false;
     h->streams_ready = false;
+    h->host_flags = nullptr;
     h->launches = 0;
     h->wait_limit = kDefaultWaitLimit;
     h->capture_scores = nullptr;
@@ -306,6 +307,7 @@ void kge_destroy(kge_handle* h) {
         for (int i = 0; i < ST_COUNT; ++i) { cudaEventDestroy(h->prof.a[i]); cudaEventDestroy(h->prof.b[i]); }
     if (h->streams_ready) {
         cudaStreamDestroy(h->side[0]); cudaStreamDestroy(h->side[1]);
+        cudaFreeHost(h->host_flags);
         cudaEventDestroy(h->ev_ids); cudaEventDestroy(h->ev_loss); cudaEventDestroy(h->ev_seg); cudaEventDestroy(h->ev_t);
     }
     delete h;
@@ -400,6 +402,7 @@ int kge_bind(kge_handle* h, float* ent, float* rel, float* relw, float* ent_stat
         KGE_CUDA_CHECK(h, cudaStreamCreateWithFlags(&h->side[1], cudaStreamNonBlocking));
         cudaEvent_t* evs[4] = {&h->ev_ids, &h->ev_loss, &h->ev_seg, &h->ev_t};
         for (cudaEvent_t* e : evs) KGE_CUDA_CHECK(h, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+        KGE_CUDA_CHECK(h, cudaHostAlloc(reinterpret_cast<void**>(&h->host_flags), 64, cudaHostAllocDefault));
         h->streams_ready = true;
     }
     h->bound = true;

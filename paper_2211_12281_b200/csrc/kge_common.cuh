@@ -146,6 +146,7 @@ struct kge_handle {
     int split_mh, split_mt; // K splits of the two dM contractions (heads; tails and negatives)
     bool features_bound;
     bool streams_ready;
+    int32_t* host_flags;    // pinned words full-entity scoring reads its flags back into (made by kge_bind; NULL: pageable memory)
     cudaStream_t side[2];
     cudaEvent_t ev_ids, ev_loss, ev_seg, ev_t;
     bool eb_valid;          // the bf16 copy of the entity table (tensor-core inference) matches the table

@@ -999,8 +999,9 @@ int run_score_all_topk(kge_handle* h, const int32_t* qh, const int32_t* qr, int3
             KGE_LAUNCH_CHECK(h);
             at = p.e_hi;
         }
-        int32_t flags[6];
-        KGE_CUDA_CHECK(h, cudaMemcpyAsync(flags, h->ws.status + 1, sizeof(flags), cudaMemcpyDeviceToHost, s));
+        int32_t words[6];
+        int32_t* const flags = h->host_flags ? h->host_flags : words;
+        KGE_CUDA_CHECK(h, cudaMemcpyAsync(flags, h->ws.status + 1, sizeof(words), cudaMemcpyDeviceToHost, s));
         KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
         if (!flags[0]) break;
         lo = flags[5];

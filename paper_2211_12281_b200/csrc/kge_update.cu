@@ -140,6 +140,48 @@ __global__ void __launch_bounds__(SEG_THREADS) segment_kernel(DedupParams p) {
     if (tid == 0) { L.seg[carry_sm] = n; *L.count = carry_sm; }
 }
 
+// The same for lists of at most SORT_TILE ids, in one launch instead of three: one CTA per list sorts it in shared memory
+// (no more places than the list needs) and reads the segments off.  At such sizes a step is bound by its launches.
+__global__ void __launch_bounds__(SORT_TILE) dedup_small_kernel(DedupParams p) {
+    __shared__ uint64_t k[SORT_TILE];
+    __shared__ int32_t warp_tot[SORT_TILE / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const IdList& L = blockIdx.x == 0 ? p.ent : p.rel;
+    const int n = L.n();
+    int n2 = 32;
+    while (n2 < n) n2 <<= 1;
+    for (int i = tid; i < n2; i += blockDim.x) k[i] = i < n ? ((uint64_t)(uint32_t)checked_id(L.raw(i), L.rows, p.status) << 32) | (uint32_t)i : ~0ull;
+    __syncthreads();
+    for (int size = 2; size <= n2; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            if (tid < n2 / 2) {
+                const int lo = 2 * tid - (tid & (stride - 1)), hi = lo + stride;
+                const bool up = (lo & size) == 0;
+                const uint64_t x = k[lo], y = k[hi];
+                if ((x > y) == up) { k[lo] = y; k[hi] = x; }
+            }
+            __syncthreads();
+        }
+    const bool in = tid < n;
+    const uint64_t key = in ? k[tid] : 0ull;
+    const int32_t id = (int32_t)(key >> 32);
+    const bool head = in && (tid == 0 || (int32_t)(k[tid - 1] >> 32) != id);
+    const unsigned mask = __ballot_sync(0xffffffffu, head);
+    if (lane == 0) warp_tot[warp] = __popc(mask);
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { const int t = warp_tot[w]; if (w < warp) before += t; total += t; }
+    if (in) {
+        const int u = before + __popc(mask & (0xffffffffu >> (31 - lane))) - 1;
+        L.perm[tid] = (int32_t)(uint32_t)key; L.sorted[tid] = id;
+        if (head) { L.uniq[u] = id; L.seg[u] = tid; }
+        L.seg_of[tid] = u;
+        L.seg_done[tid] = 0;
+        if (L.seg_done2) L.seg_done2[tid] = 0;
+    }
+    if (tid == 0) { L.seg[total] = n; *L.count = total; }
+}
+
 struct UpdateJob {
     float* table; float* state;        // [rows, width], optimiser state
     const float* grads;                // [n, width] gradient rows by source position
@@ -390,6 +432,13 @@ int launch_dedup(kge_handle* h, const int32_t* heads, const int32_t* rels, const
     dp.ent_tiles = dedup_tiles(2 * B + N);
     dp.status = w.status;
     const int tiles = dp.ent_tiles + dedup_tiles(B);
+    if (2 * B + N <= SORT_TILE) {
+        stage_begin(h, ST_RANK, s);
+        dedup_small_kernel<<<2, (2 * B + N + 31) / 32 * 32, 0, s>>>(dp);
+        stage_end(h, ST_RANK, s);
+        KGE_LAUNCH_CHECK(h);
+        return KGE_OK;
+    }
     stage_begin(h, ST_RANK, s);
     tile_sort_kernel<<<tiles, SORT_THREADS, 0, s>>>(dp);
     KGE_LAUNCH_CHECK(h);

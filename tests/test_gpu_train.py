@@ -501,3 +501,12 @@ def test_one_pass_backward_shapes(oracle64, score, p, d, B, N):
     gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
     orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
     _check_step(gpu, orc, 0, orc.sample(0))
+
+
+# lists sorted in one launch (up to 1,024 ids: a power of two, between two, the largest) and the first size that is not
+@pytest.mark.parametrize("B,N", [(4, 8), (16, 32), (260, 4), (256, 512), (256, 516)])
+def test_touched_ids_at_the_one_launch_size(oracle64, B, N):
+    prob = Problem(E=150, R=5, T=9000, d=32, score="distmult", B=B, N=N, P=2, lr=0.05, graph_seed=37)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0))
