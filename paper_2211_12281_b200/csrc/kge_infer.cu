@@ -66,8 +66,8 @@ __device__ __forceinline__ void canon_update(float& acc, float4 q, float4 t) {
 }
 
 __device__ __forceinline__ float4 canon_th_x(float u, float4 w, float4 q, float4 t) {
-    return make_float4(__fmaf_rn(u, w.x, __fsub_rn(q.x, t.x)), __fmaf_rn(u, w.y, __fsub_rn(q.y, t.y)),
-                       __fmaf_rn(u, w.z, __fsub_rn(q.z, t.z)), __fmaf_rn(u, w.w, __fsub_rn(q.w, t.w)));
+    const float2 a = sub2(make_float2(q.x, q.y), make_float2(t.x, t.y)), b = sub2(make_float2(q.z, q.w), make_float2(t.z, t.w));
+    return make_float4(__fmaf_rn(u, w.x, a.x), __fmaf_rn(u, w.y, a.y), __fmaf_rn(u, w.z, b.x), __fmaf_rn(u, w.w, b.y));
 }
 __device__ __forceinline__ void canon_th_acc(int kind, float& acc, float4 x) {
     if (kind == KIND_TH_L1) {

@@ -38,6 +38,12 @@ namespace {
 __device__ __forceinline__ float4 f4z() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 // acc += w where a > b: a compare into a predicate and a predicated add.  (A float mask, set.gt giving 1.0 or 0.0,
 // times w in a multiply-add is the same count without the predicate registers and was measured 5-16 % slower.)
+// Four differences in two instructions (see sub2): these loops are bound by issue slots rather than by the pipe.  Score block
+// at B = N = 8192, d = 128: 1640 -> 1531 us (p = 2 at 4096: 377 -> 323); the threshold's multiply-add packed as well: 1551.
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) {
+    const float2 lo = sub2(make_float2(a.x, a.y), make_float2(b.x, b.y)), hi = sub2(make_float2(a.z, a.w), make_float2(b.z, b.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
 __device__ __forceinline__ void add_if_gt(float& acc, float a, float b, float w) {
     asm("{\n .reg .pred p;\n setp.gt.f32 p, %1, %2;\n @p add.f32 %0, %0, %3;\n}\n" : "+f"(acc) : "f"(a), "f"(b), "f"(w));
 }
@@ -170,7 +176,7 @@ __global__ void __launch_bounds__(HB_THREADS, 2) th_block_kernel(ThFwdParams p) 
                             const float uu = u[i][j];
                             const float4 thr = make_float4(fmaf(uu, wv[i].x, qv[i].x), fmaf(uu, wv[i].y, qv[i].y),
                                                            fmaf(uu, wv[i].z, qv[i].z), fmaf(uu, wv[i].w, qv[i].w));
-                            const float4 x = make_float4(thr.x - tv[j].x, thr.y - tv[j].y, thr.z - tv[j].z, thr.w - tv[j].w);
+                            const float4 x = sub4(thr, tv[j]);
                             if (P1) {
                                 acc[i][j] += fabsf(x.x); acc[i][j] += fabsf(x.y); acc[i][j] += fabsf(x.z); acc[i][j] += fabsf(x.w);
                                 add_if_gt(cw[i][j], thr.x, tv[j].x, wv[i].x); add_if_gt(cw[i][j], thr.y, tv[j].y, wv[i].y);
@@ -412,7 +418,7 @@ __global__ void __launch_bounds__(HA_THREADS, 2) th_accum_kernel(ThAccArgs a) {
                                 acc2[i].z = fmaf(cw[i], bv.z, acc2[i].z); acc2[i].w = fmaf(cw[i], bv.w, acc2[i].w);
                             }
                         } else {     // acc = -sum g x, acc2 = sum (c t - u g x)
-                            const float4 x = make_float4(thr.x - bv.x, thr.y - bv.y, thr.z - bv.z, thr.w - bv.w);
+                            const float4 x = sub4(thr, bv);
                             acc[i].x = fmaf(-gw[i], x.x, acc[i].x); acc[i].y = fmaf(-gw[i], x.y, acc[i].y);
                             acc[i].z = fmaf(-gw[i], x.z, acc[i].z); acc[i].w = fmaf(-gw[i], x.w, acc[i].w);
                             if (TCC) {
@@ -437,8 +443,9 @@ __global__ void __launch_bounds__(HA_THREADS, 2) th_accum_kernel(ThAccArgs a) {
                                 acc2[i].z = fmaf(cw[i], wv.z, acc2[i].z); acc2[i].w = fmaf(cw[i], wv.w, acc2[i].w);
                             }
                         } else if (TCC) {   // acc = sum g x
-                            acc[i].x = fmaf(gw[i], thr.x - A[i].x, acc[i].x); acc[i].y = fmaf(gw[i], thr.y - A[i].y, acc[i].y);
-                            acc[i].z = fmaf(gw[i], thr.z - A[i].z, acc[i].z); acc[i].w = fmaf(gw[i], thr.w - A[i].w, acc[i].w);
+                            const float4 x = sub4(thr, A[i]);
+                            acc[i].x = fmaf(gw[i], x.x, acc[i].x); acc[i].y = fmaf(gw[i], x.y, acc[i].y);
+                            acc[i].z = fmaf(gw[i], x.z, acc[i].z); acc[i].w = fmaf(gw[i], x.w, acc[i].w);
                         } else {     // acc = sum (g x + c w)
                             acc[i].x = fmaf(cw[i], wv.x, fmaf(gw[i], thr.x - A[i].x, acc[i].x)); acc[i].y = fmaf(cw[i], wv.y, fmaf(gw[i], thr.y - A[i].y, acc[i].y));
                             acc[i].z = fmaf(cw[i], wv.z, fmaf(gw[i], thr.z - A[i].z, acc[i].z)); acc[i].w = fmaf(cw[i], wv.w, fmaf(gw[i], thr.w - A[i].w, acc[i].w));
