@@ -628,6 +628,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const int item_end = min(p.items, item_begin + *cta_items);
+    if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD) grid_dependency_wait();     // (launched while the kernel before it drains)
 
     // Full-entity scoring with rows of at most 128 coordinates: the column (entity) tile of the
     // current run of items sits in a buffer of its own (2 x 32 KB) and the rest of the stage memory
@@ -881,7 +882,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    if (FORM != DUAL_STEP) { grid_dependency_wait(); allow_dependents(); }
+    grid_dependency_wait();
+    if (FORM != DUAL_STEP) allow_dependents();     // (in a step the SMs left over serve the id sort, not waiting CTAs)
 
     if (warp == 0) {
         if (lane == 0) {
@@ -1222,6 +1224,8 @@ struct CombineParams {
 
 __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    grid_dependency_wait();
+    allow_dependents();
     if (b >= p.B) return;
     const float4* row = p.stat_part + (int64_t)b * p.pieces;
     const float fp = p.fpos[b];
@@ -1253,19 +1257,35 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     p.row_stat[b] = make_float2(m, 1.f / z);
 }
 
-// Norm expansion only: row sums and column sums of the written dL/dF from their pieces,
-// added in ascending piece order.
-__global__ void __launch_bounds__(256) grad_sums_kernel(const float* grow_part, int row_pieces, float* Grow, int B,
+// Norm expansion only: row sums and column sums of the written dL/dF from their pieces, in a fixed order.  CTAs
+// [0, row_ctas): a warp per row, its pieces side by side; the others: 32 columns, eight warps sharing the pieces.  (One
+// thread per row and per column, one piece after the other: 19 us at B = N = 8192.)
+__global__ void __launch_bounds__(256) grad_sums_kernel(const float* grow_part, int row_pieces, float* Grow, int B, int row_ctas,
                                                         const float* gcol_part, int col_pieces, float* Gcol, int N) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < B) {
+    __shared__ float part[8][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    grid_dependency_wait();
+    allow_dependents();
+    if ((int)blockIdx.x < row_ctas) {
+        const int i = blockIdx.x * 8 + warp;
+        if (i >= B) return;
         float t = 0.f;
-        for (int j = 0; j < row_pieces; ++j) t += grow_part[(int64_t)i * row_pieces + j];
-        Grow[i] = t;
-    } else if (i - B < N) {
-        const int n = i - B;
-        float t = 0.f;
-        for (int j = 0; j < col_pieces; ++j) t += gcol_part[(int64_t)j * N + n];
+        for (int j = lane; j < row_pieces; j += 32) t += grow_part[(int64_t)i * row_pieces + j];
+        t = warp_sum(t);
+        if (lane == 0) Grow[i] = t;
+        return;
+    }
+    const int n = ((int)blockIdx.x - row_ctas) * 32 + lane;
+    float t = 0.f;
+    if (n < N) {
+#pragma unroll 8
+        for (int j = warp; j < col_pieces; j += 8) t += gcol_part[(int64_t)j * N + n];
+    }
+    part[warp][lane] = t;
+    __syncthreads();
+    if (warp == 0 && n < N) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) t += part[w][lane];
         Gcol[n] = t;
     }
 }
@@ -1286,6 +1306,9 @@ cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB,
         return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN, A_MN, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + extra_max));
     });
     if (e != cudaSuccess) return e;
+    if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD)
+        return launch_dependent(tc_gemm_kernel<EPI, BN, A_MN, B_MN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem + extra_smem, s,
+                                *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
     tc_gemm_kernel<EPI, BN, A_MN, B_MN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem + extra_smem, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
     return cudaSuccess;
@@ -1356,13 +1379,14 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
     stage_begin(h, ST_LOSS, s);
     CombineParams cp{p.stat_part, p.row_pieces, p.M, w.fpos, c.loss, c.gamma, c.ce_correction, c.loss_scale,
                      reinterpret_cast<float2*>(w.row_stat), w.Lrow, w.gpos};
-    stats_combine_kernel<<<(p.M * 32 + 255) / 256, 256, 0, s>>>(cp);
+    KGE_CUDA_CHECK(h, launch_dependent(stats_combine_kernel, dim3((p.M * 32 + 255) / 256), dim3(256), 0, s, cp));
     KGE_LAUNCH_CHECK(h);
     KGE_CUDA_CHECK(h, launch_fused(EPI_GRAD, p.l2 != 0, ce, h, p, s));
     KGE_LAUNCH_CHECK(h);
     if (p.l2) {
-        grad_sums_kernel<<<(p.M + p.N + 255) / 256, 256, 0, s>>>(w.grow_part, p.row_pieces, w.Grow, p.M,
-                                                                 w.gcol_part, 4 * p.tiles_m, w.Gcol, p.N);
+        const int row_ctas = (p.M + 7) / 8;
+        KGE_CUDA_CHECK(h, launch_dependent(grad_sums_kernel, dim3(row_ctas + (p.N + 31) / 32), dim3(256), 0, s, w.grow_part, p.row_pieces, w.Grow, p.M,
+                                           row_ctas, w.gcol_part, 4 * p.tiles_m, w.Gcol, p.N));
         KGE_LAUNCH_CHECK(h);
     }
     stage_end(h, ST_LOSS, s);
@@ -1395,14 +1419,9 @@ cudaError_t launch_gemm_dual(kge_handle* h, const unsigned char* tmA0, const uns
     const int total = q0.items + q1.items;
     const int rounds = (total + h->num_sms - 1) / h->num_sms;
     const int grid = (total + rounds - 1) / rounds;
-    if (FORM != DUAL_STEP)
-        return launch_dependent(tc_gemm_dual_kernel<BN, PAIR, FORM>, dim3(grid), dim3(32 * (2 + TC_EPI_WARPS)), smem, s,
-                                *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
-                                *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
-    tc_gemm_dual_kernel<BN, PAIR, FORM><<<grid, 32 * (2 + TC_EPI_WARPS), smem, s>>>(
-        *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
-        *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
-    return cudaSuccess;
+    return launch_dependent(tc_gemm_dual_kernel<BN, PAIR, FORM>, dim3(grid), dim3(32 * (2 + TC_EPI_WARPS)), smem, s,
+                            *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
+                            *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
 }
 }  // namespace
 
