@@ -5,7 +5,7 @@
 #include <new>
 #include <vector>
 
-#include "kge_common.cuh"
+#include "kge_sample.cuh"
 
 using namespace kge;
 
@@ -540,12 +540,12 @@ int kge_train_step(kge_handle* h, uint64_t step, float lr, const int32_t* heads,
     int rc;
     if (given == 0) {
         if (!h->graph_loaded) return KGE_ERR_NOT_READY;
-        // The gather kernel can draw the batch itself when the 8 query warps of a CTA share a
-        // triple bucket and the bucket's cumulative weights fit its shared memory.
+        // The gather kernel can draw the batch itself when the 8 query warps of a CTA draw from at most
+        // two triple buckets whose cumulative weights fit its shared memory.
         const kge_config& c = h->cfg;
         const int buckets = c.head_part < 0 ? c.num_parts * c.num_parts : c.num_parts;
         // (with an encoder the features of the batch are projected first: its first kernel draws the batch the same way)
-        fused = fork && (c.batch / buckets) % 8 == 0 && c.num_relations + 1 <= 4096;
+        fused = fork && fused_sample_smem(c.num_relations, c.batch / buckets) >= 0;
         if (!fused) {
             rc = launch_sample(h, step, w.heads, w.rels, w.tails, w.negs, s);
             if (rc != KGE_OK) return rc;

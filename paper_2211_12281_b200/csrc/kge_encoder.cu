@@ -44,7 +44,7 @@ __device__ __forceinline__ void copy_row(uint4* dst, const uint4* src, int n, in
 // B = 512, N = 1024, d = 256, F = 768): CTAs [0, pos_ctas) the feature rows of eight positives' heads and tails (a warp
 // each; with fused_sample it draws its positive first), then those of eight negatives each, then the bf16 copies of the matrices.
 __global__ void __launch_bounds__(256) encoder_prepare_kernel(PrepareParams p) {
-    extern __shared__ uint64_t bucket_wcum[];   // fused sampling: cumulative weights of this CTA's bucket
+    extern __shared__ uint64_t bucket_wcum[];   // fused sampling: cumulative weights of this CTA's buckets
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int blk = blockIdx.x;
     grid_dependency_wait();
@@ -54,13 +54,12 @@ __global__ void __launch_bounds__(256) encoder_prepare_kernel(PrepareParams p) {
     if (blk < p.pos_ctas) {
         const int b = blk * 8 + warp;
         int32_t ih, ir, it;
-        if (p.fused_sample) {            // (the host checks that the slots of a bucket are a multiple of 8)
-            const int64_t base = sample_bucket_base(p.sp, blk * 8 / p.slots_per_bucket);
-            if (p.sp.sample_mode == 0)
-                for (int r = threadIdx.x; r <= (int)p.sp.R; r += blockDim.x) bucket_wcum[r] = p.sp.wcum[base + r];
+        if (p.fused_sample) {
+            stage_bucket_weights(p.sp, p.slots_per_bucket, blk * 8, bucket_wcum);
             __syncthreads();
+            if (b >= p.B) return;
             if (lane == 0) {
-                sample_positive(p.sp, b, base, bucket_wcum, ih, ir, it);
+                sample_positive_staged(p.sp, p.slots_per_bucket, blk * 8, b, bucket_wcum, ih, ir, it);
                 p.sp.heads[b] = ih; p.sp.rels[b] = ir; p.sp.tails[b] = it;
             }
             ih = __shfl_sync(0xffffffffu, ih, 0); it = __shfl_sync(0xffffffffu, it, 0);
@@ -187,7 +186,7 @@ int launch_encoder_forward(kge_handle* h, const int32_t* heads, const int32_t* t
     p.status = w.status;
     const int64_t cast_ctas = ((p.MT ? 2 : 1) * p.m4 + 255) / 256;
     KGE_CUDA_CHECK(h, launch_dependent(encoder_prepare_kernel, dim3((unsigned)(p.pos_ctas + p.neg_ctas + cast_ctas)), dim3(256),
-                                       fused_sample ? (size_t)(c.num_relations + 1) * 8 : 0, s, p));
+                                       fused_sample ? (size_t)fused_sample_smem(c.num_relations, p.slots_per_bucket) : 0, s, p));
     KGE_LAUNCH_CHECK(h);
     return launch_tc_dual_nt(h, h->tm_fh, h->tm_mh, h->tm_ft, c.feat_shared ? h->tm_mh : h->tm_mt, B, B + N, d, F, w.proj,
                              w.proj + (size_t)B * d, s);

@@ -69,6 +69,29 @@ __device__ __forceinline__ void sample_positive(const SampleParams& p, int slot,
     h = p.gh[idx]; r = p.gr[idx]; t = p.gt[idx];
 }
 
+// The cumulative weights of the one or two buckets that eight consecutive batch slots from w0 on draw from (the host checks
+// that a bucket has at least eight slots), fetched side by side by the whole CTA: [R + 1] words each in `sm`.  No barrier.
+__device__ __forceinline__ void stage_bucket_weights(const SampleParams& p, int slots_per_bucket, int w0, uint64_t* sm) {
+    if (p.sample_mode != 0) return;
+    const int s0 = w0 / slots_per_bucket, s1 = (w0 + 7 < p.B ? w0 + 7 : p.B - 1) / slots_per_bucket;
+    const int64_t b0 = sample_bucket_base(p, s0), b1 = sample_bucket_base(p, s1);
+    for (int r = threadIdx.x; r <= (int)p.R; r += blockDim.x) {
+        sm[r] = p.wcum[b0 + r];
+        if (s1 != s0) sm[p.R + 1 + r] = p.wcum[b1 + r];
+    }
+}
+// Positive of slot `slot` of those eight, from the staged weights.
+__device__ __forceinline__ void sample_positive_staged(const SampleParams& p, int slots_per_bucket, int w0, int slot, const uint64_t* sm,
+                                                       int32_t& h, int32_t& r, int32_t& t) {
+    const int own = slot / slots_per_bucket;
+    sample_positive(p, slot, sample_bucket_base(p, own), own == w0 / slots_per_bucket ? sm : sm + p.R + 1, h, r, t);
+}
+// Bytes those weights take, or -1 where a kernel of eight slots per CTA does not draw the batch itself.
+inline int64_t fused_sample_smem(int64_t R, int slots_per_bucket) {
+    const int64_t words = (R + 1) * (slots_per_bucket % 8 == 0 ? 1 : 2);
+    return slots_per_bucket >= 8 && words <= 4096 ? words * 8 : -1;
+}
+
 // Negative of slot n: uniform in partition n div (N / P).
 __device__ __forceinline__ int32_t sample_negative(const SampleParams& p, int n) {
     const int j = n / (p.N / p.P);

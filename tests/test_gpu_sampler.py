@@ -43,6 +43,18 @@ def test_step_that_samples_its_own_batch_uses_the_oracles_batch(oracle64, name):
     assert gpu.kge.get_status() == 0
 
 
+# slots per bucket: 150 (thread blocks that straddle two buckets), 9 and 8 (the fewest), 7 (too few: sampled in a launch of
+# its own), uniform sampling across a straddled boundary, more weights than two buckets may stage
+@pytest.mark.parametrize("B,P,R,mode", [(600, 2, 20, 0), (36, 2, 20, 0), (72, 3, 20, 0), (28, 2, 20, 0), (100, 2, 20, 1), (100, 2, 2100, 0)])
+def test_step_that_samples_across_bucket_boundaries(oracle64, B, P, R, mode):
+    prob = Problem(E=999, R=R, T=60000, d=16, score="transe", B=B, N=6 * P, P=P, sample_mode=mode, relation_zipf=1.0, graph_seed=41)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    for step in (0, 3, 2**32 + 5):
+        gpu.kge.train_step(step, 0.01)
+        assert (gpu.kge.debug_export("BATCH") == np.concatenate(orc.sample(step))).all(), step
+    assert gpu.kge.get_status() == 0
+
+
 def test_graph_load_reports_empty_bucket_and_bad_ids():
     import paper_2211_12281_b200 as K
     prob = Problem(E=40, R=5, T=4, d=16, score="transe", B=8, N=4, P=2)
