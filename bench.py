@@ -106,10 +106,11 @@ MIX_NAMES = {MIX_FMA: "fma", MIX_SUB_ABS: "sub+abs-add", MIX_CMP_ADD: "compare+p
 # mixes of instructions / measured rate of that mix (special-function instructions run beside the others: the larger
 # of the two times counts).
 STAGE_OPS = {
-    "transe1": dict(block=[(2, MIX_SUB_ABS)], accum=[(4, MIX_CMP_ADD)]),
-    "transe2": dict(block=[(2, MIX_FMA)], accum=[(4, MIX_FMA)]),
+    # (backward of the distance kinds: both sides in one pass, the difference formed once)
+    "transe1": dict(block=[(2, MIX_SUB_ABS)], accum=[(3, MIX_CMP_ADD)]),
+    "transe2": dict(block=[(2, MIX_FMA)], accum=[(3, MIX_FMA)]),
     # per real coordinate: two subtractions, a product and a multiply-add per complex component, then half a square root
-    "rotate1": dict(block=[(2, MIX_SUB_ABS), (0.5, MIX_FMA), (0.5, MIX_SFU)], accum=[(2, MIX_SUB_ABS), (1, MIX_FMA), (2, MIX_FMA), (1.0, MIX_SFU)]),
+    "rotate1": dict(block=[(2, MIX_SUB_ABS), (0.5, MIX_FMA), (0.5, MIX_SFU)], accum=[(1, MIX_SUB_ABS), (1.5, MIX_FMA), (2, MIX_FMA), (0.5, MIX_SFU)]),
     "distmult1": dict(block=[(1, MIX_FMA)], accum=[(2, MIX_FMA)]),
     "complex1": dict(block=[(1, MIX_FMA)], accum=[(2, MIX_FMA)]),
     # TransH p = 1.  forward: w.t (fma), threshold fma(u, w, q), residual and |.| accumulate (sub + abs-add), the pair's

@@ -16,6 +16,10 @@
 // A CTA works on a rectangle: the query rows [q_begin, q_end), a tile of PB_R x groups rows at a time, against its
 // columns.  Every column range gives one slab of dQ, every row range one of dT; the chain kernel adds the slabs in
 // order.  No atomics: results are bit-reproducible.
+//
+// Measured against a pass per side: TransE p = 1, 1024 x 1024 x 128 31.4 -> 25.1 us, 4096 x 4096 389 -> 362; p = 2, 4096 x 4096
+// 410 -> 330; 512 x 1024 x 256 36 -> 25; RotatE moduli 600 x 1500 x 200 118 -> 56, 2048 x 2048 x 200 500 -> 236.  Rows of fewer
+// than 32 floats keep the pass per side: a group is then so narrow that a thread would stage sixteen or more weights per chunk.
 #include <algorithm>
 
 #include "kge_common.cuh"
@@ -73,7 +77,7 @@ inline size_t pb_smem(int d4, int groups) {
 }
 
 // C: rows of the other side per chunk; WPT: weights of a chunk a thread brings in; D4: the row width when 256 threads are
-// whole groups of it (addresses and the groups' reduction are then constants: 4.5 -> 3.8 instructions per element at p = 1), or 0.
+// whole groups of it (addresses and the groups' reduction are then constants: 4.5 -> 4.1 instructions per element at p = 1), or 0.
 template <int KIND, int C, int WPT, int D4>
 __global__ void __launch_bounds__(256, 2) pair_backward_kernel(PairBackParams p) {
     extern __shared__ __align__(128) unsigned char pb_smem_raw[];
