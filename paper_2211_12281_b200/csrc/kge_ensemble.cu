@@ -116,7 +116,8 @@ __device__ bool ens_hash_query(const EnsParams& p, const int q, const int log2_s
                 const uint32_t sh = (uint32_t)(ml[u] & 3) * 8u;
                 if (want >= 0 && (need || (atomicAdd(&cell[(ml[u] >> 2) * slots + h], (uint32_t)(e - ml[u] * p.K + 1) << sh) >> sh & 0xffu) != 0u)) bad = 1;
             }
-            if (*reinterpret_cast<volatile int*>(&bad)) break;
+            // (by vote: the lanes read the flag at different times, and those that stay vote with the whole warp again)
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bad))) break;
         }
         __syncthreads();
         if (bad) return false;

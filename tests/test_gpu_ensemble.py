@@ -57,6 +57,23 @@ def test_ensemble_union_sizes(oracle64, M, nq, K, E, power):
     assert (sc == o_sc).all()
 
 
+# 20 lists of 254 places are 4,064 entries in the first block of models, several rounds of the insertion loop: an entity twice in
+# one list, or a union beyond the table, is seen in the first of them by some lanes of a warp only, with rounds still to come
+@pytest.mark.parametrize("twice", [True, False])
+def test_ensemble_gives_up_on_a_table_with_rounds_to_come(oracle64, twice):
+    rng = np.random.default_rng(7)
+    M, nq, K = 20, 64, 254
+    E = 260 if twice else 1_000_000
+    lists = np.stack([np.stack([rng.permutation(E)[:K] if twice else rng.integers(0, E, K) for _ in range(nq)]) for _ in range(M)]).astype(np.int32)
+    if twice:
+        for q in range(nq):
+            lists[q % 2, q, 3 + q] = lists[q % 2, q, q]
+    ids, sc = _gpu_ensemble(lists, -0.5, 10)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, -0.5, 10)
+    assert (ids == o_ids).all()
+    assert (sc == o_sc).all()
+
+
 def test_ensemble_fewer_candidates_than_places_and_limits(oracle64):
     import torch
     import paper_2211_12281_b200 as K
