@@ -14,8 +14,10 @@
 // that order), in fp64; n rounds of a block-wide maximum then pick the result.  The rank scores k^p
 // come from a table the caller fills with kge_ensemble_rank_scores, so the sums are plain IEEE
 // additions of given numbers in a fixed order: the result does not depend on any device math library.
-// A query whose union does not fit the table, or with an entity twice in one list, is left to a second
-// launch, which has a larger table and, behind that, a sort of all entries by (entity id, model, position).
+// A query whose union would fill more than three quarters of the table is left to a second launch, which
+// gathers it in a larger table, as many passes over the lists as its entries can need: a pass takes the
+// entities whose hash falls into its part, so every sum keeps its order.  A query with an entity twice in
+// one list (and lists of more than 254 places) is left to a third, which sorts all entries by (entity id, model, position).
 #include <algorithm>
 #include <cmath>
 
@@ -24,10 +26,10 @@
 namespace kge {
 namespace {
 
-constexpr int ENS_THREADS = 512;            // the sort
+constexpr int ENS_THREADS = 1024;           // at most
 constexpr int ENS_MAX_ENTRIES = 16384;      // M * K per query (85 models x top-100 = 8,500 fits)
 constexpr int ENS_MAX_K = 254;              // positions are kept as bytes (position + 1); longer lists are sorted
-constexpr int ENS_LEFT = -2;                // first output id of a query the first launch left to the second
+constexpr int ENS_LEFT = -2, ENS_SORT = -3;    // first output id of a query left to the second launch (too large a union) or to the sort
 
 struct EnsParams {
     const int32_t* lists;      // [M, nq, K]
@@ -35,6 +37,8 @@ struct EnsParams {
     int M, nq, K, top_n, n2;   // n2 = M * K rounded up to a power of two
     int32_t* out_ids; double* out_scores;
     int log2_slots;            // first launch: slots of the hash table
+    int left_log2, log2_parts; // second launch: slots of its table, passes over the lists
+    int sort_here;             // second launch: its memory holds the sort too
     uint32_t inv_k;            // ceil(2^32 / K): e / K = umulhi(e, inv_k) for every entry index e of a block of models; 0: K = 1
 };
 
@@ -44,12 +48,15 @@ __device__ __forceinline__ bool ens_before(double sa, int32_t ia, double sb, int
 // Hash form.  Shared memory per slot: entity id, fp64 sum, MB position bytes, one entry of the list of
 // occupied slots.  The cell words of a slot lie `slots` words apart, so that the slots a warp touches
 // (random, one model) spread over the banks.
-// Returns false (all threads) if the union does not fit or a list names an entity twice.
+// A table that may overflow is given up at three quarters of its slots, after the block of models that takes it
+// beyond or where a probe grows long: linear probing costs tens of steps per entry from there on (thousands near the
+// last slot: 85 lists of 100 random ids for 15,000 queries took 134 ms that way, the sort alone 37).
 // ------------------------------------------------------------------------------------------
 template <int MB>
 constexpr size_t ens_slot_bytes() { return sizeof(double) + sizeof(int32_t) + MB + sizeof(uint16_t); }
 template <int MB>
-inline size_t ens_hash_smem(int slots, int K) { return (size_t)slots * ens_slot_bytes<MB>() + (size_t)(K + 1) * sizeof(double); }
+constexpr size_t ens_hash_smem(int slots, int K) { return (size_t)slots * ens_slot_bytes<MB>() + (size_t)(K + 1) * sizeof(double); }
+enum { ENS_BAD_FULL = 1, ENS_BAD_TWICE = 2 };
 
 // Order-preserving map of a double to an unsigned integer (no NaN).
 __device__ __forceinline__ uint64_t ens_ordered(double s) {
@@ -60,145 +67,177 @@ __device__ __forceinline__ double ens_unordered(uint64_t k) {
     return __longlong_as_double((long long)((k >> 63) ? k & 0x7fffffffffffffffull : ~k));
 }
 
+// The table of the entities of query q whose hash falls into part `part` of 2^log2_parts.
 template <int MB>
-__device__ bool ens_hash_query(const EnsParams& p, const int q, const int log2_slots, unsigned char* smem) {
-    constexpr int WORDS = MB / 4;
-    const int slots = 1 << log2_slots, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
-    double* sum = reinterpret_cast<double*>(smem);                              // [slots]
-    double* tab = sum + slots;                                                  // [K + 1] absent score, then positions 1 .. K
-    int32_t* key = reinterpret_cast<int32_t*>(tab + p.K + 1);                   // [slots] entity id or -1
-    uint32_t* cell = reinterpret_cast<uint32_t*>(key + slots);                  // [WORDS][slots] bytes: position + 1 in the block's models
-    uint16_t* used = reinterpret_cast<uint16_t*>(cell + (size_t)WORDS * slots); // [slots] occupied slots, in order of arrival
-    __shared__ int n_used, bad;
-    __shared__ uint64_t red_s[2][32];
-    __shared__ int32_t red_i[2][32];
-    for (int i = tid; i < slots; i += nthr) key[i] = -1;
-    for (int i = tid; i < slots * WORDS; i += nthr) cell[i] = 0u;
-    for (int i = tid; i <= p.K; i += nthr) tab[i] = p.table[i == 0 ? p.K : i - 1];
-    if (tid == 0) { n_used = 0; bad = 0; }
-    __syncthreads();
-    const double absent = tab[0];
-    double before = 0.0;                    // an entity's sum over the models ahead of the block it first appears in
-    int seen = 0;                           // occupied slots after the blocks so far
-    for (int m0 = 0; m0 < p.M; m0 += MB) {
-        const int mb = min(MB, p.M - m0), entries = mb * p.K;
-        const int32_t* src = p.lists + ((int64_t)m0 * p.nq + q) * p.K;
-        const int64_t step = (int64_t)(p.nq - 1) * p.K;                         // list m + 1 begins `step` further than list m ends
-        for (int e0 = 0; e0 < entries; e0 += 4 * nthr) {
-            int32_t id[4];
-            int ml[4];
+struct EnsTable {
+    double* sum;          // [slots]
+    double* tab;          // [K + 1] absent score, then positions 1 .. K
+    int32_t* key;         // [slots] entity id or -1
+    uint32_t* cell;       // [MB / 4][slots] bytes: position + 1 in the block's models
+    uint16_t* used;       // [slots] occupied slots, in order of arrival
+    int n;                // of them
+
+    __device__ EnsTable(unsigned char* smem, int slots, int K)
+        : sum(reinterpret_cast<double*>(smem)), tab(sum + slots), key(reinterpret_cast<int32_t*>(tab + K + 1)),
+          cell(reinterpret_cast<uint32_t*>(key + slots)), used(reinterpret_cast<uint16_t*>(cell + (size_t)(MB / 4) * slots)), n(0) {}
+
+    // 0, or (all threads) why the table was given up: more than `limit` entities, or an entity twice in one list.
+    __device__ int gather(const EnsParams& p, const int q, const int log2_slots, const int limit, const int part, const int log2_parts) {
+        constexpr int WORDS = MB / 4;
+        const int slots = 1 << log2_slots, tid = threadIdx.x, nthr = blockDim.x;
+        __shared__ int n_used, twice;
+        for (int i = tid; i < slots; i += nthr) key[i] = -1;
+        for (int i = tid; i < slots * WORDS; i += nthr) cell[i] = 0u;
+        for (int i = tid; i <= p.K; i += nthr) tab[i] = p.table[i == 0 ? p.K : i - 1];
+        if (tid == 0) { n_used = 0; twice = 0; }
+        __syncthreads();
+        const double absent = tab[0];
+        double before = 0.0;                    // an entity's sum over the models ahead of the block it first appears in
+        int seen = 0;                           // occupied slots after the blocks so far
+        for (int m0 = 0; m0 < p.M; m0 += MB) {
+            const int mb = min(MB, p.M - m0), entries = mb * p.K;
+            const int32_t* src = p.lists + ((int64_t)m0 * p.nq + q) * p.K;
+            const int64_t step = (int64_t)(p.nq - 1) * p.K;                     // list m + 1 begins `step` further than list m ends
+            for (int e0 = 0; e0 < entries; e0 += 4 * nthr) {
+                int32_t id[4];
+                int ml[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {                                       // four loads in flight
-                const int e = e0 + u * nthr + tid;
-                ml[u] = p.inv_k ? (int)__umulhi((uint32_t)e, p.inv_k) : e;
-                id[u] = e < entries ? src[e + ml[u] * step] : -1;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                // the warp probes together: left to themselves, the lanes that need one probe more run the rest of the body on their own
-                const int e = e0 + u * nthr + tid, want = id[u];
-                uint32_t h = (uint32_t)want * 0x9E3779B1u >> (32 - log2_slots);
-                int32_t k = want < 0 ? want : *reinterpret_cast<volatile int32_t*>(key + h);       // (unused places of a list hold -1)
-                bool need = k != want;
-                for (int probe = 0; probe < slots && __any_sync(0xffffffffu, need); ++probe) {
-                    if (need && k == -1) {
-                        k = atomicCAS(key + h, -1, want);
-                        if (k == -1) { used[atomicAdd(&n_used, 1)] = (uint16_t)h; k = want; }
-                    }
-                    need = need && k != want;
-                    if (need) {
-                        h = (h + 1) & (uint32_t)(slots - 1);
-                        k = *reinterpret_cast<volatile int32_t*>(key + h);
-                        need = k != want;
-                    }
-                    if ((probe & 15) == 15 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bad))) break;
+                for (int u = 0; u < 4; ++u) {                                   // four loads in flight
+                    const int e = e0 + u * nthr + tid;
+                    ml[u] = p.inv_k ? (int)__umulhi((uint32_t)e, p.inv_k) : e;
+                    id[u] = e < entries ? src[e + ml[u] * step] : -1;
                 }
-                const uint32_t sh = (uint32_t)(ml[u] & 3) * 8u;
-                if (want >= 0 && (need || (atomicAdd(&cell[(ml[u] >> 2) * slots + h], (uint32_t)(e - ml[u] * p.K + 1) << sh) >> sh & 0xffu) != 0u)) bad = 1;
-            }
-            // (by vote: the lanes read the flag at different times, and those that stay vote with the whole warp again)
-            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bad))) break;
-        }
-        __syncthreads();
-        if (bad) return false;
-        const int total = n_used;
-        for (int i = tid; i < total; i += nthr) {
-            const int h = used[i];
-            double s = i < seen ? sum[h] : before;
-            for (int w = 0; 4 * w < mb; ++w) {
-                const uint32_t c = cell[w * slots + h];
-                cell[w * slots + h] = 0u;
-                if (c == 0u && absent == 0.0) continue;                         // (s is never -0: adding 0 leaves it as it is)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (4 * w + j < mb) s += tab[c >> (8 * j) & 0xffu];
+                for (int u = 0; u < 4; ++u) {
+                    // the warp probes together: left to themselves, the lanes that need one probe more run the rest of the body on their own
+                    const int e = e0 + u * nthr + tid;
+                    int want = id[u];
+                    const uint32_t hash = (uint32_t)want * 0x9E3779B1u;
+                    uint32_t h = hash >> (32 - log2_slots);
+                    if (log2_parts && (int)(hash >> (32 - log2_slots - log2_parts) & ((1u << log2_parts) - 1u)) != part) want = -1;
+                    int32_t k = want < 0 ? want : *reinterpret_cast<volatile int32_t*>(key + h);   // (unused places of a list hold -1)
+                    bool need = k != want;
+                    for (int probe = 0; probe < slots && __any_sync(0xffffffffu, need); ++probe) {
+                        if (need && k == -1) {
+                            k = atomicCAS(key + h, -1, want);
+                            if (k == -1) {
+                                used[atomicAdd(&n_used, 1)] = (uint16_t)h; k = want;
+                            }
+                        }
+                        need = need && k != want;
+                        if (need) {
+                            h = (h + 1) & (uint32_t)(slots - 1);
+                            k = *reinterpret_cast<volatile int32_t*>(key + h);
+                            need = k != want;
+                        }
+                        // (by vote: a lane on its own would leave the others to vote without it)
+                        if ((probe & 15) == 15 && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&twice) != 0 || *reinterpret_cast<volatile int*>(&n_used) > limit)) break;
+                    }
+                    const uint32_t sh = (uint32_t)(ml[u] & 3) * 8u;
+                    if (want >= 0 && !need && (atomicAdd(&cell[(ml[u] >> 2) * slots + h], (uint32_t)(e - ml[u] * p.K + 1) << sh) >> sh & 0xffu) != 0u)
+                        twice = 1;
+                }
             }
-            sum[h] = s;
+            __syncthreads();
+            if (twice) return ENS_BAD_TWICE;
+            const int total = n_used;
+            if (total > limit) return ENS_BAD_FULL;
+            for (int i = tid; i < total; i += nthr) {
+                const int h = used[i];
+                double s = i < seen ? sum[h] : before;
+                for (int w = 0; 4 * w < mb; ++w) {
+                    const uint32_t c = cell[w * slots + h];
+                    cell[w * slots + h] = 0u;
+                    if (c == 0u && absent == 0.0) continue;                     // (s is never -0: adding 0 leaves it as it is)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (4 * w + j < mb) s += tab[c >> (8 * j) & 0xffu];
+                }
+                sum[h] = s;
+            }
+            seen = total;
+            if (absent != 0.0) for (int m = 0; m < mb; ++m) before += absent;
+            __syncthreads();
         }
-        seen = total;
-        if (absent != 0.0) for (int m = 0; m < mb; ++m) before += absent;
-        __syncthreads();
+        n = seen;
+        return 0;
     }
-    // a thread's best candidate stays in registers until it is taken
-    auto best_of_mine = [&](uint64_t& bs, int32_t& bi, int& bp) {
+
+    // This thread's best entity that is not taken: its ordered score (0: none), id and slot.
+    __device__ void best_of_mine(uint64_t& bs, int32_t& bi, int& bp) const {
         bs = 0; bi = INT32_MAX; bp = -1;
-        for (int i = tid; i < seen; i += nthr) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
             const int h = used[i];
             if (key[h] < 0) continue;
             const uint64_t s = ens_ordered(sum[h]);
             if (bp < 0 || s > bs || (s == bs && key[h] < bi)) { bs = s; bi = key[h]; bp = h; }
         }
-    };
+    }
+};
+
+// Warp maximum under (score descending, id ascending): the score's two halves, then the id.
+__device__ __forceinline__ void ens_warp_best(uint64_t s, int32_t id, uint64_t& os, int32_t& oi) {
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32) == hi ? (uint32_t)s : 0u);
+    os = (uint64_t)hi << 32 | lo;
+    oi = __reduce_min_sync(0xffffffffu, s == os ? id : INT32_MAX);
+}
+
+// The table's entities from the best on, one per round, to `take(round, score, id)` (called by all threads with the same
+// values; no score maps to 0) until it returns false or none is left.  A thread's best stays in registers until it is taken.
+template <int MB, class Take>
+__device__ void ens_select(EnsTable<MB>& t, Take take) {
+    __shared__ uint64_t red_s[2][32];
+    __shared__ int32_t red_i[2][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     uint64_t bs; int32_t bi; int bp;
-    best_of_mine(bs, bi, bp);
-    // warp maximum under (score descending, id ascending): the score's two halves, then the id
-    auto warp_best = [&](uint64_t s, int32_t id, uint64_t& os, int32_t& oi) {
-        const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32));
-        const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(s >> 32) == hi ? (uint32_t)s : 0u);
-        os = (uint64_t)hi << 32 | lo;
-        oi = __reduce_min_sync(0xffffffffu, s == os ? id : INT32_MAX);
-    };
+    t.best_of_mine(bs, bi, bp);
     uint64_t ws; int32_t wi;                // the warp's best
-    warp_best(bs, bi, ws, wi);
-    for (int r = 0; r < p.top_n; ++r) {
+    ens_warp_best(bs, bi, ws, wi);
+    for (int r = 0;; ++r) {
         if (lane == 0) { red_s[r & 1][warp] = ws; red_i[r & 1][warp] = wi; }
         __syncthreads();
         uint64_t s; int32_t id;
-        warp_best(lane < nwarps ? red_s[r & 1][lane] : 0ull, lane < nwarps ? red_i[r & 1][lane] : INT32_MAX, s, id);   // (every warp for itself)
-        const bool have = s != 0ull;                                            // (no score maps to 0)
-        if (tid == 0) {
-            p.out_ids[(int64_t)q * p.top_n + r] = have ? id : -1;               // fewer candidates than places: -1 and -inf
-            if (p.out_scores) p.out_scores[(int64_t)q * p.top_n + r] = have ? ens_unordered(s) : -INFINITY;
-        }
-        if (have && s == ws && id == wi) {                                      // taken (ids are distinct: one warp, one thread)
-            if (bp >= 0 && bi == id) { key[bp] = -1; best_of_mine(bs, bi, bp); }
+        ens_warp_best(lane < nwarps ? red_s[r & 1][lane] : 0ull, lane < nwarps ? red_i[r & 1][lane] : INT32_MAX, s, id);   // (every warp for itself)
+        if (!take(r, s, id)) return;
+        if (s != 0ull && s == ws && id == wi) {                                 // taken (ids are distinct: one warp, one thread)
+            if (bp >= 0 && bi == id) { t.key[bp] = -1; t.best_of_mine(bs, bi, bp); }
             __syncwarp();
-            warp_best(bs, bi, ws, wi);
+            ens_warp_best(bs, bi, ws, wi);
         }
     }
-    return true;
 }
 
-// First launch: one CTA per query, 16 models at a time, at most 1,024 slots (31 KB: seven CTAs per SM).  85 x top-100 lists of
-// 15,000 queries: 36.7 ms as a sort, 0.93 ms with 32 models at a time (four CTAs), 0.87 with 8, 0.81 with 16; 128 threads 1.00 ms.
-// Bound by instruction issue (about 48,000 warp instructions a query, 74 % of the slots), not by the 510 MB of lists (78 us).
-constexpr int ENS_MB = 16, ENS_MAX_LOG2 = 10;
+__device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64_t s, int32_t id) {
+    p.out_ids[(int64_t)q * p.top_n + r] = s != 0ull ? id : -1;                  // fewer candidates than places: -1 and -inf
+    if (p.out_scores) p.out_scores[(int64_t)q * p.top_n + r] = s != 0ull ? ens_unordered(s) : -INFINITY;
+}
+
+// The whole of a query in one table.
 template <int MB>
-__global__ void __launch_bounds__(256) ensemble_hash_kernel(EnsParams p) {
-    extern __shared__ __align__(16) unsigned char ens_smem[];
-    allow_dependents();
-    if (!ens_hash_query<MB>(p, blockIdx.x, p.log2_slots, ens_smem) && threadIdx.x == 0) p.out_ids[(int64_t)blockIdx.x * p.top_n] = ENS_LEFT;
+__device__ int ens_hash_query(const EnsParams& p, const int q, const int log2_slots, const int limit, unsigned char* smem) {
+    EnsTable<MB> t(smem, 1 << log2_slots, p.K);
+    const int bad = t.gather(p, q, log2_slots, limit, 0, 0);
+    if (bad) return bad;
+    ens_select(t, [&](int r, uint64_t s, int32_t id) {
+        if (r >= p.top_n) return false;
+        if (threadIdx.x == 0) ens_put(p, q, r, s, id);
+        return true;
+    });
+    return 0;
 }
 
-// The general form: all entries of query q sorted by (entity id, model, position) in shared memory.
+// The general form: all entries of query q sorted by (entity id, model, position) in shared memory.  NT: the threads of the
+// CTA where they are known, or 0.
+template <int NT>
 __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* ens_smem) {
     uint64_t* key = reinterpret_cast<uint64_t*>(ens_smem);                      // [n2] (id, model, position); later the candidates' scores
     int32_t* cid = reinterpret_cast<int32_t*>(key + p.n2);                      // [n2] candidate id at the first entry of its run, else -1
     __shared__ double red_s[ENS_THREADS / 32];
     __shared__ int32_t red_i[ENS_THREADS / 32], red_pos[ENS_THREADS / 32];
     __shared__ int32_t win_pos;
-    const int tid = threadIdx.x, n = p.M * p.K;
-    for (int i = tid; i < p.n2; i += ENS_THREADS) {
+    const int tid = threadIdx.x, nthr = NT ? NT : (int)blockDim.x, n = p.M * p.K;
+    for (int i = tid; i < p.n2; i += nthr) {
         uint64_t k = ~0ull;
         if (i < n) {
             const int m = i / p.K, pos = i - m * p.K;
@@ -210,7 +249,7 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
     __syncthreads();
     for (int size = 2; size <= p.n2; size <<= 1)
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < p.n2 / 2; t += ENS_THREADS) {
+            for (int t = tid; t < p.n2 / 2; t += nthr) {
                 const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
                 const bool up = (lo & size) == 0;
                 const uint64_t x = key[lo], y = key[hi];
@@ -219,7 +258,7 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
             __syncthreads();
         }
     // runs of equal ids: mark their first entries (reads only)
-    for (int i = tid; i < p.n2; i += ENS_THREADS) {
+    for (int i = tid; i < p.n2; i += nthr) {
         const uint64_t k = key[i];
         const bool head = k != ~0ull && (i == 0 || (key[i - 1] >> 32) != (k >> 32));
         cid[i] = head ? (int32_t)(k >> 32) : -1;
@@ -227,7 +266,7 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
     __syncthreads();
     // every run is summed by the thread of its first entry, which then keeps the score in that entry's place
     const double absent = p.table[p.K];
-    for (int i = tid; i < p.n2; i += ENS_THREADS) {
+    for (int i = tid; i < p.n2; i += nthr) {
         if (cid[i] < 0) continue;
         const uint32_t id = (uint32_t)cid[i];
         int j = i;
@@ -245,7 +284,7 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
     __syncthreads();
     for (int r = 0; r < p.top_n; ++r) {
         double bs = -INFINITY; int32_t bi = INT32_MAX, bp = -1;
-        for (int i = tid; i < p.n2; i += ENS_THREADS) {
+        for (int i = tid; i < p.n2; i += nthr) {
             const int32_t id = cid[i];
             if (id < 0) continue;
             const double s = __longlong_as_double((long long)key[i]);
@@ -260,7 +299,7 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
         if ((tid & 31) == 0) { red_s[tid >> 5] = bs; red_i[tid >> 5] = bi; red_pos[tid >> 5] = bp; }
         __syncthreads();
         if (tid == 0) {
-            for (int w = 1; w < ENS_THREADS / 32; ++w)
+            for (int w = 1; w < nthr / 32; ++w)
                 if (red_pos[w] >= 0 && (bp < 0 || ens_before(red_s[w], red_i[w], bs, bi))) { bs = red_s[w]; bi = red_i[w]; bp = red_pos[w]; }
             p.out_ids[(int64_t)q * p.top_n + r] = bp >= 0 ? bi : -1;          // fewer candidates than places: -1 and -inf
             if (p.out_scores) p.out_scores[(int64_t)q * p.top_n + r] = bp >= 0 ? bs : -INFINITY;
@@ -273,33 +312,114 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
 }
 
 // Lists of more than ENS_MAX_K places: every query takes the general form.
-__global__ void __launch_bounds__(ENS_THREADS) ensemble_sort_kernel(EnsParams p) {
+template <int NT>
+__global__ void __launch_bounds__(NT) ensemble_sort_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
-    ens_sort_query(p, blockIdx.x, ens_smem);
+    ens_sort_query<NT>(p, blockIdx.x, ens_smem);
 }
 
-// Second launch: the queries the first one left (usually none), shared out over the CTAs.
-constexpr int ENS_BIG_MB = 8, ENS_BIG_LOG2 = 13;      // 8,192 slots, eight models at a time: 180 KB
-__global__ void __launch_bounds__(ENS_THREADS) ensemble_left_kernel(EnsParams p) {
-    extern __shared__ __align__(16) unsigned char ens_smem[];
+// The queries that earlier launches left, shared out over the CTAs: `serve(query, left to the sort)`, called by all threads.
+template <class Serve>
+__device__ void ens_left(const EnsParams& p, bool table, bool sort, Serve serve) {
     __shared__ int32_t todo[ENS_THREADS];
     __shared__ int n_todo;
-    grid_dependency_wait();
-    for (int64_t base = blockIdx.x; base < p.nq; base += (int64_t)gridDim.x * ENS_THREADS) {
+    for (int64_t base = blockIdx.x; base < p.nq; base += (int64_t)gridDim.x * blockDim.x) {
         __syncthreads();
         if (threadIdx.x == 0) n_todo = 0;
         __syncthreads();
         const int64_t q = base + (int64_t)gridDim.x * threadIdx.x;
-        if (q < p.nq && p.out_ids[q * p.top_n] == ENS_LEFT) todo[atomicAdd(&n_todo, 1)] = (int32_t)q;
+        const int32_t mark = q < p.nq ? p.out_ids[q * p.top_n] : 0;
+        if ((table && mark == ENS_LEFT) || (sort && mark == ENS_SORT)) todo[atomicAdd(&n_todo, 1)] = mark == ENS_LEFT ? (int32_t)q : ~(int32_t)q;
         __syncthreads();
         const int n = n_todo;
         for (int i = 0; i < n; ++i) {
+            const int32_t entry = todo[i];
             __syncthreads();
-            const bool done = ens_hash_query<ENS_BIG_MB>(p, todo[i], ENS_BIG_LOG2, ens_smem);
-            __syncthreads();
-            if (!done) ens_sort_query(p, todo[i], ens_smem);
+            serve(entry < 0 ? ~entry : entry, entry < 0);
         }
     }
+}
+
+template <int NT>
+__device__ __noinline__ void ens_sort_call(const EnsParams& p, int q, unsigned char* smem) { ens_sort_query<NT>(p, q, smem); }
+
+// The queries left to the sort, where the second launch's memory is more than the sort's.  Four times as many CTAs as are resident,
+// so that those of an SM are not all in the same phase (15,000 queries of 30 lists of 100, every one sorted: 5.69 -> 5.06 ms; a
+// CTA per query, as where all are sorted from the start, 4.57).
+__global__ void __launch_bounds__(512) ensemble_sort_left_kernel(EnsParams p) {
+    extern __shared__ __align__(16) unsigned char ens_smem[];
+    grid_dependency_wait();
+    ens_left(p, false, true, [&](int q, bool) { ens_sort_call<512>(p, q, ens_smem); });
+}
+
+// Lists so short that a table of 1.5 slots per entry fits (M K <= 682): one launch, no table overflows, and a query with an
+// entity twice in one list is sorted where it stands (the sort needs no more memory than the table).
+constexpr int ENS_MB = 16, ENS_MAX_LOG2 = 10;
+__global__ void __launch_bounds__(256) ensemble_small_kernel(EnsParams p) {
+    extern __shared__ __align__(16) unsigned char ens_smem[];
+    if (!ens_hash_query<ENS_MB>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
+    __syncthreads();
+    ens_sort_query<0>(p, blockIdx.x, ens_smem);
+}
+
+// Longer lists, first launch: one CTA per query, 16 models at a time, 1,024 slots (31 KB: seven CTAs per SM).  85 x top-100 lists of
+// 15,000 queries, unions of 300: 36.7 ms as a sort, 0.93 ms with 32 models at a time (four CTAs), 0.87 with 8, 0.81 with 16; 128 threads
+// 1.00 ms.  Bound by instruction issue (about 48,000 warp instructions a query, 74 % of the slots), not by the 510 MB of lists (78 us).
+__global__ void __launch_bounds__(256) ensemble_hash_kernel(EnsParams p) {
+    extern __shared__ __align__(16) unsigned char ens_smem[];
+    allow_dependents();
+    const int bad = ens_hash_query<ENS_MB>(p, blockIdx.x, ENS_MAX_LOG2, 3 << (ENS_MAX_LOG2 - 2), ens_smem);
+    if (bad && threadIdx.x == 0) p.out_ids[(int64_t)blockIdx.x * p.top_n] = bad == ENS_BAD_TWICE ? ENS_SORT : ENS_LEFT;
+}
+
+// Second launch: the queries with larger unions.  Up to 8,192 slots (180 KB), eight models at a time.  Up to ENS_BIG_PART
+// entries the table takes whatever the lists hold, in one pass; beyond, the passes are as many as give each at most ENS_BIG_PART
+// entries if their hashes spread evenly (a query whose hashes favour one part that much is sorted), and the best n of the passes
+// so far wait in shared memory.  85 x top-100 lists of 15,000 queries, all left here: unions of 1,000 6.4 ms, 3,600 8.3, 6,500
+// 10.0, where the sort takes 37.8.
+constexpr int ENS_BIG_MB = 8, ENS_BIG_LOG2 = 13, ENS_BIG_PART = 5400, ENS_BIG_TOP = ENS_THREADS;
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) ensemble_left_kernel(EnsParams p) {
+    extern __shared__ __align__(16) unsigned char ens_smem[];
+    grid_dependency_wait();
+    allow_dependents();
+    ens_left(p, true, p.sort_here != 0, [&](int q, bool sort) {
+        if (sort) {
+        } else if (p.log2_parts == 0) {
+            sort = ens_hash_query<ENS_BIG_MB>(p, q, p.left_log2, 1 << p.left_log2, ens_smem) != 0;
+        } else if (p.top_n > ENS_BIG_TOP) {
+            sort = true;
+        } else {                             // (1,024 threads, 8,192 slots)
+            const int tid = threadIdx.x;
+            uint64_t* run_s = reinterpret_cast<uint64_t*>(ens_smem);            // [top_n] ordered scores, 0: free
+            int32_t* run_i = reinterpret_cast<int32_t*>(run_s + ENS_BIG_TOP);
+            EnsTable<ENS_BIG_MB> t(reinterpret_cast<unsigned char*>(run_i + ENS_BIG_TOP), 1 << ENS_BIG_LOG2, p.K);
+            if (tid < p.top_n) { run_s[tid] = 0; run_i[tid] = INT32_MAX; }
+            for (int part = 0; part < 1 << p.log2_parts; ++part) {
+                sort = t.gather(p, q, ENS_BIG_LOG2, 3 << (ENS_BIG_LOG2 - 2), part, p.log2_parts) != 0;
+                if (sort) break;
+                ens_select(t, [&](int, uint64_t s, int32_t id) {
+                    const uint64_t last_s = run_s[p.top_n - 1]; const int32_t last_i = run_i[p.top_n - 1];
+                    if (s == 0ull || s < last_s || (s == last_s && id > last_i)) return false;
+                    // into its place: everything behind it moves one on
+                    const bool in = tid < p.top_n, mine_first = in && (run_s[tid] > s || (run_s[tid] == s && run_i[tid] < id));
+                    const bool prev_first = in && (tid == 0 || run_s[tid - 1] > s || (run_s[tid - 1] == s && run_i[tid - 1] < id));
+                    const uint64_t ps = in && tid > 0 ? run_s[tid - 1] : 0ull; const int32_t pi = in && tid > 0 ? run_i[tid - 1] : 0;
+                    __syncthreads();
+                    if (in && !mine_first) { run_s[tid] = prev_first ? s : ps; run_i[tid] = prev_first ? id : pi; }
+                    return true;
+                });
+                __syncthreads();
+            }
+            if (!sort && tid < p.top_n) ens_put(p, q, tid, run_s[tid], run_i[tid]);
+        }
+        if (sort && p.sort_here) {
+            __syncthreads();
+            ens_sort_call<NT>(p, q, ens_smem);
+        } else if (sort && threadIdx.x == 0) {
+            p.out_ids[(int64_t)q * p.top_n] = ENS_SORT;
+        }
+    });
 }
 
 }  // namespace
@@ -328,32 +448,54 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
     while (p.n2 < num_models * k_list) p.n2 <<= 1;
     p.out_ids = out_ids; p.out_scores = out_scores;
     const size_t sort_smem = (size_t)p.n2 * (sizeof(uint64_t) + sizeof(int32_t));
+    // (5 lists of 300 places, 3,000 queries: 512 threads 432 us, 256 372; 12 lists 904 and 960; 16,384 entries: 512 threads 37.8 ms, 1,024 35.3)
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    constexpr size_t parts_smem = ens_hash_smem<ENS_BIG_MB>(1 << ENS_BIG_LOG2, ENS_MAX_K) + ENS_BIG_TOP * (sizeof(uint64_t) + sizeof(int32_t));
     static DeviceOnce configured;
     cudaError_t e = once_per_device(configured, [] {
         constexpr int sort_max = (int)(ENS_MAX_ENTRIES * (sizeof(uint64_t) + sizeof(int32_t)));
-        static_assert((1 << ENS_BIG_LOG2) * ens_slot_bytes<ENS_BIG_MB>() + (ENS_MAX_K + 1) * sizeof(double) <= sort_max, "the larger table fits where the sort does");
-        cudaError_t e0 = cudaFuncSetAttribute(ensemble_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_max);
-        if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(ensemble_left_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_max);
-        if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(ensemble_hash_kernel<ENS_MB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)ens_hash_smem<ENS_MB>(1 << ENS_MAX_LOG2, ENS_MAX_K));
+        static_assert(parts_smem <= sort_max, "the larger table fits where the sort does");
+        cudaError_t e0 = cudaSuccess;
+        for (void (*k)(EnsParams) : {ensemble_sort_kernel<256>, ensemble_sort_kernel<512>, ensemble_sort_kernel<ENS_THREADS>, ensemble_sort_left_kernel,
+                                     ensemble_left_kernel<256>, ensemble_left_kernel<512>, ensemble_left_kernel<ENS_THREADS>})
+            if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_max);
         return e0;
     });
     if (e != cudaSuccess) return KGE_ERR_CUDA;
     if (k_list > ENS_MAX_K) {
-        ensemble_sort_kernel<<<nq, ENS_THREADS, sort_smem, s>>>(p);
+        if (p.n2 <= 2048) ensemble_sort_kernel<256><<<nq, 256, sort_smem, s>>>(p);
+        else if (p.n2 <= 8192) ensemble_sort_kernel<512><<<nq, 512, sort_smem, s>>>(p);
+        else ensemble_sort_kernel<ENS_THREADS><<<nq, ENS_THREADS, sort_smem, s>>>(p);
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
     p.inv_k = (uint32_t)((((uint64_t)1 << 32) + k_list - 1) / k_list);
     p.log2_slots = 5;
-    while (p.log2_slots < ENS_MAX_LOG2 && 2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
-    const int threads = p.log2_slots >= 9 ? 256 : (p.log2_slots >= 7 ? 128 : 64);
-    ensemble_hash_kernel<ENS_MB><<<nq, threads, ens_hash_smem<ENS_MB>(1 << p.log2_slots, k_list), s>>>(p);
+    while (2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
+    if (p.log2_slots <= ENS_MAX_LOG2) {
+        const int threads = p.log2_slots >= 9 ? 256 : (p.log2_slots >= 7 ? 128 : 64);
+        ensemble_small_kernel<<<nq, threads, ens_hash_smem<ENS_MB>(1 << p.log2_slots, k_list), s>>>(p);
+        return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
+    }
+    ensemble_hash_kernel<<<nq, 256, ens_hash_smem<ENS_MB>(1 << ENS_MAX_LOG2, k_list), s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return KGE_ERR_CUDA;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;
-    const size_t big_smem = std::max(sort_smem, ens_hash_smem<ENS_BIG_MB>(1 << ENS_BIG_LOG2, k_list));
-    e = launch_dependent(ensemble_left_kernel, dim3((unsigned)std::min(nq, sms)), dim3(ENS_THREADS), big_smem, s, p);
+    p.log2_parts = 0; p.left_log2 = ENS_MAX_LOG2 + 1;
+    while (p.left_log2 < ENS_BIG_LOG2 && 3 << (p.left_log2 - 2) < num_models * k_list) ++p.left_log2;
+    while (num_models * k_list > ENS_BIG_PART << p.log2_parts) ++p.log2_parts;
+    auto launch_left = [&](void (*kernel)(EnsParams), int threads, size_t smem, int waves) {
+        const int per_sm = std::max(1, std::min(2048 / threads, (int)(224 * 1024 / (smem + 8 * 1024))));
+        return launch_dependent(kernel, dim3((unsigned)std::min<int64_t>(nq, (int64_t)sms * per_sm * waves)), dim3(threads), smem, s, p);
+    };
+    const size_t table_smem = p.log2_parts > 0 ? parts_smem : ens_hash_smem<ENS_BIG_MB>(1 << p.left_log2, k_list);
+    // (where the sort takes much less memory than the table, and so more CTAs of it share an SM, it is a launch of its own)
+    const bool sort_apart = p.left_log2 > ENS_MAX_LOG2 + 1 && p.n2 <= 8192;
+    p.sort_here = sort_apart ? 0 : 1;
+    const size_t left_smem = sort_apart ? table_smem : std::max(table_smem, sort_smem);
+    if (p.left_log2 == ENS_MAX_LOG2 + 1) e = launch_left(ensemble_left_kernel<256>, 256, left_smem, 2);
+    else if (p.left_log2 == ENS_MAX_LOG2 + 2) e = launch_left(ensemble_left_kernel<512>, 512, left_smem, 1);
+    else e = launch_left(ensemble_left_kernel<ENS_THREADS>, ENS_THREADS, left_smem, 1);
+    if (e == cudaSuccess && sort_apart) e = launch_left(ensemble_sort_left_kernel, 512, sort_smem, 4);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
 }
 

@@ -39,8 +39,8 @@ def test_ensemble_against_oracle(oracle64, M, nq, K, E, power):
     assert (sc == o_sc).all()
 
 
-# unions at and beyond the first launch's table (1,024 slots), the larger table (8,192 slots) and the sort behind it; one
-# place per list; the longest list kept as bytes and the first that is sorted; blocks of 32 models with a remainder of one
+# unions up to and beyond what the first launch's table takes (768 of 1,024 slots), one, two and four passes of the larger
+# table; one place per list; the longest list kept as bytes and the first that is sorted; blocks of 16 models with a remainder
 @pytest.mark.parametrize("M,nq,K,E", [(33, 7, 31, 1024), (11, 150, 94, 100_000), (85, 3, 96, 1_000_000), (90, 3, 100, 1_000_000), (160, 2, 102, 1 << 30),
                                       (40, 9, 1, 12), (4, 5, 254, 300), (4, 5, 255, 300), (65, 40, 2, 5)])
 @pytest.mark.parametrize("power", [-0.5, 1.0])
@@ -72,6 +72,59 @@ def test_ensemble_gives_up_on_a_table_with_rounds_to_come(oracle64, twice):
     o_ids, o_sc = oracle64.ensemble_topk(lists, -0.5, 10)
     assert (ids == o_ids).all()
     assert (sc == o_sc).all()
+
+
+@pytest.mark.parametrize("power", [-0.5, 1.0])
+@pytest.mark.parametrize("union", [767, 768, 769])
+def test_ensemble_union_of_exactly_what_the_table_takes(oracle64, union, power):
+    rng = np.random.default_rng(union)
+    M, nq, K = 85, 6, 100
+    flat = np.stack([np.concatenate([rng.permutation(union) for _ in range(12)])[:M * K] for _ in range(nq)])    # 8,500 places: every id
+    lists = np.ascontiguousarray(flat.reshape(nq, M, K).transpose(1, 0, 2)).astype(np.int32) + 1_000_000
+    for q in range(nq):                                 # (a list across the seam of two permutations may name an id twice: make it distinct)
+        for m in range(M):
+            if len(set(lists[m, q])) < K:
+                lists[m, q] = 1_000_000 + rng.permutation(union)[:K]
+    assert all(len(np.unique(lists[:, q])) == union for q in range(nq))
+    ids, sc = _gpu_ensemble(lists, power, 10)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, power, 10)
+    assert (ids == o_ids).all() and (sc == o_sc).all()
+
+
+def _ids_of_one_part(rng, n):
+    """Entity ids whose multiplicative hash has the bit below the larger table's 13 slot bits clear."""
+    inverse = pow(0x9E3779B1, -1, 1 << 32)
+    h = np.unique(rng.integers(0, 1 << 32, 8 * n, dtype=np.uint64)) & ~np.uint64(1 << 18)
+    ids = np.unique((h * np.uint64(inverse)) & np.uint64(0xffffffff))
+    ids = ids[ids < (1 << 31)]
+    return rng.permutation(ids)[:n].astype(np.int32)
+
+
+@pytest.mark.parametrize("form", ["one pass", "two passes", "one part of two overflows", "more places than the larger table keeps"])
+def test_ensemble_large_unions(oracle64, form):
+    rng = np.random.default_rng(3)
+    M, nq, K, top_n = (54 if form == "one pass" else 85), 4, 100, 10
+    if form.startswith("one part"):
+        lists = np.stack([_ids_of_one_part(rng, M * K).reshape(M, K) for _ in range(nq)], axis=1)
+    else:
+        lists = np.stack([rng.permutation(1 << 20)[:M * K].reshape(M, K) for _ in range(nq)], axis=1).astype(np.int32)
+    if form.startswith("more"):
+        top_n = 1100
+    ids, sc = _gpu_ensemble(lists, -0.5, top_n)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, -0.5, top_n)
+    assert (ids == o_ids).all() and (sc == o_sc).all()
+
+
+# lists short enough for one launch (682 places), and the first that are not: an entity twice in a list, more places than
+# entities, more than one warp's worth of queries
+@pytest.mark.parametrize("M,K", [(2, 10), (1, 254), (22, 31), (31, 22), (33, 21)])
+@pytest.mark.parametrize("power", [-1.0, 0.5])
+def test_ensemble_an_entity_twice_in_short_lists(oracle64, M, K, power):
+    rng = np.random.default_rng(M)
+    lists = rng.integers(0, 3 * K, (M, 50, K)).astype(np.int32)
+    ids, sc = _gpu_ensemble(lists, power, K + 3)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, power, K + 3)
+    assert (ids == o_ids).all() and (sc == o_sc).all()
 
 
 def test_ensemble_fewer_candidates_than_places_and_limits(oracle64):
