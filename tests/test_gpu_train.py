@@ -510,3 +510,14 @@ def test_touched_ids_at_the_one_launch_size(oracle64, B, N):
     gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
     orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
     _check_step(gpu, orc, 0, orc.sample(0))
+
+
+# score block with few and with many CTAs (two per SM: stages of 128 floats up to there, of 64 beyond), rows that end at, before
+# and after a stage
+@pytest.mark.parametrize("B,N", [(20, 68), (330, 2050)])
+@pytest.mark.parametrize("score,d", [("distmult", 60), ("distmult", 124), ("distmult", 128), ("transe", 132), ("distmult", 260), ("transe", 384)])
+def test_score_block_stages(oracle64, score, d, B, N):
+    prob = Problem(E=3000, R=7, T=20000, d=d, score=score, p_norm=2, loss="softmax", B=B, N=N, P=1, gamma=0.0, lr=0.05, graph_seed=26)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0))
