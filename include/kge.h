@@ -56,7 +56,7 @@ typedef enum {
     KGE_ERR_BAD_ARG = -1,        /* NULL / out-of-range argument, misaligned pointer */
     KGE_ERR_DIVISIBILITY = -2,   /* B % P^2 (or B % P with head_part >= 0) or N % P != 0 */
     KGE_ERR_EMPTY_BUCKET = -3,   /* a triple bucket T_{i,j} or entity partition E_j that must be sampled is empty */
-    KGE_ERR_WORKSPACE = -4,      /* workspace missing or smaller than kge_workspace_bytes() */
+    KGE_ERR_WORKSPACE = -4,      /* workspace missing or too small (see kge_bind) */
     KGE_ERR_UNSUPPORTED = -5,    /* combination not implemented */
     KGE_ERR_NOT_READY = -6,      /* tables not bound / graph not loaded */
     KGE_ERR_CUDA = -7,           /* a CUDA runtime call failed (see kge_last_cuda_error) */
@@ -111,7 +111,9 @@ size_t kge_workspace_bytes(const kge_handle* h, int64_t num_triples, int32_t max
 /*
  * Attach caller-owned device memory.  ent [E, d]; rel [R, d] (RotatE [R, d/2]); relw [R, d]
  * for TransH, else NULL; *_state as described above or NULL for SGD; workspace of at
- * least kge_workspace_bytes() bytes, 256-byte aligned.  The workspace must be the one sized
+ * least kge_workspace_bytes() bytes, 256-byte aligned (a smaller one is accepted as long as the
+ * backward fits with fewer partial slabs: TransE and RotatE then take a pass over the pairs per
+ * side instead of one pass for both).  The workspace must be the one sized
  * with the same (num_triples, max_queries, topk).  Zero-fills the workspace header
  * asynchronously on `stream`.
  */

@@ -71,6 +71,33 @@ int pick_split_tc(int rows, int cols, int depth, int num_sms) {
     return (kb + per - 1) / per;
 }
 
+// How the backward is divided.  `compact`: as the smallest accepted workspace holds it.  The one-pass backward of the distance
+// kinds leaves more partial slabs (rectangles of pairs: fp32 TransE at 4,096 x 4,096 x 128 175 MB of workspace against 110), and the
+// negatives' matrix gradient has splits of its own number.
+void pick_plan(kge_handle* h, bool compact) {
+    const kge_config& c = h->cfg;
+    h->pair_backward = !compact && pair_backward_serves(h);
+    // resident CTAs per SM of the TransH accumulation kernels: two (128 registers x 256 threads, 70-90 KB of shared memory);
+    // with the c sums on the tensor cores a CTA of the negatives' side owns 64 rows
+    if (c.score == KGE_TRANSH) {
+        h->split_q = pick_split_waves(c.batch, c.num_neg, h->num_sms, 2);
+        h->split_t = pick_split_waves(c.num_neg, c.batch, h->num_sms, 2, h->th_tc ? 64 : 32);
+    } else {
+        h->split_q = pick_split(c.batch, c.num_neg, h->num_sms);
+        h->split_t = pick_split(c.num_neg, c.batch, h->num_sms);
+    }
+    if (h->pair_backward) pair_backward_split(c.batch, c.num_neg, c.dim / 4, h->num_sms, &h->split_q, &h->split_t);
+    if (c.prec == KGE_PREC_BF16_TC) {   // the backward contractions run as 128 x 128 tensor-core tiles split over K
+        h->split_q = pick_split_tc(c.batch, c.dim, c.num_neg, h->num_sms);
+        h->split_t = pick_split_tc(c.num_neg, c.dim, c.batch, h->num_sms);
+    }
+    h->split_mh = h->split_mt = 1;
+    if (c.feat_dim > 0) {   // dM = dE^T . F: [d, F] over the role's slots, split over the slots so that every SM has a tile
+        h->split_mh = pick_split_tc(c.dim, c.feat_dim, c.batch, h->num_sms);
+        h->split_mt = compact ? h->split_mh : pick_split_tc(c.dim, c.feat_dim, c.batch + c.num_neg, h->num_sms);
+    }
+}
+
 size_t layout(const kge_handle* h, char* base, int64_t T, int32_t maxq, int32_t topk, Workspace* out) {
     const kge_config& c = h->cfg;
     const size_t B = c.batch, N = c.num_neg, d = c.dim, kw = h->kw;
@@ -270,20 +297,7 @@ int kge_create(const kge_config* cfg, kge_handle** out) {
     // 0 automatic, 1 always where the shapes allow, 2 never)
     h->th_tc = c.score == KGE_TRANSH && c.prec == KGE_PREC_FP32 && c.dim % 32 == 0 && c.contract != 2 &&
                (c.contract == 1 || (int64_t)c.batch * c.num_neg >= ((int64_t)1 << 22));
-    // resident CTAs per SM of the TransH accumulation kernels: two (128 registers x 256 threads, 70-90 KB of shared memory);
-    // with the c sums on the tensor cores a CTA of the negatives' side owns 64 rows
-    if (c.score == KGE_TRANSH) {
-        h->split_q = pick_split_waves(c.batch, c.num_neg, h->num_sms, 2);
-        h->split_t = pick_split_waves(c.num_neg, c.batch, h->num_sms, 2, h->th_tc ? 64 : 32);
-    } else {
-        h->split_q = pick_split(c.batch, c.num_neg, h->num_sms);
-        h->split_t = pick_split(c.num_neg, c.batch, h->num_sms);
-    }
-    if (pair_backward_serves(h)) pair_backward_split(c.batch, c.num_neg, c.dim / 4, h->num_sms, &h->split_q, &h->split_t);
-    if (c.prec == KGE_PREC_BF16_TC) {   // the backward contractions run as 128 x 128 tensor-core tiles split over K
-        h->split_q = pick_split_tc(c.batch, c.dim, c.num_neg, h->num_sms);
-        h->split_t = pick_split_tc(c.num_neg, c.dim, c.batch, h->num_sms);
-    }
+    pick_plan(h, false);
     h->th_gsplit = 1;
     if (h->th_tc) {   // K splits: as many as still give every SM at most one tile, each at least eight 64-wide slices deep, at most 4
         const int bn = 2 * c.dim > 128 ? 256 : 128;
@@ -291,12 +305,7 @@ int kge_create(const kge_config* cfg, kge_handle** out) {
         const int kb = 2 * ((std::min(c.batch, c.num_neg) + 63) / 64);
         h->th_gsplit = std::max(1, std::min(std::min(h->num_sms / tiles, kb / 8), 4));
     }
-    h->split_mh = h->split_mt = 1;
     h->features_bound = false;
-    if (c.feat_dim > 0) {   // dM = dE^T . F: [d, F] over the role's slots, split over the slots so that every SM has a tile
-        h->split_mh = pick_split_tc(c.dim, c.feat_dim, c.batch, h->num_sms);
-        h->split_mt = pick_split_tc(c.dim, c.feat_dim, c.batch + c.num_neg, h->num_sms);
-    }
     *out = h;
     return KGE_OK;
 }
@@ -337,7 +346,9 @@ int kge_profile_read(kge_handle* h, double* ms, int64_t* launches, int reset) {
 
 size_t kge_workspace_bytes(const kge_handle* h, int64_t num_triples, int32_t max_queries, int32_t topk) {
     if (!h || num_triples < 0 || max_queries < 0 || topk < 0) return 0;
-    return layout(h, nullptr, num_triples, max_queries, topk, nullptr);
+    kge_handle preferred = *h;                  // (a bound handle may hold the compact plan)
+    pick_plan(&preferred, false);
+    return layout(&preferred, nullptr, num_triples, max_queries, topk, nullptr);
 }
 
 int kge_bind(kge_handle* h, float* ent, float* rel, float* relw, float* ent_state, float* rel_state,
@@ -352,8 +363,16 @@ int kge_bind(kge_handle* h, float* ent, float* rel, float* relw, float* ent_stat
     if (misaligned(ent, 16) || misaligned(rel, 16) || misaligned(relw, 16) || misaligned(ent_state, 16) ||
         misaligned(rel_state, 16) || misaligned(relw_state, 16) || misaligned(workspace, 256))
         return KGE_ERR_BAD_ARG;
-    if (!workspace || workspace_bytes < layout(h, nullptr, num_triples, max_queries, topk, nullptr))
-        return KGE_ERR_WORKSPACE;
+    if (!workspace) return KGE_ERR_WORKSPACE;
+    // a workspace that holds the compact plan only is taken as well: two passes instead of one in the distance kinds' backward
+    kge_handle plan = *h;
+    pick_plan(&plan, false);
+    if (workspace_bytes < layout(&plan, nullptr, num_triples, max_queries, topk, nullptr)) {
+        pick_plan(&plan, true);
+        if (workspace_bytes < layout(&plan, nullptr, num_triples, max_queries, topk, nullptr)) return KGE_ERR_WORKSPACE;
+    }
+    h->pair_backward = plan.pair_backward;
+    h->split_q = plan.split_q; h->split_t = plan.split_t; h->split_mh = plan.split_mh; h->split_mt = plan.split_mt;
     h->ent = ent; h->rel = rel; h->relw = relw;
     h->ent_state = ent_state; h->rel_state = rel_state; h->relw_state = relw_state;
     h->ws_base = static_cast<char*>(workspace);

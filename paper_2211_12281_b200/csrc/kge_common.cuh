@@ -124,6 +124,7 @@ struct kge_handle {
     int64_t num_triples;
     int32_t max_queries, topk;
     int split_q, split_t;   // column splits of the two backward accumulations
+    bool pair_backward;     // both of them in one pass over the pairs (set with the splits: the workspace may be too small for its slabs)
     bool th_tc;             // TransH: sum_n c_bn t_n and sum_b c_bn w_b as tensor-core contractions of bf16 splits
     int th_gsplit;          // K splits of each of those contractions (each leaves two partial slabs)
     bool bound, graph_loaded;

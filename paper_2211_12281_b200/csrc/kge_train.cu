@@ -1213,10 +1213,10 @@ cudaError_t launch_accum_tma_inst(const AccArgs& aq, const AccArgs& at, cudaStre
 
 template <int KIND>
 cudaError_t launch_accum_tma_kind(const AccArgs& aq, const AccArgs& at, cudaStream_t s) {
-    // (distance kinds come here with rows of less than 32 floats only, see pair_backward_serves)
-    if (KIND != KIND_DOT || aq.d4 <= 32) return launch_accum_tma_inst<KIND, 1>(aq, at, s);
-    if (aq.d4 <= 64) return launch_accum_tma_inst<KIND == KIND_DOT ? KIND : KIND_DOT, 2>(aq, at, s);
-    return launch_accum_tma_inst<KIND == KIND_DOT ? KIND : KIND_DOT, 4>(aq, at, s);
+    // (distance kinds come here with rows of less than 32 floats, see pair_backward_serves, or in a small workspace)
+    if (aq.d4 <= 32) return launch_accum_tma_inst<KIND, 1>(aq, at, s);
+    if (aq.d4 <= 64) return launch_accum_tma_inst<KIND, 2>(aq, at, s);
+    return launch_accum_tma_inst<KIND, 4>(aq, at, s);
 }
 
 // dQ and dT of the pair kinds whose operands are plain rows, in one launch.
@@ -1332,7 +1332,7 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     at.out = p.w.dTpart; at.out2 = nullptr; at.csum = p.w.Cpart;
     if (p.kind != KIND_TH_L1 && p.kind != KIND_TH_L2) {
         stage_begin(h, ST_ACCUM_Q, s);
-        if (pair_backward_serves(h)) {
+        if (h->pair_backward) {
             const int rc = launch_pair_backward(h, s);
             if (rc != KGE_OK) return rc;
         } else {

@@ -521,3 +521,31 @@ def test_score_block_stages(oracle64, score, d, B, N):
     gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
     orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
     _check_step(gpu, orc, 0, orc.sample(0))
+
+
+@pytest.mark.parametrize("score,p,d,B,N", [("transe", 1, 128, 600, 700), ("transe", 2, 256, 300, 600), ("rotate", 2, 400, 256, 516), ("transe", 1, 64, 2048, 256)])
+def test_a_workspace_without_room_for_the_one_pass_backward(oracle64, score, p, d, B, N):
+    """A workspace smaller than the preferred size binds down to the size that a pass per side needs, trains the same step, and
+    is refused one byte below; what kge_workspace_bytes says does not depend on what is bound."""
+    prob = Problem(E=3000, R=6, T=20000, d=d, score=score, p_norm=p, loss="logsigmoid", B=B, N=N, P=2, gamma=4.0, adv_temp=0.5, lr=0.05, graph_seed=29)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    need = gpu.kge.workspace_bytes(prob.T, 0, 0)
+    space = gpu.torch.empty(need + 512, dtype=gpu.torch.uint8, device=gpu.ent.device)
+    first = space[(-space.data_ptr()) % 256:]
+
+    def bind(size):
+        try:
+            gpu.kge.bind(gpu.ent, gpu.rel, None, num_triples=prob.T, workspace=first[:size])
+        except gpu.K.KgeError:
+            return False
+        return True
+
+    lo, hi = 256, need                                    # refused, accepted
+    assert not bind(lo) and bind(hi)
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if bind(mid) else (mid, hi)
+    assert hi < need and bind(hi) and gpu.kge.workspace_bytes(prob.T, 0, 0) == need
+    gpu.kge.graph_load(prob.h, prob.r, prob.t)
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0))
