@@ -8,7 +8,7 @@
 // into one of two accumulators in tensor memory and owns the allocation, warps 2-17 drain the
 // other accumulator meanwhile (a warp may only touch the 32 lanes of its own quarter; four warps
 // share a quarter, a quarter of the columns each) and apply the epilogue:
-//   EPI_STORE   C = acc (the backward contractions)
+//   EPI_STORE   C = acc (the score block as a test reads it)
 //   EPI_STATS   no score leaves the chip: per row and 64-column piece the running maximum, the sum
 //               of exponentials and the weighted loss sum of Section 3.1 "Loss Functions"; the
 //               score is the contraction (DistMult, ComplEx) or, for TransE with p = 2, the
@@ -574,10 +574,8 @@ __device__ __forceinline__ void tc_item_next(const TcGemmParams& p, TcItem& it) 
     }
 }
 
-// BN: columns per tile (128, or 256 for the backward contractions of wide rows); A_MN / B_MN:
-// the operand is read MN-major (its tensor map has the contraction index as rows), which is how
-// dL/dF, Q and T serve as transposed operands without a transposed copy.
-template <int EPI, int BN = 128, bool A_MN = false, bool B_MN = false>
+// BN: columns per tile, 128 or 256.
+template <int EPI, int BN = 128>
 __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
                                                              const __grid_constant__ CUtensorMap tmB, TcGemmParams p) {
     constexpr uint32_t TC_STAGE_BYTES = tc_stage_bytes(BN);
@@ -725,19 +723,9 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                     const bool load_a = !(have && !p.m_fastest), load_b = !(have && p.m_fastest);
                     mbar_arrive_expect_tx(&full[s], (load_a ? TC_A_BYTES : 0u) + (load_b ? TC_STAGE_BYTES - TC_A_BYTES : 0u));
                     const int k0 = (kb0 + kb) * TC_BK;
-                    if (!load_a) {
-                    } else if (A_MN) {
-#pragma unroll
-                        for (int g = 0; g < TC_BM / 64; ++g) tma_load_2d(sa + g * TC_MN_GROUP_BYTES, &tmA, it.m0 + 64 * g, k0, &full[s]);
-                    } else {
-                        tma_load_2d(sa, &tmA, k0, it.m0, &full[s]);
-                    }
+                    if (load_a) tma_load_2d(sa, &tmA, k0, it.m0, &full[s]);
                     unsigned char* sb = sa + TC_A_BYTES;
-                    if (!load_b) {
-                    } else if (B_MN) {
-#pragma unroll
-                        for (int g = 0; g < BN / 64; ++g) tma_load_2d(sb + g * TC_MN_GROUP_BYTES, &tmB, it.n0 + 64 * g, k0, &full[s]);
-                    } else {
+                    if (load_b) {
 #pragma unroll
                         for (int g = 0; g < BN / 128; ++g)   // boxes of 128 rows, one after the other
                             tma_load_2d(sb + g * (128 * TC_BK * 2), &tmB, k0, (int)p.n_base + it.n0 + 128 * g, &full[s]);
@@ -747,7 +735,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN, A_MN, B_MN);
+            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN, false, false);
             int ring = 0;
             bool ok = true;
             TcItem it = tc_item(p, item_begin);
@@ -765,8 +753,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                     const uint32_t sa = smem_u32(base + (size_t)s * TC_STAGE_BYTES);
 #pragma unroll
                     for (int k = 0; k < TC_BK / 16; ++k) {   // one MMA covers 16 of K: 32 bytes of a K-major row, 16 rows MN-major
-                        const uint64_t ad = A_MN ? umma_desc_mn_sw128(sa + k * 2048) : umma_desc_k_sw128(sa + k * 32);
-                        const uint64_t bd = B_MN ? umma_desc_mn_sw128(sa + TC_A_BYTES + k * 2048) : umma_desc_k_sw128(sa + TC_A_BYTES + k * 32);
+                        const uint64_t ad = umma_desc_k_sw128(sa + k * 32), bd = umma_desc_k_sw128(sa + TC_A_BYTES + k * 32);
                         umma_bf16(tmem_acc, ad, bd, idesc, (kb | k) != 0);
                     }
                     umma_commit(&empty[s]);            // the stage is free once these MMAs have read it
@@ -1293,7 +1280,7 @@ __global__ void __launch_bounds__(256) grad_sums_kernel(const float* grow_part, 
 }  // namespace
 
 namespace {
-template <int EPI, int BN = 128, bool A_MN = false, bool B_MN = false>
+template <int EPI, int BN = 128>
 cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB, const TcGemmParams& p, int num_sms, cudaStream_t s,
                              size_t extra_smem = 0) {
     constexpr size_t smem = tc_smem_bytes(BN);
@@ -1303,13 +1290,13 @@ cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB,
     if ((EPI & 3) == EPI_GRAD || (EPI & 3) == EPI_STORE) extra_smem = extra_max;
     static DeviceOnce configured;
     const cudaError_t e = once_per_device(configured, [] {
-        return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN, A_MN, B_MN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + extra_max));
+        return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + extra_max));
     });
     if (e != cudaSuccess) return e;
     if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD)
-        return launch_dependent(tc_gemm_kernel<EPI, BN, A_MN, B_MN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem + extra_smem, s,
+        return launch_dependent(tc_gemm_kernel<EPI, BN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem + extra_smem, s,
                                 *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
-    tc_gemm_kernel<EPI, BN, A_MN, B_MN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem + extra_smem, s>>>(
+    tc_gemm_kernel<EPI, BN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem + extra_smem, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
     return cudaSuccess;
 }
