@@ -24,7 +24,7 @@ def _infer(gpu, qh, qr, tt, K):
                                      ("transh", 1), ("transh", 2), ("rotate", 2), ("rotate", 1), ("rotate_real_l1", 1)])
 def test_topk_rank_mrr_against_fp32_oracle(oracle32, oracle64, score, p):
     import kge_synth
-    E, R, d, K, nq = 5000, 9, 40, 10, 70          # chunks 1024, 1024, 2048, 904; ragged tiles
+    E, R, d, K, nq = 5000, 9, 40, 10, 70          # chunks 1024 and 3976; ragged tiles
     prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=p, B=4, N=4, P=1, graph_seed=11)
     prob.ent[3000] = prob.ent[17]; prob.ent[4999] = prob.ent[17]; prob.ent[1] = prob.ent[0]   # exact ties
     qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=11)
@@ -61,7 +61,7 @@ def test_topk_rank_mrr_against_fp32_oracle(oracle32, oracle64, score, p):
 
 @pytest.mark.parametrize("score,p,d", [("transe", 1, 128), ("distmult", 1, 40), ("transe", 2, 64), ("complex", 1, 128)])
 def test_five_query_tiles_with_a_ragged_last_one(oracle32, score, p, d):
-    """300 queries (a ragged fifth 64-query tile) against 3,000 entities (ragged last tile, chunks 1024 + 1024 + 952)
+    """300 queries (a ragged fifth 64-query tile) against 3,000 entities (ragged last tile, chunks 1024 + 1976)
     with exact ties: ids, scores and ranks bit-exact against the fp32 oracle."""
     import kge_synth
     E, R, K, nq = 3000, 9, 10, 300
@@ -166,7 +166,7 @@ def test_rising_scores_take_the_overflow_path(oracle32):
 @pytest.mark.parametrize("score,p,K", [("transe", 1, 10), ("transe", 2, 100), ("distmult", 1, 129)])
 def test_row_widths_at_the_edges_of_a_staged_box(oracle32, score, p, d, K):
     """Rows that end at, before and after the 32-float boxes and 64-float stages of the score tile; lists of up to 128 places
-    (cut down before they are sorted) and one more; 65 queries (a second tile of one row), 2,500 entities in three chunks."""
+    (cut down before they are sorted) and one more; 65 queries (a second tile of one row), 2,500 entities in two chunks (K = 129: three)."""
     import kge_synth
     E, R, nq = 2500, 5, 65
     prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=p, B=4, N=4, P=1, graph_seed=31)
@@ -199,3 +199,21 @@ def test_scores_that_rise_along_a_stretch(oracle32, score, tc, d, lo, hi, K):
     ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
     o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, None, qh, qr, K, true_tails=tt)
     assert (ids == o_ids).all() and (ranks == o_ranks).all() and (sc == o_sc).all()
+
+
+@pytest.mark.parametrize("score,p,d", [("transe", 1, 40), ("transe", 2, 96), ("distmult", 1, 132), ("complex", 1, 28), ("transh", 1, 40), ("transh", 2, 36)])
+@pytest.mark.parametrize("K", [10, 100])
+def test_several_filtered_chunks(oracle32, score, p, d, K):
+    """17,000 entities: chunks of 1,024, then four (K = 100: two) times what went before, so that the running lists are merged,
+    and the thresholds tightened, at least twice after the first selection."""
+    import kge_synth
+    E, R, nq = 17_000, 5, 66
+    prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=p, B=4, N=4, P=1, graph_seed=33)
+    prob.ent[16_990] = prob.ent[17]; prob.ent[6000] = prob.ent[17]
+    qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=33)
+    tt[0] = qh[0]; tt[1] = 16_990; qh[2] = 17
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K, true_tails=tt)
+    assert (ids == o_ids).all() and (ranks == o_ranks).all()
+    assert (sc == o_sc).all() or np.allclose(sc, o_sc, rtol=1e-6)

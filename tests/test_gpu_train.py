@@ -512,6 +512,53 @@ def test_touched_ids_at_the_one_launch_size(oracle64, B, N):
     _check_step(gpu, orc, 0, orc.sample(0))
 
 
+# kinks of the distance kinds in the one-pass backward (rows of 32 floats and more): exact ties of single coordinates, complex
+# residuals that are exactly zero, and whole rows at distance zero
+@pytest.mark.parametrize("score,p", [("transe", 1), ("transe", 2), ("rotate", 1), ("rotate", 2)])
+def test_one_pass_backward_at_exact_zeros(oracle64_tie, score, p):
+    prob = Problem(E=60, R=4, T=3000, d=64, score=score, p_norm=p, loss="logsigmoid", B=32, N=40, P=2, gamma=4.0, adv_temp=0.5, lr=0.05, graph_seed=15)
+    rng = np.random.default_rng(15)
+    prob.ent = rng.integers(-2, 3, prob.ent.shape).astype(np.float32)                      # whole numbers: differences are exact
+    prob.rel = np.zeros_like(prob.rel) if score == "rotate" else rng.integers(-1, 2, prob.rel.shape).astype(np.float32)
+    prob.rel[0] = 0.0
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64_tie)
+    batch = orc.sample(0)
+    batch[1][:8] = 0
+    batch[3][:8] = batch[0][:8]                          # q = h exactly, and h among the negatives: every residual of the pair is zero
+    B, N, d = prob.B, prob.N, prob.d
+    want = orc.grads(batch)
+    gpu.kge.train_step(0, prob.lr, *[gpu.dev_i32(a) for a in batch])
+    assert gpu.kge.get_status() == 0
+    ge = gpu.kge.debug_export("GRAD_ENT").reshape(2 * B + N, d)
+    scale = max(np.abs(want["dh"]).max(), np.abs(want["dtneg"]).max())
+    for got, key in ((ge[:B], "dh"), (ge[B:2 * B], "dtpos"), (ge[2 * B:], "dtneg")):
+        assert_close(got, want[key], atol=2e-5 * scale, what=key)
+
+
+@pytest.mark.parametrize("score,p,d,B,N", [("transe", 1, 64, 300, 520), ("transe", 2, 128, 520, 132), ("rotate", 1, 200, 140, 1030)])
+def test_one_pass_backward_run_twice_bit_identical(score, p, d, B, N):
+    prob = Problem(E=5000, R=6, T=40000, d=d, score=score, p_norm=p, loss="logsigmoid", opt="adagrad", B=B, N=N, P=2, gamma=6.0, adv_temp=1.0, lr=0.05, graph_seed=22)
+    tables = []
+    for _ in range(2):
+        gpu = GpuSide(prob)
+        for step in range(3):
+            gpu.kge.train_step(step, prob.lr)
+        assert gpu.kge.get_status() == 0
+        tables.append(gpu.tables()[:2])
+    assert all((a == b).all() for a, b in zip(*tables))
+
+
+# rows of 257 to 2,048 scores: a warp per row where the rows fill the GPU eight to a CTA (1,184 on 148 SMs), else a CTA per row;
+# beyond 1,536 scores the eight rows of a CTA take more than 48 KB
+@pytest.mark.parametrize("B,N", [(1200, 300), (1200, 2048), (1180, 300), (1180, 2048), (60, 260)])
+@pytest.mark.parametrize("loss,a", [("logsigmoid", 1.0), ("logsigmoid", 0.5), ("softmax", 0.0)])
+def test_loss_rows_on_both_sides_of_the_row_count(oracle64, B, N, loss, a):
+    prob = Problem(E=3000, R=7, T=20000, d=32, score="transe", p_norm=2, loss=loss, B=B, N=N, P=2, gamma=4.0, adv_temp=a, lr=0.05, graph_seed=27)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0))
+
+
 # score block with few and with many CTAs (two per SM: stages of 128 floats up to there, of 64 beyond), rows that end at, before
 # and after a stage
 @pytest.mark.parametrize("B,N", [(20, 68), (330, 2050)])
