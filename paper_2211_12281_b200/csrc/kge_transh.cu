@@ -36,14 +36,14 @@ namespace kge {
 namespace {
 
 __device__ __forceinline__ float4 f4z() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-// acc += w where a > b: a compare into a predicate and a predicated add.  (A float mask, set.gt giving 1.0 or 0.0,
-// times w in a multiply-add is the same count without the predicate registers and was measured 5-16 % slower.)
 // Four differences in two instructions (see sub2): these loops are bound by issue slots rather than by the pipe.  Score block
 // at B = N = 8192, d = 128: 1640 -> 1531 us (p = 2 at 4096: 377 -> 323); the threshold's multiply-add packed as well: 1551.
 __device__ __forceinline__ float4 sub4(float4 a, float4 b) {
     const float2 lo = sub2(make_float2(a.x, a.y), make_float2(b.x, b.y)), hi = sub2(make_float2(a.z, a.w), make_float2(b.z, b.w));
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
+// acc += w where a > b: a compare into a predicate and a predicated add.  (A float mask, set.gt giving 1.0 or 0.0,
+// times w in a multiply-add is the same count without the predicate registers and was measured 5-16 % slower.)
 __device__ __forceinline__ void add_if_gt(float& acc, float a, float b, float w) {
     asm("{\n .reg .pred p;\n setp.gt.f32 p, %1, %2;\n @p add.f32 %0, %0, %3;\n}\n" : "+f"(acc) : "f"(a), "f"(b), "f"(w));
 }
