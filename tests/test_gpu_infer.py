@@ -217,3 +217,22 @@ def test_several_filtered_chunks(oracle32, score, p, d, K):
     o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K, true_tails=tt)
     assert (ids == o_ids).all() and (ranks == o_ranks).all()
     assert (sc == o_sc).all() or np.allclose(sc, o_sc, rtol=1e-6)
+
+
+@pytest.mark.parametrize("score,d", [("transe", 16), ("transe", 84), ("transh", 36)])
+@pytest.mark.parametrize("nq", [1, 63, 64, 65])
+def test_ranks_of_few_queries(oracle32, score, d, nq):
+    """Rank counts of a tile's rows, whole and ragged, in every tile kernel; without true tails nothing is counted."""
+    import kge_synth
+    E, R, K = 1500, 5, 3
+    prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=1, B=4, N=4, P=1, graph_seed=35)
+    qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=35)
+    tt[0] = E - 1
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K, true_tails=tt)
+    assert (ids == o_ids).all() and (ranks == o_ranks).all()
+    t = gpu.torch
+    ids2, sc2 = t.empty((nq, K), dtype=t.int32, device=gpu.ent.device), t.empty((nq, K), dtype=t.float32, device=gpu.ent.device)
+    gpu.kge.score_all_topk(gpu.dev_i32(qh), gpu.dev_i32(qr), K, None, ids2, sc2)
+    assert (ids2.cpu().numpy() == ids).all() and (sc2.cpu().numpy() == sc).all()
