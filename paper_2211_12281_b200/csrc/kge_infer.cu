@@ -245,6 +245,11 @@ __global__ void __launch_bounds__(32 * SETUP_WARPS) query_setup_kernel(InferPara
 
 constexpr int IQ = 64, IE = 64, IKC = 32, ILD = IKC + 4;
 
+// Whether a candidate list overflowed earlier in this call: asked by one thread before the first load, so that what was queued
+// behind costs little more than its launch.  (A plain load: the CTAs of a launch find it in their SM's cache, which is empty when
+// the launch begins; one that misses a change during the launch does work that is redone.)
+__device__ __forceinline__ int call_given_up(const InferParams& p) { return p.first ? 0 : p.w.status[1]; }
+
 // Largest float below x (x finite).
 __device__ __forceinline__ float float_below(float x) {
     if (x == 0.f) return __uint_as_float(0x80000001u);
@@ -399,10 +404,12 @@ __global__ void __launch_bounds__(256) score_tile_kernel(InferParams p) {
     const float4* Tg = reinterpret_cast<const float4*>(p.ent);
 
     __shared__ float4 cuts[IQ];
-    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
+    __shared__ int skip;
     grid_dependency_wait();
     allow_dependents();
-    if (tid == 0) skip = p.w.status[1];
+    if (tid == 0) skip = call_given_up(p);
+    __syncthreads();
+    if (skip) return;
     if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barriers of the loop below)
     float acc[4][4], u[4][4];
 #pragma unroll
@@ -429,7 +436,6 @@ __global__ void __launch_bounds__(256) score_tile_kernel(InferParams p) {
                 if (TH) *reinterpret_cast<float4*>(&Ws[row * ILD + c4 * 4]) = wv;
             }
             __syncthreads();
-            if (skip) return;
 #pragma unroll
             for (int kk = 0; kk < IKC; kk += 4) {
                 float4 qv[4], tv[4], wv[4];
@@ -481,10 +487,13 @@ __global__ void __launch_bounds__(256) score_tile_tma_kernel(InferParams p) {
     const int q0 = qt * IQ;
     const int64_t e0 = p.e_lo + et * IE;
 
+    __shared__ int skip;
     if (tid == 0) { mbar_init(bar, ROWS); mbar_init_fence(); }
-    __syncthreads();
     grid_dependency_wait();
     allow_dependents();
+    if (tid == 0) skip = call_given_up(p);
+    __syncthreads();
+    if (skip) return;
     if (tid < ROWS) {                            // thread r owns row r
         const bool isq = tid < IQ;
         const int64_t g = isq ? q0 + tid : e0 + (tid - IQ);
@@ -499,8 +508,6 @@ __global__ void __launch_bounds__(256) score_tile_tma_kernel(InferParams p) {
         }
     }
     __shared__ float4 cuts[IQ];
-    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
-    if (tid == 128) skip = p.w.status[1];
     if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barrier that follows the wait)
 
     float acc[4][4];
@@ -516,7 +523,6 @@ __global__ void __launch_bounds__(256) score_tile_tma_kernel(InferParams p) {
         (void)mbar_wait_bounded(bar, 0u, p.wait_limit);
         return;
     }
-    if (skip) return;
     const float* Qs = base;
     const float* Ts = Qs + IQ * ld;
 #pragma unroll 2
@@ -594,9 +600,12 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
         for (int st = 0; st < nstage; ++st) mbar_init(&bars[st], 1);
         mbar_init_fence();
     }
-    __syncthreads();
+    __shared__ int skip;
     grid_dependency_wait();
     allow_dependents();
+    if (tid == 0) skip = call_given_up(p);
+    __syncthreads();
+    if (skip) return;
     auto issue = [&](int chunk, int stage) {     // (a box that begins beyond the row is left out)
         if (tid != 0) return;
         unsigned char* qs = base + (size_t)stage * ITB_STAGE_BYTES;
@@ -613,8 +622,6 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
     issue(0, 0);
     if (nchunk > 1) issue(1, 1);
     __shared__ float4 cuts[IQ];
-    __shared__ int skip;                 // (one thread's reading: the flag may change while this launch runs)
-    if (tid == 128) skip = p.w.status[1];
     if (tid >= 256 - IQ) score_tile_row_cuts(p, q0, e0, tid - (256 - IQ), cuts);     // (read after the barrier that follows the first wait)
 
     float acc[4][4];
@@ -630,8 +637,8 @@ __global__ void __launch_bounds__(256, 3) score_tile_tensor_kernel(const __grid_
         const int stage = chunk % nstage;
         const bool ok = mbar_wait_bounded(&bars[stage], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
         const bool all = __syncthreads_and(ok);
-        if (!all || skip) {
-            if (!all && tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
+        if (!all) {
+            if (tid == 0) set_status(p.w.status, KGE_ERR_TIMEOUT);
             for (int st = 0; st < min(nstage, nchunk); ++st) (void)mbar_wait_bounded(&bars[st], (uint32_t)(chunk / nstage) & 1u, p.wait_limit);
             return;
         }
@@ -978,18 +985,20 @@ int run_score_all_topk(kge_handle* h, const int32_t* qh, const int32_t* qr, int3
     // some 50 us of selection, start-up and drain each; four times as long is 7.
     //
     // The chunks are queued without waiting for one another.  A list that fills up (scores rising along the table) sets
-    // status[1]: what is queued behind does nothing, status[6] says how far the call has come, and the chunk is redone in
-    // shorter pieces (pieces of one list's worth cannot overflow).
+    // status[1]: what is queued behind does nothing, status[6] says how far the call has come, and it goes on from there with
+    // chunks an eighth as long (those of one list's worth cannot overflow), a few queued at a time.  Once they pass they grow
+    // again, after twice as many queues each time that this proved too early.
     const int64_t max_chunk = std::max<int64_t>(kCandCap, std::min<int64_t>((int64_t)1 << 22, (int64_t)0x7fffffff / p.q_tiles * IE / 2));
     const int64_t grow = std::max(1, std::min(4, 256 / k));
-    int64_t piece = max_chunk, piece_until = 0;      // entities below piece_until go in chunks of at most `piece`
-    auto chunk_len = [&](int64_t lo) {
-        const int64_t len = std::min(std::max<int64_t>(lo * grow, kCandCap), lo < piece_until ? piece : max_chunk);
-        return std::min(len, p.E - lo);
-    };
+    constexpr int kFew = 16;
+    int64_t most = max_chunk;                        // longest chunk for now
+    int passed = 0, patience = 1;
+    bool grown = false;
+    auto chunk_len = [&](int64_t lo) { return std::min(std::min(std::max<int64_t>(lo * grow, kCandCap), most), p.E - lo); };
     int64_t lo = 0;
     while (lo < p.E) {
-        for (int64_t at = lo; at < p.E;) {
+        int64_t at = lo;
+        for (int queued = 0; at < p.E && (most == max_chunk || queued < kFew); ++queued) {
             p.e_lo = at; p.e_hi = at + chunk_len(at);
             p.first = at == 0; p.last = p.e_hi == p.E;
             if (tc) {
@@ -1007,13 +1016,19 @@ int run_score_all_topk(kge_handle* h, const int32_t* qh, const int32_t* qr, int3
         int32_t* const flags = h->host_flags ? h->host_flags : words;
         KGE_CUDA_CHECK(h, cudaMemcpyAsync(flags, h->ws.status + 1, sizeof(words), cudaMemcpyDeviceToHost, s));
         KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
-        if (!flags[0]) break;
-        lo = flags[5];
-        const int64_t len = chunk_len(lo);
-        piece_until = std::max(piece_until, lo + len);
-        piece = std::max<int64_t>(kCandCap, (len / 8 + kCandCap - 1) / kCandCap * kCandCap);
-        reset_chunk_kernel<<<qblocks, 128, 0, s>>>(p);
-        KGE_LAUNCH_CHECK(h);
+        if (flags[0]) {
+            lo = flags[5];
+            most = std::max<int64_t>(kCandCap, (chunk_len(lo) / 8 + kCandCap - 1) / kCandCap * kCandCap);
+            patience = grown ? std::min(2 * patience, 64) : 1;
+            passed = 0;
+            grown = false;
+            reset_chunk_kernel<<<qblocks, 128, 0, s>>>(p);
+            KGE_LAUNCH_CHECK(h);
+        } else {
+            lo = at;
+            if (most < max_chunk) grown = ++passed >= patience;
+            if (grown) { most = std::min(8 * most, max_chunk); passed = 0; }
+        }
     }
     return KGE_OK;
 }

@@ -236,3 +236,29 @@ def test_ranks_of_few_queries(oracle32, score, d, nq):
     ids2, sc2 = t.empty((nq, K), dtype=t.int32, device=gpu.ent.device), t.empty((nq, K), dtype=t.float32, device=gpu.ent.device)
     gpu.kge.score_all_topk(gpu.dev_i32(qh), gpu.dev_i32(qr), K, None, ids2, sc2)
     assert (ids2.cpu().numpy() == ids).all() and (sc2.cpu().numpy() == sc).all()
+
+
+@pytest.mark.parametrize("score,tc,d", [("transe", False, 64), ("transh", False, 32), ("distmult", False, 16), ("distmult", True, 64)])
+def test_a_rise_after_a_restart(oracle32, score, tc, d):
+    """Two stretches of rising scores: the chunks that were cut down in the first have grown again when the second fills the
+    lists, and the second begins inside a chunk of a few queued ones."""
+    E, K = 150_000, 7
+    prob = Problem(E=E, R=2, T=50, d=d, score=score, p_norm=1, B=4, N=4, P=1, graph_seed=13, tc=tc)
+    step = np.zeros(E, np.float32)
+    step[2000:5000] = 0.25 + np.arange(3000, dtype=np.float32) // 24 / 512.0          # up to 0.494
+    step[90_000:130_000] = 0.5 + np.arange(40_000, dtype=np.float32) // 160 / 512.0   # up to 0.986
+    prob.ent[:] = 0.0
+    if score == "distmult":
+        prob.ent[:, 0] = 0.25 + step.astype(np.float32) if not tc else np.round((0.25 + step) * 128) / 128
+        prob.rel[:] = 1.0
+    else:
+        prob.ent[:, 0] = step                             # distance to the query's 2 (a head of 0 and a relation of 2) falls along the stretch
+        prob.rel[:] = 0.0; prob.rel[:, 0] = 2.0
+        if prob.relw is not None:
+            prob.relw[:] = 0.0; prob.relw[:, 1] = 1.0
+    gpu = GpuSide(prob, max_queries=70, topk=K, load_graph=False)
+    rng = np.random.default_rng(5)
+    qh, qr, tt = rng.integers(0, 1500, 66), rng.integers(0, 2, 66), rng.integers(0, E, 66)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K, true_tails=tt)
+    assert (ids == o_ids).all() and (ranks == o_ranks).all() and (sc == o_sc).all()
