@@ -1309,8 +1309,10 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     if (p.N == 256) KGE_CUDA_CHECK(h, (launch_dependent(loss_reg_kernel<1, 2>, dim3((p.B + warps / 2 - 1) / (warps / 2)), dim3(LOSS_THREADS), 0, s, p)));
     else if (p.N == 512) KGE_CUDA_CHECK(h, (launch_dependent(loss_reg_kernel<1, 4>, dim3((p.B + warps / 4 - 1) / (warps / 4)), dim3(LOSS_THREADS), 0, s, p)));
     else if (p.N == 1024) KGE_CUDA_CHECK(h, (launch_dependent(loss_reg_kernel<2, 4>, dim3((p.B + warps / 4 - 1) / (warps / 4)), dim3(LOSS_THREADS), 0, s, p)));
-    // (fewer rows than fill the GPU at eight to a CTA: a CTA per row instead, 600 rows of 1,500 scores 12 -> 7 us)
-    else if (p.N <= LOSS_WARP_MAX_N && (p.N & 3) == 0 && (p.N <= 256 || p.B >= 8 * h->num_sms)) {
+    // (a CTA per row where long rows are fewer than fill the GPU at eight to a CTA.  TransE p = 1 step, d = 32, warp against CTA per
+    // row: 300 rows of 260 scores 35.6 and 38.9 us, 900 of 516 48.2 and 50.3, 300 of 768 45.1 and 47.4: a warp at every number
+    // of rows up to 1,024 scores.  Beyond it depends: 96 rows of 1,500 48.8 and 45.5, 300 51.6 and 55.7, 600 60.9 and 61.7, 1,180 67.5 and 63.4)
+    else if (p.N <= LOSS_WARP_MAX_N && (p.N & 3) == 0 && (p.N <= 1024 || p.B >= 8 * h->num_sms)) {
         constexpr int rows = LOSS_THREADS / 32;
         KGE_CUDA_CHECK(h, launch_dependent(loss_warp_kernel, dim3((p.B + rows - 1) / rows), dim3(LOSS_THREADS), (size_t)rows * p.N * 4, s, p));
     } else {

@@ -548,9 +548,9 @@ def test_one_pass_backward_run_twice_bit_identical(score, p, d, B, N):
     assert all((a == b).all() for a, b in zip(*tables))
 
 
-# rows of 257 to 2,048 scores: a warp per row where the rows fill the GPU eight to a CTA (1,184 on 148 SMs), else a CTA per row;
-# beyond 1,536 scores the eight rows of a CTA take more than 48 KB
-@pytest.mark.parametrize("B,N", [(1200, 300), (1200, 2048), (1180, 300), (1180, 2048), (60, 260)])
+# rows of up to 2,048 scores: a warp per row, or a CTA per row where rows of over 1,024 scores are fewer than fill the GPU eight to
+# a CTA (1,184 on 148 SMs); beyond 1,536 scores the eight rows of a CTA take more than 48 KB
+@pytest.mark.parametrize("B,N", [(1200, 300), (1200, 2048), (1180, 300), (1180, 2048), (60, 260), (300, 1020), (300, 1028)])
 @pytest.mark.parametrize("loss,a", [("logsigmoid", 1.0), ("logsigmoid", 0.5), ("softmax", 0.0)])
 def test_loss_rows_on_both_sides_of_the_row_count(oracle64, B, N, loss, a):
     prob = Problem(E=3000, R=7, T=20000, d=32, score="transe", p_norm=2, loss=loss, B=B, N=N, P=2, gamma=4.0, adv_temp=a, lr=0.05, graph_seed=27)
