@@ -86,7 +86,7 @@ void pick_plan(kge_handle* h, bool compact) {
         h->split_q = pick_split(c.batch, c.num_neg, h->num_sms);
         h->split_t = pick_split(c.num_neg, c.batch, h->num_sms);
     }
-    if (h->pair_backward) pair_backward_split(c.batch, c.num_neg, c.dim / 4, h->num_sms, &h->split_q, &h->split_t);
+    if (h->pair_backward) pair_backward_split(h->kind, c.batch, c.num_neg, c.dim / 4, h->num_sms, &h->split_q, &h->split_t);
     if (c.prec == KGE_PREC_BF16_TC) {   // the backward contractions run as 128 x 128 tensor-core tiles split over K
         h->split_q = pick_split_tc(c.batch, c.dim, c.num_neg, h->num_sms);
         h->split_t = pick_split_tc(c.num_neg, c.dim, c.batch, h->num_sms);

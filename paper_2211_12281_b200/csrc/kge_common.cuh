@@ -234,7 +234,7 @@ int th_contract_slabs(const kge_handle* h);          // partial slabs the tensor
 int launch_th_contract_gemm(kge_handle* h, cudaStream_t s);
 // Backward of the distance kinds, both sides in one pass (kge_pair_backward.cu).
 bool pair_backward_serves(const kge_handle* h);
-void pair_backward_split(int B, int N, int d4, int num_sms, int* split_q, int* split_t);
+void pair_backward_split(int kind, int B, int N, int d4, int num_sms, int* split_q, int* split_t);
 int launch_pair_backward(kge_handle* h, cudaStream_t s);
 int launch_tc_forward(kge_handle* h, cudaStream_t s);
 int launch_tc_gemm_terms(kge_handle* h, const unsigned char* tmA, const unsigned char* tmB, int M, int N, int tstride, float* C,

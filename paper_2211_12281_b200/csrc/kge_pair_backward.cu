@@ -241,11 +241,15 @@ bool pair_backward_serves(const kge_handle* h) {
 
 // Column ranges (split_q: slabs of dQ) and row ranges (split_t: slabs of dT).  The CTAs of one wave fill the GPU; among the
 // divisions that do, the one whose longest CTA plus the slabs' traffic is shortest: a chunk row costs about 0.11 us per
-// CTA and SM-resident CTA pair at 256 threads, a tile's start about 24 such rows, a slab is written and read at some 5 TB/s.
-void pair_backward_split(int B, int N, int d4, int num_sms, int* split_q, int* split_t) {
+// CTA and SM-resident CTA pair at 256 threads (moduli 0.24), a tile's start about 24 such rows, a slab is written and read at some
+// 5 TB/s.  More than 64 column ranges, where the rows leave places for them, have to gain more than the chain kernel's rounds over their
+// slabs cost (eight slabs a round, some 1.2 us): 64 x 16,384 x 128 in 64 ranges 126 us a step (RotatE 207), in 128 113 (151), in 256 126
+// (129); 64 x 4,096 x 128 in 64 ranges 56 us, in 128 60 (RotatE 81 and 76).
+void pair_backward_split(int kind, int B, int N, int d4, int num_sms, int* split_q, int* split_t) {
     const int groups = pb_groups(B, d4), threads = pb_threads(d4, groups), q_tiles = (B + PB_R * groups - 1) / (PB_R * groups);
     const int ctas_per_sm = std::max(1, std::min({65536 / (threads * 128), (int)(224 * 1024 / (pb_smem(d4, groups) + 1024)), 16}));
     const int slots = num_sms * ctas_per_sm;
+    const double width = ctas_per_sm * (threads / 256.0), slab_us = d4 * 32.0 / 5e6;
     double best = 1e30;
     *split_q = *split_t = 1;
     for (int sq = 1; sq <= std::min(q_tiles, 64); ++sq) {
@@ -254,8 +258,16 @@ void pair_backward_split(int B, int N, int d4, int num_sms, int* split_q, int* s
         const int want = std::max(1, std::min({slots / rows, 64, (N + 15) / 16}));
         const int per = (N + want - 1) / want, cols = (N + per - 1) / per;
         const int waves = (rows * cols + slots - 1) / slots;
-        const double us = 0.11 * ctas_per_sm * (threads / 256.0) * waves * tiles * (per + 24) + ((double)rows * N + (double)cols * B) * d4 * 32.0 / 5e6;
+        const double us = 0.11 * width * waves * tiles * (per + 24) + ((double)rows * N + (double)cols * B) * slab_us;
         if (us < best) { best = us; *split_q = cols; *split_t = rows; }
+    }
+    const int cols64 = *split_q, rows = *split_t, tiles = (q_tiles + rows - 1) / rows;
+    double gain = 0.0;
+    for (int want = std::min(slots / rows, (N + 15) / 16); want > 64; want /= 2) {
+        const int per = (N + want - 1) / want, cols = (N + per - 1) / per;
+        const double us = (kind == KIND_CL1 ? 0.24 : 0.11) * width * tiles * ((N + cols64 - 1) / cols64 - per) - (double)(cols - cols64) * B * slab_us -
+                          1.2 * ((cols + 7) / 8 - (cols64 + 7) / 8);
+        if (us > gain) { gain = us; *split_q = cols; }
     }
 }
 
