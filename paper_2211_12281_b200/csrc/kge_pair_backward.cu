@@ -42,8 +42,6 @@ struct PairBackParams {
     int wait_limit;
 };
 
-__device__ __forceinline__ float pb_rsqrt(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-
 __device__ __forceinline__ void add_both_if_gt(float& aq, float& at, float q, float t, float w) {
     asm("{\n .reg .pred p;\n setp.gt.f32 p, %2, %3;\n @p add.f32 %0, %0, %4;\n @p add.f32 %1, %1, %4;\n}\n" : "+f"(aq), "+f"(at) : "f"(q), "f"(t), "f"(w));
 }
@@ -61,8 +59,8 @@ __device__ __forceinline__ void pair_back(float4& aq, float4& at, float4 q, floa
     const float2 a = sub2(make_float2(t.x, t.y), make_float2(q.x, q.y)), b = sub2(make_float2(t.z, t.w), make_float2(q.z, q.w));
     float wa = w, wb = w;
     if (KIND == KIND_CL1) {
-        wa *= pb_rsqrt(fmaxf(fmaf(a.x, a.x, a.y * a.y), 1e-37f));
-        wb *= pb_rsqrt(fmaxf(fmaf(b.x, b.x, b.y * b.y), 1e-37f));
+        wa *= approx_rsqrt(fmaxf(fmaf(a.x, a.x, a.y * a.y), 1e-37f));
+        wb *= approx_rsqrt(fmaxf(fmaf(b.x, b.x, b.y * b.y), 1e-37f));
     }
     aq.x = fmaf(wa, a.x, aq.x); aq.y = fmaf(wa, a.y, aq.y); aq.z = fmaf(wb, b.x, aq.z); aq.w = fmaf(wb, b.y, aq.w);
     at.x = fmaf(wa, a.x, at.x); at.y = fmaf(wa, a.y, at.y); at.z = fmaf(wb, b.x, at.z); at.w = fmaf(wb, b.y, at.w);

@@ -258,9 +258,6 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
 // ------------------------------------------------------------------------------------------
 constexpr int TN = 64;   // negative columns per score tile
 
-__device__ __forceinline__ float approx_sqrt(float x) { float r; asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-__device__ __forceinline__ float approx_rsqrt(float x) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-
 template <int KIND>
 __device__ __forceinline__ void pair_update(float& acc, float4 q, float4 t) {
     if (KIND == KIND_DOT) {

@@ -199,7 +199,6 @@ struct UpdateParams {
     float lr, beta1, beta2, eps, corr1, corr2;   // corr = 1 - beta^t
 };
 
-__device__ __forceinline__ float approx_sqrt(float x) { float r; asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 __device__ __forceinline__ float approx_rcp(float x) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
 template <typename V> struct VecOps;
