@@ -40,6 +40,7 @@ struct EnsParams {
     int left_log2, log2_parts; // second launch: slots of its table, passes over the lists
     int sort_here;             // second launch: its memory holds the sort too
     uint32_t inv_k;            // ceil(2^32 / K): e / K = umulhi(e, inv_k) for every entry index e of a block of models; 0: K = 1
+    uint32_t inv_quads;        // the same for the quads of a list, ceil(K / 4); 0: one
 };
 
 __device__ __forceinline__ bool ens_before(double sa, int32_t ia, double sb, int32_t ib) { return sa > sb || (sa == sb && ia < ib); }
@@ -213,6 +214,226 @@ __device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64
     if (p.out_scores) p.out_scores[(int64_t)q * p.top_n + r] = s != 0ull ? ens_unordered(s) : -INFINITY;
 }
 
+// ------------------------------------------------------------------------------------------
+// Unions of at most ENS_REGS entities per thread.  A thread takes four places of one list at a time, whose first probes
+// are in flight together; what a lane has left over of its four is probed one step at a time by the whole warp, so that a
+// warp's rounds are those of its unluckiest lane's four and not of its unluckiest lane four times.  The table is sparse
+// (2,048 slots for 768 entities) for the same reason.  The sums stay in registers: entity i of the order of arrival belongs
+// to thread i mod threads, which adds its rank scores model by model.  The rank scores lie in ENS_COPIES copies side by side,
+// a lane reads its own: a random look-up in one copy would meet three others in its bank.  An entity twice in one list
+// loses one of its two bytes (position + 1), so that the bytes read add up to less than the bytes written.
+// ------------------------------------------------------------------------------------------
+constexpr int ENS_REGS = 3, ENS_COPIES = 8, ENS_CAND = 64, ENS_CUT_TOP = 16;
+template <int MB>
+constexpr size_t ens_union_smem(int slots, int K) {
+    return (size_t)(K + 1) * ENS_COPIES * sizeof(double) + (size_t)slots * (sizeof(int32_t) + MB) + (size_t)slots * sizeof(uint16_t);
+}
+
+// V: places of a list that lie on one boundary of a load (4, 2 or 1).  Returns 0, or (all threads) why the table was given up.
+template <int MB, int V>
+__device__ int ens_union_query(const EnsParams& p, const int q, const int log2_slots, const int limit, unsigned char* smem) {
+    constexpr int WORDS = MB / 4;
+    const int slots = 1 << log2_slots, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, K = p.K;
+    double* tab = reinterpret_cast<double*>(smem);                              // [K + 1][copies] absent score, then positions 1 .. K
+    int32_t* key = reinterpret_cast<int32_t*>(tab + (size_t)(K + 1) * ENS_COPIES);   // [slots] entity id or -1
+    uint32_t* cell = reinterpret_cast<uint32_t*>(key + slots);                  // [MB / 4][slots] bytes: position + 1 in the block's models
+    uint16_t* used = reinterpret_cast<uint16_t*>(cell + (size_t)WORDS * slots);      // [slots] occupied slots, in order of arrival
+    __shared__ int n_used, lost;
+    for (int i = tid; i < slots; i += nthr) key[i] = -1;
+    for (int i = tid; i < slots * WORDS; i += nthr) cell[i] = 0u;
+    for (int i = tid; i < (K + 1) * ENS_COPIES; i += nthr) tab[i] = p.table[i < ENS_COPIES ? K : i / ENS_COPIES - 1];
+    if (tid == 0) { n_used = 0; lost = 0; }
+    const int quads = (K + 3) >> 2, per_block = min(MB, nthr / quads);           // quads of a list; models per block: a quad per thread
+    const int ml = p.inv_quads ? (int)__umulhi((uint32_t)tid, p.inv_quads) : tid, pos = 4 * (tid - ml * quads);
+    const int64_t list_step = (int64_t)p.nq * K;
+    const int32_t* src = p.lists + ((int64_t)ml * p.nq + q) * K + pos;
+    auto fetch = [&](int m0, int32_t (&id)[4]) {
+        const bool in = ml < per_block && m0 + ml < p.M;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) id[u] = -1;
+        if (!in) return;
+        if constexpr (V == 4) {
+            const int4 x = *reinterpret_cast<const int4*>(src);
+            id[0] = x.x; id[1] = x.y; id[2] = x.z; id[3] = x.w;
+        } else if constexpr (V == 2) {
+            const int2 x = *reinterpret_cast<const int2*>(src);
+            id[0] = x.x; id[1] = x.y;
+            if (pos + 2 < K) { const int2 y = *reinterpret_cast<const int2*>(src + 2); id[2] = y.x; id[3] = y.y; }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) if (pos + u < K) id[u] = src[u];
+        }
+    };
+    int32_t next[4];
+    fetch(0, next);
+    __syncthreads();
+    const double* mytab = tab + (lane & (ENS_COPIES - 1));
+    const double absent = tab[0];
+    double before = 0.0, sum[ENS_REGS];     // before: an entity's sum over the models ahead of the block it first appears in
+    int slot[ENS_REGS];
+#pragma unroll
+    for (int r = 0; r < ENS_REGS; ++r) { sum[r] = 0.0; slot[r] = 0; }
+    int seen = 0;                           // occupied slots after the blocks so far
+    uint32_t bytes = 0;                     // positions written less positions read
+    unsigned char* mycell = reinterpret_cast<unsigned char*>(cell + (size_t)(ml >> 2) * slots) + (ml & 3);
+    for (int m0 = 0; m0 < p.M; m0 += per_block) {
+        const int mb = min(per_block, p.M - m0);
+        int32_t want[4], k[4];
+        uint32_t h[4];
+        uint32_t left = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            want[u] = next[u];
+            h[u] = (uint32_t)want[u] * 0x9E3779B1u >> (32 - log2_slots);
+            k[u] = reinterpret_cast<volatile int32_t*>(key)[h[u]];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (want[u] >= 0 && k[u] != want[u]) left |= 1u << u;               // (unused places of a list hold -1)
+        while (__any_sync(0xffffffffu, left != 0u)) {                           // (a slot is always free: see the launch)
+            if (left) {
+                const bool b0 = left & 1u, b1 = left & 2u, b2 = left & 4u;
+                const int32_t w = b0 ? want[0] : (b1 ? want[1] : (b2 ? want[2] : want[3]));
+                uint32_t g = b0 ? h[0] : (b1 ? h[1] : (b2 ? h[2] : h[3]));
+                int32_t x = reinterpret_cast<volatile int32_t*>(key)[g];
+                if (x == -1) {
+                    x = atomicCAS(key + g, -1, w);
+                    if (x == -1) { used[atomicAdd(&n_used, 1)] = (uint16_t)g; x = w; }
+                }
+                if (x == w) left &= left - 1u;
+                else {
+                    g = (g + 1) & (uint32_t)(slots - 1);
+                    if (b0) h[0] = g; else if (b1) h[1] = g; else if (b2) h[2] = g; else h[3] = g;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (want[u] >= 0) {
+                mycell[4 * h[u]] = (unsigned char)(pos + 1 + u);
+                bytes += (uint32_t)(pos + 1 + u);
+            }
+        src += per_block * list_step;
+        fetch(m0 + per_block, next);                                            // on its way while this block is summed
+        __syncthreads();
+        const int total = n_used;
+        if (total > limit) return ENS_BAD_FULL;
+#pragma unroll
+        for (int r = 0; r < ENS_REGS; ++r) {
+            const int i = r * nthr + tid;
+            if (i >= total) break;
+            if (i >= seen) { slot[r] = used[i]; sum[r] = before; }
+            double s = sum[r];
+#pragma unroll
+            for (int w = 0; w < WORDS; ++w) {
+                if (4 * w >= mb) break;
+                const uint32_t c = cell[w * slots + slot[r]];
+                if (c == 0u && absent == 0.0) continue;                         // (s is never -0: adding 0 leaves it as it is)
+                cell[w * slots + slot[r]] = 0u;
+                bytes -= __dp4a(c, 0x01010101u, 0u);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (4 * w + j < mb) s += mytab[(c >> (8 * j) & 0xffu) * ENS_COPIES];
+            }
+            sum[r] = s;
+        }
+        seen = total;
+        if (absent != 0.0) for (int m = 0; m < mb; ++m) before += absent;
+        __syncthreads();
+    }
+    bytes = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0 && bytes) atomicAdd(&lost, (int)bytes);
+
+    // The best top_n.  Up to ENS_CUT_TOP: the top_n-th best of 32 groups' best scores (upper halves) is a bound that at least top_n
+    // entities reach; those that do, hardly more, are ranked against one another.  Otherwise, and where too many reach it: a round per place.
+    uint64_t os[ENS_REGS];                  // ordered scores, 0: none or taken
+    int32_t id[ENS_REGS];
+    uint32_t top_hi = 0;
+#pragma unroll
+    for (int r = 0; r < ENS_REGS; ++r) {
+        const bool in = r * nthr + tid < seen;
+        os[r] = in ? ens_ordered(sum[r]) : 0ull;
+        id[r] = in ? key[slot[r]] : INT32_MAX;
+        top_hi = max(top_hi, (uint32_t)(os[r] >> 32));
+    }
+    __shared__ uint64_t cand_s[ENS_CAND];
+    __shared__ int32_t cand_i[ENS_CAND];
+    __shared__ uint32_t group_hi[32];
+    __shared__ uint32_t cut;
+    __shared__ int n_cand;
+    if (p.top_n <= ENS_CUT_TOP) {
+        const int per_group = nthr >> 5;                                        // 2, 4 or 8 lanes
+        for (int o = per_group >> 1; o > 0; o >>= 1) top_hi = max(top_hi, __shfl_xor_sync(0xffffffffu, top_hi, o));
+        if ((tid & (per_group - 1)) == 0) group_hi[tid / per_group] = top_hi;
+        if (tid == 0) n_cand = 0;
+    }
+    __syncthreads();
+    if (lost) return ENS_BAD_TWICE;
+    if (p.top_n <= ENS_CUT_TOP) {
+        if (tid < 32) {
+            uint32_t v = group_hi[tid], c = 0;
+            for (int found = 0; found < p.top_n;) {
+                c = __reduce_max_sync(0xffffffffu, v);
+                if (c == 0u) break;
+                const bool hit = v == c;
+                found += __popc(__ballot_sync(0xffffffffu, hit));
+                if (hit) v = 0u;
+            }
+            if (tid == 0) cut = c;
+        }
+        __syncthreads();
+        const uint32_t c = cut;
+#pragma unroll
+        for (int r = 0; r < ENS_REGS; ++r)
+            if (os[r] != 0ull && (uint32_t)(os[r] >> 32) >= c) {
+                const int at = atomicAdd(&n_cand, 1);
+                if (at < ENS_CAND) { cand_s[at] = os[r]; cand_i[at] = id[r]; }
+            }
+        __syncthreads();
+        const int n = n_cand;
+        if (n <= ENS_CAND) {
+            if (tid < max(n, p.top_n)) {
+                int rank = tid;
+                if (tid < n) {
+                    const uint64_t s = cand_s[tid];
+                    const int32_t e = cand_i[tid];
+                    rank = 0;
+                    for (int j = 0; j < n; ++j) rank += cand_s[j] > s || (cand_s[j] == s && cand_i[j] < e);
+                    if (rank < p.top_n) ens_put(p, q, rank, s, e);
+                } else {
+                    ens_put(p, q, rank, 0ull, 0);
+                }
+            }
+            return 0;
+        }
+    }
+    __shared__ uint64_t red_s[2][32];
+    __shared__ int32_t red_i[2][32];
+    const int warp = tid >> 5, nwarps = nthr >> 5;
+    uint64_t ws; int32_t wi;                // the warp's best
+    auto warp_best = [&] {
+        uint64_t bs = 0; int32_t bi = INT32_MAX;
+#pragma unroll
+        for (int r = 0; r < ENS_REGS; ++r)
+            if (os[r] > bs || (os[r] == bs && id[r] < bi)) { bs = os[r]; bi = id[r]; }
+        ens_warp_best(bs, bi, ws, wi);
+    };
+    warp_best();
+    for (int r = 0; r < p.top_n; ++r) {
+        if (lane == 0) { red_s[r & 1][warp] = ws; red_i[r & 1][warp] = wi; }
+        __syncthreads();
+        uint64_t s; int32_t e;
+        ens_warp_best(lane < nwarps ? red_s[r & 1][lane] : 0ull, lane < nwarps ? red_i[r & 1][lane] : INT32_MAX, s, e);   // (every warp for itself)
+        if (tid == 0) ens_put(p, q, r, s, e);
+        if (s != 0ull && s == ws && e == wi) {                                  // taken (ids are distinct: one warp, one thread)
+#pragma unroll
+            for (int u = 0; u < ENS_REGS; ++u) if (id[u] == e) { os[u] = 0ull; id[u] = INT32_MAX; }
+            warp_best();
+        }
+    }
+    return 0;
+}
+
 // The whole of a query in one table.
 template <int MB>
 __device__ int ens_hash_query(const EnsParams& p, const int q, const int log2_slots, const int limit, unsigned char* smem) {
@@ -311,6 +532,9 @@ __device__ void ens_sort_query(const EnsParams& p, const int q, unsigned char* e
     }
 }
 
+template <int NT>
+__device__ __noinline__ void ens_sort_call(const EnsParams& p, int q, unsigned char* smem) { ens_sort_query<NT>(p, q, smem); }
+
 // Lists of more than ENS_MAX_K places: every query takes the general form.
 template <int NT>
 __global__ void __launch_bounds__(NT) ensemble_sort_kernel(EnsParams p) {
@@ -340,9 +564,6 @@ __device__ void ens_left(const EnsParams& p, bool table, bool sort, Serve serve)
     }
 }
 
-template <int NT>
-__device__ __noinline__ void ens_sort_call(const EnsParams& p, int q, unsigned char* smem) { ens_sort_query<NT>(p, q, smem); }
-
 // The queries left to the sort, where the second launch's memory is more than the sort's.  Four times as many CTAs as are resident,
 // so that those of an SM are not all in the same phase (15,000 queries of 30 lists of 100, every one sorted: 5.69 -> 5.06 ms; a
 // CTA per query, as where all are sorted from the start, 4.57).
@@ -354,21 +575,24 @@ __global__ void __launch_bounds__(512) ensemble_sort_left_kernel(EnsParams p) {
 
 // Lists so short that a table of 1.5 slots per entry fits (M K <= 682): one launch, no table overflows, and a query with an
 // entity twice in one list is sorted where it stands (the sort needs no more memory than the table).
-constexpr int ENS_MB = 16, ENS_MAX_LOG2 = 10;
+constexpr int ENS_SMALL_MB = 16, ENS_SMALL_LOG2 = 10;
+template <int V>
 __global__ void __launch_bounds__(256) ensemble_small_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
-    if (!ens_hash_query<ENS_MB>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
+    if (!ens_union_query<ENS_SMALL_MB, V>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
     __syncthreads();
-    ens_sort_query<0>(p, blockIdx.x, ens_smem);
+    ens_sort_call<0>(p, blockIdx.x, ens_smem);
 }
 
-// Longer lists, first launch: one CTA per query, 16 models at a time, 1,024 slots (31 KB: seven CTAs per SM).  85 x top-100 lists of
-// 15,000 queries, unions of 300: 36.7 ms as a sort, 0.93 ms with 32 models at a time (four CTAs), 0.87 with 8, 0.81 with 16; 128 threads
-// 1.00 ms.  Bound by instruction issue (about 48,000 warp instructions a query, 74 % of the slots), not by the 510 MB of lists (78 us).
+// Longer lists, first launch: one CTA of 256 threads per query.  A block of models is at most 256 quads, 1,024 places, so that with
+// ENS_LIMIT entities before it a slot is always free.
+constexpr int ENS_LOG2 = 11, ENS_LIMIT = 256 * ENS_REGS, ENS_MB = 12;
+static_assert(ENS_LIMIT + 1024 < 1 << ENS_LOG2, "a probe ends");
+template <int V>
 __global__ void __launch_bounds__(256) ensemble_hash_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
     allow_dependents();
-    const int bad = ens_hash_query<ENS_MB>(p, blockIdx.x, ENS_MAX_LOG2, 3 << (ENS_MAX_LOG2 - 2), ens_smem);
+    const int bad = ens_union_query<ENS_MB, V>(p, blockIdx.x, ENS_LOG2, ENS_LIMIT, ens_smem);
     if (bad && threadIdx.x == 0) p.out_ids[(int64_t)blockIdx.x * p.top_n] = bad == ENS_BAD_TWICE ? ENS_SORT : ENS_LEFT;
 }
 
@@ -456,6 +680,10 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
         constexpr int sort_max = (int)(ENS_MAX_ENTRIES * (sizeof(uint64_t) + sizeof(int32_t)));
         static_assert(parts_smem <= sort_max, "the larger table fits where the sort does");
         cudaError_t e0 = cudaSuccess;
+        constexpr int union_max = (int)std::max(ens_union_smem<ENS_MB>(1 << ENS_LOG2, ENS_MAX_K), ens_union_smem<ENS_SMALL_MB>(1 << ENS_SMALL_LOG2, ENS_MAX_K));
+        for (void (*k)(EnsParams) : {ensemble_small_kernel<1>, ensemble_small_kernel<2>, ensemble_small_kernel<4>,
+                                     ensemble_hash_kernel<1>, ensemble_hash_kernel<2>, ensemble_hash_kernel<4>})
+            if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, union_max);
         for (void (*k)(EnsParams) : {ensemble_sort_kernel<256>, ensemble_sort_kernel<512>, ensemble_sort_kernel<ENS_THREADS>, ensemble_sort_left_kernel,
                                      ensemble_left_kernel<256>, ensemble_left_kernel<512>, ensemble_left_kernel<ENS_THREADS>})
             if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_max);
@@ -469,18 +697,25 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
     p.inv_k = (uint32_t)((((uint64_t)1 << 32) + k_list - 1) / k_list);
+    const int quads = (k_list + 3) / 4;
+    p.inv_quads = quads == 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + quads - 1) / quads);
+    auto pick = [&](void (*k4)(EnsParams), void (*k2)(EnsParams), void (*k1)(EnsParams)) {    // the widest load that every quad's address allows
+        const uintptr_t at = reinterpret_cast<uintptr_t>(lists);
+        return k_list % 4 == 0 && at % 16 == 0 ? k4 : (k_list % 2 == 0 && at % 8 == 0 ? k2 : k1);
+    };
     p.log2_slots = 5;
     while (2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
-    if (p.log2_slots <= ENS_MAX_LOG2) {
+    if (p.log2_slots <= ENS_SMALL_LOG2) {
         const int threads = p.log2_slots >= 9 ? 256 : (p.log2_slots >= 7 ? 128 : 64);
-        ensemble_small_kernel<<<nq, threads, ens_hash_smem<ENS_MB>(1 << p.log2_slots, k_list), s>>>(p);
+        pick(ensemble_small_kernel<4>, ensemble_small_kernel<2>, ensemble_small_kernel<1>)
+            <<<nq, threads, std::max(ens_union_smem<ENS_SMALL_MB>(1 << p.log2_slots, k_list), sort_smem), s>>>(p);
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
-    ensemble_hash_kernel<<<nq, 256, ens_hash_smem<ENS_MB>(1 << ENS_MAX_LOG2, k_list), s>>>(p);
+    pick(ensemble_hash_kernel<4>, ensemble_hash_kernel<2>, ensemble_hash_kernel<1>)<<<nq, 256, ens_union_smem<ENS_MB>(1 << ENS_LOG2, k_list), s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return KGE_ERR_CUDA;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;
-    p.log2_parts = 0; p.left_log2 = ENS_MAX_LOG2 + 1;
+    p.log2_parts = 0; p.left_log2 = ENS_LOG2;
     while (p.left_log2 < ENS_BIG_LOG2 && 3 << (p.left_log2 - 2) < num_models * k_list) ++p.left_log2;
     while (num_models * k_list > ENS_BIG_PART << p.log2_parts) ++p.log2_parts;
     auto launch_left = [&](void (*kernel)(EnsParams), int threads, size_t smem, int waves) {
@@ -489,11 +724,11 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
     };
     const size_t table_smem = p.log2_parts > 0 ? parts_smem : ens_hash_smem<ENS_BIG_MB>(1 << p.left_log2, k_list);
     // (where the sort takes much less memory than the table, and so more CTAs of it share an SM, it is a launch of its own)
-    const bool sort_apart = p.left_log2 > ENS_MAX_LOG2 + 1 && p.n2 <= 8192;
+    const bool sort_apart = p.left_log2 > ENS_LOG2 && p.n2 <= 8192;
     p.sort_here = sort_apart ? 0 : 1;
     const size_t left_smem = sort_apart ? table_smem : std::max(table_smem, sort_smem);
-    if (p.left_log2 == ENS_MAX_LOG2 + 1) e = launch_left(ensemble_left_kernel<256>, 256, left_smem, 2);
-    else if (p.left_log2 == ENS_MAX_LOG2 + 2) e = launch_left(ensemble_left_kernel<512>, 512, left_smem, 1);
+    if (p.left_log2 == ENS_LOG2) e = launch_left(ensemble_left_kernel<256>, 256, left_smem, 2);
+    else if (p.left_log2 == ENS_LOG2 + 1) e = launch_left(ensemble_left_kernel<512>, 512, left_smem, 1);
     else e = launch_left(ensemble_left_kernel<ENS_THREADS>, ENS_THREADS, left_smem, 1);
     if (e == cudaSuccess && sort_apart) e = launch_left(ensemble_sort_left_kernel, 512, sort_smem, 4);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
