@@ -62,9 +62,8 @@ int pick_split_waves(int rows, int cols, int num_sms, int ctas_per_sm, int rows_
 // Tensor-core contraction [rows, cols] over `depth` on persistent CTAs (one per SM): as many K
 // splits as still give every SM at most one tile (or one split when there are more tiles than
 // SMs), each at least four 64-wide slices deep, at most 16, none empty.
-int pick_split_tc(int rows, int cols, int depth, int num_sms) {
-    const int bn = tc_backward_tile_cols(cols);
-    const int tiles = ((rows + 127) / 128) * ((cols + bn - 1) / bn);
+int pick_split_tc(int rows, int cols, int depth, int num_sms, bool xcol = false) {
+    const int tiles = ((rows + 127) / 128) * tc_backward_col_tiles(cols, xcol);
     const int kb = (depth + 63) / 64;
     const int want = std::max(1, std::min(std::min(num_sms / tiles, std::max(1, kb / 4)), 16));
     const int per = (kb + want - 1) / want;
@@ -88,8 +87,8 @@ void pick_plan(kge_handle* h, bool compact) {
     }
     if (h->pair_backward) pair_backward_split(h->kind, c.batch, c.num_neg, c.dim / 4, h->num_sms, &h->split_q, &h->split_t);
     if (c.prec == KGE_PREC_BF16_TC) {   // the backward contractions run as 128 x 128 tensor-core tiles split over K
-        h->split_q = pick_split_tc(c.batch, c.dim, c.num_neg, h->num_sms);
-        h->split_t = pick_split_tc(c.num_neg, c.dim, c.batch, h->num_sms);
+        h->split_q = pick_split_tc(c.batch, c.dim, c.num_neg, h->num_sms, h->kind == KIND_L2);
+        h->split_t = pick_split_tc(c.num_neg, c.dim, c.batch, h->num_sms, h->kind == KIND_L2);
     }
     h->split_mh = h->split_mt = 1;
     if (c.feat_dim > 0) {   // dM = dE^T . F: [d, F] over the role's slots, split over the slots so that every SM has a tile
@@ -136,15 +135,13 @@ size_t layout(const kge_handle* h, char* base, int64_t T, int32_t maxq, int32_t 
     w.tn2 = tc ? cv.take<float>(N) : nullptr;
     const size_t ldN = (N + 7) / 8 * 8;
     w.Gb = tc ? cv.take<uint16_t>(B * ldN) : nullptr;
-    w.Gcol = tc ? cv.take<float>(N) : nullptr;
-    const size_t tiles_n = (N + 127) / 128, tiles_m = (B + 127) / 128;
+    const size_t tiles_n = (N + 127) / 128;
     w.stat_part = tc ? cv.take<float>(B * tc_pieces_per_tile() * tiles_n * 4) : nullptr;
     w.row_stat = tc ? cv.take<float>(B * 2) : nullptr;
-    w.grow_part = tc ? cv.take<float>(B * tc_pieces_per_tile() * tiles_n) : nullptr;
-    w.gcol_part = tc ? cv.take<float>(4 * tiles_m * N) : nullptr;
+    w.xsum_q = w.stat_part;      // (a split is at least 256 negatives deep: [Sq, B] fits)
     w.Grow = cv.take<float>(B);
     w.Cpart = cv.take<float>((size_t)h->split_t * N);
-    w.F = cv.take<float>(B * N);
+    w.F = tc ? nullptr : cv.take<float>(B * N);
     w.U = th ? cv.take<float>(B * N) : nullptr;
     w.Cc = th ? cv.take<float>(B * N) : nullptr;
     w.wsum = th ? cv.take<float>(B) : nullptr;
@@ -160,6 +157,7 @@ size_t layout(const kge_handle* h, char* base, int64_t T, int32_t maxq, int32_t 
     w.dWpart = th ? cv.take<float>(((size_t)h->split_q + xs) * B * d) : nullptr;
     w.dTpart = cv.take<float>(((size_t)h->split_t + xs) * N * d);
     w.grad_ent = cv.take<float>((2 * B + N) * d);
+    w.Xq = tc ? reinterpret_cast<uint16_t*>(w.grad_ent) : nullptr;
     w.grad_rel = cv.take<float>(B * kw);
     w.grad_relw = th ? cv.take<float>(B * d) : nullptr;
     const size_t ne = 2 * B + N;
@@ -390,6 +388,7 @@ int kge_bind(kge_handle* h, float* ent, float* rel, float* relw, float* ent_stat
         if (rc == KGE_OK) rc = tc_make_operand_map(h, h->tm_g64, h->ws.Gb, B, N, ldN, 64);
         if (rc == KGE_OK) rc = tc_make_operand_map(h, h->tm_t64, h->ws.Tb, N, d, d, 64);
         if (rc == KGE_OK) rc = tc_make_operand_map(h, h->tm_q64, h->ws.Qb, B, d, d, 64);
+        if (rc == KGE_OK) rc = tc_make_operand_map(h, h->tm_x64, h->ws.Xq, B, 64, 64, 64);
         if (rc == KGE_OK && h->ws.Eb) {
             rc = tc_make_operand_map(h, h->tm_iq, h->ws.iqb, max_queries, d, d, 128);
             if (rc == KGE_OK) rc = tc_make_operand_map(h, h->tm_eb, h->ws.Eb, h->cfg.num_entities, d, d, 128);
@@ -912,16 +911,19 @@ int kge_debug_export(kge_handle* h, int tap, void* dst, size_t bytes, void* stre
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (tap == KGE_TAP_G && h->cfg.prec == KGE_PREC_BF16_TC) {
-        // the tensor-core path keeps dL/dF only as bf16 [B, ldN]: widen it on the host
+        // the tensor-core path keeps dL/dF only as bf16 [B, ldN] up to a factor per row: widened on the host
         const size_t B = h->cfg.batch, N = h->cfg.num_neg, ldN = (N + 7) / 8 * 8;
         std::vector<uint16_t> tmp(B * ldN);
+        std::vector<float> factor(B);
         KGE_CUDA_CHECK(h, cudaMemcpyAsync(tmp.data(), w.Gb, tmp.size() * 2, cudaMemcpyDeviceToHost, s));
+        KGE_CUDA_CHECK(h, cudaMemcpyAsync(factor.data(), w.Grow, B * 4, cudaMemcpyDeviceToHost, s));
         KGE_CUDA_CHECK(h, cudaStreamSynchronize(s));
         float* out = static_cast<float*>(dst);
         for (size_t b = 0; b < B; ++b)
             for (size_t n = 0; n < N; ++n) {
                 const uint32_t bits = (uint32_t)tmp[b * ldN + n] << 16;
                 std::memcpy(&out[b * N + n], &bits, 4);
+                out[b * N + n] *= factor[b];
             }
         return KGE_OK;
     }

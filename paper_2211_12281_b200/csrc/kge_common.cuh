@@ -58,13 +58,13 @@ struct Workspace {
     float *dMpart;                         // [split_mh + split_mt][d, F] partial gradients of M_H, M_T
     float *reg_s3;                         // [2B+N] sum of |e_k|^3 of the gathered rows [heads | tails | negs] (L3 regulariser), or NULL
     uint16_t *Qb, *Tb;                     // [B,d], [N,d] bf16 copies of Q and Tneg (tensor-core scoring)
-    uint16_t *Gb;                          // bf16 [B,ldN] dL/dF (ldN = N rounded up to 8)
-    float *Gcol;                           // [N] column sums of dL/dF (TransE p=2 on tensor cores)
+    uint16_t *Gb;                          // bf16 [B,ldN] dL/dF up to a factor per row, Grow (ldN = N rounded up to 8)
     float *stat_part, *row_stat;           // [B, pieces, 4], [B, 2] loss statistics of the fused tensor-core forward
-    float *grow_part, *gcol_part;          // [B, pieces], [4*tiles_m, N] partial sums of dL/dF
+    uint16_t *Xq;                          // [B, 64] bf16, TransE p=2 on tensor cores: the row factors as two terms (in grad_ent, which is written later)
+    float *xsum_q;                         // [Sq, B] sums of dL/dF per query and split, without the row's factor (in stat_part, which is read before)
     float *qn2, *tn2;                      // [B], [N] squared norms of the fp32 rows (TransE p=2 by norm expansion)
-    float *Grow;                           // [B] row sums of dL/dF (TransE p=1 backward)
-    float *Cpart;                          // [St, N] column sums of dL/dF per row split (TransE p=1 backward)
+    float *Grow;                           // [B] row sums of dL/dF (TransE p=1 backward); tensor cores: what the rows of Gb are still to be multiplied by
+    float *Cpart;                          // [St, N] column sums of dL/dF per row split (TransE p=1 backward; p=2 on tensor cores)
     float *F;                              // [B,N] scores, overwritten by dL/dF
     float *U, *Cc;                         // [B,N] TransH: w.t and the contraction c' = sum_k s_k w_k of every pair
     float *wsum;                           // [B] TransH: sum of the unit normal's coordinates
@@ -133,8 +133,8 @@ struct kge_handle {
     // Side streams and events of the training step: the sort of the touched ids and one of the
     // two backward accumulations run beside the main stream's kernels (created by kge_bind).
     // TMA tensor maps (tensor-core path): Qb, Tb (128-row boxes) for the scores; Gb (128-row boxes) and Tb (64-row boxes,
-    // read MN-major) for dQ; Gb and Qb (64-row boxes, read MN-major) for dT
-    alignas(64) unsigned char tm_q[128], tm_t[128], tm_g[128], tm_g64[128], tm_t64[128], tm_q64[128];
+    // read MN-major) for dQ; Gb and Qb (64-row boxes, read MN-major) for dT, with Xq as one more column
+    alignas(64) unsigned char tm_q[128], tm_t[128], tm_g[128], tm_g64[128], tm_t64[128], tm_q64[128], tm_x64[128];
     alignas(64) unsigned char tm_cs[128], tm_cs64[128], tm_ts64[128], tm_ws64[128], tm_w3[128], tm_t3[128];   // TransH splits: Csb K-major / MN-major, Tsb, Wsb
     alignas(64) unsigned char tm_iq[128], tm_eb[128];   // inference: bf16 query vectors and bf16 entity table
     alignas(64) unsigned char tm_iq32[128], tm_ent32[128];   // inference on CUDA cores: fp32 query vectors and entity table in 64-row x 32-float boxes
@@ -223,6 +223,8 @@ int tc_make_operand_map(kge_handle* h, void* map_out, const void* base, int64_t 
 // Tensor map of a row-major fp32 matrix [rows, cols] read in boxes of 64 rows x 32 floats with the 128-byte swizzle.
 int tc_make_f32_tile_map(kge_handle* h, void* map_out, const void* base, int64_t rows, int64_t cols);
 int tc_backward_tile_cols(int cols);
+int tc_backward_col_tiles(int cols, bool xcol);
+constexpr int TC_REDO_FLAG = 7;      // status word: a row of dL/dF is left to the second round of this step
 int tc_pieces_per_tile();
 // The dT contraction of the dot-product kinds with a single K split is the negatives' gradient rows: it writes them in place.
 bool tc_negatives_direct(const kge_handle* h);

@@ -9,12 +9,11 @@
 // other accumulator meanwhile (a warp may only touch the 32 lanes of its own quarter; four warps
 // share a quarter, a quarter of the columns each) and apply the epilogue:
 //   EPI_STORE   C = acc (the score block as a test reads it)
-//   EPI_STATS   no score leaves the chip: per row and 64-column piece the running maximum, the sum
-//               of exponentials and the weighted loss sum of Section 3.1 "Loss Functions"; the
+//   EPI_LOSS    no score leaves the chip: dL/dF up to a factor of the row as bf16, for the two backward contractions, and per row
+//               and 64-column piece the sum of exponentials and the weighted loss sum of Section 3.1 "Loss Functions"; the
 //               score is the contraction (DistMult, ComplEx) or, for TransE with p = 2, the
 //               norm expansion -sqrt(max(|q|^2 + |t|^2 - 2 acc, 0))
-//   EPI_GRAD    scores recomputed, dL/dF formed from the finished row statistics and written as
-//               bf16 in both orientations for the two backward contractions
+//   EPI_GRAD    dL/dF of the few rows, if any, whose scores lie too far from what EPI_LOSS took as their reference
 // Every wait on a barrier is bounded; a wait that runs out records KGE_ERR_TIMEOUT, tells the
 // other warps to stop, and the CTA still releases its tensor memory before it returns.
 #include <cuda.h>
@@ -41,8 +40,8 @@ constexpr int TC_PIECE = TC_BN / TC_EPI_GROUPS;           // columns of a 128-wi
 // measured against eight, C3 passes 41.5 / 58.0 -> 39.4 / 53.8 us, the special-function-bound C4 passes 98.7 / 154.7 -> 98.9 / 135.8 us,
 // although sixteen warps leave 96 registers per thread and the norm-expansion variants spill a little.
 constexpr int TC_FUSED_WARPS_256 = 16;
-__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 3 = EPI_TOPK, 1 / 2 = the fused loss epilogues
-    return (epi & 3) == 3 ? TC_EPI_WARPS_TOPK : ((((epi & 3) == 1 || (epi & 3) == 2) && bn == 256) ? TC_FUSED_WARPS_256 : TC_EPI_WARPS);
+__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 3 = EPI_TOPK, 1 = the fused loss epilogue
+    return (epi & 3) == 3 ? TC_EPI_WARPS_TOPK : (((epi & 3) == 1 && bn == 256) ? TC_FUSED_WARPS_256 : TC_EPI_WARPS);
 }
 __host__ __device__ constexpr int tc_threads(int epi, int bn = 128) { return 32 * (2 + tc_epi_warps(epi, bn)); }
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;
@@ -51,8 +50,8 @@ __host__ __device__ constexpr uint32_t tc_stage_bytes(int bn) { return TC_A_BYTE
 __host__ __device__ constexpr size_t tc_smem_bytes(int bn) { return 1024 + (size_t)TC_STAGES * tc_stage_bytes(bn) + 256; }
 constexpr int TC_BEAT_ROWS_MAX = 8 * 1024;                 // queries whose rank counts fit in shared memory beside the 256-column stages
 
-enum { EPI_STORE = 0, EPI_STATS = 1, EPI_GRAD = 2, EPI_TOPK = 3, EPI_L2 = 4, EPI_CE = 8,    // L2 / CE: flags of the fused loss epilogues
-       EPI_A1 = 16 };   // log-sigmoid loss of a distance score with self-adversarial temperature exactly 1 (see tc_stats_chunk)
+enum { EPI_STORE = 0, EPI_LOSS = 1, EPI_GRAD = 2, EPI_TOPK = 3, EPI_L2 = 4, EPI_CE = 8,    // L2 / CE: flags of the fused loss epilogues
+       EPI_A1 = 16 };   // log-sigmoid loss of a distance score with self-adversarial temperature exactly 1 (see tc_loss_chunk)
 
 struct TcGemmParams {
     int M, N, K;
@@ -64,15 +63,14 @@ struct TcGemmParams {
     const float *row_norm2, *col_norm2;   // norm expansion: |q_b|^2 [M], |t_n|^2 [N]
     int32_t* status;
     int wait_limit;                       // tries of a bounded barrier wait
-    // fused loss epilogues (EPI_STATS, EPI_GRAD): the score is acc, or for l2 != 0 the distance score above
+    // fused loss epilogues (EPI_LOSS, EPI_GRAD): the score is acc, or for l2 != 0 the distance score above
     int l2, loss;
     float gamma, adv_temp, ce_c, loss_scale;
-    int row_pieces;                       // pieces of TC_PIECE columns per row of stat_part / grow_part
-    float4* stat_part;                    // [M, row_pieces] per column piece: (max, sum exp, weighted loss sum, -)
-    const float2* row_stat;               // [M] (max, 1 / normaliser) of the whole row
+    int row_pieces;                       // pieces of TC_PIECE columns per row of stat_part
+    float4* stat_part;                    // [M, row_pieces] per column piece: (base-2 reference, sum exp, weighted loss sum, -)
+    const float2* row_stat;               // [M] EPI_LOSS: (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser), 0: row is finished
+    const int32_t* redo;                  // EPI_GRAD: whether there is any row to do
     uint16_t* Gb; int64_t ldg;            // [M, ldg] bf16 dL/dF (divided by the distance for l2)
-    float* grow_part;                     // [M, row_pieces] sums of the written values per column piece
-    float* gcol_part;                     // [4 * tiles_m, N] sums per 32-row piece (l2 only)
     // full-entity scoring (EPI_TOPK): rows are queries, columns the entities [n_base, n_base + N)
     int m_fastest;                        // walk the row tiles of one column tile first (the column tile stays in L2)
     int64_t n_base;
@@ -157,6 +155,14 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, float (&v)[32]) 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) { tmem_ld32_issue(taddr, v); tmem_ld_wait(); }
 
+// Two columns.
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, float (&v)[2]) {
+    uint32_t a, b;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n" : "=r"(a), "=r"(b) : "r"(taddr));
+    tmem_ld_wait();
+    v[0] = __uint_as_float(a); v[1] = __uint_as_float(b);
+}
+
 struct TcItem { int z, m0, n0; };   // K split, first row, first column
 
 constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
@@ -165,16 +171,18 @@ __device__ __forceinline__ float fast_log2(float y) { float r; asm("lg2.approx.f
 __device__ __forceinline__ float fast_rcp(float y) { float r; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y)); return r; }
 __device__ __forceinline__ float fast_rsqrt(float y) { float r; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y)); return r; }
 
+// Maximum of three in one instruction.
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // The fused epilogues evaluate one transcendental per special-function instruction: their
 // inputs come from bf16 operands, so the approximate forms (relative error about 2^-22) are
 // far inside the error of the scores, and an epilogue of a d = 128 contraction is bound by
 // exactly these instructions.
-// softplus(z) = max(z, 0) + log(1 + exp(-|z|))
-__device__ __forceinline__ float tc_softplus(float z) {
-    const float e = fast_exp2(-fabsf(z) * kLog2e);
-    return fmaf(fast_log2(1.f + e), kLn2, fmaxf(z, 0.f));
-}
-// sigmoid(z) from the same exponential
+// sigmoid(z)
 __device__ __forceinline__ float tc_sigmoid(float z) {
     const float e = fast_exp2(-fabsf(z) * kLog2e);
     const float r = fast_rcp(1.f + e);
@@ -200,7 +208,7 @@ __device__ __forceinline__ float tc_score(const TcGemmParams& p, float acc, floa
 // Per-row inputs of an epilogue, read before the accumulator is waited for.
 struct TcRowState {
     float rn;                 // squared norm of the row (norm expansion)
-    float2 st;                // EPI_GRAD: the row's (base-2 maximum, 1 / normaliser)
+    float2 st;                // EPI_LOSS: the row's (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser)
     float thr, ft;            // EPI_TOPK: current k-th best score, score of the true tail
     int32_t thr_id, tt;       //           its id, the true tail's id
 };
@@ -209,7 +217,7 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
     TcRowState r{0.f, make_float2(0.f, 0.f), INFINITY, 0.f, 0, -1};
     if (row >= p.M) return r;   // rows outside the problem: no true tail, a threshold nothing exceeds
     if ((EPI & EPI_L2) != 0) r.rn = p.row_norm2[row];
-    if ((EPI & 3) == EPI_GRAD) r.st = p.row_stat[row];
+    if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) r.st = p.row_stat[row];
     if ((EPI & 3) == EPI_TOPK) {
         r.thr = p.thr[row]; r.thr_id = p.thr_id[row];
         if (p.tt) { r.ft = p.ftrue[row]; r.tt = p.tt[row]; }
@@ -217,177 +225,216 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
     return r;
 }
 
-// One chunk of 32 scores of the first pass.  FULL: all 32 columns lie inside the problem (no
-// per-element masking); otherwise the first `valid` do.
-// A1 (distance scores f <= 0, log-sigmoid loss, temperature a = 1): the weight exponential and the loss term share one
-// exponential.  With e = 2^(y - m) the weight term, exp(gamma + f) = K e with K = exp(gamma) 2^m (one special-function
-// instruction per chunk and lane; K <= exp(gamma) because f <= 0), and softplus(gamma + f) = log(1 + K e): three
-// special-function instructions per score (distance, exponential, logarithm) instead of four.
-template <bool L2, bool CE, bool FULL, bool A1 = false>
-__device__ __forceinline__ void tc_stats_chunk(const TcGemmParams& p, float (&v)[32], float rn, int ncol, int valid,
-                                               float k1, float k0, float& m, float& z, float& l) {
-    // four independent chains each for the maximum and the sums: a single chain of 32 dependent
-    // operations would leave the few epilogue warps waiting on their own results
-    float cmv[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+// The loss in one pass over the scores.  Per row, dL/dF is a function of the score over the row's normaliser Z, which is known
+// only when the row has been seen; so what is written is dL/dF without that factor, E = e(f) u(f) with e = 2^(y - ref), y the
+// base-2 exponent (a f log2 e for the self-adversarial weights, (f + c) log2 e for the sampled softmax) and u the rest
+// (sigmoid(gamma + f), the reciprocal distance), and the factor loss_scale / Z joins afterwards: dQ's rows are multiplied by
+// it, and dT's contraction takes q_b times it as its operand (both see as many roundings to bf16 as with the factor in E).
+// bf16 and fp32 share their exponent range, so any reference within it serves: `ref` is the largest y among eight of the row's
+// negatives (the gather kernel computes them), a lower bound of the maximum up to rounding.  A chunk of 32 scores that exceeds it
+// by more than 2^TC_REF_SPAN takes its own maximum instead, which keeps the statistics in range, and the row is found by
+// stats_combine_kernel and its E written again, over the true maximum and with the factor, by an EPI_GRAD launch that
+// otherwise ends at once.  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
+// softmax 4,096 x 16,384 x 256 34 + 53 us, TransE-L2 8,192 x 8,192 x 128 67 + 94 us.)
+constexpr float TC_REF_SPAN = 80.f;
+
+// One chunk of 32 scores.  FULL: all 32 columns lie inside the problem (no per-element masking); otherwise the first `valid`
+// do.  k0: the exponent's constant less the reference.  Returns what was subtracted beyond the reference.
+// A1 (distance scores f <= 0, log-sigmoid loss, temperature a = 1): with K = exp(gamma) 2^ref, exp(gamma + f) = K e =: t, so
+// softplus(gamma + f) = log(1 + t) and sigmoid(gamma + f) = t / (1 + t): four special-function instructions per score
+// (distance, exponential, logarithm, reciprocal).
+// An L2 score is at most 0, so only a row whose reference is far below (`low`) can exceed it by much, and the chunk's maximum
+// is looked for only in a warp that holds such a row; the other scores' maximum is a tree of three-input maxima.
+template <bool L2, bool CE, bool FULL, bool A1>
+__device__ __forceinline__ float tc_loss_chunk(const TcGemmParams& p, const float (&v)[32], float rn, int ncol, int valid,
+                                               float k1, float k0, float ref, bool low, float& z, float& l, uint32_t (&g2)[16]) {
+    float cn[32];
+    if (L2) {
+        if (FULL) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        if (L2) v[i] = (FULL || i < valid) ? tc_score<true>(p, v[i], rn, ncol + i) : 0.f;
-        const float y = fmaf(v[i], k1, k0);        // exponent in base 2
-        if (CE) v[i] = y;                          // the sampled softmax does not need the score itself again
-        cmv[i & 3] = fmaxf(cmv[i & 3], (FULL || i < valid) ? y : -INFINITY);
+            for (int i = 0; i < 8; ++i) {
+                const float4 c = __ldg(reinterpret_cast<const float4*>(p.col_norm2 + ncol) + i);
+                cn[4 * i] = rn + c.x; cn[4 * i + 1] = rn + c.y; cn[4 * i + 2] = rn + c.z; cn[4 * i + 3] = rn + c.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) cn[i] = i < valid ? rn + __ldg(p.col_norm2 + ncol + i) : 1.f;
+        }
     }
-    const float cm = fmaxf(fmaxf(cmv[0], cmv[1]), fmaxf(cmv[2], cmv[3]));
-    if (cm > m) { const float r = fast_exp2(m - cm); z *= r; l *= r; m = cm; }
+    auto score = [&](int i, float& inv) {
+        if (!L2) { inv = 0.f; return v[i]; }
+        const float s2 = fmaxf(fmaf(-2.f, v[i], cn[i]), 0.f);
+        inv = s2 > 0.f ? fast_rsqrt(s2) : 0.f;
+        return -s2 * inv;
+    };
+    float fm = -INFINITY;
+    if (!L2) {
+        float vm[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = FULL || 8 * j + i < valid ? v[8 * j + i] : -INFINITY;
+            vm[j] = max3(max3(x[0], x[1], x[2]), max3(x[3], x[4], x[5]), fmaxf(x[6], x[7]));
+        }
+        fm = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
+    } else if (__any_sync(0xffffffffu, low)) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            float inv;
+            const float f = score(i, inv);
+            if (FULL || i < valid) fm = fmaxf(fm, f);
+        }
+    }
+    const float ym = fmaf(fm, k1, k0), shift = ym > TC_REF_SPAN ? ym : 0.f;      // (k1 >= 0)
+    const float kk = k0 - shift;
+    const float kexp = A1 ? fast_exp2(fmaf(p.gamma, kLog2e, ref + shift)) : 0.f;
     float zv[4] = {0.f, 0.f, 0.f, 0.f}, lv[4] = {0.f, 0.f, 0.f, 0.f};
-    const float kexp = A1 ? fast_exp2(fmaf(p.gamma, kLog2e, m)) : 0.f;      // exp(gamma) 2^m
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        float e = fast_exp2((CE ? v[i] : fmaf(v[i], k1, k0)) - m);
-        if (!FULL && i >= valid) e = 0.f;
+    auto one = [&](int i) {
+        if (!FULL && i >= valid) return 0.f;
+        float inv;
+        const float f = score(i, inv);
+        const float e = fast_exp2(fmaf(f, k1, kk));
         zv[i & 3] += e;
-        if (A1) lv[i & 3] = fmaf(e, kLn2 * fast_log2(fmaf(kexp, e, 1.f)), lv[i & 3]);
-        else if (!CE) lv[i & 3] = fmaf(e, tc_softplus(p.gamma + v[i]), lv[i & 3]);
+        float g = L2 ? e * inv : e;
+        if (A1) {
+            const float t = kexp * e, t1 = 1.f + t;
+            lv[i & 3] = fmaf(e, fast_log2(t1), lv[i & 3]);
+            g *= t * fast_rcp(t1);
+        } else if (!CE) {
+            // softplus(x) = max(x, 0) + log(1 + exp(-|x|)) and sigmoid(x) from one exponential
+            const float x = p.gamma + f, w = fast_exp2(-fabsf(x) * kLog2e), w1 = 1.f + w, r = fast_rcp(w1);
+            lv[i & 3] = fmaf(e, fmaf(fmaxf(x, 0.f), kLog2e, fast_log2(w1)), lv[i & 3]);
+            g *= x >= 0.f ? r : w * r;
+        }
+        return g;
+    };
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const float a = one(2 * i), b = one(2 * i + 1);
+        const __nv_bfloat162 pr = __floats2bfloat162_rn(a, b);
+        g2[i] = *reinterpret_cast<const uint32_t*>(&pr);
     }
-    z += (zv[0] + zv[1]) + (zv[2] + zv[3]);
-    if (!CE) l += (lv[0] + lv[1]) + (lv[2] + lv[3]);
+    z = (zv[0] + zv[1]) + (zv[2] + zv[3]);
+    if (!CE) l = kLn2 * ((lv[0] + lv[1]) + (lv[2] + lv[3]));
+    return shift;
 }
 
-// First pass of the fused loss: running (max, sum of exponentials, exponentially weighted loss
-// sum) over this thread's 64 columns of one row, rescaled whenever the maximum moves.  The
-// exponent is x = a f for the self-adversarial weights and x = f + c for the sampled softmax;
-// it is carried in base 2 (y = x log2 e), so an exponential is one ex2 of a difference.
+// A warp's 32 rows x 32 columns of bf16 on their way to memory: through `stage` (2 KB of shared memory of its own), so that a store
+// instruction writes whole 32-byte sectors, eight rows x 64 contiguous bytes instead of 16 bytes in each of 32 rows.  The 16-byte chunk c
+// of row r sits at chunk c ^ ((r >> 1) & 3) of the row: both the row-wise writes and the 8-row reads then touch every bank once.
+// `rows`: the rows (lanes) to be written; `valid`: columns inside the problem.
+__device__ __forceinline__ void tc_put_bf16(const TcGemmParams& p, int row0, int ncol, int valid, uint32_t rows, const uint32_t (&g2)[16], uint4* stage) {
+    const int lane = threadIdx.x & 31;
+    if (valid == 32) {
+        const int sw = (lane >> 1) & 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) stage[lane * 4 + (i ^ sw)] = make_uint4(g2[4 * i], g2[4 * i + 1], g2[4 * i + 2], g2[4 * i + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = i * 8 + (lane >> 2), c = lane & 3;
+            const uint4 val = stage[r * 4 + (c ^ ((r >> 1) & 3))];
+            if (rows >> r & 1u) *reinterpret_cast<uint4*>(p.Gb + (int64_t)(row0 + r) * p.ldg + ncol + c * 8) = val;
+        }
+        __syncwarp();
+    } else if (rows >> lane & 1u) {
+        uint16_t* dst = p.Gb + (int64_t)(row0 + lane) * p.ldg + ncol;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) if (i < valid) dst[i] = (uint16_t)(g2[i >> 1] >> ((i & 1) * 16));
+    }
+}
+
+// This thread's 64 columns of one row.
 template <bool L2, bool CE, bool A1>
-__device__ __forceinline__ void tc_epilogue_stats(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr) {
-    const float rn = rs.rn;
-    const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = CE ? p.ce_c * kLog2e : 0.f;
-    float m = -INFINITY, z = 0.f, l = 0.f;
+__device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, uint4* stage) {
     static_assert(TC_PIECE == 64, "two chunks of 32 columns per piece");
-    float v0[32], v1[32];
-    tmem_ld32_issue(taddr, v0);                // both chunks are requested before the first is used
-    tmem_ld32_issue(taddr + 32u, v1);
-    tmem_ld_wait();
-    if (row < p.M) {
-        const int ncol = it.n0 + col_off;
-        const int valid0 = min(32, p.N - ncol), valid1 = min(32, p.N - ncol - 32);   // columns inside the problem (may be <= 0)
-        if (valid0 == 32) tc_stats_chunk<L2, CE, true, A1>(p, v0, rn, ncol, valid0, k1, k0, m, z, l);
-        else if (valid0 > 0) tc_stats_chunk<L2, CE, false, A1>(p, v0, rn, ncol, valid0, k1, k0, m, z, l);
-        if (valid1 == 32) tc_stats_chunk<L2, CE, true, A1>(p, v1, rn, ncol + 32, valid1, k1, k0, m, z, l);
-        else if (valid1 > 0) tc_stats_chunk<L2, CE, false, A1>(p, v1, rn, ncol + 32, valid1, k1, k0, m, z, l);
+    const bool rin = row < p.M;
+    const float rn = rs.rn, ref = rs.st.x;
+    const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = (CE ? p.ce_c * kLog2e : 0.f) - ref;
+    const bool low = L2 && k0 > TC_REF_SPAN;
+    const uint32_t rows = __ballot_sync(0xffffffffu, rin);
+    const int row0 = row - (int)(threadIdx.x & 31);
+    float m = ref, z = 0.f, l = 0.f;
+    auto chunk = [&](const float (&v)[32], int c0) {
+        const int ncol = it.n0 + c0, valid = min(32, p.N - ncol);             // (the same for every lane; may be <= 0)
+        if (valid <= 0) return;
+        uint32_t g2[16];
+        float cz, cl = 0.f, shift;
+        if (valid == 32) shift = tc_loss_chunk<L2, CE, true, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cz, cl, g2);
+        else shift = tc_loss_chunk<L2, CE, false, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cz, cl, g2);
+        const float cm = ref + shift;
+        if (cm == m) { z += cz; l += cl; }
+        else {
+            const float mm = fmaxf(m, cm), ra = fast_exp2(m - mm), rb = fast_exp2(cm - mm);
+            z = z * ra + cz * rb; l = l * ra + cl * rb; m = mm;
+        }
+        tc_put_bf16(p, row0, ncol, valid, rows, g2, stage);
+    };
+    if (L2) {                                  // (both chunks at once spill here)
+#pragma unroll 1
+        for (int c = 0; c < TC_PIECE; c += 32) {
+            float v[32];
+            tmem_ld32(taddr + (uint32_t)c, v);
+            chunk(v, col_off + c);
+        }
+    } else {
+        float v0[32], v1[32];
+        tmem_ld32_issue(taddr, v0);            // both chunks are requested before the first is used
+        tmem_ld32_issue(taddr + 32u, v1);
+        tmem_ld_wait();
+        chunk(v0, col_off);
+        chunk(v1, col_off + 32);
     }
     const int piece = (it.n0 + col_off) / TC_PIECE;
-    if (row < p.M && piece < p.row_pieces) p.stat_part[(int64_t)row * p.row_pieces + piece] = make_float4(m, z, l, 0.f);
+    if (rin && piece < p.row_pieces) p.stat_part[(int64_t)row * p.row_pieces + piece] = make_float4(m, z, l, 0.f);
 }
-
-__device__ __forceinline__ float bf16_value(uint16_t bits) { return __uint_as_float((uint32_t)bits << 16); }
 
 // dL/dF of one pair from its accumulator: scale = loss_scale / normaliser, k0 already holds minus
 // the row's base-2 maximum.
-// A1: sigmoid(gamma + f) = t / (1 + t) with t = exp(gamma + f) = krow e, e the weight exponential 2^(y - max) and
-// krow = exp(gamma) 2^max per row: one reciprocal instead of an exponential and a reciprocal.
-template <bool L2, bool CE, bool A1>
-__device__ __forceinline__ float tc_grad_one(const TcGemmParams& p, float acc, float rn, int col, float k1, float k0, float scale, float krow) {
+template <bool L2, bool CE>
+__device__ __forceinline__ float tc_grad_one(const TcGemmParams& p, float acc, float rn, int col, float k1, float k0, float scale) {
     float inv;
     const float f = tc_score_inv<L2>(p, acc, rn, col, inv);
-    const float e = fast_exp2(fmaf(f, k1, k0));
-    float g = scale * e;
-    if (A1) { const float t = krow * e; g *= t * fast_rcp(1.f + t); }
-    else if (!CE) g *= tc_sigmoid(p.gamma + f);
+    float g = scale * fast_exp2(fmaf(f, k1, k0));
+    if (!CE) g *= tc_sigmoid(p.gamma + f);
     if (L2) g *= inv;
     return g;
 }
 
-// Second pass: dL/dF from the recomputed score and the row's final (base-2 max, 1 / normaliser),
-// written as bf16 for the two backward contractions (which read it K-major and MN-major).
-// A warp's 32 rows x 32 columns of bf16 pass through `stage` (2 KB of shared memory of its own)
-// on their way out, so that a store instruction writes whole 32-byte sectors: eight rows x 64
-// contiguous bytes instead of 16 bytes in each of 32 rows.  The 16-byte chunk c of row r sits at
-// chunk c ^ ((r >> 1) & 3) of the row: both the row-wise writes and the 8-row reads then touch
-// every bank once.
-template <bool L2, bool CE, bool A1>
+// The rows that EPI_LOSS could not finish: dL/dF from the recomputed score and the row's final (base-2 max, 1 / normaliser).
+template <bool L2, bool CE>
 __device__ __forceinline__ void tc_epilogue_grad(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr,
                                                  uint4* stage) {
-    const bool rin = row < p.M;
-    const float rn = rs.rn;
-    const float2 st = rs.st;
-    const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = (CE ? p.ce_c * kLog2e : 0.f) - st.x;
-    const float scale = p.loss_scale * st.y;
-    const float krow = A1 ? fast_exp2(fmaf(p.gamma, kLog2e, st.x)) : 0.f;     // exp(gamma) 2^(row maximum)
-    const int lane = threadIdx.x & 31;
-    float rsum = 0.f;
+    const bool todo = row < p.M && rs.st.y != 0.f;
+    const uint32_t rows = __ballot_sync(0xffffffffu, todo);
+    if (rows == 0u) return;
+    const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = (CE ? p.ce_c * kLog2e : 0.f) - rs.st.x;
+    const float scale = p.loss_scale * rs.st.y;
 #pragma unroll 1
     for (int c0 = col_off; c0 < col_off + TC_PIECE; c0 += 32) {
         float v[32];
         tmem_ld32(taddr + (uint32_t)(c0 - col_off), v);
-        const int ncol = it.n0 + c0;
-        const int valid = rin ? min(32, p.N - ncol) : 0;
-        uint32_t g2[16];     // bf16 pairs in memory order
-        if (valid == 32) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = tc_grad_one<L2, CE, A1>(p, v[i], rn, ncol + i, k1, k0, scale, krow);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = i < valid ? tc_grad_one<L2, CE, A1>(p, v[i], rn, ncol + i, k1, k0, scale, krow) : 0.f;
-        }
+        const int ncol = it.n0 + c0, valid = min(32, p.N - ncol);
+        if (valid <= 0) return;
+        uint32_t g2[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const __nv_bfloat162 pr = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            float g[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                g[j] = todo && 2 * i + j < valid ? tc_grad_one<L2, CE>(p, v[2 * i + j], rs.rn, ncol + 2 * i + j, k1, k0, scale) : 0.f;
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(g[0], g[1]);
             g2[i] = *reinterpret_cast<const uint32_t*>(&pr);
         }
-        if (ncol + 32 <= p.N) {       // warp-uniform: all 32 columns lie inside the problem
-            const int sw = (lane >> 1) & 3;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                stage[lane * 4 + (i ^ sw)] = make_uint4(g2[4 * i], g2[4 * i + 1], g2[4 * i + 2], g2[4 * i + 3]);
-            __syncwarp();
-            const int row0 = row - lane;             // first of this warp's 32 rows
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = i * 8 + (lane >> 2), c = lane & 3;
-                const uint4 val = stage[r * 4 + (c ^ ((r >> 1) & 3))];
-                if (row0 + r < p.M) *reinterpret_cast<uint4*>(p.Gb + (int64_t)(row0 + r) * p.ldg + ncol + c * 8) = val;
-            }
-            __syncwarp();
-        } else if (valid > 0) {
-            uint16_t* dst = p.Gb + (int64_t)row * p.ldg + ncol;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) if (i < valid) dst[i] = (uint16_t)(g2[i >> 1] >> ((i & 1) * 16));
-        }
-        if (L2) {   // the norm expansion also needs the sums of what the contractions will see
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                v[i] = bf16_value((uint16_t)(g2[i >> 1] >> ((i & 1) * 16)));
-                rsum += v[i];
-            }
-            // Sums over this warp's 32 rows (rows outside the problem hold zeros) of all 32 columns
-            // at once: each exchange halves the columns a lane still carries, so 31 shuffles do
-            // what 32 separate warp sums need 160 for; lane c ends with the sum of column c.
-#pragma unroll
-            for (int half = 16; half >= 1; half >>= 1) {
-                const bool upper = (lane & half) != 0;
-#pragma unroll
-                for (int j = 0; j < half; ++j) {
-                    const float send = upper ? v[j] : v[j + half], keep = upper ? v[j + half] : v[j];
-                    v[j] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-                }
-            }
-            if (ncol + lane < p.N)
-                p.gcol_part[(int64_t)((it.m0 / TC_BM) * 4 + ((row - it.m0) >> 5)) * p.N + ncol + lane] = v[0];
-        }
+        tc_put_bf16(p, row - (int)(threadIdx.x & 31), ncol, valid, rows, g2, stage);
     }
-    const int piece = (it.n0 + col_off) / TC_PIECE;
-    if (L2 && rin && piece < p.row_pieces) p.grow_part[(int64_t)row * p.row_pieces + piece] = rsum;
 }
 
 // 1.0f if a > b, else 0.0f, in one instruction.
 __device__ __forceinline__ float one_if_gt(float a, float b) {
     float r;
     asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-// Maximum of three in one instruction.
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 
@@ -509,11 +556,12 @@ __device__ __forceinline__ void tc_epilogue_topk(const TcGemmParams& p, const Tc
 template <int EPI, int WIDTH>
 __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, int32_t* beat_sm) {
     static_assert((EPI & 3) == EPI_STORE || (EPI & 3) == EPI_TOPK || WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
-    if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD) {
+    if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) {
 #pragma unroll 1
         for (int c = 0; c < WIDTH; c += TC_PIECE) {
-            if ((EPI & 3) == EPI_STATS) tc_epilogue_stats<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c);
-            else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, reinterpret_cast<uint4*>(beat_sm));
+            uint4* stage = reinterpret_cast<uint4*>(beat_sm);
+            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
+            else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
         }
         return;
     }
@@ -582,11 +630,10 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     constexpr int NACC = 512 / BN;                      // fp32 accumulators in tensor memory, used in turn: all 512 columns
     constexpr uint32_t TC_TMEM_COLS = NACC * BN;
     constexpr int EW = tc_epi_warps(EPI, BN), EG = EW / 4, TC_THREADS = tc_threads(EPI, BN);
-    // In the gradient pass of the norm-expansion kinds (bound by special-function instructions, with row- and
+    // In the loss pass of the norm-expansion kinds (bound by special-function instructions, with row- and
     // column-dependent loads) the epilogue warps form two groups that take the CTA's items in turn, so the epilogues
-    // of consecutive items overlap: measured faster there (136 against 146 us at B = N = 8192) and slower or equal
-    // in every other pass, which stay one group.
-    constexpr int EGRP = ((EPI & EPI_L2) != 0 && (EPI & 3) == EPI_GRAD && EG % 2 == 0) ? 2 : 1;
+    // of consecutive items overlap; every other pass was measured slower or equal that way and stays one group.
+    constexpr int EGRP = ((EPI & EPI_L2) != 0 && (EPI & 3) == EPI_LOSS && EG % 2 == 0) ? 2 : 1;
     constexpr int GW = EW / EGRP, GCOLS = BN / (GW / 4);       // warps per group; columns per warp
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* base = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
@@ -603,6 +650,11 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     if ((EPI & 3) == EPI_TOPK)
         for (int i = threadIdx.x; i < p.beat_rows; i += TC_THREADS) beat_sm[i] = 0;
 
+    if ((EPI & 3) == EPI_GRAD) {                        // (nothing in flight writes the flag)
+        grid_dependency_wait();
+        allow_dependents();
+        if (*p.redo == 0) return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int per_cta = (p.items + gridDim.x - 1) / gridDim.x;
     const int item_begin = blockIdx.x * per_cta;
@@ -626,7 +678,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const int item_end = min(p.items, item_begin + *cta_items);
-    if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD) grid_dependency_wait();     // (launched while the kernel before it drains)
+    if ((EPI & 3) == EPI_LOSS) grid_dependency_wait();     // (launched while the kernel before it drains)
 
     // Full-entity scoring with rows of at most 128 coordinates: the column (entity) tile of the
     // current run of items sits in a buffer of its own (2 x 32 KB) and the rest of the stage memory
@@ -779,8 +831,8 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
             tc_fence_after();
             if (!ok || *stop) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * GCOLS);
-            // scratch after the barriers: the rank counts of EPI_TOPK, or 2 / 4 KB per epilogue warp for EPI_GRAD's / EPI_STORE's stores
-            int32_t* scratch = (EPI & 3) == EPI_GRAD ? beat_sm + (warp - 2) * (TC_GRAD_STAGE_BYTES / 4)
+            // scratch after the barriers: the rank counts of EPI_TOPK, or 2 / 4 KB per epilogue warp for the stores of bf16 / fp32 tiles
+            int32_t* scratch = (EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD ? beat_sm + (warp - 2) * (TC_GRAD_STAGE_BYTES / 4)
                              : ((EPI & 3) == EPI_STORE ? beat_sm + (warp - 2) * (TC_STORE_STAGE_BYTES / 4) : beat_sm);
             tc_epilogue<EPI, GCOLS>(p, it, it.m0 + quarter * 32 + lane, rs, cgrp * GCOLS, taddr, scratch);
             tc_fence_before();
@@ -816,20 +868,28 @@ struct DualProb {
     int seg_kb, a_seg_x;
     // fold > 0: output column c goes to column c % fold of slab c / fold (slabs fold_stride floats apart)
     int fold; int64_t fold_stride;
+    // XCOL: groups of 64 columns of B per tile; extra[split][row] receives the extra column
+    int groups; float* extra;
 };
 
 // PAIR: the A operand has two K segments that meet the same slices of the B operand (two-term splits of dL/dF-like
 // coefficients against one [x1 | x2] operand).  A stage then holds both segments' A tiles beside the one B tile and both
 // are multiplied into the accumulator, so a B slice is fetched once instead of once per segment (a third fewer operand
 // bytes per flop); K runs over one segment's slices.  Three stages instead of four fit.
+// XCOL (norm expansion): the B operand has one more column than the output: ones in problem 0, the factor of every row of dL/dF
+// as two bf16 terms in problem 1 (box tmX), which gives the sums of dL/dF over its rows and columns exactly as the contractions
+// see it.  The box of 64 columns that holds it follows a tile's `groups` boxes; the last tile's MMAs are 16 columns wider
+// for it.  The ones lie in shared memory from the start: problem 0's copies leave that box alone, and a CTA's items of problem 1
+// come after those of problem 0.
 // FORM: how the operands of both problems are read.  DUAL_STEP: as above.  DUAL_NT: A and B K-major (the encoder's two
 // projections).  DUAL_TN: A and B MN-major (the encoder's two matrix gradients).
 enum { DUAL_STEP = 0, DUAL_NT = 1, DUAL_TN = 2 };
-template <int BN, bool PAIR = false, int FORM = DUAL_STEP>
+template <int BN, bool PAIR = false, int FORM = DUAL_STEP, bool XCOL = false>
 __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kernel(const __grid_constant__ CUtensorMap tmA0,
                                                                                     const __grid_constant__ CUtensorMap tmB0,
                                                                                     const __grid_constant__ CUtensorMap tmA1,
                                                                                     const __grid_constant__ CUtensorMap tmB1,
+                                                                                    const __grid_constant__ CUtensorMap tmX,
                                                                                     DualProb q0, DualProb q1, int32_t* status, int wait_limit) {
     constexpr uint32_t A_BYTES = PAIR ? 2 * TC_A_BYTES : TC_A_BYTES;      // A tile(s) of a stage; the B tile follows
     constexpr uint32_t STAGE_BYTES = tc_stage_bytes(BN) + (PAIR ? TC_A_BYTES : 0u);
@@ -852,9 +912,18 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     auto prob_of = [&](int item) { return item < q0.items ? 0 : 1; };
     auto item_of = [&](const DualProb& q, int local_item) {
         const int tn = local_item % q.tiles_n, r = local_item / q.tiles_n;
-        return TcItem{r / q.tiles_m, (r % q.tiles_m) * TC_BM, tn * BN};
+        return TcItem{r / q.tiles_m, (r % q.tiles_m) * TC_BM, tn * (XCOL ? 64 * q.groups : BN)};
     };
+    auto last_tile = [&](const DualProb& q, const TcItem& it) { return it.n0 + 64 * q.groups >= q.N; };
 
+    if (XCOL) {     // K row r of the box: 128 bytes, 16-byte piece c at c ^ (r & 7)
+        for (int i = threadIdx.x; i < STAGES * 512; i += blockDim.x) {
+            const int r = i >> 3 & 63, c = i & 7;
+            *reinterpret_cast<uint4*>(base + (size_t)(i >> 9) * STAGE_BYTES + A_BYTES + q0.groups * TC_MN_GROUP_BYTES + r * 128 + c * 16) =
+                make_uint4(c == (r & 7) ? 0x3F80u : 0u, 0u, 0u, 0u);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EW); }
@@ -886,7 +955,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                     const int s = ring % STAGES;
                     if (!mbar_wait_idle(&empty[s], ((ring / STAGES) & 1) ^ 1, wait_limit)) { *stop = 1; set_status(status, KGE_ERR_TIMEOUT); break; }
                     unsigned char* sa = base + (size_t)s * STAGE_BYTES;
-                    mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
+                    const bool load_x = XCOL && which && last_tile(q, it);
+                    mbar_arrive_expect_tx(&full[s], XCOL ? A_BYTES + (uint32_t)(q.groups + (load_x ? 1 : 0)) * TC_MN_GROUP_BYTES : STAGE_BYTES);
                     const int kblk = kb0 + kb, seg = PAIR ? 0 : kblk / q.seg_kb;
                     const int k0 = kblk * TC_BK, kseg = (kblk - seg * q.seg_kb) * TC_BK;
 #pragma unroll
@@ -903,6 +973,9 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                     if (FORM == DUAL_NT) {
 #pragma unroll
                         for (int g = 0; g < BN / 128; ++g) tma_load_2d(sa + A_BYTES + g * (128 * TC_BK * 2), tb, kseg, it.n0 + 128 * g, &full[s]);
+                    } else if (XCOL) {
+                        for (int g = 0; g < q.groups; ++g) tma_load_2d(sa + A_BYTES + g * TC_MN_GROUP_BYTES, tb, it.n0 + 64 * g, kseg, &full[s]);
+                        if (load_x) tma_load_2d(sa + A_BYTES + q.groups * TC_MN_GROUP_BYTES, &tmX, 0, kseg, &full[s]);
                     } else {
 #pragma unroll
                         for (int g = 0; g < BN / 64; ++g) tma_load_2d(sa + A_BYTES + g * TC_MN_GROUP_BYTES, tb, it.n0 + 64 * g, kseg, &full[s]);
@@ -921,6 +994,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                 const TcItem it = item_of(q, which ? item - q0.items : item);
                 const int nkb = min(q.kb_per_split, q.kb_total - it.z * q.kb_per_split);
                 const int buf = local % NACC;
+                const int cols = 64 * q.groups + (last_tile(q, it) ? 16 : 0);       // XCOL
+                const uint32_t idesc = XCOL ? umma_idesc_bf16(TC_BM, cols, which != 0, true) : 0u;
                 if (!mbar_wait_idle(&acc_empty[buf], ((local / NACC) & 1) ^ 1, wait_limit)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t tmem_acc = tmem_base + (uint32_t)buf * BN;
@@ -937,7 +1012,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                             const bool a_mn = FORM == DUAL_TN || (FORM == DUAL_STEP && which);
                             const uint64_t ad = a_mn ? umma_desc_mn_sw128(aa + k * 2048) : umma_desc_k_sw128(aa + k * 32);
                             const uint64_t bd = FORM == DUAL_NT ? umma_desc_k_sw128(sa + A_BYTES + k * 32) : umma_desc_mn_sw128(sa + A_BYTES + k * 2048);
-                            umma_bf16(tmem_acc, ad, bd, a_mn ? idesc_mn : idesc_k, (kb | k | half) != 0);
+                            umma_bf16(tmem_acc, ad, bd, XCOL ? idesc : (a_mn ? idesc_mn : idesc_k), (kb | k | half) != 0);
                         }
                     }
                     umma_commit(&empty[s]);
@@ -960,12 +1035,13 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
             const DualProb q = which ? q1 : q0;
             const TcItem it = item_of(q, which ? item - q0.items : item);
             const int row = it.m0 + quarter * 32 + lane;
-            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * COLS);
+            const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN);
             float* const Cout = q.C + (int64_t)it.z * q.split_stride;
+            // (XCOL: a tile's columns are fewer than BN; the groups of warps take them 32 by 32 in turn)
 #pragma unroll 1
-            for (int c0 = cgrp * COLS; c0 < (cgrp + 1) * COLS; c0 += 32) {
+            for (int c0 = cgrp * (XCOL ? 32 : COLS); c0 < (XCOL ? 64 * q.groups : (cgrp + 1) * COLS); c0 += XCOL ? 32 * EG : 32) {
                 float v[32];
-                tmem_ld32(taddr + (uint32_t)(c0 - cgrp * COLS), v);
+                tmem_ld32(taddr + (uint32_t)c0, v);
                 const int ncol = it.n0 + c0;
                 float* piece = Cout + ncol;                    // column ncol of row 0 of this item's slab
                 if (q.fold > 0) piece += (int64_t)(ncol / q.fold) * (q.fold_stride - q.fold);   // (32-column pieces never straddle a fold)
@@ -986,6 +1062,11 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
 #pragma unroll
                     for (int i = 0; i < 32; ++i) if (ncol + i < q.N) dst[i] = v[i];
                 }
+            }
+            if (XCOL && cgrp == EG - 1 && last_tile(q, it)) {
+                float x[2];
+                tmem_ld2(taddr + (uint32_t)(64 * q.groups), x);
+                if (row < q.M) q.extra[(int64_t)it.z * q.M + row] = x[0] + x[1];    // (problem 0: the second column is zero)
             }
             tc_fence_before();
             __syncwarp();
@@ -1199,14 +1280,19 @@ int tc_make_f32_tile_map(kge_handle* h, void* map_out, const void* base, int64_t
 
 namespace {
 
-// One warp per positive merges the per-piece statistics of its row (and the positive score,
-// which the sampled softmax normalises over too) into the row's final (max, 1 / normaliser),
-// the per-positive loss and dL/df+.
+// One warp per positive merges the per-piece statistics of its row (and the positive score, which the sampled softmax
+// normalises over too) into the per-positive loss, dL/df+ and the row's factor loss_scale / Z, and multiplies the row of the dT
+// contraction's operand by it.  A row with a piece that left its reference (see tc_loss_chunk) keeps its operand and a factor of
+// one; its (max, 1 / Z) go to the launch that writes its dL/dF.
 struct CombineParams {
     const float4* stat_part; int pieces; int B;
     const float* fpos;
     int loss; float gamma, ce_c, loss_scale;
     float2* row_stat; float *Lrow, *gpos;
+    float* row_scale;                     // [B] what a row of dL/dF is still to be multiplied by
+    const float4* Q; uint2* Qb; int d4;   // [B, d] query vectors; their bf16 copies
+    uint32_t* Xq;                         // norm expansion: [B, 64] bf16, the factor as two terms beside the operand's columns, or NULL
+    int32_t* redo;
 };
 
 __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
@@ -1215,24 +1301,37 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     allow_dependents();
     if (b >= p.B) return;
     const float4* row = p.stat_part + (int64_t)b * p.pieces;
-    const float fp = p.fpos[b];
+    const float fp = p.fpos[b], ref = p.row_stat[b].x;
     const bool ce = p.loss == KGE_LOSS_SAMPLED_SOFTMAX;
-    // the pieces carry their maxima and exponent sums in base 2 (exponent times log2 e)
+    // the pieces carry their references and exponent sums in base 2 (exponent times log2 e)
     float m = -INFINITY;
-    for (int j = lane; j < p.pieces; j += 32) m = fmaxf(m, row[j].x);
+    bool good = true;
+    for (int j = lane; j < p.pieces; j += 32) { const float x = row[j].x; m = fmaxf(m, x); good = good && x == ref; }
     m = warp_max(m);
     if (ce) m = fmaxf(m, fp * kLog2e);
     float z = 0.f, l = 0.f;
     for (int j = lane; j < p.pieces; j += 32) {
         const float4 s = row[j];
-        const float r = exp2f(s.x - m);    // a piece without valid columns has max = -inf: weight 0
+        const float r = exp2f(s.x - m);
         z += s.y * r; l += s.z * r;
     }
     z = warp_sum(z); l = warp_sum(l);
+    if (ce) z += exp2f(fp * kLog2e - m);
+    good = __all_sync(0xffffffffu, good) && m == ref && z >= 1e-30f && z < INFINITY;
+    const float scale = good ? p.loss_scale / z : 1.f;
+    if (good)
+        for (int c = lane; c < p.d4; c += 32) {
+            const float4 q = p.Q[(int64_t)b * p.d4 + c];
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(scale * q.x, scale * q.y), hi = __floats2bfloat162_rn(scale * q.z, scale * q.w);
+            p.Qb[(int64_t)b * p.d4 + c] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        }
+    if (p.Xq) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(scale), lo = __float2bfloat16_rn(scale - __bfloat162float(hi));
+        p.Xq[(int64_t)b * 32 + lane] = lane == 0 ? (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16 : 0u;
+    }
     if (lane != 0) return;
     if (ce) {
         const float epos = exp2f(fp * kLog2e - m);
-        z += epos;
         p.Lrow[b] = -fp + (m + log2f(z)) * 0.6931471805599453f;
         p.gpos[b] = p.loss_scale * (epos / z - 1.f);
     } else {
@@ -1241,40 +1340,9 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
         p.Lrow[b] = sp + l / z;
         p.gpos[b] = -p.loss_scale * sg;
     }
-    p.row_stat[b] = make_float2(m, 1.f / z);
-}
-
-// Norm expansion only: row sums and column sums of the written dL/dF from their pieces, in a fixed order.  CTAs
-// [0, row_ctas): a warp per row, its pieces side by side; the others: 32 columns, eight warps sharing the pieces.  (One
-// thread per row and per column, one piece after the other: 19 us at B = N = 8192.)
-__global__ void __launch_bounds__(256) grad_sums_kernel(const float* grow_part, int row_pieces, float* Grow, int B, int row_ctas,
-                                                        const float* gcol_part, int col_pieces, float* Gcol, int N) {
-    __shared__ float part[8][32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    grid_dependency_wait();
-    allow_dependents();
-    if ((int)blockIdx.x < row_ctas) {
-        const int i = blockIdx.x * 8 + warp;
-        if (i >= B) return;
-        float t = 0.f;
-        for (int j = lane; j < row_pieces; j += 32) t += grow_part[(int64_t)i * row_pieces + j];
-        t = warp_sum(t);
-        if (lane == 0) Grow[i] = t;
-        return;
-    }
-    const int n = ((int)blockIdx.x - row_ctas) * 32 + lane;
-    float t = 0.f;
-    if (n < N) {
-#pragma unroll 8
-        for (int j = warp; j < col_pieces; j += 8) t += gcol_part[(int64_t)j * N + n];
-    }
-    part[warp][lane] = t;
-    __syncthreads();
-    if (warp == 0 && n < N) {
-#pragma unroll
-        for (int w = 1; w < 8; ++w) t += part[w][lane];
-        Gcol[n] = t;
-    }
+    p.row_scale[b] = scale;
+    p.row_stat[b] = make_float2(m, good ? 0.f : 1.f / z);
+    if (!good) *p.redo = 1;
 }
 
 }  // namespace
@@ -1285,15 +1353,15 @@ cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB,
                              size_t extra_smem = 0) {
     constexpr size_t smem = tc_smem_bytes(BN);
     constexpr size_t extra_max = (EPI & 3) == EPI_TOPK ? (size_t)TC_BEAT_ROWS_MAX * 4
-                               : ((EPI & 3) == EPI_GRAD ? (size_t)tc_epi_warps(EPI, BN) * TC_GRAD_STAGE_BYTES
+                               : ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD ? (size_t)tc_epi_warps(EPI, BN) * TC_GRAD_STAGE_BYTES
                                : ((EPI & 3) == EPI_STORE ? (size_t)tc_epi_warps(EPI, BN) * TC_STORE_STAGE_BYTES : 0));
-    if ((EPI & 3) == EPI_GRAD || (EPI & 3) == EPI_STORE) extra_smem = extra_max;
+    if ((EPI & 3) != EPI_TOPK) extra_smem = extra_max;
     static DeviceOnce configured;
     const cudaError_t e = once_per_device(configured, [] {
         return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + extra_max));
     });
     if (e != cudaSuccess) return e;
-    if ((EPI & 3) == EPI_STATS || (EPI & 3) == EPI_GRAD)
+    if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD)
         return launch_dependent(tc_gemm_kernel<EPI, BN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem + extra_smem, s,
                                 *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
     tc_gemm_kernel<EPI, BN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem + extra_smem, s>>>(
@@ -1301,34 +1369,32 @@ cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB,
     return cudaSuccess;
 }
 
-// Scores Q . T^T with one of the fused loss epilogues, in tiles of BN columns.
+// Scores Q . T^T with the fused loss epilogue, in tiles of BN columns.
 template <int BN>
-cudaError_t launch_fused_bn(int pass, bool l2, bool ce, kge_handle* h, const TcGemmParams& p, cudaStream_t s) {
-    // the shared-exponential form of the log-sigmoid distance epilogues: temperature exactly 1, exp(gamma) finite
-    if (l2 && !ce && p.adv_temp == 1.f && p.gamma <= 80.f) {
-        if (pass == EPI_GRAD) return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_A1, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        return launch_gemm_inst<EPI_STATS | EPI_L2 | EPI_A1, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-    }
-    const int key = (pass == EPI_GRAD ? 4 : 0) | (l2 ? 2 : 0) | (ce ? 1 : 0);
-    switch (key) {
-        case 0: return launch_gemm_inst<EPI_STATS, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 1: return launch_gemm_inst<EPI_STATS | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 2: return launch_gemm_inst<EPI_STATS | EPI_L2, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 3: return launch_gemm_inst<EPI_STATS | EPI_L2 | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 4: return launch_gemm_inst<EPI_GRAD, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 5: return launch_gemm_inst<EPI_GRAD | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 6: return launch_gemm_inst<EPI_GRAD | EPI_L2, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        default: return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+cudaError_t launch_loss_bn(bool l2, bool ce, kge_handle* h, const TcGemmParams& p, cudaStream_t s) {
+    // the shared-exponential form of the log-sigmoid distance epilogue: temperature exactly 1, exp(gamma) finite
+    if (l2 && !ce && p.adv_temp == 1.f && p.gamma <= 80.f) return launch_gemm_inst<EPI_LOSS | EPI_L2 | EPI_A1, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+    switch ((l2 ? 2 : 0) | (ce ? 1 : 0)) {
+        case 0: return launch_gemm_inst<EPI_LOSS, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 1: return launch_gemm_inst<EPI_LOSS | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 2: return launch_gemm_inst<EPI_LOSS | EPI_L2, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        default: return launch_gemm_inst<EPI_LOSS | EPI_L2 | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
     }
 }
-cudaError_t launch_fused(int pass, bool l2, bool ce, kge_handle* h, const TcGemmParams& p, cudaStream_t s) {
-    return p.bn == 256 ? launch_fused_bn<256>(pass, l2, ce, h, p, s) : launch_fused_bn<128>(pass, l2, ce, h, p, s);
+// The rows that launch could not finish (in tiles of 128 columns: hardly ever more than a look at the flag).
+cudaError_t launch_redo(bool l2, bool ce, kge_handle* h, TcGemmParams p, cudaStream_t s) {
+    p.bn = TC_BN; p.tiles_n = (p.N + TC_BN - 1) / TC_BN; p.items = p.tiles_m * p.tiles_n;
+    switch ((l2 ? 2 : 0) | (ce ? 1 : 0)) {
+        case 0: return launch_gemm_inst<EPI_GRAD>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 1: return launch_gemm_inst<EPI_GRAD | EPI_CE>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 2: return launch_gemm_inst<EPI_GRAD | EPI_L2>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        default: return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_CE>(h->tm_q, h->tm_t, p, h->num_sms, s);
+    }
 }
 }  // namespace
 
-// Forward of the tensor-core path without the B x N score block ever leaving the chip:
-//   pass 1  scores -> per-piece statistics;  merge per row -> loss, dL/df+, (max, 1 / normaliser)
-//   pass 2  scores again -> dL/dF as bf16, as it is and transposed, for the backward contractions
+// Forward of the tensor-core path without the B x N score block ever leaving the chip: scores -> dL/dF up to a factor per row, as
+// bf16, and per-piece statistics; merge per row -> loss, dL/df+, the factor; the rows that take another round, if any.
 int launch_tc_forward(kge_handle* h, cudaStream_t s) {
     const kge_config& c = h->cfg;
     Workspace& w = h->ws;
@@ -1347,7 +1413,7 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
     p.gamma = c.gamma; p.adv_temp = c.adv_temp; p.ce_c = c.ce_correction; p.loss_scale = c.loss_scale;
     p.stat_part = reinterpret_cast<float4*>(w.stat_part); p.row_stat = reinterpret_cast<const float2*>(w.row_stat);
     p.Gb = w.Gb; p.ldg = (c.num_neg + 7) / 8 * 8;
-    p.grow_part = w.grow_part; p.gcol_part = w.gcol_part;
+    p.redo = w.status + TC_REDO_FLAG;
     const bool ce = c.loss == KGE_LOSS_SAMPLED_SOFTMAX;
     if (h->capture_scores) {
         // debug tap: this path never stores the score block, so an extra contraction writes it (fp32 [B, N]) with the
@@ -1360,27 +1426,23 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
         KGE_LAUNCH_CHECK(h);
     }
     stage_begin(h, ST_BLOCK, s);
-    KGE_CUDA_CHECK(h, launch_fused(EPI_STATS, p.l2 != 0, ce, h, p, s));
+    KGE_CUDA_CHECK(h, p.bn == 256 ? launch_loss_bn<256>(p.l2 != 0, ce, h, p, s) : launch_loss_bn<128>(p.l2 != 0, ce, h, p, s));
     stage_end(h, ST_BLOCK, s);
     KGE_LAUNCH_CHECK(h);
     stage_begin(h, ST_LOSS, s);
     CombineParams cp{p.stat_part, p.row_pieces, p.M, w.fpos, c.loss, c.gamma, c.ce_correction, c.loss_scale,
-                     reinterpret_cast<float2*>(w.row_stat), w.Lrow, w.gpos};
+                     reinterpret_cast<float2*>(w.row_stat), w.Lrow, w.gpos, w.Grow, reinterpret_cast<const float4*>(w.Q),
+                     reinterpret_cast<uint2*>(w.Qb), c.dim / 4, p.l2 ? reinterpret_cast<uint32_t*>(w.Xq) : nullptr, w.status + TC_REDO_FLAG};
     KGE_CUDA_CHECK(h, launch_dependent(stats_combine_kernel, dim3((p.M * 32 + 255) / 256), dim3(256), 0, s, cp));
     KGE_LAUNCH_CHECK(h);
-    KGE_CUDA_CHECK(h, launch_fused(EPI_GRAD, p.l2 != 0, ce, h, p, s));
+    KGE_CUDA_CHECK(h, launch_redo(p.l2 != 0, ce, h, p, s));
     KGE_LAUNCH_CHECK(h);
-    if (p.l2) {
-        const int row_ctas = (p.M + 7) / 8;
-        KGE_CUDA_CHECK(h, launch_dependent(grad_sums_kernel, dim3(row_ctas + (p.N + 31) / 32), dim3(256), 0, s, w.grow_part, p.row_pieces, w.Grow, p.M,
-                                           row_ctas, w.gcol_part, 4 * p.tiles_m, w.Gcol, p.N));
-        KGE_LAUNCH_CHECK(h);
-    }
     stage_end(h, ST_LOSS, s);
     return KGE_OK;
 }
 
 namespace {
+// bn: columns per tile.
 DualProb dual_prob(int M, int N, int K, int split, float* C, int64_t ldc, int bn) {
     DualProb q{};
     q.M = M; q.N = N;
@@ -1390,25 +1452,27 @@ DualProb dual_prob(int M, int N, int K, int split, float* C, int64_t ldc, int bn
     q.items = q.tiles_m * q.tiles_n * ((q.kb_total + q.kb_per_split - 1) / q.kb_per_split);
     q.C = C; q.ldc = ldc; q.split_stride = (int64_t)M * ldc;
     q.seg_kb = q.kb_total; q.a_seg_x = 0; q.fold = 0; q.fold_stride = 0;
+    q.groups = bn / 64; q.extra = nullptr;
     return q;
 }
-template <int BN, bool PAIR = false, int FORM = DUAL_STEP>
+template <int BN, bool PAIR = false, int FORM = DUAL_STEP, bool XCOL = false>
 cudaError_t launch_gemm_dual(kge_handle* h, const unsigned char* tmA0, const unsigned char* tmB0, const unsigned char* tmA1,
-                             const unsigned char* tmB1, const DualProb& q0, const DualProb& q1, cudaStream_t s) {
+                             const unsigned char* tmB1, const DualProb& q0, const DualProb& q1, cudaStream_t s, const unsigned char* tmX = nullptr) {
     constexpr size_t smem = (PAIR ? 1024 + (size_t)3 * (tc_stage_bytes(BN) + TC_A_BYTES) + 256 : tc_smem_bytes(BN)) +
                             (size_t)TC_EPI_WARPS * TC_STORE_STAGE_BYTES;      // + the epilogue warps' store staging
     static DeviceOnce configured;
     const cudaError_t e = once_per_device(configured, [] {
-        return cudaFuncSetAttribute(tc_gemm_dual_kernel<BN, PAIR, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaFuncSetAttribute(tc_gemm_dual_kernel<BN, PAIR, FORM, XCOL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     // as few CTAs as give the same number of rounds: SMs left over serve the id sort that runs beside this launch
     const int total = q0.items + q1.items;
     const int rounds = (total + h->num_sms - 1) / h->num_sms;
     const int grid = (total + rounds - 1) / rounds;
-    return launch_dependent(tc_gemm_dual_kernel<BN, PAIR, FORM>, dim3(grid), dim3(32 * (2 + TC_EPI_WARPS)), smem, s,
+    return launch_dependent(tc_gemm_dual_kernel<BN, PAIR, FORM, XCOL>, dim3(grid), dim3(32 * (2 + TC_EPI_WARPS)), smem, s,
                             *reinterpret_cast<const CUtensorMap*>(tmA0), *reinterpret_cast<const CUtensorMap*>(tmB0),
-                            *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1), q0, q1, h->ws.status, h->wait_limit);
+                            *reinterpret_cast<const CUtensorMap*>(tmA1), *reinterpret_cast<const CUtensorMap*>(tmB1),
+                            *reinterpret_cast<const CUtensorMap*>(tmX ? tmX : tmB1), q0, q1, h->ws.status, h->wait_limit);
 }
 }  // namespace
 
@@ -1456,6 +1520,15 @@ bool tc_negatives_direct(const kge_handle* h) {
 // Columns per tile of a backward contraction whose output rows are `cols` wide.
 int tc_backward_tile_cols(int cols) { return cols > 128 ? 256 : 128; }
 
+// 64-column groups per tile and tiles of a backward contraction of the norm expansion, whose last tile needs room for one more
+// group (see tc_gemm_dual_kernel): at most three groups in a tile of 256 columns.
+static int tc_xcol_groups(int cols) { const int g = (cols + 63) / 64, tiles = (g + 2) / 3; return (g + tiles - 1) / tiles; }
+// Column tiles of a backward contraction; `xcol`: of the norm expansion.
+int tc_backward_col_tiles(int cols, bool xcol) {
+    const int bn = xcol ? 64 * tc_xcol_groups(cols) : tc_backward_tile_cols(cols);
+    return (cols + bn - 1) / bn;
+}
+
 // Column pieces per 128-wide tile for which the fused forward keeps separate statistics.
 int tc_pieces_per_tile() { return TC_EPI_GROUPS; }
 
@@ -1473,9 +1546,15 @@ int launch_tc_backward(kge_handle* h, cudaStream_t s, cudaStream_t side) {
     (void)side;
     // one split and no correction term: the negatives' rows are final, so they go where the update reads them
     float* dT_out = tc_negatives_direct(h) ? w.grad_ent + (size_t)2 * B * d : w.dTpart;
-    const int bn = tc_backward_tile_cols(d);
-    const DualProb q0 = dual_prob(B, d, N, h->split_q, w.dQpart, d, bn), q1 = dual_prob(N, d, B, h->split_t, dT_out, d, bn);
+    const bool xcol = h->kind == KIND_L2;
+    const int bn = xcol ? 64 * tc_xcol_groups(d) : tc_backward_tile_cols(d);
+    DualProb q0 = dual_prob(B, d, N, h->split_q, w.dQpart, d, bn), q1 = dual_prob(N, d, B, h->split_t, dT_out, d, bn);
+    q0.extra = w.xsum_q; q1.extra = w.Cpart;
     stage_begin(h, ST_ACCUM_Q, s);        // (both contractions: the profile reports them as one stage)
+    if (xcol)
+        KGE_CUDA_CHECK(h, bn > 64 ? (launch_gemm_dual<256, false, DUAL_STEP, true>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s, h->tm_x64))
+                                  : (launch_gemm_dual<128, false, DUAL_STEP, true>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s, h->tm_x64)));
+    else
     KGE_CUDA_CHECK(h, bn == 256 ? launch_gemm_dual<256>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s)
                                 : launch_gemm_dual<128>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s));
     stage_end(h, ST_ACCUM_Q, s);

@@ -25,7 +25,8 @@ struct TrainParams {
     int fused_sample;   // the gather kernel draws the batch itself (ids land in sp.heads ...) instead of reading it
     int slots_per_bucket;
     SampleParams sp;
-    int tc_l2;          // TransE p = 2 with tensor-core backward: the splits hold C.T and C^T.Q, C = dL/dF / distance
+    int tc;             // tensor-core backward: dQ's splits lack the row's factor Grow
+    int tc_l2;          // TransE p = 2 on it: the splits hold C.T and C^T.Q, C = dL/dF / distance, and Cpart / xsum_q the sums of C
     int neg_direct;     // the dT contraction wrote the negatives' gradient rows itself (one K split, no correction term)
     int wait_limit;     // tries of a bounded barrier wait
     const float* proj;  // feature-projection encoder: [2B+N, d] M e_F of the slots [heads | tails | negs], added to the rows read; or NULL
@@ -249,6 +250,50 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
         if (p.kind == KIND_L1 || p.kind == KIND_CL1 || p.kind == KIND_TH_L1) f = -acc;
         else if (p.kind == KIND_L2 || p.kind == KIND_TH_L2) f = -sqrtf(acc);
         p.w.fpos[b] = f;
+    }
+    if (p.w.row_stat) {
+        // tensor cores: the row's reference, the largest exponent among eight of its negatives (and the positive, which the
+        // sampled softmax sums too)
+        constexpr int SAMPLES = 8;
+        const int slot = (int)((int64_t)(lane & (SAMPLES - 1)) * p.N / SAMPLES);
+        const int32_t mine = p.fused_sample ? sample_negative(p.sp, slot) : p.negs[slot];
+        float part[SAMPLES];
+#pragma unroll
+        for (int j = 0; j < SAMPLES; ++j) {
+            const int64_t id = checked_id(__shfl_sync(0xffffffffu, mine, j), p.E, p.w.status);
+            const int n = __shfl_sync(0xffffffffu, slot, j);
+            part[j] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kMaxChunks; ++i) {
+                const int c = lane + 32 * i;
+                if (c >= d4) continue;
+                float4 v = reinterpret_cast<const float4*>(p.ent)[id * d4 + c];
+                if (p.proj) v = f4add(v, reinterpret_cast<const float4*>(p.proj)[(int64_t)(2 * p.B + n) * d4 + c]);
+                part[j] += pair_partial(p.kind, q[i], v);
+            }
+        }
+        // the eight sums side by side: every exchange halves the sums a lane carries
+#pragma unroll
+        for (int half = SAMPLES / 2; half >= 1; half >>= 1) {
+            const bool upper = (lane & half) != 0;
+#pragma unroll
+            for (int j = 0; j < half; ++j) {
+                const float send = upper ? part[j] : part[j + half], keep = upper ? part[j + half] : part[j];
+                part[j] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+            }
+        }
+        float f = part[0];
+        f += __shfl_xor_sync(0xffffffffu, f, 8);
+        f += __shfl_xor_sync(0xffffffffu, f, 16);
+        if (p.kind == KIND_L2) f = -sqrtf(f);
+        const bool ce = p.loss == KGE_LOSS_SAMPLED_SOFTMAX;
+        constexpr float kLog2e = 1.4426950408889634f;
+        float y = warp_max(fmaf(f, ce ? kLog2e : p.adv_temp * kLog2e, ce ? p.ce_c * kLog2e : 0.f));
+        if (ce) y = fmaxf(y, __shfl_sync(0xffffffffu, p.kind == KIND_L2 ? -sqrtf(acc) : acc, 0) * kLog2e);
+        if (lane == 0) {
+            reinterpret_cast<float2*>(p.w.row_stat)[b] = make_float2(fmaxf(y, -1e30f), 0.f);
+            if (b == 0) p.w.status[TC_REDO_FLAG] = 0;
+        }
     }
 }
 
@@ -996,14 +1041,14 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     if (warp >= p.B) {
         const int n = warp - p.B;
         const float4* part = reinterpret_cast<const float4*>(p.w.dTpart);
-        float wsum = 0.f;   // TransE p = 1: the splits hold P, the gradient is 2 P - (column sum of dL/dF)
-        if (p.kind == KIND_L1) wsum = sum_splits(p.w.Cpart + n, p.N, p.split_t);
+        float wsum = 0.f;   // column sum of dL/dF.  TransE p = 1: the splits hold P, the gradient is 2 P - (column sum)
+        if (p.kind == KIND_L1 || p.tc_l2) wsum = sum_splits(p.w.Cpart + n, p.N, p.split_t);
         const float creg = p.w.reg_s3 ? reg_coef(p.reg_lambda, p.reg_form, p.w.reg_s3[2 * p.B + n]) : 0.f;
         for (int c = lane; c < d4; c += 32) {
             float4 s = sum_splits(part + (int64_t)n * d4 + c, (int64_t)p.N * d4, p.split_t + p.th_slabs);
             if (p.kind == KIND_L1) s = make_float4(2.f * s.x - wsum, 2.f * s.y - wsum, 2.f * s.z - wsum, 2.f * s.w - wsum);
             if (p.tc_l2) {   // dT_n = sum_b C_bn (q_b - t_n) = (C^T Q)_n - (column sum of C) t_n
-                const float cs = p.w.Gcol[n];
+                const float cs = wsum;
                 const float4 t = reinterpret_cast<const float4*>(p.w.Tneg)[(int64_t)n * d4 + c];
                 s = make_float4(s.x - cs * t.x, s.y - cs * t.y, s.z - cs * t.z, s.w - cs * t.w);
             }
@@ -1020,6 +1065,8 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     const float4* trow = reinterpret_cast<const float4*>(p.ent) + tid * d4;
     const float4* qrow = reinterpret_cast<const float4*>(p.w.Q) + (int64_t)b * d4;
     const float gp = p.w.gpos[b], fp = p.w.fpos[b];
+    const float factor = p.tc ? p.w.Grow[b] : 1.f;
+    const float xrow = p.tc_l2 ? factor * sum_splits(p.w.xsum_q + b, p.B, p.split_q) : 0.f;
 
     float4 h[kMaxChunks], t[kMaxChunks], q[kMaxChunks], dq[kMaxChunks], dt[kMaxChunks];
 #pragma unroll
@@ -1037,8 +1084,9 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
             const float rs = p.w.Grow[b];
             s = make_float4(rs - 2.f * s.x, rs - 2.f * s.y, rs - 2.f * s.z, rs - 2.f * s.w);
         }
+        if (p.tc) s = f4scale(factor, s);
         if (p.tc_l2 && in) {             // dQ_b = sum_n C_bn (t_n - q_b) = (C T)_b - (row sum of C) q_b
-            const float rs = p.w.Grow[b];
+            const float rs = xrow;
             s = make_float4(s.x - rs * q[i].x, s.y - rs * q[i].y, s.z - rs * q[i].z, s.w - rs * q[i].w);
         }
         dq[i] = s; dt[i] = f4zero();
@@ -1246,7 +1294,8 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     p.sp = make_sample_params(h, step);
     p.sp.heads = h->ws.heads; p.sp.rels = h->ws.rels; p.sp.tails = h->ws.tails; p.sp.negs = h->ws.negs;
     p.slots_per_bucket = c.batch / (c.head_part < 0 ? c.num_parts * c.num_parts : c.num_parts);
-    p.tc_l2 = c.prec == KGE_PREC_BF16_TC && p.kind == KIND_L2;
+    p.tc = c.prec == KGE_PREC_BF16_TC;
+    p.tc_l2 = p.tc && p.kind == KIND_L2;
     p.neg_direct = tc_negatives_direct(h) ? 1 : 0;
     p.wait_limit = h->wait_limit;
     p.reg_lambda = c.reg_lambda; p.reg_form = c.reg_form;
