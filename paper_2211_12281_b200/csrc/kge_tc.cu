@@ -29,9 +29,7 @@ namespace {
 
 constexpr int TC_BM = 128, TC_BN = 128, TC_BK = 64;      // BK bf16 = one 128-byte swizzle row
 constexpr int TC_STAGES = 4;
-constexpr int TC_RING_MAX = 8;                            // barriers are laid out for the deepest ring (resident column tile, below)
 constexpr int TC_EPI_WARPS = 8;                           // epilogue warps of the training kernels: TC_EPI_GROUPS per tensor-memory lane quarter
-constexpr int TC_EPI_WARPS_TOPK = 16;                     // the filter epilogue of full-entity scoring profits from more
 constexpr int TC_EPI_GROUPS = TC_EPI_WARPS / 4;
 constexpr int TC_GRAD_STAGE_BYTES = 2048;                 // per epilogue warp: 32 rows x 32 bf16 columns on their way to memory
 constexpr int TC_STORE_STAGE_BYTES = 4096;                // the same for EPI_STORE's 32 rows x 32 fp32 columns
@@ -40,17 +38,16 @@ constexpr int TC_PIECE = TC_BN / TC_EPI_GROUPS;           // columns of a 128-wi
 // measured against eight, C3 passes 41.5 / 58.0 -> 39.4 / 53.8 us, the special-function-bound C4 passes 98.7 / 154.7 -> 98.9 / 135.8 us,
 // although sixteen warps leave 96 registers per thread and the norm-expansion variants spill a little.
 constexpr int TC_FUSED_WARPS_256 = 16;
-__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 3 = EPI_TOPK, 1 = the fused loss epilogue
-    return (epi & 3) == 3 ? TC_EPI_WARPS_TOPK : (((epi & 3) == 1 && bn == 256) ? TC_FUSED_WARPS_256 : TC_EPI_WARPS);
+__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 1 = the fused loss epilogue
+    return (epi & 3) == 1 && bn == 256 ? TC_FUSED_WARPS_256 : TC_EPI_WARPS;
 }
 __host__ __device__ constexpr int tc_threads(int epi, int bn = 128) { return 32 * (2 + tc_epi_warps(epi, bn)); }
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;
 constexpr uint32_t TC_MN_GROUP_BYTES = 64 * TC_BK * 2;    // MN-major operand: 64 contiguous elements x 64 K rows per TMA box
 __host__ __device__ constexpr uint32_t tc_stage_bytes(int bn) { return TC_A_BYTES + (uint32_t)bn * TC_BK * 2; }
 __host__ __device__ constexpr size_t tc_smem_bytes(int bn) { return 1024 + (size_t)TC_STAGES * tc_stage_bytes(bn) + 256; }
-constexpr int TC_BEAT_ROWS_MAX = 8 * 1024;                 // queries whose rank counts fit in shared memory beside the 256-column stages
 
-enum { EPI_STORE = 0, EPI_LOSS = 1, EPI_GRAD = 2, EPI_TOPK = 3, EPI_L2 = 4, EPI_CE = 8,    // L2 / CE: flags of the fused loss epilogues
+enum { EPI_STORE = 0, EPI_LOSS = 1, EPI_GRAD = 2, EPI_L2 = 4, EPI_CE = 8,    // L2 / CE: flags of the fused loss epilogues
        EPI_A1 = 16 };   // log-sigmoid loss of a distance score with self-adversarial temperature exactly 1 (see tc_loss_chunk)
 
 struct TcGemmParams {
@@ -71,19 +68,6 @@ struct TcGemmParams {
     const float2* row_stat;               // [M] EPI_LOSS: (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser), 0: row is finished
     const int32_t* redo;                  // EPI_GRAD: whether there is any row to do
     uint16_t* Gb; int64_t ldg;            // [M, ldg] bf16 dL/dF (divided by the distance for l2)
-    // full-entity scoring (EPI_TOPK): rows are queries, columns the entities [n_base, n_base + N)
-    int m_fastest;                        // walk the row tiles of one column tile first (the column tile stays in L2)
-    int64_t n_base;
-    int64_t id_base;                      // the caller's id of table row 0 (sharded inference)
-    const float *thr, *ftrue;             // [M] current k-th best score; score of the true tail
-    const int32_t *thr_id, *tt;           // [M] its id; true tail ids (or NULL)
-    int32_t *cand_cnt, *beat_tmp;         // [M] candidates appended in this chunk; entities ordered before the true tail
-    float* cand_score; int32_t* cand_id;  // [M, cand_cap]
-    int cand_cap;
-    int32_t* overflow;                    // set when a candidate list is full: the call's later launches do nothing
-    int first;                            // first chunk: nothing is filtered, the scores go to the candidate lists in entity order
-    int beat_rows;                        // rows whose rank counts are gathered in shared memory first (0: global atomics)
-    int resident_b;                       // EPI_TOPK: the column tile has a buffer of its own and the ring holds row tiles only
 };
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar) {
@@ -209,19 +193,13 @@ __device__ __forceinline__ float tc_score(const TcGemmParams& p, float acc, floa
 struct TcRowState {
     float rn;                 // squared norm of the row (norm expansion)
     float2 st;                // EPI_LOSS: the row's (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser)
-    float thr, ft;            // EPI_TOPK: current k-th best score, score of the true tail
-    int32_t thr_id, tt;       //           its id, the true tail's id
 };
 template <int EPI>
 __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int row) {
-    TcRowState r{0.f, make_float2(0.f, 0.f), INFINITY, 0.f, 0, -1};
-    if (row >= p.M) return r;   // rows outside the problem: no true tail, a threshold nothing exceeds
+    TcRowState r{0.f, make_float2(0.f, 0.f)};
+    if (row >= p.M) return r;
     if ((EPI & EPI_L2) != 0) r.rn = p.row_norm2[row];
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) r.st = p.row_stat[row];
-    if ((EPI & 3) == EPI_TOPK) {
-        r.thr = p.thr[row]; r.thr_id = p.thr_id[row];
-        if (p.tt) { r.ft = p.ftrue[row]; r.tt = p.tt[row]; }
-    }
     return r;
 }
 
@@ -446,126 +424,20 @@ __device__ __forceinline__ float float_below(float x) {
     return __uint_as_float(x > 0.f ? b - 1u : b + 1u);
 }
 
-// Full-entity scoring (Section 3.1 "Inference"): a score survives into the query's candidate
-// list if it is ordered before the query's current k-th best under (score descending, entity
-// id ascending); entities ordered before the true tail are counted for its rank.
-// Within a run of 32 consecutive entity ids that does not contain the reference id, "ordered
-// before (f0, id0)" is a plain comparison: f >= f0 if the run lies below id0, f > f0 if above;
-// f >= f0 is written f > (largest float below f0).  Only the run that contains the reference
-// id takes the element-by-element form, so the common case costs a compare-and-count per score
-// for the rank and one maximum per score for the candidate test.
-template <int WIDTH>
-__device__ __forceinline__ void tc_epilogue_topk(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, int32_t* beat_sm) {
-    const bool rin = row < p.M;
-    // rows outside the problem stay in the loop (the warp votes below need every lane): their state
-    // holds no true tail and a threshold nothing exceeds
-    const float thr = rs.thr, ft = rs.ft; const int32_t thr_id = rs.thr_id, tt = rs.tt;
-    const float thr_lo = float_below(thr), ft_lo = float_below(ft);
-    const int lane = threadIdx.x & 31;
-    int beat = 0;
-    auto chunk = [&](float (&v)[32], int c0) {
-        const int ncol = it.n0 + c0;
-        const int valid = min(32, p.N - ncol);          // the same for every lane
-        if (valid <= 0) return;
-        const int32_t e0 = (int32_t)(p.n_base + p.id_base + ncol);
-        if (valid != 32) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) if (i >= valid) v[i] = -INFINITY;   // never counted, never a candidate
-        }
-        // rank of the true tail.  The branch is taken by the whole warp (a vote), so that the
-        // element-by-element form stays out of the instruction stream of the common case.
-        if (p.tt) {
-            const bool inside = tt >= e0 && tt < e0 + 32;
-            if (!__any_sync(0xffffffffu, inside)) {
-                // counted in floating point (exact: at most 8 per chain) on four independent chains:
-                // the comparison yields 1.0f and the additions go to the FMA pipe
-                const float c = tt >= e0 + 32 ? ft_lo : ft;
-                float n[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int i = 0; i < 32; ++i) n[i & 3] += one_if_gt(v[i], c);
-                if (tt >= 0) beat += (int)((n[0] + n[1]) + (n[2] + n[3]));
-            } else if (tt >= 0) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int32_t e = e0 + i;
-                    if (e != tt && (v[i] > ft || (v[i] == ft && e < tt))) ++beat;
-                }
-            }
-        }
-        if (p.first) {         // (a chunk starts at a multiple of 32 columns: whole 128-byte pieces of the row's list)
-            if (rin) {
-                float4* dst = reinterpret_cast<float4*>(p.cand_score + (int64_t)row * p.cand_cap + ncol);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-            }
-            return;
-        }
-        // candidates: anything ordered before the current k-th best
-        float vm[4];           // a tree of three-input maxima, not a chain of 31
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            vm[j] = max3(max3(v[8 * j], v[8 * j + 1], v[8 * j + 2]), max3(v[8 * j + 3], v[8 * j + 4], v[8 * j + 5]), fmaxf(v[8 * j + 6], v[8 * j + 7]));
-        const float vmax = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
-        // Rare once the threshold has tightened, but one warp of the sixteen that share a tile
-        // meets it at most tiles, and the tile waits for its slowest warp.  So the warp takes the
-        // flagged lanes one at a time and spreads that lane's 32 scores over its 32 lanes (one
-        // shuffle per score): the ordering test and the append then run once per lane, not 32
-        // times in a row.
-        unsigned pending = __ballot_sync(0xffffffffu, vmax > thr_lo);
-        while (pending) {
-            const int src = __ffs(pending) - 1;
-            pending &= pending - 1;
-            float f = 0.f;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const float t = __shfl_sync(0xffffffffu, v[i], src);
-                if (lane == i) f = t;
-            }
-            const float thr_s = __shfl_sync(0xffffffffu, thr, src);
-            const int32_t id_s = __shfl_sync(0xffffffffu, thr_id, src);
-            const int row_s = __shfl_sync(0xffffffffu, row, src);
-            const int32_t e = e0 + lane;
-            if (f > thr_s || (f == thr_s && e < id_s && f != -INFINITY)) {     // (padded columns hold -inf and never pass)
-                const int slot = atomicAdd(&p.cand_cnt[row_s], 1);
-                if (slot < p.cand_cap) {
-                    p.cand_score[(int64_t)row_s * p.cand_cap + slot] = f;
-                    p.cand_id[(int64_t)row_s * p.cand_cap + slot] = e;
-                } else {
-                    *p.overflow = 1;   // the host redoes this chunk in shorter pieces
-                }
-            }
-        }
-    };
-    static_assert(WIDTH % 64 == 0, "two chunks of 32 columns are requested from tensor memory at a time");
-#pragma unroll 1
-    for (int c0 = col_off; c0 < col_off + WIDTH; c0 += 64) {
-        float v0[32], v1[32];
-        tmem_ld32_issue(taddr + (uint32_t)(c0 - col_off), v0);
-        tmem_ld32_issue(taddr + (uint32_t)(c0 - col_off) + 32u, v1);
-        tmem_ld_wait();
-        chunk(v0, c0);
-        chunk(v1, c0 + 32);
-    }
-    if (rin && beat > 0) {
-        if (row < p.beat_rows) atomicAdd(&beat_sm[row], beat); else atomicAdd(&p.beat_tmp[row], beat);
-    }
-}
-
 // Epilogue of one warp on one item: WIDTH columns [col_off, col_off + WIDTH) of the tile row held by
 // this thread's tensor-memory lane (taddr points at the first of them).
 template <int EPI, int WIDTH>
-__device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, int32_t* beat_sm) {
-    static_assert((EPI & 3) == EPI_STORE || (EPI & 3) == EPI_TOPK || WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
+__device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, void* scratch) {
+    static_assert((EPI & 3) == EPI_STORE || WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) {
 #pragma unroll 1
         for (int c = 0; c < WIDTH; c += TC_PIECE) {
-            uint4* stage = reinterpret_cast<uint4*>(beat_sm);
+            uint4* stage = static_cast<uint4*>(scratch);
             if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
             else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
         }
         return;
     }
-    if ((EPI & 3) == EPI_TOPK) { tc_epilogue_topk<WIDTH>(p, it, row, rs, col_off, taddr, beat_sm); return; }
     float* const Cout = p.C + (int64_t)it.z * p.split_stride;
     const float rn = rs.rn;
 #pragma unroll 1
@@ -581,7 +453,7 @@ __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem&
             // (warp-uniform) a lane holds 32 columns of its own row: stored as they are, every instruction would touch
             // 32 rows with 16 bytes each.  Through shared memory (128-byte rows, 16-byte pieces XOR-swizzled by row) an
             // instruction writes four rows' whole 128 bytes.
-            float4* st = reinterpret_cast<float4*>(beat_sm);
+            float4* st = static_cast<float4*>(scratch);
             const int lane = threadIdx.x & 31, sw = lane & 7, row0 = row - lane;
 #pragma unroll
             for (int i = 0; i < 8; ++i) st[lane * 8 + (i ^ sw)] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
@@ -604,21 +476,15 @@ __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem&
 // Work item = (K split, row tile, column tile), column tile fastest.  A CTA takes a contiguous
 // run of items, so consecutive items mostly share their A rows (kept warm in L2).
 __device__ __forceinline__ TcItem tc_item(const TcGemmParams& p, int64_t item) {
-    if (p.m_fastest) return TcItem{0, (int)(item % p.tiles_m) * TC_BM, (int)(item / p.tiles_m) * p.bn};
     const int tn = (int)(item % p.tiles_n), r = (int)(item / p.tiles_n);
     return TcItem{r / p.tiles_m, (r % p.tiles_m) * TC_BM, tn * p.bn};
 }
 // The same walk one item at a time: the divisions are paid once per CTA, not once per item and warp.
 __device__ __forceinline__ void tc_item_next(const TcGemmParams& p, TcItem& it) {
-    if (p.m_fastest) {
-        it.m0 += TC_BM;
-        if (it.m0 >= p.tiles_m * TC_BM) { it.m0 = 0; it.n0 += p.bn; }
-    } else {
-        it.n0 += p.bn;
-        if (it.n0 >= p.tiles_n * p.bn) {
-            it.n0 = 0; it.m0 += TC_BM;
-            if (it.m0 >= p.tiles_m * TC_BM) { it.m0 = 0; ++it.z; }
-        }
+    it.n0 += p.bn;
+    if (it.n0 >= p.tiles_n * p.bn) {
+        it.n0 = 0; it.m0 += TC_BM;
+        if (it.m0 >= p.tiles_m * TC_BM) { it.m0 = 0; ++it.z; }
     }
 }
 
@@ -638,17 +504,12 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* base = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
     uint64_t* full = reinterpret_cast<uint64_t*>(base + (size_t)TC_STAGES * TC_STAGE_BYTES);
-    uint64_t* empty = full + TC_RING_MAX;
-    uint64_t* acc_full = empty + TC_RING_MAX;    // [NACC] accumulator buffer written
+    uint64_t* empty = full + TC_STAGES;
+    uint64_t* acc_full = empty + TC_STAGES;    // [NACC] accumulator buffer written
     uint64_t* acc_empty = acc_full + NACC;       // [NACC] accumulator buffer drained by all epilogue warps
-    uint64_t* b_full = acc_empty + NACC;         // resident column tile: loaded / no longer read by any MMA
-    uint64_t* b_free = b_full + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(b_free + 1);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + NACC);
     volatile uint32_t* stop = tmem_slot + 1;     // set by a warp whose wait ran out
-    volatile int* cta_items = reinterpret_cast<volatile int*>(tmem_slot + 2);
-    int32_t* beat_sm = reinterpret_cast<int32_t*>(base + (size_t)TC_STAGES * TC_STAGE_BYTES + 256);   // [beat_rows], EPI_TOPK
-    if ((EPI & 3) == EPI_TOPK)
-        for (int i = threadIdx.x; i < p.beat_rows; i += TC_THREADS) beat_sm[i] = 0;
+    unsigned char* scratch_sm = base + (size_t)TC_STAGES * TC_STAGE_BYTES + 256;
 
     if ((EPI & 3) == EPI_GRAD) {                        // (nothing in flight writes the flag)
         grid_dependency_wait();
@@ -661,10 +522,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     const int kb_total = (p.K + TC_BK - 1) / TC_BK;
 
     if (threadIdx.x == 0) {
-        // full-entity scoring after a list overflowed: no items (one thread's reading: the flag may change while this launch runs)
-        *cta_items = (EPI & 3) == EPI_TOPK && *reinterpret_cast<volatile int32_t*>(p.overflow) ? 0 : per_cta;
-        for (int s = 0; s < TC_RING_MAX; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        mbar_init(b_full, 1); mbar_init(b_free, 1);
+        for (int s = 0; s < TC_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], GW); }
         *stop = 0;
         mbar_init_fence();
@@ -677,86 +535,16 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const int item_end = min(p.items, item_begin + *cta_items);
+    const int item_end = min(p.items, item_begin + per_cta);
     if ((EPI & 3) == EPI_LOSS) grid_dependency_wait();     // (launched while the kernel before it drains)
 
-    // Full-entity scoring with rows of at most 128 coordinates: the column (entity) tile of the
-    // current run of items sits in a buffer of its own (2 x 32 KB) and the rest of the stage memory
-    // is a ring of eight 16 KB row-tile slices, four items deep.  With the column tile kept inside
-    // the ring stages instead, only two items were in flight and the MMAs waited for copies.
-    const bool resident = (EPI & 3) == EPI_TOPK && BN == 256 && p.resident_b != 0;
-    constexpr uint32_t RES_B_BYTES = 2u * 256u * TC_BK * 2u;          // two slices of the column tile
-    constexpr int RES_RING = 8;
-    if (warp == 0 && resident) {
-        if (lane == 0) {
-            int ring = 0, btile = 0, cur_n0 = -1;
-            TcItem it = tc_item(p, item_begin);
-            for (int item = item_begin; item < item_end && !*stop; ++item, tc_item_next(p, it)) {
-                bool ok = true;
-                if (it.n0 != cur_n0) {      // a new column tile: every MMA on the previous one must be done
-                    cur_n0 = it.n0;
-                    ok = mbar_wait_idle(b_free, (btile & 1) ^ 1, p.wait_limit);
-                    if (ok) {
-                        mbar_arrive_expect_tx(b_full, (uint32_t)kb_total * (256u * TC_BK * 2u));
-                        for (int kb = 0; kb < kb_total; ++kb)
-#pragma unroll
-                            for (int g = 0; g < 2; ++g)
-                                tma_load_2d(base + (size_t)kb * (256 * TC_BK * 2) + g * (128 * TC_BK * 2), &tmB, kb * TC_BK,
-                                            (int)p.n_base + it.n0 + 128 * g, b_full);
-                        ++btile;
-                    }
-                }
-                for (int kb = 0; kb < kb_total && ok; ++kb, ++ring) {
-                    const int s = ring % RES_RING;
-                    ok = mbar_wait_idle(&empty[s], ((ring / RES_RING) & 1) ^ 1, p.wait_limit);
-                    if (!ok) break;
-                    mbar_arrive_expect_tx(&full[s], TC_A_BYTES);
-                    tma_load_2d(base + RES_B_BYTES + (size_t)s * TC_A_BYTES, &tmA, kb * TC_BK, it.m0, &full[s]);
-                }
-                if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); break; }
-            }
-        }
-    } else if (warp == 1 && resident) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN, false, false);
-            int ring = 0, btile = 0, cur_n0 = -1;
-            bool ok = true;
-            TcItem it = tc_item(p, item_begin);
-            for (int item = item_begin, local = 0; item < item_end && ok && !*stop; ++item, ++local) {
-                const int buf = local % NACC;
-                if (it.n0 != cur_n0) {
-                    cur_n0 = it.n0;
-                    if (!mbar_wait_idle(b_full, btile & 1, p.wait_limit)) { ok = false; break; }
-                    ++btile;
-                }
-                if (!mbar_wait_idle(&acc_empty[buf], ((local / NACC) & 1) ^ 1, p.wait_limit)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t tmem_acc = tmem_base + (uint32_t)buf * BN;
-                for (int kb = 0; kb < kb_total; ++kb, ++ring) {
-                    const int s = ring % RES_RING;
-                    if (!mbar_wait_idle(&full[s], (ring / RES_RING) & 1, p.wait_limit)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t sa = smem_u32(base + RES_B_BYTES + (size_t)s * TC_A_BYTES);
-                    const uint32_t sb = smem_u32(base + (size_t)kb * (256 * TC_BK * 2));
-#pragma unroll
-                    for (int k = 0; k < TC_BK / 16; ++k)
-                        umma_bf16(tmem_acc, umma_desc_k_sw128(sa + k * 32), umma_desc_k_sw128(sb + k * 32), idesc, (kb | k) != 0);
-                    umma_commit(&empty[s]);
-                }
-                umma_commit(&acc_full[buf]);           // also after a failed wait, so the epilogue warps wake up
-                tc_item_next(p, it);
-                if (item + 1 >= item_end || it.n0 != cur_n0) umma_commit(b_free);   // the last MMAs that read this column tile
-            }
-            if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
-        }
-    } else if (warp == 0) {
+    if (warp == 0) {
         if (lane == 0) {
             int ring = 0;    // slices issued so far: stage = ring % STAGES, phase = ring / STAGES
             // Without K splits and with a slice count that divides the ring, slice kb of every item
-            // lands in the same stages, so the operand that consecutive items share (the row tile
-            // when column tiles vary fastest, the column tile otherwise) is still there from the item
-            // before: it is fetched again only when it changes.  keep[s] = first row (or column) of
-            // the shared operand held by stage s.
+            // lands in the same stages, so the row tile that consecutive items share is still there from
+            // the item before: it is fetched again only when it changes.  keep[s] = first row of the tile
+            // held by stage s.
             const bool reuse = p.kb_per_split == kb_total && TC_STAGES % kb_total == 0;
             int keep[TC_STAGES];
 #pragma unroll
@@ -768,20 +556,16 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                     const int s = ring % TC_STAGES;
                     if (!mbar_wait_idle(&empty[s], ((ring / TC_STAGES) & 1) ^ 1, p.wait_limit)) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); break; }
                     unsigned char* sa = base + (size_t)s * TC_STAGE_BYTES;
-                    const int shared_at = p.m_fastest ? it.n0 : it.m0;
                     bool have = false;
 #pragma unroll
-                    for (int q = 0; q < TC_STAGES; ++q) if (q == s) { have = reuse && keep[q] == shared_at; keep[q] = shared_at; }
-                    const bool load_a = !(have && !p.m_fastest), load_b = !(have && p.m_fastest);
-                    mbar_arrive_expect_tx(&full[s], (load_a ? TC_A_BYTES : 0u) + (load_b ? TC_STAGE_BYTES - TC_A_BYTES : 0u));
+                    for (int q = 0; q < TC_STAGES; ++q) if (q == s) { have = reuse && keep[q] == it.m0; keep[q] = it.m0; }
+                    mbar_arrive_expect_tx(&full[s], have ? TC_STAGE_BYTES - TC_A_BYTES : TC_STAGE_BYTES);
                     const int k0 = (kb0 + kb) * TC_BK;
-                    if (load_a) tma_load_2d(sa, &tmA, k0, it.m0, &full[s]);
+                    if (!have) tma_load_2d(sa, &tmA, k0, it.m0, &full[s]);
                     unsigned char* sb = sa + TC_A_BYTES;
-                    if (load_b) {
 #pragma unroll
-                        for (int g = 0; g < BN / 128; ++g)   // boxes of 128 rows, one after the other
-                            tma_load_2d(sb + g * (128 * TC_BK * 2), &tmB, k0, (int)p.n_base + it.n0 + 128 * g, &full[s]);
-                    }
+                    for (int g = 0; g < BN / 128; ++g)   // boxes of 128 rows, one after the other
+                        tma_load_2d(sb + g * (128 * TC_BK * 2), &tmB, k0, it.n0 + 128 * g, &full[s]);
                 }
             }
         }
@@ -831,9 +615,8 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
             tc_fence_after();
             if (!ok || *stop) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * GCOLS);
-            // scratch after the barriers: the rank counts of EPI_TOPK, or 2 / 4 KB per epilogue warp for the stores of bf16 / fp32 tiles
-            int32_t* scratch = (EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD ? beat_sm + (warp - 2) * (TC_GRAD_STAGE_BYTES / 4)
-                             : ((EPI & 3) == EPI_STORE ? beat_sm + (warp - 2) * (TC_STORE_STAGE_BYTES / 4) : beat_sm);
+            // scratch after the barriers: 2 or 4 KB per epilogue warp for the stores of bf16 or fp32 tiles
+            void* scratch = scratch_sm + (warp - 2) * ((EPI & 3) == EPI_STORE ? TC_STORE_STAGE_BYTES : TC_GRAD_STAGE_BYTES);
             tc_epilogue<EPI, GCOLS>(p, it, it.m0 + quarter * 32 + lane, rs, cgrp * GCOLS, taddr, scratch);
             tc_fence_before();
             __syncwarp();
@@ -844,8 +627,6 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     __syncthreads();
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_TMEM_COLS) : "memory");
-    if ((EPI & 3) == EPI_TOPK)     // hand this CTA's rank counts over (integer adds: the result does not depend on the order)
-        for (int i = threadIdx.x; i < p.beat_rows; i += TC_THREADS) { const int32_t b = beat_sm[i]; if (b) atomicAdd(&p.beat_tmp[i], b); }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -900,8 +681,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* base = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
     uint64_t* full = reinterpret_cast<uint64_t*>(base + (size_t)STAGES * STAGE_BYTES);
-    uint64_t* empty = full + TC_RING_MAX;
-    uint64_t* acc_full = empty + TC_RING_MAX;
+    uint64_t* empty = full + TC_STAGES;
+    uint64_t* acc_full = empty + TC_STAGES;
     uint64_t* acc_empty = acc_full + NACC;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + NACC);
     volatile uint32_t* stop = tmem_slot + 1;
@@ -1228,6 +1009,302 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
 }
 
+// ------------------------------------------------------------------------------------------
+// Full-entity scoring (Section 3.1 "Inference"): a score survives into the query's candidate list if it is ordered before the query's
+// current k-th best under (score descending, entity id ascending); entities ordered before the true tail are counted for its rank.
+//
+// The queries stay and the entities pass by.  A CTA keeps MT tiles of 128 queries in shared memory and runs 256-entity tiles past them,
+// 64 coordinates (32 KB) at a time through a ring; each (query tile, entity tile) is one accumulator of 256 columns, two in
+// turn, and each accumulator has eight epilogue warps of its own (32 queries x 128 entities each).  What an epilogue needs of its
+// query (threshold, true tail's score, ids) and its rank count are then registers for hundreds of tiles.  With the entity tile kept and the
+// queries passing by, as before, every tile read them from L2 and added its counts to shared memory: 39.8 ms for 15,000 x
+// 8 M x 128, 3,000 cycles per 128 x 256 tile against the MMAs' 1,024, most of it latency.
+// MT = 2 for rows of at most 128 coordinates halves the entity bytes a SM reads per score (32 bytes a clock at the
+// MMAs' full rate); longer rows leave no room for the second tile's ring.
+// All CTAs walk the table one superblock of some 32 MB after the other, each through its own contiguous run of the superblock's (query
+// group, entity tile) pairs, query group slowest, so that the table is read from HBM once and a CTA changes queries rarely.
+// ------------------------------------------------------------------------------------------
+constexpr int SCAN_BN = 256, SCAN_WARPS = 16, SCAN_THREADS = 32 * (2 + SCAN_WARPS), SCAN_RING_MAX = 8;
+constexpr uint32_t SCAN_SLICE_BYTES = SCAN_BN * TC_BK * 2;
+constexpr size_t SCAN_SMEM_MAX = 227 * 1024;
+
+struct ScanParams {
+    int M, N, slices, tiles_m, groups, tiles_n, sb_tiles, ring;     // groups of MT query tiles; tiles per superblock
+    int64_t n_base, id_base;              // first table row of this launch; the caller's id of table row 0 (sharded inference)
+    const float *thr, *ftrue;             // [M] current k-th best score; score of the true tail
+    const int32_t *thr_id, *tt;           // [M] its id; true tail ids (or NULL)
+    int32_t *cand_cnt, *beat_tmp;         // [M] candidates appended in this launch; entities ordered before the true tail
+    float* cand_score; int32_t* cand_id;  // [M, cand_cap]
+    int cand_cap;
+    int32_t* overflow;                    // set when a candidate list is full: the call's later launches do nothing
+    int32_t* status; int wait_limit;
+};
+
+// Waits for this thread's outstanding tensor-memory loads; the registers pass through, so that nothing that uses them moves ahead.
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]),
+                   "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]),
+                   "+f"(v[21]), "+f"(v[22]), "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]),
+                   "+f"(v[31])::"memory");
+}
+
+// One query as its lane holds it.
+struct ScanRow {
+    float thr, thr_lo, ft, ft_lo;         // k-th best score, largest float below it; the same of the true tail's score
+    int32_t thr_id, tt, row;
+    int beat;
+};
+
+// Calls f(query group, entity tile) for this CTA's pairs until it returns false.
+template <class F>
+__device__ __forceinline__ void scan_walk(const ScanParams& p, F f) {
+    for (int sb = 0; sb < p.tiles_n; sb += p.sb_tiles) {
+        const int tiles = min(p.sb_tiles, p.tiles_n - sb);
+        const int64_t pairs = (int64_t)p.groups * tiles;
+        const int64_t begin = pairs * blockIdx.x / gridDim.x, end = pairs * (blockIdx.x + 1) / gridDim.x;
+        int g = (int)(begin / tiles), e = (int)(begin % tiles);
+        for (int64_t i = begin; i < end; ++i) {
+            if (!f(g, sb + e)) return;
+            if (++e == tiles) { e = 0; ++g; }
+        }
+    }
+}
+
+// 32 scores of one query against the entities [e0, e0 + 32) from tile column `ncol` on.  Within a run of entity ids that does not contain the
+// reference id, "ordered before (f0, id0)" is a plain comparison: f >= f0 if the run lies below id0, f > f0 if above; f >= f0
+// is written f > (largest float below f0).  `cut`: that bound of the true tail, unless the true tail is among the warp's ids
+// (`exact`); n: the count so far, in floating point on four chains (exact, and the additions go to the FMA pipe).
+template <bool FIRST>
+__device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], ScanRow& r, int ncol, float cut, bool exact, float (&n)[4]) {
+    const int lane = threadIdx.x & 31, valid = p.N - ncol;             // the same for every lane
+    if (valid <= 0) return;
+    const int32_t e0 = (int32_t)(p.n_base + p.id_base + ncol);
+    if (valid < 32) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) if (i >= valid) v[i] = -INFINITY;   // never counted, never a candidate
+    }
+    if (!exact) {
+        if (p.tt) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) n[i & 3] += one_if_gt(v[i], cut);
+        }
+    } else if (r.tt >= 0) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int32_t e = e0 + i;
+            if (e != r.tt && (v[i] > r.ft || (v[i] == r.ft && e < r.tt))) ++r.beat;
+        }
+    }
+    if constexpr (FIRST) {               // (a chunk starts at a multiple of 32 columns: whole 128-byte pieces of the row's list)
+        if (r.row < p.M) {
+            float4* dst = reinterpret_cast<float4*>(p.cand_score + (int64_t)r.row * p.cand_cap + ncol);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+        return;
+    } else {
+    float vm[4];               // a tree of three-input maxima, not a chain of 31
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        vm[j] = max3(max3(v[8 * j], v[8 * j + 1], v[8 * j + 2]), max3(v[8 * j + 3], v[8 * j + 4], v[8 * j + 5]), fmaxf(v[8 * j + 6], v[8 * j + 7]));
+    const float vmax = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
+    // Rare once the threshold has tightened.  The warp takes the flagged lanes one at a time and spreads that lane's 32 scores over its
+    // 32 lanes (one shuffle per score): the ordering test and the append then run once per lane, not 32 times in a row.
+    unsigned pending = __ballot_sync(0xffffffffu, vmax > r.thr_lo);
+    while (pending) {
+        const int src = __ffs(pending) - 1;
+        pending &= pending - 1;
+        float f = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const float t = __shfl_sync(0xffffffffu, v[i], src);
+            if (lane == i) f = t;
+        }
+        const float thr_s = __shfl_sync(0xffffffffu, r.thr, src);
+        const int32_t id_s = __shfl_sync(0xffffffffu, r.thr_id, src), row_s = __shfl_sync(0xffffffffu, r.row, src);
+        const int32_t e = e0 + lane;
+        if (f > thr_s || (f == thr_s && e < id_s && f != -INFINITY)) {     // (padded columns hold -inf and never pass)
+            const int slot = atomicAdd(&p.cand_cnt[row_s], 1);
+            if (slot < p.cand_cap) {
+                p.cand_score[(int64_t)row_s * p.cand_cap + slot] = f;
+                p.cand_id[(int64_t)row_s * p.cand_cap + slot] = e;
+            } else {
+                *p.overflow = 1;   // the host redoes this chunk in shorter pieces
+            }
+        }
+    }
+    }
+}
+
+// FIRST: nothing is filtered yet, the scores go to the candidate lists in entity order.
+template <int MT, bool FIRST>
+__global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, ScanParams p) {
+    extern __shared__ unsigned char tc_smem_raw[];
+    unsigned char* base = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
+    unsigned char* slice0 = base + (size_t)MT * p.slices * TC_A_BYTES;
+    uint64_t* full = reinterpret_cast<uint64_t*>(slice0 + (size_t)p.ring * SCAN_SLICE_BYTES);
+    uint64_t* empty = full + SCAN_RING_MAX;
+    uint64_t* acc_full = empty + SCAN_RING_MAX;    // [2] accumulator written
+    uint64_t* acc_empty = acc_full + 2;            // [2] accumulator read by all eight of its warps
+    uint64_t* q_full = acc_empty + 2;              // query tiles loaded / no longer read by any MMA
+    uint64_t* q_free = q_full + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_free + 1);
+    volatile uint32_t* stop = tmem_slot + 1;       // set by a warp whose wait ran out
+    volatile uint32_t* given_up = tmem_slot + 2;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < SCAN_RING_MAX; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], SCAN_WARPS / 2); }
+        mbar_init(q_full, 1); mbar_init(q_free, 1);
+        *stop = 0;
+        // after a list overflowed: no pairs (one thread's reading: the flag may change while this launch runs)
+        *given_up = *reinterpret_cast<volatile int32_t*>(p.overflow) != 0;
+        mbar_init_fence();
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2u * SCAN_BN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    const bool idle = *given_up != 0;
+
+    if (idle) {
+    } else if (warp == 0) {
+        if (lane == 0) {
+            int ring = 0, phase = 1, cur = -1, changes = 0;
+            bool ok = true;
+            scan_walk(p, [&](int g, int e) {
+                if (*stop) return false;
+                if (g != cur) {                    // other queries: every MMA on the ones before must be done
+                    cur = g;
+                    if (!mbar_wait_idle(q_free, (changes & 1) ^ 1, p.wait_limit)) { ok = false; return false; }
+                    ++changes;
+                    const int tiles = min(MT, p.tiles_m - g * MT);
+                    mbar_arrive_expect_tx(q_full, (uint32_t)(tiles * p.slices) * TC_A_BYTES);
+                    for (int t = 0; t < tiles; ++t)
+                        for (int kb = 0; kb < p.slices; ++kb)
+                            tma_load_2d(base + (size_t)(t * p.slices + kb) * TC_A_BYTES, &tmA, kb * TC_BK, (g * MT + t) * TC_BM, q_full);
+                }
+                for (int kb = 0; kb < p.slices; ++kb) {
+                    if (!mbar_wait_idle(&empty[ring], phase, p.wait_limit)) { ok = false; return false; }
+                    mbar_arrive_expect_tx(&full[ring], SCAN_SLICE_BYTES);
+                    unsigned char* dst = slice0 + (size_t)ring * SCAN_SLICE_BYTES;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_2d(dst + h * (128 * TC_BK * 2), &tmB, kb * TC_BK, (int)p.n_base + e * SCAN_BN + 128 * h, &full[ring]);
+                    if (++ring == p.ring) { ring = 0; phase ^= 1; }
+                }
+                return true;
+            });
+            if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, SCAN_BN, false, false);
+            int ring = 0, phase = 0, cur = -1, changes = 0;
+            int uses[2] = {0, 0}, turn = 0;
+            bool ok = true;
+            scan_walk(p, [&](int g, int e) {
+                if (*stop) return false;
+                if (g != cur) {
+                    if (cur >= 0) umma_commit(q_free);
+                    cur = g;
+                    if (!mbar_wait_idle(q_full, changes & 1, p.wait_limit)) { ok = false; return false; }
+                    ++changes;
+                }
+                const int tiles = min(MT, p.tiles_m - g * MT);
+                int s = ring, ph = phase;
+#pragma unroll
+                for (int t = 0; t < MT; ++t) {
+                    if (t >= tiles) break;
+                    const int buf = MT == 1 ? turn : t;
+                    const int used = buf ? uses[1]++ : uses[0]++;
+                    if (!mbar_wait_idle(&acc_empty[buf], (used & 1) ^ 1, p.wait_limit)) { ok = false; return false; }
+                    tc_fence_after();
+                    s = ring; ph = phase;
+                    for (int kb = 0; kb < p.slices; ++kb) {
+                        // (the second query tile finds the slices that the first waited for)
+                        if (!mbar_wait_idle(&full[s], ph, p.wait_limit)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t sa = smem_u32(base + (size_t)(t * p.slices + kb) * TC_A_BYTES);
+                        const uint32_t sb = smem_u32(slice0 + (size_t)s * SCAN_SLICE_BYTES);
+#pragma unroll
+                        for (int k = 0; k < TC_BK / 16; ++k)
+                            umma_bf16(tmem_base + (uint32_t)buf * SCAN_BN, umma_desc_k_sw128(sa + k * 32), umma_desc_k_sw128(sb + k * 32), idesc, (kb | k) != 0);
+                        if (t + 1 == tiles) umma_commit(&empty[s]);
+                        if (++s == p.ring) { s = 0; ph ^= 1; }
+                    }
+                    umma_commit(&acc_full[buf]);       // also after a failed wait, so the epilogue warps wake up
+                    if (!ok) return false;
+                }
+                ring = s; phase = ph; turn ^= 1;
+                return true;
+            });
+            if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+        }
+    } else {
+        const int acc = (warp - 2) >> 3, quarter = warp & 3, col0 = ((warp - 2) >> 2 & 1) * 128;   // (a warp reads the lanes of its own quarter only)
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * SCAN_BN + col0);
+        int cur = -1, used = 0, turn = 0;
+        ScanRow r{INFINITY, INFINITY, 0.f, 0.f, 0, -1, 0, 0};
+        auto hand_over = [&] { if (r.beat > 0) atomicAdd(&p.beat_tmp[r.row], r.beat); r.beat = 0; };
+        bool ok = true;
+        scan_walk(p, [&](int g, int e) {
+            if (MT == 1) { turn ^= 1; if ((turn ^ 1) != acc) return true; }
+            else if (g * MT + acc >= p.tiles_m) return true;
+            if (g != cur) {
+                hand_over();
+                cur = g;
+                r.row = (g * MT + (MT == 1 ? 0 : acc)) * TC_BM + quarter * 32 + lane;
+                // rows outside the problem stay in the loop (the warp votes need every lane): no true tail, a threshold nothing exceeds
+                r.thr = INFINITY; r.thr_id = 0; r.ft = INFINITY; r.tt = -1;
+                if (r.row < p.M) {
+                    r.thr = p.thr[r.row]; r.thr_id = p.thr_id[r.row];
+                    if (p.tt) { r.ft = p.ftrue[r.row]; r.tt = p.tt[r.row]; }
+                }
+                r.thr_lo = float_below(r.thr); r.ft_lo = float_below(r.ft);
+            }
+            const int32_t id0 = (int32_t)(p.n_base + p.id_base + e * SCAN_BN + col0);
+            const bool exact = __any_sync(0xffffffffu, r.tt >= id0 && r.tt < id0 + 128);
+            const float cut = r.tt < 0 ? INFINITY : (r.tt >= id0 + 128 ? r.ft_lo : r.ft);
+            ok = mbar_wait_bounded(&acc_full[acc], used & 1, p.wait_limit);
+            ++used;
+            tc_fence_after();
+            if (!ok || *stop) { ok = false; return false; }
+            float n[4] = {0.f, 0.f, 0.f, 0.f};
+            float va[32], vb[32];                  // the next 32 columns are on their way while these are looked at
+            tmem_ld32_issue(taddr, va);
+#pragma unroll 1
+            for (int c = 0; c < 128; c += 64) {
+                tmem_ld_wait(va);
+                tmem_ld32_issue(taddr + (uint32_t)(c + 32), vb);
+                scan_chunk<FIRST>(p, va, r, e * SCAN_BN + col0 + c, cut, exact, n);
+                tmem_ld_wait(vb);
+                if (c == 0) tmem_ld32_issue(taddr + 64u, va);
+                else {                             // everything is in registers: the accumulator is free
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[acc]);
+                }
+                scan_chunk<FIRST>(p, vb, r, e * SCAN_BN + col0 + c + 32, cut, exact, n);
+            }
+            r.beat += (int)((n[0] + n[1]) + (n[2] + n[3]));
+            return true;
+        });
+        if (!ok && lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+        hand_over();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2u * SCAN_BN) : "memory");
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -1349,22 +1426,17 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
 
 namespace {
 template <int EPI, int BN = 128>
-cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB, const TcGemmParams& p, int num_sms, cudaStream_t s,
-                             size_t extra_smem = 0) {
-    constexpr size_t smem = tc_smem_bytes(BN);
-    constexpr size_t extra_max = (EPI & 3) == EPI_TOPK ? (size_t)TC_BEAT_ROWS_MAX * 4
-                               : ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD ? (size_t)tc_epi_warps(EPI, BN) * TC_GRAD_STAGE_BYTES
-                               : ((EPI & 3) == EPI_STORE ? (size_t)tc_epi_warps(EPI, BN) * TC_STORE_STAGE_BYTES : 0));
-    if ((EPI & 3) != EPI_TOPK) extra_smem = extra_max;
+cudaError_t launch_gemm_inst(const unsigned char* tmA, const unsigned char* tmB, const TcGemmParams& p, int num_sms, cudaStream_t s) {
+    constexpr size_t smem = tc_smem_bytes(BN) + (size_t)tc_epi_warps(EPI, BN) * ((EPI & 3) == EPI_STORE ? TC_STORE_STAGE_BYTES : TC_GRAD_STAGE_BYTES);
     static DeviceOnce configured;
     const cudaError_t e = once_per_device(configured, [] {
-        return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem + extra_max));
+        return cudaFuncSetAttribute(tc_gemm_kernel<EPI, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD)
-        return launch_dependent(tc_gemm_kernel<EPI, BN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem + extra_smem, s,
+        return launch_dependent(tc_gemm_kernel<EPI, BN>, dim3(std::min(p.items, num_sms)), dim3(tc_threads(EPI, BN)), smem, s,
                                 *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
-    tc_gemm_kernel<EPI, BN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem + extra_smem, s>>>(
+    tc_gemm_kernel<EPI, BN><<<std::min(p.items, num_sms), tc_threads(EPI, BN), smem, s>>>(
         *reinterpret_cast<const CUtensorMap*>(tmA), *reinterpret_cast<const CUtensorMap*>(tmB), p);
     return cudaSuccess;
 }
@@ -1614,22 +1686,36 @@ int launch_cast_bf16(kge_handle* h, const float* src, uint16_t* dst, int64_t cou
 // rows [e_lo, e_hi) of the entity table, survivors appended to the candidate lists.
 int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, const int32_t* true_tails, int64_t id_base, int first, cudaStream_t s) {
     const Workspace& w = h->ws;
-    TcGemmParams p{};
-    p.M = nq; p.N = (int)(e_hi - e_lo); p.K = h->cfg.dim;
-    p.kb_per_split = (p.K + TC_BK - 1) / TC_BK;
-    p.bn = 256;      // a row tile of queries is shared by 256 entities
-    p.tiles_m = (p.M + TC_BM - 1) / TC_BM; p.tiles_n = (p.N + p.bn - 1) / p.bn;
-    if ((int64_t)p.tiles_m * p.tiles_n > 0x7fffffff) return KGE_ERR_BAD_ARG;
-    p.items = p.tiles_m * p.tiles_n;
+    ScanParams p{};
+    p.M = nq; p.N = (int)(e_hi - e_lo);
+    p.slices = (h->cfg.dim + TC_BK - 1) / TC_BK;
+    p.tiles_m = (nq + TC_BM - 1) / TC_BM; p.tiles_n = (p.N + SCAN_BN - 1) / SCAN_BN;
+    const int mt = p.slices <= 2 && p.tiles_m > 1 ? 2 : 1;
+    p.groups = (p.tiles_m + mt - 1) / mt;
+    const size_t fixed = 1024 + 256 + (size_t)mt * p.slices * TC_A_BYTES;
+    p.ring = (int)std::min<size_t>(SCAN_RING_MAX, (SCAN_SMEM_MAX - fixed) / SCAN_SLICE_BYTES);
+    const int grid = (int)std::min<int64_t>((int64_t)p.groups * p.tiles_n, h->num_sms);
+    // superblocks of about 32 MB, but at least 32 pairs per CTA in each
+    const int64_t tile_bytes = (int64_t)SCAN_BN * h->cfg.dim * 2;
+    const int64_t sb = std::max<int64_t>((int64_t)(32 << 20) / tile_bytes, ((int64_t)32 * grid + p.groups - 1) / p.groups);
+    const int64_t n_sb = (p.tiles_n + sb - 1) / sb;
+    p.sb_tiles = (int)((p.tiles_n + n_sb - 1) / n_sb);
     p.status = w.status; p.wait_limit = h->wait_limit;
-    p.m_fastest = 1; p.n_base = e_lo; p.id_base = id_base;
+    p.n_base = e_lo; p.id_base = id_base;
     p.thr = w.thr; p.thr_id = w.thr_id; p.ftrue = w.iftrue; p.tt = true_tails;
     p.cand_cnt = w.cand_cnt; p.beat_tmp = w.beat_tmp; p.cand_score = w.cand_score; p.cand_id = w.cand_id;
-    p.cand_cap = kCandCap; p.overflow = w.status + 1; p.first = first;
-    p.beat_rows = std::min(nq, TC_BEAT_ROWS_MAX);   // the other rows count with global atomics
-    p.resident_b = p.kb_per_split <= 2 ? 1 : 0;     // the column tile's two slices fit beside an eight-stage ring of row-tile slices
+    p.cand_cap = kCandCap; p.overflow = w.status + 1;
+    static DeviceOnce configured;
+    KGE_CUDA_CHECK(h, once_per_device(configured, [] {
+        cudaError_t e = cudaSuccess;
+        for (auto k : {tc_scan_kernel<1, false>, tc_scan_kernel<1, true>, tc_scan_kernel<2, false>, tc_scan_kernel<2, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCAN_SMEM_MAX);
+        return e;
+    }));
     // (the table's tensor map covers all rows; the kernel offsets its row coordinate by n_base)
-    KGE_CUDA_CHECK(h, (launch_gemm_inst<EPI_TOPK, 256>(h->tm_iq, h->tm_eb, p, h->num_sms, s, (size_t)p.beat_rows * 4)));
+    auto kernel = mt == 2 ? (first ? tc_scan_kernel<2, true> : tc_scan_kernel<2, false>) : (first ? tc_scan_kernel<1, true> : tc_scan_kernel<1, false>);
+    kernel<<<grid, SCAN_THREADS, fixed + (size_t)p.ring * SCAN_SLICE_BYTES, s>>>(*reinterpret_cast<const CUtensorMap*>(h->tm_iq),
+                                                                                 *reinterpret_cast<const CUtensorMap*>(h->tm_eb), p);
     KGE_LAUNCH_CHECK(h);
     return KGE_OK;
 }
