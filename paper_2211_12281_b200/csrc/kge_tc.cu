@@ -137,6 +137,14 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, float (&v)[32]) 
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Waits for this thread's outstanding tensor-memory loads; the registers pass through, so that nothing that uses them moves ahead.
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]),
+                   "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]),
+                   "+f"(v[21]), "+f"(v[22]), "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]),
+                   "+f"(v[31])::"memory");
+}
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) { tmem_ld32_issue(taddr, v); tmem_ld_wait(); }
 
 // Two columns.
@@ -323,9 +331,10 @@ __device__ __forceinline__ void tc_put_bf16(const TcGemmParams& p, int row0, int
     }
 }
 
-// This thread's 64 columns of one row.
-template <bool L2, bool CE, bool A1>
-__device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, uint4* stage) {
+// This thread's 64 columns of one row.  `release`: called once the accumulator has been read.
+template <bool L2, bool CE, bool A1, class Release>
+__device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, uint4* stage,
+                                                 Release release) {
     static_assert(TC_PIECE == 64, "two chunks of 32 columns per piece");
     const bool rin = row < p.M;
     const float rn = rs.rn, ref = rs.st.x;
@@ -354,13 +363,15 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
         for (int c = 0; c < TC_PIECE; c += 32) {
             float v[32];
             tmem_ld32(taddr + (uint32_t)c, v);
+            if (c + 32 == TC_PIECE) release();
             chunk(v, col_off + c);
         }
     } else {
         float v0[32], v1[32];
         tmem_ld32_issue(taddr, v0);            // both chunks are requested before the first is used
         tmem_ld32_issue(taddr + 32u, v1);
-        tmem_ld_wait();
+        tmem_ld_wait(v0); tmem_ld_wait(v1);
+        release();                             // the next item is multiplied under this one's arithmetic
         chunk(v0, col_off);
         chunk(v1, col_off + 32);
     }
@@ -426,16 +437,18 @@ __device__ __forceinline__ float float_below(float x) {
 
 // Epilogue of one warp on one item: WIDTH columns [col_off, col_off + WIDTH) of the tile row held by
 // this thread's tensor-memory lane (taddr points at the first of them).
-template <int EPI, int WIDTH>
-__device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, void* scratch) {
+template <int EPI, int WIDTH, class Release>
+__device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, void* scratch, Release release) {
     static_assert((EPI & 3) == EPI_STORE || WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) {
 #pragma unroll 1
         for (int c = 0; c < WIDTH; c += TC_PIECE) {
             uint4* stage = static_cast<uint4*>(scratch);
-            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
+            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage,
+                                                                                                                                    [&] { if (c + TC_PIECE == WIDTH) release(); });
             else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
         }
+        if ((EPI & 3) == EPI_GRAD) release();
         return;
     }
     float* const Cout = p.C + (int64_t)it.z * p.split_stride;
@@ -471,6 +484,7 @@ __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem&
             for (int i = 0; i < 32; ++i) if (ncol + i < p.N) dst[i] = v[i];
         }
     }
+    release();
 }
 
 // Work item = (K split, row tile, column tile), column tile fastest.  A CTA takes a contiguous
@@ -617,10 +631,11 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * GCOLS);
             // scratch after the barriers: 2 or 4 KB per epilogue warp for the stores of bf16 or fp32 tiles
             void* scratch = scratch_sm + (warp - 2) * ((EPI & 3) == EPI_STORE ? TC_STORE_STAGE_BYTES : TC_GRAD_STAGE_BYTES);
-            tc_epilogue<EPI, GCOLS>(p, it, it.m0 + quarter * 32 + lane, rs, cgrp * GCOLS, taddr, scratch);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            tc_epilogue<EPI, GCOLS>(p, it, it.m0 + quarter * 32 + lane, rs, cgrp * GCOLS, taddr, scratch, [&] {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            });
         }
     }
     tc_fence_before();
@@ -1015,14 +1030,17 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
 //
 // The queries stay and the entities pass by.  A CTA keeps MT tiles of 128 queries in shared memory and runs 256-entity tiles past them,
 // 64 coordinates (32 KB) at a time through a ring; each (query tile, entity tile) is one accumulator of 256 columns, two in
-// turn, and each accumulator has eight epilogue warps of its own (32 queries x 128 entities each).  What an epilogue needs of its
-// query (threshold, true tail's score, ids) and its rank count are then registers for hundreds of tiles.  With the entity tile kept and the
+// turn; the sixteen epilogue warps (32 queries x 64 entities each) take an accumulator into registers and hand it back before they
+// look at it, so that its next tile is multiplied meanwhile.  What an epilogue needs of its queries (threshold, true tail's
+// score and id) and its rank count are registers for hundreds of tiles.  With the entity tile kept and the
 // queries passing by, as before, every tile read them from L2 and added its counts to shared memory: 39.8 ms for 15,000 x
 // 8 M x 128, 3,000 cycles per 128 x 256 tile against the MMAs' 1,024, most of it latency.
 // MT = 2 for rows of at most 128 coordinates halves the entity bytes a SM reads per score (32 bytes a clock at the
 // MMAs' full rate); longer rows leave no room for the second tile's ring.
-// All CTAs walk the table one superblock of some 32 MB after the other, each through its own contiguous run of the superblock's (query
-// group, entity tile) pairs, query group slowest, so that the table is read from HBM once and a CTA changes queries rarely.
+// The table is to be read from HBM once.  Few query groups: as many CTAs for each, the CTAs of one entity range side by side.  Many:
+// all CTAs walk the table one superblock of some 32 MB after the other, each through its own contiguous run of the superblock's (query
+// group, entity tile) pairs, query group slowest, so that a CTA changes queries rarely.  (300 queries x 1 M x 320, three groups:
+// superblocks that give every CTA enough pairs are then larger than L2 and each group reads the table for itself, 399 us.)
 // ------------------------------------------------------------------------------------------
 constexpr int SCAN_BN = 256, SCAN_WARPS = 16, SCAN_THREADS = 32 * (2 + SCAN_WARPS), SCAN_RING_MAX = 8;
 constexpr uint32_t SCAN_SLICE_BYTES = SCAN_BN * TC_BK * 2;
@@ -1030,6 +1048,7 @@ constexpr size_t SCAN_SMEM_MAX = 227 * 1024;
 
 struct ScanParams {
     int M, N, slices, tiles_m, groups, tiles_n, sb_tiles, ring;     // groups of MT query tiles; tiles per superblock
+    int ctas_per_group;                   // 0: superblocks
     int64_t n_base, id_base;              // first table row of this launch; the caller's id of table row 0 (sharded inference)
     const float *thr, *ftrue;             // [M] current k-th best score; score of the true tail
     const int32_t *thr_id, *tt;           // [M] its id; true tail ids (or NULL)
@@ -1040,25 +1059,39 @@ struct ScanParams {
     int32_t* status; int wait_limit;
 };
 
-// Waits for this thread's outstanding tensor-memory loads; the registers pass through, so that nothing that uses them moves ahead.
-__device__ __forceinline__ void tmem_ld_wait(float (&v)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]),
-                   "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]),
-                   "+f"(v[21]), "+f"(v[22]), "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]),
-                   "+f"(v[31])::"memory");
-}
-
-// One query as its lane holds it.
+// One query as its lane holds it: k-th best score, score and id of the true tail, entities before it so far, and one candidate
+// (score, id) on its way to the query's list (no score: -inf).
 struct ScanRow {
-    float thr, thr_lo, ft, ft_lo;         // k-th best score, largest float below it; the same of the true tail's score
-    int32_t thr_id, tt, row;
-    int beat;
+    float thr, ft;
+    int32_t tt, beat;
+    float cand;
+    int32_t cand_id;
 };
+// Puts the lanes' candidates into their lists.  All lanes at once: one wait for the atomics.
+__device__ __forceinline__ void scan_flush(const ScanParams& p, ScanRow& r, int row) {
+    if (r.cand != -INFINITY) {
+        const int slot = atomicAdd(&p.cand_cnt[row], 1);
+        if (slot < p.cand_cap) {
+            p.cand_score[(int64_t)row * p.cand_cap + slot] = r.cand;
+            p.cand_id[(int64_t)row * p.cand_cap + slot] = r.cand_id;
+        } else {
+            *p.overflow = 1;   // the host redoes this chunk in shorter pieces
+        }
+        r.cand = -INFINITY;
+    }
+    __syncwarp();
+}
 
 // Calls f(query group, entity tile) for this CTA's pairs until it returns false.
 template <class F>
 __device__ __forceinline__ void scan_walk(const ScanParams& p, F f) {
+    if (p.ctas_per_group) {
+        const int g = blockIdx.x / p.ctas_per_group, c = blockIdx.x % p.ctas_per_group;
+        const int end = (int)((int64_t)p.tiles_n * (c + 1) / p.ctas_per_group);
+        for (int e = (int)((int64_t)p.tiles_n * c / p.ctas_per_group); e < end; ++e)
+            if (!f(g, e)) return;
+        return;
+    }
     for (int sb = 0; sb < p.tiles_n; sb += p.sb_tiles) {
         const int tiles = min(p.sb_tiles, p.tiles_n - sb);
         const int64_t pairs = (int64_t)p.groups * tiles;
@@ -1071,13 +1104,13 @@ __device__ __forceinline__ void scan_walk(const ScanParams& p, F f) {
     }
 }
 
-// 32 scores of one query against the entities [e0, e0 + 32) from tile column `ncol` on.  Within a run of entity ids that does not contain the
-// reference id, "ordered before (f0, id0)" is a plain comparison: f >= f0 if the run lies below id0, f > f0 if above; f >= f0
+// 32 scores of query `row` against the entities [e0, e0 + 32) from tile column `ncol` on.  Within a run of entity ids that does not contain
+// the reference id, "ordered before (f0, id0)" is a plain comparison: f >= f0 if the run lies below id0, f > f0 if above; f >= f0
 // is written f > (largest float below f0).  `cut`: that bound of the true tail, unless the true tail is among the warp's ids
 // (`exact`); n: the count so far, in floating point on four chains (exact, and the additions go to the FMA pipe).
 template <bool FIRST>
-__device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], ScanRow& r, int ncol, float cut, bool exact, float (&n)[4]) {
-    const int lane = threadIdx.x & 31, valid = p.N - ncol;             // the same for every lane
+__device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], ScanRow& r, int row, int ncol, float cut, bool exact, float (&n)[4]) {
+    const int valid = p.N - ncol;                                      // the same for every lane
     if (valid <= 0) return;
     const int32_t e0 = (int32_t)(p.n_base + p.id_base + ncol);
     if (valid < 32) {
@@ -1096,44 +1129,39 @@ __device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], 
             if (e != r.tt && (v[i] > r.ft || (v[i] == r.ft && e < r.tt))) ++r.beat;
         }
     }
-    if constexpr (FIRST) {               // (a chunk starts at a multiple of 32 columns: whole 128-byte pieces of the row's list)
-        if (r.row < p.M) {
-            float4* dst = reinterpret_cast<float4*>(p.cand_score + (int64_t)r.row * p.cand_cap + ncol);
+    if constexpr (FIRST) {     // (a chunk starts at a multiple of 32 columns: whole 128-byte pieces of the row's list)
+        if (row < p.M) {
+            float4* dst = reinterpret_cast<float4*>(p.cand_score + (int64_t)row * p.cand_cap + ncol);
 #pragma unroll
             for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
-        return;
     } else {
-    float vm[4];               // a tree of three-input maxima, not a chain of 31
+        float vm[4];           // a tree of three-input maxima, not a chain of 31
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-        vm[j] = max3(max3(v[8 * j], v[8 * j + 1], v[8 * j + 2]), max3(v[8 * j + 3], v[8 * j + 4], v[8 * j + 5]), fmaxf(v[8 * j + 6], v[8 * j + 7]));
-    const float vmax = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
-    // Rare once the threshold has tightened.  The warp takes the flagged lanes one at a time and spreads that lane's 32 scores over its
-    // 32 lanes (one shuffle per score): the ordering test and the append then run once per lane, not 32 times in a row.
-    unsigned pending = __ballot_sync(0xffffffffu, vmax > r.thr_lo);
-    while (pending) {
-        const int src = __ffs(pending) - 1;
-        pending &= pending - 1;
-        float f = 0.f;
+        for (int j = 0; j < 4; ++j)
+            vm[j] = max3(max3(v[8 * j], v[8 * j + 1], v[8 * j + 2]), max3(v[8 * j + 3], v[8 * j + 4], v[8 * j + 5]), fmaxf(v[8 * j + 6], v[8 * j + 7]));
+        const float vmax = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
+        // Rare once the threshold has tightened, but one warp of sixteen meets it at most tiles, and the tile waits for the slowest of
+        // them.  So nothing here waits for memory: a lane keeps its candidate until the query's next one comes, and then the warp
+        // hands all it holds to the lists (every candidate at once with an atomic of its own: 11.8 ms for 15,000 x 2 M x 128, the
+        // MMAs alone 6.0).
+        unsigned hits = 0u;
+        if (!__any_sync(0xffffffffu, vmax >= r.thr)) return;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float t = __shfl_sync(0xffffffffu, v[i], src);
-            if (lane == i) f = t;
-        }
-        const float thr_s = __shfl_sync(0xffffffffu, r.thr, src);
-        const int32_t id_s = __shfl_sync(0xffffffffu, r.thr_id, src), row_s = __shfl_sync(0xffffffffu, r.row, src);
-        const int32_t e = e0 + lane;
-        if (f > thr_s || (f == thr_s && e < id_s && f != -INFINITY)) {     // (padded columns hold -inf and never pass)
-            const int slot = atomicAdd(&p.cand_cnt[row_s], 1);
-            if (slot < p.cand_cap) {
-                p.cand_score[(int64_t)row_s * p.cand_cap + slot] = f;
-                p.cand_id[(int64_t)row_s * p.cand_cap + slot] = e;
-            } else {
-                *p.overflow = 1;   // the host redoes this chunk in shorter pieces
+        for (int i = 0; i < 32; ++i) if (v[i] >= r.thr) hits |= 1u << i;
+        if (valid < 32) hits &= (1u << valid) - 1u;
+        while (__any_sync(0xffffffffu, hits != 0u)) {
+            if (hits != 0u) {
+                const int at = __ffs(hits) - 1;
+                float f = v[0];
+#pragma unroll
+                for (int i = 1; i < 32; ++i) if (at == i) f = v[i];
+                // (the k-th best score itself: before it only with a smaller id)
+                if (f == r.thr && !(e0 + at < p.thr_id[row])) hits &= hits - 1u;
+                else if (r.cand == -INFINITY) { r.cand = f; r.cand_id = e0 + at; hits &= hits - 1u; }
             }
+            if (__any_sync(0xffffffffu, hits != 0u)) scan_flush(p, r, row);
         }
-    }
     }
 }
 
@@ -1146,7 +1174,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
     uint64_t* full = reinterpret_cast<uint64_t*>(slice0 + (size_t)p.ring * SCAN_SLICE_BYTES);
     uint64_t* empty = full + SCAN_RING_MAX;
     uint64_t* acc_full = empty + SCAN_RING_MAX;    // [2] accumulator written
-    uint64_t* acc_empty = acc_full + 2;            // [2] accumulator read by all eight of its warps
+    uint64_t* acc_empty = acc_full + 2;            // [2] accumulator read by all epilogue warps
     uint64_t* q_full = acc_empty + 2;              // query tiles loaded / no longer read by any MMA
     uint64_t* q_free = q_full + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_free + 1);
@@ -1156,7 +1184,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < SCAN_RING_MAX; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], SCAN_WARPS / 2); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], SCAN_WARPS); }
         mbar_init(q_full, 1); mbar_init(q_free, 1);
         *stop = 0;
         // after a list overflowed: no pairs (one thread's reading: the flag may change while this launch runs)
@@ -1248,56 +1276,67 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
             if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
         }
     } else {
-        const int acc = (warp - 2) >> 3, quarter = warp & 3, col0 = ((warp - 2) >> 2 & 1) * 128;   // (a warp reads the lanes of its own quarter only)
-        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * SCAN_BN + col0);
-        int cur = -1, used = 0, turn = 0;
-        ScanRow r{INFINITY, INFINITY, 0.f, 0.f, 0, -1, 0, 0};
-        auto hand_over = [&] { if (r.beat > 0) atomicAdd(&p.beat_tmp[r.row], r.beat); r.beat = 0; };
+        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * 64;            // (a warp reads the lanes of its own quarter only)
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
+        int cur = -1, turn = 0;
+        uint32_t parity = 0;                       // bit b: parity of accumulator b's next full phase
+        ScanRow rows[MT];
+#pragma unroll
+        for (int t = 0; t < MT; ++t) rows[t] = ScanRow{INFINITY, INFINITY, -1, 0, -INFINITY, 0};
+        auto row_of = [&](int g, int t) { return (g * MT + t) * TC_BM + quarter * 32 + lane; };
+        auto hand_over = [&] {
+#pragma unroll
+            for (int t = 0; t < MT; ++t) {
+                if (rows[t].beat > 0) atomicAdd(&p.beat_tmp[row_of(cur, t)], rows[t].beat);
+                scan_flush(p, rows[t], row_of(cur, t));
+            }
+        };
         bool ok = true;
         scan_walk(p, [&](int g, int e) {
-            if (MT == 1) { turn ^= 1; if ((turn ^ 1) != acc) return true; }
-            else if (g * MT + acc >= p.tiles_m) return true;
             if (g != cur) {
-                hand_over();
+                if (cur >= 0) hand_over();
                 cur = g;
-                r.row = (g * MT + (MT == 1 ? 0 : acc)) * TC_BM + quarter * 32 + lane;
-                // rows outside the problem stay in the loop (the warp votes need every lane): no true tail, a threshold nothing exceeds
-                r.thr = INFINITY; r.thr_id = 0; r.ft = INFINITY; r.tt = -1;
-                if (r.row < p.M) {
-                    r.thr = p.thr[r.row]; r.thr_id = p.thr_id[r.row];
-                    if (p.tt) { r.ft = p.ftrue[r.row]; r.tt = p.tt[r.row]; }
+#pragma unroll
+                for (int t = 0; t < MT; ++t) {
+                    // rows outside the problem stay in the loop (the warp votes need every lane): no true tail, a threshold nothing exceeds
+                    const int row = row_of(g, t);
+                    rows[t] = ScanRow{INFINITY, INFINITY, -1, 0, -INFINITY, 0};
+                    if (row < p.M) {
+                        rows[t].thr = p.thr[row];
+                        if (p.tt) { rows[t].ft = p.ftrue[row]; rows[t].tt = p.tt[row]; }
+                    }
                 }
-                r.thr_lo = float_below(r.thr); r.ft_lo = float_below(r.ft);
             }
             const int32_t id0 = (int32_t)(p.n_base + p.id_base + e * SCAN_BN + col0);
-            const bool exact = __any_sync(0xffffffffu, r.tt >= id0 && r.tt < id0 + 128);
-            const float cut = r.tt < 0 ? INFINITY : (r.tt >= id0 + 128 ? r.ft_lo : r.ft);
-            ok = mbar_wait_bounded(&acc_full[acc], used & 1, p.wait_limit);
-            ++used;
-            tc_fence_after();
-            if (!ok || *stop) { ok = false; return false; }
-            float n[4] = {0.f, 0.f, 0.f, 0.f};
-            float va[32], vb[32];                  // the next 32 columns are on their way while these are looked at
-            tmem_ld32_issue(taddr, va);
 #pragma unroll 1
-            for (int c = 0; c < 128; c += 64) {
-                tmem_ld_wait(va);
-                tmem_ld32_issue(taddr + (uint32_t)(c + 32), vb);
-                scan_chunk<FIRST>(p, va, r, e * SCAN_BN + col0 + c, cut, exact, n);
-                tmem_ld_wait(vb);
-                if (c == 0) tmem_ld32_issue(taddr + 64u, va);
-                else {                             // everything is in registers: the accumulator is free
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[acc]);
-                }
-                scan_chunk<FIRST>(p, vb, r, e * SCAN_BN + col0 + c + 32, cut, exact, n);
+            for (int t = 0; t < MT; ++t) {                 // (one copy of the code: the rows change places)
+                if (MT == 2) { const ScanRow x = rows[0]; rows[0] = rows[MT - 1]; rows[MT - 1] = x; }
+                if (g * MT + t >= p.tiles_m) continue;
+                ScanRow& r = rows[MT - 1];
+                const int acc = MT == 1 ? turn : t;
+                const bool exact = __any_sync(0xffffffffu, r.tt >= id0 && r.tt < id0 + 64);
+                const float cut = r.tt < 0 ? INFINITY : (r.tt >= id0 + 64 ? float_below(r.ft) : r.ft);
+                ok = mbar_wait_bounded(&acc_full[acc], parity >> acc & 1u, p.wait_limit);
+                parity ^= 1u << acc;
+                tc_fence_after();
+                if (!ok || *stop) { ok = false; return false; }
+                float va[32], vb[32];
+                tmem_ld32_issue(taddr + (uint32_t)(acc * SCAN_BN), va);
+                tmem_ld32_issue(taddr + (uint32_t)(acc * SCAN_BN + 32), vb);
+                tmem_ld_wait(va); tmem_ld_wait(vb);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[acc]);
+                float n[4] = {0.f, 0.f, 0.f, 0.f};
+                scan_chunk<FIRST>(p, va, r, row_of(g, t), e * SCAN_BN + col0, cut, exact, n);
+                scan_chunk<FIRST>(p, vb, r, row_of(g, t), e * SCAN_BN + col0 + 32, cut, exact, n);
+                r.beat += (int)((n[0] + n[1]) + (n[2] + n[3]));
             }
-            r.beat += (int)((n[0] + n[1]) + (n[2] + n[3]));
+            turn ^= 1;
             return true;
         });
         if (!ok && lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
-        hand_over();
+        if (cur >= 0) hand_over();
     }
     tc_fence_before();
     __syncthreads();
@@ -1694,7 +1733,11 @@ int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, con
     p.groups = (p.tiles_m + mt - 1) / mt;
     const size_t fixed = 1024 + 256 + (size_t)mt * p.slices * TC_A_BYTES;
     p.ring = (int)std::min<size_t>(SCAN_RING_MAX, (SCAN_SMEM_MAX - fixed) / SCAN_SLICE_BYTES);
-    const int grid = (int)std::min<int64_t>((int64_t)p.groups * p.tiles_n, h->num_sms);
+    int grid = (int)std::min<int64_t>((int64_t)p.groups * p.tiles_n, h->num_sms);
+    // CTAs of their own for every group where that leaves at most one in sixteen idle
+    const int per_group = std::min(h->num_sms / p.groups, p.tiles_n);
+    p.ctas_per_group = per_group > 0 && (per_group == p.tiles_n || per_group * p.groups * 16 >= h->num_sms * 15) ? per_group : 0;
+    if (p.ctas_per_group) grid = p.ctas_per_group * p.groups;
     // superblocks of about 32 MB, but at least 32 pairs per CTA in each
     const int64_t tile_bytes = (int64_t)SCAN_BN * h->cfg.dim * 2;
     const int64_t sb = std::max<int64_t>((int64_t)(32 << 20) / tile_bytes, ((int64_t)32 * grid + p.groups - 1) / p.groups);
