@@ -215,7 +215,7 @@ __device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64
 }
 
 // ------------------------------------------------------------------------------------------
-// Unions of at most ENS_REGS entities per thread.  A thread takes four places of one list at a time, whose first probes
+// Unions of at most R entities per thread.  A thread takes four places of one list at a time, whose first probes
 // are in flight together; what a lane has left over of its four is probed one step at a time by the whole warp, so that a
 // warp's rounds are those of its unluckiest lane's four and not of its unluckiest lane four times.  The table is sparse
 // (2,048 slots for 768 entities) for the same reason.  The sums stay in registers: entity i of the order of arrival belongs
@@ -223,14 +223,14 @@ __device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64
 // a lane reads its own: a random look-up in one copy would meet three others in its bank.  An entity twice in one list
 // loses one of its two bytes (position + 1), so that the bytes read add up to less than the bytes written.
 // ------------------------------------------------------------------------------------------
-constexpr int ENS_REGS = 3, ENS_COPIES = 8, ENS_CAND = 64, ENS_CUT_TOP = 16;
+constexpr int ENS_COPIES = 16, ENS_CAND = 64, ENS_CUT_TOP = 16;
 template <int MB>
 constexpr size_t ens_union_smem(int slots, int K) {
     return (size_t)(K + 1) * ENS_COPIES * sizeof(double) + (size_t)slots * (sizeof(int32_t) + MB) + (size_t)slots * sizeof(uint16_t);
 }
 
 // V: places of a list that lie on one boundary of a load (4, 2 or 1).  Returns 0, or (all threads) why the table was given up.
-template <int MB, int V>
+template <int MB, int V, int R>
 __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_slots, const int limit, unsigned char* smem) {
     constexpr int WORDS = MB / 4;
     const int slots = 1 << log2_slots, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, K = p.K;
@@ -239,9 +239,13 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
     uint32_t* cell = reinterpret_cast<uint32_t*>(key + slots);                  // [MB / 4][slots] bytes: position + 1 in the block's models
     uint16_t* used = reinterpret_cast<uint16_t*>(cell + (size_t)WORDS * slots);      // [slots] occupied slots, in order of arrival
     __shared__ int n_used, lost;
-    for (int i = tid; i < slots; i += nthr) key[i] = -1;
-    for (int i = tid; i < slots * WORDS; i += nthr) cell[i] = 0u;
-    for (int i = tid; i < (K + 1) * ENS_COPIES; i += nthr) tab[i] = p.table[i < ENS_COPIES ? K : i / ENS_COPIES - 1];
+    for (int i = tid; i < slots / 4; i += nthr) reinterpret_cast<int4*>(key)[i] = make_int4(-1, -1, -1, -1);
+    for (int i = tid; i < slots * WORDS / 4; i += nthr) reinterpret_cast<int4*>(cell)[i] = make_int4(0, 0, 0, 0);
+    for (int i = tid; i < (K + 1) * (ENS_COPIES / 2); i += nthr) {
+        const int j = i / (ENS_COPIES / 2);
+        const double x = p.table[j == 0 ? K : j - 1];
+        reinterpret_cast<double2*>(tab)[i] = make_double2(x, x);
+    }
     if (tid == 0) { n_used = 0; lost = 0; }
     const int quads = (K + 3) >> 2, per_block = min(MB, nthr / quads);           // quads of a list; models per block: a quad per thread
     const int ml = p.inv_quads ? (int)__umulhi((uint32_t)tid, p.inv_quads) : tid, pos = 4 * (tid - ml * quads);
@@ -269,10 +273,10 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
     __syncthreads();
     const double* mytab = tab + (lane & (ENS_COPIES - 1));
     const double absent = tab[0];
-    double before = 0.0, sum[ENS_REGS];     // before: an entity's sum over the models ahead of the block it first appears in
-    int slot[ENS_REGS];
+    double before = 0.0, sum[R];     // before: an entity's sum over the models ahead of the block it first appears in
+    int slot[R];
 #pragma unroll
-    for (int r = 0; r < ENS_REGS; ++r) { sum[r] = 0.0; slot[r] = 0; }
+    for (int r = 0; r < R; ++r) { sum[r] = 0.0; slot[r] = 0; }
     int seen = 0;                           // occupied slots after the blocks so far
     uint32_t bytes = 0;                     // positions written less positions read
     unsigned char* mycell = reinterpret_cast<unsigned char*>(cell + (size_t)(ml >> 2) * slots) + (ml & 3);
@@ -319,7 +323,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
         const int total = n_used;
         if (total > limit) return ENS_BAD_FULL;
 #pragma unroll
-        for (int r = 0; r < ENS_REGS; ++r) {
+        for (int r = 0; r < R; ++r) {
             const int i = r * nthr + tid;
             if (i >= total) break;
             if (i >= seen) { slot[r] = used[i]; sum[r] = before; }
@@ -346,11 +350,11 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
 
     // The best top_n.  Up to ENS_CUT_TOP: the top_n-th best of 32 groups' best scores (upper halves) is a bound that at least top_n
     // entities reach; those that do, hardly more, are ranked against one another.  Otherwise, and where too many reach it: a round per place.
-    uint64_t os[ENS_REGS];                  // ordered scores, 0: none or taken
-    int32_t id[ENS_REGS];
+    uint64_t os[R];                  // ordered scores, 0: none or taken
+    int32_t id[R];
     uint32_t top_hi = 0;
 #pragma unroll
-    for (int r = 0; r < ENS_REGS; ++r) {
+    for (int r = 0; r < R; ++r) {
         const bool in = r * nthr + tid < seen;
         os[r] = in ? ens_ordered(sum[r]) : 0ull;
         id[r] = in ? key[slot[r]] : INT32_MAX;
@@ -384,7 +388,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
         __syncthreads();
         const uint32_t c = cut;
 #pragma unroll
-        for (int r = 0; r < ENS_REGS; ++r)
+        for (int r = 0; r < R; ++r)
             if (os[r] != 0ull && (uint32_t)(os[r] >> 32) >= c) {
                 const int at = atomicAdd(&n_cand, 1);
                 if (at < ENS_CAND) { cand_s[at] = os[r]; cand_i[at] = id[r]; }
@@ -414,7 +418,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
     auto warp_best = [&] {
         uint64_t bs = 0; int32_t bi = INT32_MAX;
 #pragma unroll
-        for (int r = 0; r < ENS_REGS; ++r)
+        for (int r = 0; r < R; ++r)
             if (os[r] > bs || (os[r] == bs && id[r] < bi)) { bs = os[r]; bi = id[r]; }
         ens_warp_best(bs, bi, ws, wi);
     };
@@ -427,7 +431,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
         if (tid == 0) ens_put(p, q, r, s, e);
         if (s != 0ull && s == ws && e == wi) {                                  // taken (ids are distinct: one warp, one thread)
 #pragma unroll
-            for (int u = 0; u < ENS_REGS; ++u) if (id[u] == e) { os[u] = 0ull; id[u] = INT32_MAX; }
+            for (int u = 0; u < R; ++u) if (id[u] == e) { os[u] = 0ull; id[u] = INT32_MAX; }
             warp_best();
         }
     }
@@ -575,24 +579,26 @@ __global__ void __launch_bounds__(512) ensemble_sort_left_kernel(EnsParams p) {
 
 // Lists so short that a table of 1.5 slots per entry fits (M K <= 682): one launch, no table overflows, and a query with an
 // entity twice in one list is sorted where it stands (the sort needs no more memory than the table).
-constexpr int ENS_SMALL_MB = 16, ENS_SMALL_LOG2 = 10;
-template <int V>
-__global__ void __launch_bounds__(256) ensemble_small_kernel(EnsParams p) {
+// T threads (fewer where the lists need fewer).
+constexpr int ENS_SMALL_MB = 16, ENS_SMALL_LOG2 = 10, ENS_ENTITIES = 768;
+template <int V, int T>
+__global__ void __launch_bounds__(T) ensemble_small_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
-    if (!ens_union_query<ENS_SMALL_MB, V>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
+    if (!ens_union_query<ENS_SMALL_MB, V, ENS_ENTITIES / T>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
     __syncthreads();
     ens_sort_call<0>(p, blockIdx.x, ens_smem);
 }
 
-// Longer lists, first launch: one CTA of 256 threads per query.  A block of models is at most 256 quads, 1,024 places, so that with
-// ENS_LIMIT entities before it a slot is always free.
-constexpr int ENS_LOG2 = 11, ENS_LIMIT = 256 * ENS_REGS, ENS_MB = 12;
-static_assert(ENS_LIMIT + 1024 < 1 << ENS_LOG2, "a probe ends");
-template <int V>
-__global__ void __launch_bounds__(256) ensemble_hash_kernel(EnsParams p) {
+// Longer lists, first launch: one CTA of T threads per query.  A block of models is at most T quads, 1,024 places, so that with
+// ENS_ENTITIES entities before it a slot is always free.  Lists of more than 64 places fill 256 threads with eight models, shorter
+// ones with sixteen, those of up to 32 places 128 threads.
+constexpr int ENS_LOG2 = 11;
+static_assert(ENS_ENTITIES + 1024 < 1 << ENS_LOG2, "a probe ends");
+template <int MB, int V, int T>
+__global__ void __launch_bounds__(T) ensemble_hash_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
     allow_dependents();
-    const int bad = ens_union_query<ENS_MB, V>(p, blockIdx.x, ENS_LOG2, ENS_LIMIT, ens_smem);
+    const int bad = ens_union_query<MB, V, ENS_ENTITIES / T>(p, blockIdx.x, ENS_LOG2, ENS_ENTITIES, ens_smem);
     if (bad && threadIdx.x == 0) p.out_ids[(int64_t)blockIdx.x * p.top_n] = bad == ENS_BAD_TWICE ? ENS_SORT : ENS_LEFT;
 }
 
@@ -680,9 +686,13 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
         constexpr int sort_max = (int)(ENS_MAX_ENTRIES * (sizeof(uint64_t) + sizeof(int32_t)));
         static_assert(parts_smem <= sort_max, "the larger table fits where the sort does");
         cudaError_t e0 = cudaSuccess;
-        constexpr int union_max = (int)std::max(ens_union_smem<ENS_MB>(1 << ENS_LOG2, ENS_MAX_K), ens_union_smem<ENS_SMALL_MB>(1 << ENS_SMALL_LOG2, ENS_MAX_K));
-        for (void (*k)(EnsParams) : {ensemble_small_kernel<1>, ensemble_small_kernel<2>, ensemble_small_kernel<4>,
-                                     ensemble_hash_kernel<1>, ensemble_hash_kernel<2>, ensemble_hash_kernel<4>})
+        constexpr int union_max = (int)std::max(std::max(ens_union_smem<8>(1 << ENS_LOG2, ENS_MAX_K), ens_union_smem<16>(1 << ENS_LOG2, 64)),
+                                                ens_union_smem<ENS_SMALL_MB>(1 << ENS_SMALL_LOG2, ENS_MAX_K));
+        for (void (*k)(EnsParams) : {ensemble_small_kernel<1, 128>, ensemble_small_kernel<2, 128>, ensemble_small_kernel<4, 128>,
+                                     ensemble_small_kernel<1, 256>, ensemble_small_kernel<2, 256>, ensemble_small_kernel<4, 256>,
+                                     ensemble_hash_kernel<8, 1, 256>, ensemble_hash_kernel<8, 2, 256>, ensemble_hash_kernel<8, 4, 256>,
+                                     ensemble_hash_kernel<16, 1, 256>, ensemble_hash_kernel<16, 2, 256>, ensemble_hash_kernel<16, 4, 256>,
+                                     ensemble_hash_kernel<16, 1, 128>, ensemble_hash_kernel<16, 2, 128>, ensemble_hash_kernel<16, 4, 128>})
             if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, union_max);
         for (void (*k)(EnsParams) : {ensemble_sort_kernel<256>, ensemble_sort_kernel<512>, ensemble_sort_kernel<ENS_THREADS>, ensemble_sort_left_kernel,
                                      ensemble_left_kernel<256>, ensemble_left_kernel<512>, ensemble_left_kernel<ENS_THREADS>})
@@ -706,12 +716,15 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
     p.log2_slots = 5;
     while (2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
     if (p.log2_slots <= ENS_SMALL_LOG2) {
-        const int threads = p.log2_slots >= 9 ? 256 : (p.log2_slots >= 7 ? 128 : 64);
-        pick(ensemble_small_kernel<4>, ensemble_small_kernel<2>, ensemble_small_kernel<1>)
-            <<<nq, threads, std::max(ens_union_smem<ENS_SMALL_MB>(1 << p.log2_slots, k_list), sort_smem), s>>>(p);
+        const int threads = p.log2_slots >= 9 ? (k_list <= 32 ? 128 : 256) : (p.log2_slots >= 7 && k_list > 32 ? 128 : 64);
+        const size_t smem = std::max(ens_union_smem<ENS_SMALL_MB>(1 << p.log2_slots, k_list), sort_smem);
+        if (threads <= 128) pick(ensemble_small_kernel<4, 128>, ensemble_small_kernel<2, 128>, ensemble_small_kernel<1, 128>)<<<nq, threads, smem, s>>>(p);
+        else pick(ensemble_small_kernel<4, 256>, ensemble_small_kernel<2, 256>, ensemble_small_kernel<1, 256>)<<<nq, threads, smem, s>>>(p);
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
-    pick(ensemble_hash_kernel<4>, ensemble_hash_kernel<2>, ensemble_hash_kernel<1>)<<<nq, 256, ens_union_smem<ENS_MB>(1 << ENS_LOG2, k_list), s>>>(p);
+    if (k_list > 64) pick(ensemble_hash_kernel<8, 4, 256>, ensemble_hash_kernel<8, 2, 256>, ensemble_hash_kernel<8, 1, 256>)<<<nq, 256, ens_union_smem<8>(1 << ENS_LOG2, k_list), s>>>(p);
+    else if (k_list > 32) pick(ensemble_hash_kernel<16, 4, 256>, ensemble_hash_kernel<16, 2, 256>, ensemble_hash_kernel<16, 1, 256>)<<<nq, 256, ens_union_smem<16>(1 << ENS_LOG2, k_list), s>>>(p);
+    else pick(ensemble_hash_kernel<16, 4, 128>, ensemble_hash_kernel<16, 2, 128>, ensemble_hash_kernel<16, 1, 128>)<<<nq, 128, ens_union_smem<16>(1 << ENS_LOG2, k_list), s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return KGE_ERR_CUDA;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;
