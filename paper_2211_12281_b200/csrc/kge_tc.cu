@@ -200,11 +200,12 @@ __device__ __forceinline__ float tc_score(const TcGemmParams& p, float acc, floa
 // Per-row inputs of an epilogue, read before the accumulator is waited for.
 struct TcRowState {
     float rn;                 // squared norm of the row (norm expansion)
+    float cn[2];              // EPI_LOSS, norm expansion: squared norms of this lane's column of each of the warp's chunks of 32
     float2 st;                // EPI_LOSS: the row's (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser)
 };
 template <int EPI>
 __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int row) {
-    TcRowState r{0.f, make_float2(0.f, 0.f)};
+    TcRowState r{0.f, {}, make_float2(0.f, 0.f)};
     if (row >= p.M) return r;
     if ((EPI & EPI_L2) != 0) r.rn = p.row_norm2[row];
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) r.st = p.row_stat[row];
@@ -216,8 +217,8 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
 // base-2 exponent (a f log2 e for the self-adversarial weights, (f + c) log2 e for the sampled softmax) and u the rest
 // (sigmoid(gamma + f), the reciprocal distance), and the factor loss_scale / Z joins afterwards: dQ's rows are multiplied by
 // it, and dT's contraction takes q_b times it as its operand (both see as many roundings to bf16 as with the factor in E).
-// bf16 and fp32 share their exponent range, so any reference within it serves: `ref` is the largest y among eight of the row's
-// negatives (the gather kernel computes them), a lower bound of the maximum up to rounding.  A chunk of 32 scores that exceeds it
+// bf16 and fp32 share their exponent range, so any reference within it serves: `ref` is the larger y of two of the row's
+// negatives (the gather kernel computes them), a lower bound of the maximum up to rounding and a constant.  A chunk of 32 scores that exceeds it
 // by more than 2^TC_REF_SPAN takes its own maximum instead, which keeps the statistics in range, and the row is found by
 // stats_combine_kernel and its E written again, over the true maximum and with the factor, by an EPI_GRAD launch that
 // otherwise ends at once.  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
@@ -225,7 +226,8 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
 constexpr float TC_REF_SPAN = 80.f;
 
 // One chunk of 32 scores.  FULL: all 32 columns lie inside the problem (no per-element masking); otherwise the first `valid`
-// do.  k0: the exponent's constant less the reference.  Returns what was subtracted beyond the reference.
+// do.  k0: the exponent's constant less the reference; cn: the columns' squared norms (shared memory, norm expansion).  Returns what was
+// subtracted beyond the reference.
 // A1 (distance scores f <= 0, log-sigmoid loss, temperature a = 1): with K = exp(gamma) 2^ref, exp(gamma + f) = K e =: t, so
 // softplus(gamma + f) = log(1 + t) and sigmoid(gamma + f) = t / (1 + t): four special-function instructions per score
 // (distance, exponential, logarithm, reciprocal).
@@ -233,23 +235,10 @@ constexpr float TC_REF_SPAN = 80.f;
 // is looked for only in a warp that holds such a row; the other scores' maximum is a tree of three-input maxima.
 template <bool L2, bool CE, bool FULL, bool A1>
 __device__ __forceinline__ float tc_loss_chunk(const TcGemmParams& p, const float (&v)[32], float rn, int ncol, int valid,
-                                               float k1, float k0, float ref, bool low, float& z, float& l, uint32_t (&g2)[16]) {
-    float cn[32];
-    if (L2) {
-        if (FULL) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const float4 c = __ldg(reinterpret_cast<const float4*>(p.col_norm2 + ncol) + i);
-                cn[4 * i] = rn + c.x; cn[4 * i + 1] = rn + c.y; cn[4 * i + 2] = rn + c.z; cn[4 * i + 3] = rn + c.w;
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) cn[i] = i < valid ? rn + __ldg(p.col_norm2 + ncol + i) : 1.f;
-        }
-    }
+                                               float k1, float k0, float ref, bool low, const float* cn, float& z, float& l, uint32_t (&g2)[16]) {
     auto score = [&](int i, float& inv) {
         if (!L2) { inv = 0.f; return v[i]; }
-        const float s2 = fmaxf(fmaf(-2.f, v[i], cn[i]), 0.f);
+        const float s2 = fmaxf(fmaf(-2.f, v[i], rn + cn[i]), 0.f);
         inv = s2 > 0.f ? fast_rsqrt(s2) : 0.f;
         return -s2 * inv;
     };
@@ -343,19 +332,22 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
     const uint32_t rows = __ballot_sync(0xffffffffu, rin);
     const int row0 = row - (int)(threadIdx.x & 31);
     float m = ref, z = 0.f, l = 0.f;
-    auto chunk = [&](const float (&v)[32], int c0) {
+    auto chunk = [&](const float (&v)[32], int c0, float cnorm) {
         const int ncol = it.n0 + c0, valid = min(32, p.N - ncol);             // (the same for every lane; may be <= 0)
         if (valid <= 0) return;
+        const float* cn = reinterpret_cast<const float*>(stage);
+        if (L2) { reinterpret_cast<float*>(stage)[threadIdx.x & 31] = cnorm; __syncwarp(); }
         uint32_t g2[16];
         float cz, cl = 0.f, shift;
-        if (valid == 32) shift = tc_loss_chunk<L2, CE, true, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cz, cl, g2);
-        else shift = tc_loss_chunk<L2, CE, false, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cz, cl, g2);
+        if (valid == 32) shift = tc_loss_chunk<L2, CE, true, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cn, cz, cl, g2);
+        else shift = tc_loss_chunk<L2, CE, false, A1>(p, v, rn, ncol, valid, k1, k0, ref, low, cn, cz, cl, g2);
         const float cm = ref + shift;
         if (cm == m) { z += cz; l += cl; }
         else {
             const float mm = fmaxf(m, cm), ra = fast_exp2(m - mm), rb = fast_exp2(cm - mm);
             z = z * ra + cz * rb; l = l * ra + cl * rb; m = mm;
         }
+        if (L2) __syncwarp();
         tc_put_bf16(p, row0, ncol, valid, rows, g2, stage);
     };
     if (L2) {                                  // (both chunks at once spill here)
@@ -364,7 +356,7 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
             float v[32];
             tmem_ld32(taddr + (uint32_t)c, v);
             if (c + 32 == TC_PIECE) release();
-            chunk(v, col_off + c);
+            chunk(v, col_off + c, c == 0 ? rs.cn[0] : rs.cn[1]);
         }
     } else {
         float v0[32], v1[32];
@@ -372,8 +364,8 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
         tmem_ld32_issue(taddr + 32u, v1);
         tmem_ld_wait(v0); tmem_ld_wait(v1);
         release();                             // the next item is multiplied under this one's arithmetic
-        chunk(v0, col_off);
-        chunk(v1, col_off + 32);
+        chunk(v0, col_off, 0.f);
+        chunk(v1, col_off + 32, 0.f);
     }
     const int piece = (it.n0 + col_off) / TC_PIECE;
     if (rin && piece < p.row_pieces) p.stat_part[(int64_t)row * p.row_pieces + piece] = make_float4(m, z, l, 0.f);
@@ -439,13 +431,12 @@ __device__ __forceinline__ float float_below(float x) {
 // this thread's tensor-memory lane (taddr points at the first of them).
 template <int EPI, int WIDTH, class Release>
 __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, void* scratch, Release release) {
-    static_assert((EPI & 3) == EPI_STORE || WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
+    static_assert((EPI & 3) == EPI_STORE || (EPI & 3) == EPI_LOSS ? (EPI & 3) == EPI_STORE || WIDTH == TC_PIECE : WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) {
 #pragma unroll 1
         for (int c = 0; c < WIDTH; c += TC_PIECE) {
             uint4* stage = static_cast<uint4*>(scratch);
-            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage,
-                                                                                                                                    [&] { if (c + TC_PIECE == WIDTH) release(); });
+            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage, release);
             else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
         }
         if ((EPI & 3) == EPI_GRAD) release();
@@ -510,11 +501,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     constexpr int NACC = 512 / BN;                      // fp32 accumulators in tensor memory, used in turn: all 512 columns
     constexpr uint32_t TC_TMEM_COLS = NACC * BN;
     constexpr int EW = tc_epi_warps(EPI, BN), EG = EW / 4, TC_THREADS = tc_threads(EPI, BN);
-    // In the loss pass of the norm-expansion kinds (bound by special-function instructions, with row- and
-    // column-dependent loads) the epilogue warps form two groups that take the CTA's items in turn, so the epilogues
-    // of consecutive items overlap; every other pass was measured slower or equal that way and stays one group.
-    constexpr int EGRP = ((EPI & EPI_L2) != 0 && (EPI & 3) == EPI_LOSS && EG % 2 == 0) ? 2 : 1;
-    constexpr int GW = EW / EGRP, GCOLS = BN / (GW / 4);       // warps per group; columns per warp
+    constexpr int GCOLS = BN / EG;                      // columns per epilogue warp
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* base = tc_smem_raw + ((1024u - (smem_u32(tc_smem_raw) & 1023u)) & 1023u);
     uint64_t* full = reinterpret_cast<uint64_t*>(base + (size_t)TC_STAGES * TC_STAGE_BYTES);
@@ -537,7 +524,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], GW); }
+        for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EW); }
         *stop = 0;
         mbar_init_fence();
     }
@@ -614,16 +601,19 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
         }
     } else {
         const int quarter = warp & 3;                  // tensor-memory lanes this warp may read
-        const int egrp = (warp - 2) / GW;              // which items
-        const int cgrp = ((warp - 2) % GW) >> 2;       // which group of the tile's columns
-        TcItem it = tc_item(p, min(item_begin + egrp, p.items - 1));
-        for (int item = item_begin + egrp, local = egrp; item < item_end; item += EGRP, local += EGRP) {
-            if (local != egrp) {
-#pragma unroll
-                for (int g = 0; g < EGRP; ++g) tc_item_next(p, it);
-            }
+        const int cgrp = (warp - 2) >> 2;              // which group of the tile's columns
+        TcItem it = tc_item(p, item_begin);
+        for (int item = item_begin, local = 0; item < item_end; ++item, ++local) {
+            if (local != 0) tc_item_next(p, it);
             // what the epilogue needs of its row does not depend on the accumulator: fetched before the wait
-            const TcRowState rs = tc_row_state<EPI>(p, it.m0 + quarter * 32 + lane);
+            TcRowState rs = tc_row_state<EPI>(p, it.m0 + quarter * 32 + lane);
+            if ((EPI & EPI_L2) != 0 && (EPI & 3) == EPI_LOSS) {
+#pragma unroll
+                for (int i = 0; i < GCOLS / 32; ++i) {
+                    const int col = it.n0 + cgrp * GCOLS + 32 * i + lane;
+                    rs.cn[i] = col < p.N ? __ldg(p.col_norm2 + col) : 1.f;
+                }
+            }
             const int buf = local % NACC;
             const bool ok = mbar_wait_bounded(&acc_full[buf], (local / NACC) & 1, p.wait_limit);
             tc_fence_after();
@@ -1424,7 +1414,8 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     bool good = true;
     for (int j = lane; j < p.pieces; j += 32) { const float x = row[j].x; m = fmaxf(m, x); good = good && x == ref; }
     m = warp_max(m);
-    if (ce) m = fmaxf(m, fp * kLog2e);
+    good = __all_sync(0xffffffffu, good);
+    if (ce && !good) m = fmaxf(m, fp * kLog2e);        // (a good row's reference is within 2^1 of it or above)
     float z = 0.f, l = 0.f;
     for (int j = lane; j < p.pieces; j += 32) {
         const float4 s = row[j];
@@ -1433,7 +1424,7 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     }
     z = warp_sum(z); l = warp_sum(l);
     if (ce) z += exp2f(fp * kLog2e - m);
-    good = __all_sync(0xffffffffu, good) && m == ref && z >= 1e-30f && z < INFINITY;
+    good = good && z >= 1e-30f && z < INFINITY;
     const float scale = good ? p.loss_scale / z : 1.f;
     if (good)
         for (int c = lane; c < p.d4; c += 32) {

@@ -85,7 +85,8 @@ __device__ __forceinline__ float pair_partial(int kind, float4 q, float4 t) {
     return f4dot(x, x);
 }
 
-template <int kMaxChunks>   // float4 slices per lane: a warp owns a row
+// TC: operands and row references of the tensor-core path.
+template <int kMaxChunks, bool TC>   // float4 slices per lane: a warp owns a row
 __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
     extern __shared__ uint64_t bucket_wcum[];   // fused sampling: cumulative weights of this CTA's buckets
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -114,17 +115,35 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
             float4 v = src[c];
             if (pj) v = f4add(v, pj[c]);       // e = e_S + M_T e_F
             dst[c] = v;
-            if (p.w.Tb) {   // tensor-core scoring: bf16 copy and the squared norm of the unrounded row
+            if (TC) {       // tensor-core scoring: bf16 copy and the squared norm of the unrounded row
                 reinterpret_cast<uint2*>(p.w.Tb)[(int64_t)n * d4 + c] = pack_bf16x4(v);
                 nrm2 += f4dot(v, v);
             }
             if (p.w.reg_s3) s3 += f4cube(v);
         }
-        if (p.w.Tb) { nrm2 = warp_sum(nrm2); if (lane == 0) p.w.tn2[n] = nrm2; }
+        if (TC) { nrm2 = warp_sum(nrm2); if (lane == 0) p.w.tn2[n] = nrm2; }
         if (p.w.reg_s3) { s3 = warp_sum(s3); if (lane == 0) p.w.reg_s3[2 * p.B + n] = s3; }
         return;
     }
     const int b = warp;
+    // tensor cores: the rows of two of the negatives.  The row's reference is the larger exponent of theirs (and of the positive, which
+    // the sampled softmax sums too); fetched first, since nothing of the positive is needed for it
+    float4 ref_row[2][kMaxChunks];
+    if (TC) {
+        const int slot = (lane & 1) ? p.N / 2 : 0;
+        const int32_t mine = p.fused_sample ? sample_negative(p.sp, slot) : p.negs[slot];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int64_t id = checked_id(__shfl_sync(0xffffffffu, mine, j), p.E, p.w.status);
+            const float4* src = reinterpret_cast<const float4*>(p.ent) + id * d4;
+#pragma unroll
+            for (int i = 0; i < kMaxChunks; ++i) {
+                const int c = lane + 32 * i;
+                ref_row[j][i] = c < d4 ? src[c] : f4zero();
+                if (p.proj && c < d4) ref_row[j][i] = f4add(ref_row[j][i], reinterpret_cast<const float4*>(p.proj)[(int64_t)(2 * p.B + (j ? p.N / 2 : 0)) * d4 + c]);
+            }
+        }
+    }
     int32_t ih, ir, it;
     if (p.fused_sample) {
         if (lane == 0) {
@@ -214,7 +233,7 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
     float4* qdst = reinterpret_cast<float4*>(p.w.Q) + (int64_t)b * d4;
 #pragma unroll
     for (int i = 0; i < kMaxChunks; ++i) { const int c = lane + 32 * i; if (c < d4) qdst[c] = q[i]; }
-    if (p.w.Qb) {
+    if (TC) {
         float nrm2 = 0.f;
 #pragma unroll
         for (int i = 0; i < kMaxChunks; ++i) {
@@ -251,47 +270,27 @@ __global__ void __launch_bounds__(256) build_kernel(TrainParams p) {
         else if (p.kind == KIND_L2 || p.kind == KIND_TH_L2) f = -sqrtf(acc);
         p.w.fpos[b] = f;
     }
-    if (p.w.row_stat) {
-        // tensor cores: the row's reference, the largest exponent among eight of its negatives (and the positive, which the
-        // sampled softmax sums too)
-        constexpr int SAMPLES = 8;
-        const int slot = (int)((int64_t)(lane & (SAMPLES - 1)) * p.N / SAMPLES);
-        const int32_t mine = p.fused_sample ? sample_negative(p.sp, slot) : p.negs[slot];
-        float part[SAMPLES];
+    if (TC) {
+        // the two sums side by side: the first exchange leaves each lane one of them
+        float part[2] = {0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < SAMPLES; ++j) {
-            const int64_t id = checked_id(__shfl_sync(0xffffffffu, mine, j), p.E, p.w.status);
-            const int n = __shfl_sync(0xffffffffu, slot, j);
-            part[j] = 0.f;
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-            for (int i = 0; i < kMaxChunks; ++i) {
-                const int c = lane + 32 * i;
-                if (c >= d4) continue;
-                float4 v = reinterpret_cast<const float4*>(p.ent)[id * d4 + c];
-                if (p.proj) v = f4add(v, reinterpret_cast<const float4*>(p.proj)[(int64_t)(2 * p.B + n) * d4 + c]);
-                part[j] += pair_partial(p.kind, q[i], v);
-            }
-        }
-        // the eight sums side by side: every exchange halves the sums a lane carries
+            for (int i = 0; i < kMaxChunks; ++i)
+                if (lane + 32 * i < d4) part[j] += pair_partial(p.kind, q[i], ref_row[j][i]);
+        const bool odd = (lane & 1) != 0;
+        float f = (odd ? part[1] : part[0]) + __shfl_xor_sync(0xffffffffu, odd ? part[0] : part[1], 1);
 #pragma unroll
-        for (int half = SAMPLES / 2; half >= 1; half >>= 1) {
-            const bool upper = (lane & half) != 0;
-#pragma unroll
-            for (int j = 0; j < half; ++j) {
-                const float send = upper ? part[j] : part[j + half], keep = upper ? part[j + half] : part[j];
-                part[j] = keep + __shfl_xor_sync(0xffffffffu, send, half);
-            }
-        }
-        float f = part[0];
-        f += __shfl_xor_sync(0xffffffffu, f, 8);
-        f += __shfl_xor_sync(0xffffffffu, f, 16);
-        if (p.kind == KIND_L2) f = -sqrtf(f);
+        for (int o = 2; o < 32; o <<= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+        if (p.kind == KIND_L2) { f = -sqrtf(f); acc = -sqrtf(acc); }
         const bool ce = p.loss == KGE_LOSS_SAMPLED_SOFTMAX;
         constexpr float kLog2e = 1.4426950408889634f;
-        float y = warp_max(fmaf(f, ce ? kLog2e : p.adv_temp * kLog2e, ce ? p.ce_c * kLog2e : 0.f));
-        if (ce) y = fmaxf(y, __shfl_sync(0xffffffffu, p.kind == KIND_L2 ? -sqrtf(acc) : acc, 0) * kLog2e);
+        float y = fmaf(f, ce ? kLog2e : p.adv_temp * kLog2e, ce ? p.ce_c * kLog2e : 0.f);
+        y = fmaxf(y, __shfl_xor_sync(0xffffffffu, y, 1));
+        if (ce) y = fmaxf(y, acc * kLog2e);
         if (lane == 0) {
-            reinterpret_cast<float2*>(p.w.row_stat)[b] = make_float2(fmaxf(y, -1e30f), 0.f);
+            // (dL/dF's values lie near the reference where scores hardly differ: at 1.75 times a power of two a bf16 is rounded half as far as just above one)
+            reinterpret_cast<float2*>(p.w.row_stat)[b] = make_float2(fmaxf(y, -1e30f) - 0.8073549f, 0.f);
             if (b == 0) p.w.status[TC_REDO_FLAG] = 0;
         }
     }
@@ -1308,9 +1307,10 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     {
         const int grid = (row_warps * 32 + 255) / 256;
         const size_t smem = fused_sample ? (size_t)fused_sample_smem(c.num_relations, p.slots_per_bucket) : 0;
-        if (nch == 1) KGE_CUDA_CHECK(h, launch_dependent(build_kernel<1>, dim3(grid), dim3(256), smem, s, p));
-        else if (nch == 2) KGE_CUDA_CHECK(h, launch_dependent(build_kernel<2>, dim3(grid), dim3(256), smem, s, p));
-        else KGE_CUDA_CHECK(h, launch_dependent(build_kernel<4>, dim3(grid), dim3(256), smem, s, p));
+        const bool tc = c.prec == KGE_PREC_BF16_TC;
+        auto kernel = nch == 1 ? (tc ? build_kernel<1, true> : build_kernel<1, false>)
+                               : (nch == 2 ? (tc ? build_kernel<2, true> : build_kernel<2, false>) : (tc ? build_kernel<4, true> : build_kernel<4, false>));
+        KGE_CUDA_CHECK(h, launch_dependent(kernel, dim3(grid), dim3(256), smem, s, p));
     }
     stage_end(h, ST_BUILD, s);
     KGE_LAUNCH_CHECK(h);
