@@ -25,8 +25,6 @@ struct TrainParams {
     int fused_sample;   // the gather kernel draws the batch itself (ids land in sp.heads ...) instead of reading it
     int slots_per_bucket;
     SampleParams sp;
-    int tc;             // tensor-core backward: dQ's splits lack the row's factor Grow
-    int tc_l2;          // TransE p = 2 on it: the splits hold C.T and C^T.Q, C = dL/dF / distance, and Cpart / xsum_q the sums of C
     int neg_direct;     // the dT contraction wrote the negatives' gradient rows itself (one K split, no correction term)
     int wait_limit;     // tries of a bounded barrier wait
     const float* proj;  // feature-projection encoder: [2B+N, d] M e_F of the slots [heads | tails | negs], added to the rows read; or NULL
@@ -1003,9 +1001,12 @@ __device__ __forceinline__ float sum_splits(const float* first, int64_t stride, 
     return s;
 }
 
-template <int kMaxChunks>
+// TC: behind the tensor-core contractions (dQ's splits lack the row's factor Grow; TransE p = 2: the splits hold C.T and C^T.Q,
+// C = dL/dF / distance, and Cpart / xsum_q the sums of C).
+template <int kMaxChunks, bool TC>
 __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     const int lane = threadIdx.x & 31;
+    const bool tc_l2 = TC && p.kind == KIND_L2;
     grid_dependency_wait();
     allow_dependents();
     if (blockIdx.x == gridDim.x - 1) {   // the extra last CTA adds up the batch loss
@@ -1041,12 +1042,12 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
         const int n = warp - p.B;
         const float4* part = reinterpret_cast<const float4*>(p.w.dTpart);
         float wsum = 0.f;   // column sum of dL/dF.  TransE p = 1: the splits hold P, the gradient is 2 P - (column sum)
-        if (p.kind == KIND_L1 || p.tc_l2) wsum = sum_splits(p.w.Cpart + n, p.N, p.split_t);
+        if (p.kind == KIND_L1 || tc_l2) wsum = sum_splits(p.w.Cpart + n, p.N, p.split_t);
         const float creg = p.w.reg_s3 ? reg_coef(p.reg_lambda, p.reg_form, p.w.reg_s3[2 * p.B + n]) : 0.f;
         for (int c = lane; c < d4; c += 32) {
             float4 s = sum_splits(part + (int64_t)n * d4 + c, (int64_t)p.N * d4, p.split_t + p.th_slabs);
             if (p.kind == KIND_L1) s = make_float4(2.f * s.x - wsum, 2.f * s.y - wsum, 2.f * s.z - wsum, 2.f * s.w - wsum);
-            if (p.tc_l2) {   // dT_n = sum_b C_bn (q_b - t_n) = (C^T Q)_n - (column sum of C) t_n
+            if (tc_l2) {   // dT_n = sum_b C_bn (q_b - t_n) = (C^T Q)_n - (column sum of C) t_n
                 const float cs = wsum;
                 const float4 t = reinterpret_cast<const float4*>(p.w.Tneg)[(int64_t)n * d4 + c];
                 s = make_float4(s.x - cs * t.x, s.y - cs * t.y, s.z - cs * t.z, s.w - cs * t.w);
@@ -1064,8 +1065,8 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
     const float4* trow = reinterpret_cast<const float4*>(p.ent) + tid * d4;
     const float4* qrow = reinterpret_cast<const float4*>(p.w.Q) + (int64_t)b * d4;
     const float gp = p.w.gpos[b], fp = p.w.fpos[b];
-    const float factor = p.tc ? p.w.Grow[b] : 1.f;
-    const float xrow = p.tc_l2 ? factor * sum_splits(p.w.xsum_q + b, p.B, p.split_q) : 0.f;
+    const float factor = TC ? p.w.Grow[b] : 1.f;
+    const float xrow = tc_l2 ? factor * sum_splits(p.w.xsum_q + b, p.B, p.split_q) : 0.f;
 
     float4 h[kMaxChunks], t[kMaxChunks], q[kMaxChunks], dq[kMaxChunks], dt[kMaxChunks];
 #pragma unroll
@@ -1083,8 +1084,8 @@ __global__ void __launch_bounds__(256) chain_kernel(TrainParams p) {
             const float rs = p.w.Grow[b];
             s = make_float4(rs - 2.f * s.x, rs - 2.f * s.y, rs - 2.f * s.z, rs - 2.f * s.w);
         }
-        if (p.tc) s = f4scale(factor, s);
-        if (p.tc_l2 && in) {             // dQ_b = sum_n C_bn (t_n - q_b) = (C T)_b - (row sum of C) q_b
+        if (TC) s = f4scale(factor, s);
+        if (tc_l2 && in) {             // dQ_b = sum_n C_bn (t_n - q_b) = (C T)_b - (row sum of C) q_b
             const float rs = xrow;
             s = make_float4(s.x - rs * q[i].x, s.y - rs * q[i].y, s.z - rs * q[i].z, s.w - rs * q[i].w);
         }
@@ -1293,8 +1294,6 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     p.sp = make_sample_params(h, step);
     p.sp.heads = h->ws.heads; p.sp.rels = h->ws.rels; p.sp.tails = h->ws.tails; p.sp.negs = h->ws.negs;
     p.slots_per_bucket = c.batch / (c.head_part < 0 ? c.num_parts * c.num_parts : c.num_parts);
-    p.tc = c.prec == KGE_PREC_BF16_TC;
-    p.tc_l2 = p.tc && p.kind == KIND_L2;
     p.neg_direct = tc_negatives_direct(h) ? 1 : 0;
     p.wait_limit = h->wait_limit;
     p.reg_lambda = c.reg_lambda; p.reg_form = c.reg_form;
@@ -1408,9 +1407,10 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
     stage_begin(h, ST_CHAIN, s);
     {
         const int grid = ((p.neg_direct ? p.B : row_warps) * 32 + 255) / 256 + 1;
-        if (nch == 1) KGE_CUDA_CHECK(h, launch_dependent(chain_kernel<1>, dim3(grid), dim3(256), 0, s, p));
-        else if (nch == 2) KGE_CUDA_CHECK(h, launch_dependent(chain_kernel<2>, dim3(grid), dim3(256), 0, s, p));
-        else KGE_CUDA_CHECK(h, launch_dependent(chain_kernel<4>, dim3(grid), dim3(256), 0, s, p));
+        const bool tc = c.prec == KGE_PREC_BF16_TC;
+        auto kernel = nch == 1 ? (tc ? chain_kernel<1, true> : chain_kernel<1, false>)
+                               : (nch == 2 ? (tc ? chain_kernel<2, true> : chain_kernel<2, false>) : (tc ? chain_kernel<4, true> : chain_kernel<4, false>));
+        KGE_CUDA_CHECK(h, launch_dependent(kernel, dim3(grid), dim3(256), 0, s, p));
     }
     stage_end(h, ST_CHAIN, s);
     KGE_LAUNCH_CHECK(h);
