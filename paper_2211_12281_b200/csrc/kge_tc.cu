@@ -1140,6 +1140,10 @@ __device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], 
 #pragma unroll
         for (int i = 0; i < 32; ++i) if (v[i] >= r.thr) hits |= 1u << i;
         if (valid < 32) hits &= (1u << valid) - 1u;
+        if (vmax == r.thr) {                       // only ties with the k-th best: before it with a smaller id
+            const int before = p.thr_id[row] - e0;
+            hits &= before >= 32 ? ~0u : (before <= 0 ? 0u : (1u << before) - 1u);
+        }
         while (__any_sync(0xffffffffu, hits != 0u)) {
             if (hits != 0u) {
                 const int at = __ffs(hits) - 1;

@@ -164,3 +164,27 @@ def test_ensemble_of_three_scoring_functions_at_top_100(oracle32, oracle64):
     ids, sc = _gpu_ensemble(lists, -0.5, 10)
     o_ids, o_sc = oracle64.ensemble_topk(lists, -0.5, 10)
     assert (ids == o_ids).all() and (sc == o_sc).all()
+
+
+# one, two and four places per load (list length and the address of the lists), 64, 128 and 256 threads, eight and sixteen models
+# at a time with a remainder, the last number of places that is cut by groups and the first that is not
+@pytest.mark.parametrize("M,K,shift", [(25, 30, 0), (25, 31, 0), (24, 32, 0), (24, 32, 1), (24, 32, 2), (24, 33, 0), (12, 64, 0), (13, 65, 0), (13, 68, 2), (90, 12, 0), (17, 101, 0), (4, 7, 0)])
+@pytest.mark.parametrize("power,top_n", [(-0.5, 16), (0.5, 17)])
+def test_ensemble_places_per_load(oracle64, M, K, shift, power, top_n):
+    import torch
+    import paper_2211_12281_b200 as lib
+    rng = np.random.default_rng(100 * M + K)
+    nq, E = 33, max(3 * K, 40)
+    names = rng.permutation(np.unique(rng.integers(0, 1 << 30, 2 * E)))[:E]
+    lists = np.stack([np.stack([names[rng.permutation(E)[:K]] for _ in range(nq)]) for _ in range(M)]).astype(np.int32)
+    lists[0, :, K - 1] = -1
+    dev = torch.device("cuda:0")
+    flat = torch.zeros(lists.size + shift, dtype=torch.int32, device=dev)
+    view = flat[shift:].view(M, nq, K)
+    view.copy_(torch.from_numpy(lists))
+    table = torch.from_numpy(lib.ensemble_rank_scores(power, K)).to(dev)
+    ids = torch.full((nq, top_n), -7, dtype=torch.int32, device=dev)
+    sc = torch.zeros((nq, top_n), dtype=torch.float64, device=dev)
+    assert lib.ensemble_topk(view, table, top_n, ids, sc) == 0
+    o_ids, o_sc = oracle64.ensemble_topk(lists, power, top_n)
+    assert (ids.cpu().numpy() == o_ids).all() and (sc.cpu().numpy() == o_sc).all()

@@ -262,3 +262,40 @@ def test_a_rise_after_a_restart(oracle32, score, tc, d):
     ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
     o_ids, o_sc, o_ranks = oracle32.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K, true_tails=tt)
     assert (ids == o_ids).all() and (ranks == o_ranks).all() and (sc == o_sc).all()
+
+
+# tensor cores: one, two and three tiles of 128 queries (two side by side for rows of up to 128 coordinates, else one), a table that ends
+# inside and at the end of a 256-entity tile, CTAs of their own for every query group and shared ones, lists that take many candidates
+@pytest.mark.parametrize("nq,E,d,K", [(1, 3001, 64, 10), (128, 4352, 128, 40), (129, 6000, 128, 1), (257, 9000, 64, 100), (385, 6001, 192, 10), (130, 20000, 384, 40),
+                                      (2900, 5000, 64, 10), (300, 1500, 512, 5)])
+def test_tensor_core_query_groups(oracle64, nq, E, d, K):
+    import kge_synth
+    prob = Problem(E=E, R=9, T=100, d=d, score="distmult", B=8, N=8, P=1, graph_seed=47, tc=True)
+    qh, qr, tt = kge_synth.make_queries(E, 9, nq, seed=47)
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    r_ids, r_sc, r_ranks = oracle64.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh, qr, K + 5, true_tails=tt)
+    for q in range(nq):
+        assert len(set(ids[q])) == K
+        for e in set(ids[q]) - set(r_ids[q, :K]):          # (near ties only: the sums' order differs)
+            assert e in set(r_ids[q])
+            f = r_sc[q][list(r_ids[q]).index(e)]
+            assert abs(f - r_sc[q, K - 1]) <= 1e-4 * abs(f) + 1e-6
+    assert_close(sc, r_sc[:, :K], atol=1e-5, what="scores")
+    assert np.abs(ranks - r_ranks).max() <= 2
+    t = gpu.torch                                          # without true tails: the same lists
+    ids2 = t.empty((nq, K), dtype=t.int32, device=gpu.ent.device); sc2 = t.empty((nq, K), dtype=t.float32, device=gpu.ent.device)
+    gpu.kge.score_all_topk(gpu.dev_i32(qh), gpu.dev_i32(qr), K, None, ids2, sc2)
+    assert (ids2.cpu().numpy() == ids).all() and (sc2.cpu().numpy() == sc).all()
+
+
+def test_tensor_core_lists_of_equal_scores(oracle64):
+    """Every entity the same row: all scores of a query are equal, and the smallest ids win without filling a candidate list."""
+    import kge_synth
+    E, nq, K = 40000, 140, 10
+    prob = Problem(E=E, R=9, T=100, d=64, score="distmult", B=8, N=8, P=1, graph_seed=49, tc=True)
+    prob.ent[:] = prob.ent[0]
+    qh, qr, tt = kge_synth.make_queries(E, 9, nq, seed=49)
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, _, _ = _infer(gpu, qh, qr, tt, K)
+    assert (ids == np.arange(K)).all()

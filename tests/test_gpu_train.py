@@ -596,3 +596,56 @@ def test_a_workspace_without_room_for_the_one_pass_backward(oracle64, score, p, 
     gpu.kge.graph_load(prob.h, prob.r, prob.t)
     orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
     _check_step(gpu, orc, 0, orc.sample(0))
+
+
+# tensor cores, norm expansion: 64-column groups of the contractions from one to seven (the extra column of the sums beside them),
+# batches at the edges of a tile, more than one K split
+@pytest.mark.parametrize("d,B,N", [(64, 1, 1), (128, 129, 65), (128, 64, 2600), (256, 130, 127), (320, 20, 1030), (384, 128, 256), (448, 40, 200)])
+@pytest.mark.parametrize("loss", ["logsigmoid", "softmax"])
+def test_tensor_core_distance_row_widths(oracle64, d, B, N, loss):
+    prob = Problem(E=4000, R=7, T=9000, d=d, score="transe", p_norm=2, loss=loss, B=B, N=N, P=1, gamma=4.0, adv_temp=0.5,
+                   ce_correction=0.3, lr=0.05, graph_seed=41, tc=True)
+    _run(oracle64, prob, steps=1)
+
+
+# Rows whose scores reach far beyond (dot products) or lie far below (distances) what their reference negatives suggest: dL/dF
+# of these rows takes the second round, the others of the same batch do not.  Scores of +-150 whose fp32 sums differ in the last bits
+# move an exponential by some 2e-5, which the losses (fp32 tolerance, cancelling against the positive score) and dL/dF (2^-8) allow;
+# taps of the distances are compared at the positions that the bf16 norm expansion resolves.
+@pytest.mark.parametrize("score,loss,scale", [("distmult", "softmax", 46.0), ("distmult", "logsigmoid", 46.0), ("complex", "softmax", 40.0),
+                                              ("transe", "softmax", 160.0)])
+def test_tensor_core_rows_that_leave_their_reference(oracle64, score, loss, scale):
+    prob = Problem(E=4000, R=7, T=9000, d=64, score=score, p_norm=2 if score == "transe" else 1, loss=loss, B=150, N=700, P=1, gamma=0.0,
+                   adv_temp=1.0, lr=1e-4, graph_seed=43, tc=True)
+    prob.ent *= np.float32(scale)
+    if score == "transe":
+        prob.rel *= np.float32(scale)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    batch = orc.sample(0)
+    want = orc.o.batch_loss(orc.cfg, orc.ent, orc.rel, orc.relw, *batch)
+    ref = np.maximum(want["F"][:, 0], want["F"][:, prob.N // 2])
+    if loss == "softmax":
+        ref = np.maximum(ref, want["fpos"])
+    beyond = want["F"].max(axis=1) - ref
+    assert (beyond > 56).any() and (beyond < 54).any()                 # (the span is 2^80 = exp(55.5))
+    g = orc.grads(batch)
+    gpu.kge.train_step(0, prob.lr)
+    assert gpu.kge.get_status() == 0
+    assert_close(gpu.kge.debug_export("LROW"), want["Lrow"], rtol=1e-4, atol=1e-3, what="losses")
+    ge = gpu.kge.debug_export("GRAD_ENT").reshape(2 * prob.B + prob.N, prob.d)
+    for got, exact, what in ((ge[:prob.B], g["dh"], "dh"), (ge[2 * prob.B:], g["dtneg"], "dtneg")):
+        assert_close(got, exact, atol=1e-2 * np.abs(exact).max(), what=what)
+
+
+# lists of more than 1,024 ids: the last tile one id long, full, and one short; an odd and an even number of tiles; one id everywhere
+@pytest.mark.parametrize("B,N,E", [(500, 25, 400), (600, 848, 5000), (600, 847, 3), (900, 1273, 50000), (1500, 1097, 1), (1024, 2048, 200)])
+def test_touched_ids_over_several_tiles(oracle64, B, N, E):
+    prob = Problem(E=E, R=3, T=9000, d=32, score="distmult", B=B, N=N, P=1, lr=1e-3, graph_seed=45)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    batch = orc.sample(0)
+    gpu.kge.train_step(0, prob.lr)
+    for pre, lst in (("ENT", np.concatenate([batch[0], batch[2], batch[3]])), ("REL", batch[1])):
+        uniq, seg, perm = orc.o.dedup(lst)
+        assert (gpu.kge.debug_export(pre + "_UNIQ") == uniq).all()
+        assert (gpu.kge.debug_export(pre + "_SEG") == seg).all()
+        assert (gpu.kge.debug_export(pre + "_PERM") == perm).all()
