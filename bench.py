@@ -134,10 +134,9 @@ def transh_on_tensor_cores(w):
     """The library's automatic choice (config field `contract` = 0) for TransH with fp32 arithmetic."""
     return w["score"] == "transh" and not w.get("tc") and w["d"] % 32 == 0 and w["B"] * w["N"] >= 1 << 22
 
-# Special-function instructions per score of the fused tensor-core epilogues (exponential, logarithm, reciprocal, reciprocal
+# Special-function instructions per score of the fused tensor-core epilogue (exponentials, logarithm, reciprocal, reciprocal
 # square root: one instruction each).
-TC_SFU_PER_SCORE = {("softmax", False): dict(block=1, loss=1), ("logsigmoid", False): dict(block=3, loss=3),
-                    ("softmax", True): dict(block=2, loss=2), ("logsigmoid", True): dict(block=4, loss=4)}
+TC_SFU_PER_SCORE = {("softmax", False): 1, ("logsigmoid", False): 4, ("softmax", True): 2, ("logsigmoid", True): 5}
 
 
 def cfg_kwargs(w, seed):
@@ -533,18 +532,18 @@ def bench_training(ctx, name, w, cpu_seconds):
     elements = float(B) * N * d
     roofs = {}                                                           # stage -> (roofline us, bound, detail)
     if w.get("tc"):
-        # each of the four tensor-core launches is one B x N x d contraction: 2 B N d flops, bf16 operands, fp32 accumulation.
-        # "block" is the statistics pass and "loss" the merge kernel plus the gradient pass; their epilogues also issue
-        # special-function instructions per score, and the larger of the two times is the pass's roof.
+        # each of the three contractions is B x N x d: 2 B N d flops, bf16 operands, fp32 accumulation.
+        # "block" is the pass over the scores (loss statistics and dL/dF); its epilogue also issues special-function
+        # instructions per score, and the larger of the two times is the pass's roof.  ("loss", the rows' merge, has none.)
         sfu = TC_SFU_PER_SCORE[(w["loss"], w["score"] == "transe")]
         if w["loss"] == "logsigmoid" and w["score"] == "transe" and w.get("adv_temp") == 1.0 and w.get("gamma", 0.0) <= 80.0:
-            sfu = dict(block=3, loss=3)      # temperature 1: the weight and the loss term share one exponential
-        for st in ("block", "loss", "accum_q", "accum_t", "accum"):
+            sfu = 4                          # temperature 1: the weight and the loss term share one exponential
+        for st in ("block", "accum_q", "accum_t", "accum"):
             if st not in per_stage_us:
                 continue
             # ("accum": both backward contractions in one launch)
             t_tc = (2 if st == "accum" else 1) * 2.0 * elements / (ctx.peaks["bf16_tflops"] * 1e12) * 1e6
-            t_sf = sfu.get(st, 0) * float(B) * N / ctx.alu[MIX_SFU] * 1e6
+            t_sf = (sfu if st == "block" else 0) * float(B) * N / ctx.alu[MIX_SFU] * 1e6
             roofs[st] = (max(t_tc, t_sf), "tensor" if t_tc >= t_sf else "sfu", {"t_tensor_us": t_tc, "t_sfu_us": t_sf})
     else:
         for st, o in ops.items():
