@@ -1140,7 +1140,10 @@ __device__ __forceinline__ void scan_chunk(const ScanParams& p, float (&v)[32], 
 #pragma unroll
         for (int i = 0; i < 32; ++i) if (v[i] >= r.thr) hits |= 1u << i;
         if (valid < 32) hits &= (1u << valid) - 1u;
-        if (vmax == r.thr) {                       // only ties with the k-th best: before it with a smaller id
+        // (the tensor map covers every query that fits the workspace: the scores of a row outside the call come from whatever an
+        // earlier call left there, and no finite or infinite threshold is above +inf)
+        if (row >= p.M) hits = 0u;
+        else if (vmax == r.thr) {                  // only ties with the k-th best: before it with a smaller id
             const int before = p.thr_id[row] - e0;
             hits &= before >= 32 ? ~0u : (before <= 0 ? 0u : (1u << before) - 1u);
         }
@@ -1292,7 +1295,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
                 cur = g;
 #pragma unroll
                 for (int t = 0; t < MT; ++t) {
-                    // rows outside the problem stay in the loop (the warp votes need every lane): no true tail, a threshold nothing exceeds
+                    // rows outside the problem stay in the loop (the warp votes need every lane): no true tail, a threshold that only +inf reaches
                     const int row = row_of(g, t);
                     rows[t] = ScanRow{INFINITY, INFINITY, -1, 0, -INFINITY, 0};
                     if (row < p.M) {

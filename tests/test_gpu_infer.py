@@ -299,3 +299,24 @@ def test_tensor_core_lists_of_equal_scores(oracle64):
     gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
     ids, _, _ = _infer(gpu, qh, qr, tt, K)
     assert (ids == np.arange(K)).all()
+
+
+@pytest.mark.parametrize("d", [64, 192])
+def test_tensor_core_queries_outside_the_call_score_infinity(d):
+    """A call with fewer queries than the workspace holds, where the rest of the query vectors' memory makes every score +inf and the
+    rest of the thresholds' ids lie beyond the table: nothing of it reaches the call, which ends and gives what a call with as
+    many queries as the workspace holds gives."""
+    import kge_synth
+    E, R, K, nq, most = 9000, 5, 10, 130, 400
+    prob = Problem(E=E, R=R, T=100, d=d, score="distmult", B=8, N=8, P=1, graph_seed=51, tc=True)
+    prob.ent = np.abs(prob.ent)                                # (no +inf - inf among the sums)
+    qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=51)
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    want = _infer(gpu, qh, qr, tt, K)
+    t = gpu.torch
+    need = gpu.kge.workspace_bytes(0, most, K)
+    space = t.full((need + 512,), 0x7F, dtype=t.uint8, device=gpu.ent.device)
+    space[::2] = 0x80                                          # 0x7F80: +inf as bf16, 0x7F807F80 as an id
+    gpu.kge.bind(gpu.ent, gpu.rel, None, max_queries=most, topk=K, workspace=space[(-space.data_ptr()) % 256:][:need])
+    for got, exact in zip(_infer(gpu, qh, qr, tt, K), want):
+        assert (got == exact).all()
