@@ -120,6 +120,23 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// A CTA that gives up may not leave copies into its shared memory, or MMAs on its tensor memory, behind: these waits are bounded by
+// the default limit even where a test has shortened the kernel's own.  (At the end of a launch that went well both are done.)
+// The last copies into each of `stages` stages, of `issued` in all.
+__device__ __forceinline__ void tc_settle_copies(uint64_t* full, int stages, int issued) {
+    for (int r = max(0, issued - stages); r < issued; ++r) mbar_wait_idle(&full[r % stages], (r / stages) & 1, kDefaultWaitLimit);
+}
+// Every MMA this thread has issued; `done` is a barrier of its own.
+__device__ __forceinline__ void tc_settle_mmas(uint64_t* done) {
+    umma_commit(done);
+    mbar_wait_idle(done, 0, kDefaultWaitLimit);
+}
+// An epilogue warp's wait for an accumulator, with one answer for all its lanes: false if it ran out or another warp gave up.
+__device__ __forceinline__ bool tc_acc_ready(uint64_t* bar, uint32_t parity, int limit, volatile uint32_t* stop) {
+    const bool ok = mbar_wait_bounded(bar, parity, limit) && !*stop;
+    return __all_sync(0xffffffffu, ok);
+}
+
 // 32 consecutive fp32 columns of this thread's tensor-memory lane.
 // (the registers are valid after tmem_ld_wait)
 __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, float (&v)[32]) {
@@ -508,7 +525,8 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     uint64_t* empty = full + TC_STAGES;
     uint64_t* acc_full = empty + TC_STAGES;    // [NACC] accumulator buffer written
     uint64_t* acc_empty = acc_full + NACC;       // [NACC] accumulator buffer drained by all epilogue warps
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + NACC);
+    uint64_t* done = acc_empty + NACC;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* stop = tmem_slot + 1;     // set by a warp whose wait ran out
     unsigned char* scratch_sm = base + (size_t)TC_STAGES * TC_STAGE_BYTES + 256;
 
@@ -525,6 +543,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EW); }
+        mbar_init(done, 1);
         *stop = 0;
         mbar_init_fence();
     }
@@ -569,6 +588,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                         tma_load_2d(sb + g * (128 * TC_BK * 2), &tmB, k0, it.n0 + 128 * g, &full[s]);
                 }
             }
+            tc_settle_copies(full, TC_STAGES, ring);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -598,6 +618,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                 umma_commit(&acc_full[buf]);           // also after a failed wait, so the epilogue warps wake up
             }
             if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+            tc_settle_mmas(done);
         }
     } else {
         const int quarter = warp & 3;                  // tensor-memory lanes this warp may read
@@ -615,9 +636,9 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
                 }
             }
             const int buf = local % NACC;
-            const bool ok = mbar_wait_bounded(&acc_full[buf], (local / NACC) & 1, p.wait_limit);
+            const bool ok = tc_acc_ready(&acc_full[buf], (local / NACC) & 1, p.wait_limit, stop);
             tc_fence_after();
-            if (!ok || *stop) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
+            if (!ok) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * GCOLS);
             // scratch after the barriers: 2 or 4 KB per epilogue warp for the stores of bf16 or fp32 tiles
             void* scratch = scratch_sm + (warp - 2) * ((EPI & 3) == EPI_STORE ? TC_STORE_STAGE_BYTES : TC_GRAD_STAGE_BYTES);
@@ -689,7 +710,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     uint64_t* empty = full + TC_STAGES;
     uint64_t* acc_full = empty + TC_STAGES;
     uint64_t* acc_empty = acc_full + NACC;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + NACC);
+    uint64_t* done = acc_empty + NACC;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* stop = tmem_slot + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -713,6 +735,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], EW); }
+        mbar_init(done, 1);
         *stop = 0;
         mbar_init_fence();
     }
@@ -768,6 +791,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                     }
                 }
             }
+            tc_settle_copies(full, STAGES, ring);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -806,6 +830,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
                 umma_commit(&acc_full[buf]);           // also after a failed wait, so the epilogue warps wake up
             }
             if (!ok) { *stop = 1; set_status(status, KGE_ERR_TIMEOUT); }
+            tc_settle_mmas(done);
         }
     } else {
         const int quarter = warp & 3;                  // tensor-memory lanes this warp may read
@@ -814,9 +839,9 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_dual_kerne
         float4* st = reinterpret_cast<float4*>(base + (size_t)STAGES * STAGE_BYTES + 256) + (size_t)(warp - 2) * (TC_STORE_STAGE_BYTES / 16);
         for (int item = blockIdx.x, local = 0; item < total; item += gridDim.x, ++local) {
             const int buf = local % NACC;
-            const bool ok = mbar_wait_bounded(&acc_full[buf], (local / NACC) & 1, wait_limit);
+            const bool ok = tc_acc_ready(&acc_full[buf], (local / NACC) & 1, wait_limit, stop);
             tc_fence_after();
-            if (!ok || *stop) { if (lane == 0) { *stop = 1; set_status(status, KGE_ERR_TIMEOUT); } break; }
+            if (!ok) { if (lane == 0) { *stop = 1; set_status(status, KGE_ERR_TIMEOUT); } break; }
             const int which = prob_of(item);
             const DualProb q = which ? q1 : q0;
             const TcItem it = item_of(q, which ? item - q0.items : item);
@@ -895,7 +920,8 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
     uint64_t* empty = full + TT_STAGES;
     uint64_t* acc_full = empty + TT_STAGES;
     uint64_t* acc_empty = acc_full + NACC;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + NACC);
+    uint64_t* done = acc_empty + NACC;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* stop = tmem_slot + 1;
     float4* store_stage = reinterpret_cast<float4*>(base + (size_t)TT_STAGES * TT_STAGE_BYTES + 256);
 
@@ -903,6 +929,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
     if (threadIdx.x == 0) {
         for (int s = 0; s < TT_STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < NACC; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], TC_EPI_WARPS); }
+        mbar_init(done, 1);
         *stop = 0;
         mbar_init_fence();
     }
@@ -932,6 +959,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
                     }
                 }
             }
+            tc_settle_copies(full, TT_STAGES, ring);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -966,6 +994,7 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
                 umma_commit(&acc_full[buf]);           // also after a failed wait, so the epilogue warps wake up
             }
             if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+            tc_settle_mmas(done);
         }
     } else {
         const int quarter = warp & 3;                  // tensor-memory lanes this warp may read
@@ -974,9 +1003,9 @@ __global__ void __launch_bounds__(32 * (2 + TC_EPI_WARPS), 1) tc_gemm_terms_kern
         float4* st = store_stage + (size_t)(warp - 2) * (TC_STORE_STAGE_BYTES / 16);
         for (int item = blockIdx.x, local = 0; item < p.items; item += gridDim.x, ++local) {
             const int buf = local % NACC;
-            const bool ok = mbar_wait_bounded(&acc_full[buf], (local / NACC) & 1, p.wait_limit);
+            const bool ok = tc_acc_ready(&acc_full[buf], (local / NACC) & 1, p.wait_limit, stop);
             tc_fence_after();
-            if (!ok || *stop) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
+            if (!ok) { if (lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); } break; }
             const int m0 = (item / p.tiles_n) * TC_BM, n0 = (item % p.tiles_n) * BN;
             const int row0 = m0 + quarter * 32, row = row0 + lane;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + cgrp * COLS);
@@ -1174,7 +1203,8 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
     uint64_t* acc_empty = acc_full + 2;            // [2] accumulator read by all epilogue warps
     uint64_t* q_full = acc_empty + 2;              // query tiles loaded / no longer read by any MMA
     uint64_t* q_free = q_full + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_free + 1);
+    uint64_t* done = q_free + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile uint32_t* stop = tmem_slot + 1;       // set by a warp whose wait ran out
     volatile uint32_t* given_up = tmem_slot + 2;
 
@@ -1182,7 +1212,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
     if (threadIdx.x == 0) {
         for (int s = 0; s < SCAN_RING_MAX; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], SCAN_WARPS); }
-        mbar_init(q_full, 1); mbar_init(q_free, 1);
+        mbar_init(q_full, 1); mbar_init(q_free, 1); mbar_init(done, 1);
         *stop = 0;
         // after a list overflowed: no pairs (one thread's reading: the flag may change while this launch runs)
         *given_up = *reinterpret_cast<volatile int32_t*>(p.overflow) != 0;
@@ -1201,7 +1231,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
     if (idle) {
     } else if (warp == 0) {
         if (lane == 0) {
-            int ring = 0, phase = 1, cur = -1, changes = 0;
+            int ring = 0, phase = 1, cur = -1, changes = 0, fills = 0;
             bool ok = true;
             scan_walk(p, [&](int g, int e) {
                 if (*stop) return false;
@@ -1223,10 +1253,13 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
                     for (int h = 0; h < 2; ++h)
                         tma_load_2d(dst + h * (128 * TC_BK * 2), &tmB, kb * TC_BK, (int)p.n_base + e * SCAN_BN + 128 * h, &full[ring]);
                     if (++ring == p.ring) { ring = 0; phase ^= 1; }
+                    ++fills;
                 }
                 return true;
             });
             if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+            tc_settle_copies(full, p.ring, fills);
+            if (changes > 0) mbar_wait_idle(q_full, (changes - 1) & 1, kDefaultWaitLimit);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -1271,6 +1304,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
                 return true;
             });
             if (!ok) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
+            tc_settle_mmas(done);
         }
     } else {
         const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * 64;            // (a warp reads the lanes of its own quarter only)
@@ -1313,10 +1347,10 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
                 const int acc = MT == 1 ? turn : t;
                 const bool exact = __any_sync(0xffffffffu, r.tt >= id0 && r.tt < id0 + 64);
                 const float cut = r.tt < 0 ? INFINITY : (r.tt >= id0 + 64 ? float_below(r.ft) : r.ft);
-                ok = mbar_wait_bounded(&acc_full[acc], parity >> acc & 1u, p.wait_limit);
+                ok = tc_acc_ready(&acc_full[acc], parity >> acc & 1u, p.wait_limit, stop);
                 parity ^= 1u << acc;
                 tc_fence_after();
-                if (!ok || *stop) { ok = false; return false; }
+                if (!ok) return false;
                 float va[32], vb[32];
                 tmem_ld32_issue(taddr + (uint32_t)(acc * SCAN_BN), va);
                 tmem_ld32_issue(taddr + (uint32_t)(acc * SCAN_BN + 32), vb);

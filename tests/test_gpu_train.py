@@ -242,6 +242,27 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(oracle64):
     assert gpu.kge.get_status() == 0
 
 
+@pytest.mark.parametrize("score,p,B,N", [("transe", 2, 2048, 2500), ("distmult", 1, 300, 700)])
+def test_tensor_core_waits_that_run_out_leave_the_context_usable(oracle64, score, p, B, N):
+    """Limits so short that a wait runs out anywhere in the loss pass or the contractions: the step reports KGE_ERR_TIMEOUT (or got by),
+    and the next step on the same handle, with the tables as they were, is right."""
+    prob = Problem(E=3000, R=7, T=20000, d=128, score=score, p_norm=p, B=B, N=N, P=1, gamma=6.0, adv_temp=1.0, lr=0.05, tc=True)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    ran_out = 0
+    for tries in (1, 1, 1, 1, 2, 4, 8, 16, 64):
+        gpu.kge.debug_set_wait_limit(tries)
+        gpu.kge.train_step(0, prob.lr)
+        status = gpu.kge.get_status()
+        assert status in (0, -11)
+        ran_out += status != 0
+    assert ran_out
+    gpu.kge.debug_set_wait_limit(0)
+    gpu.ent.copy_(gpu.torch.from_numpy(prob.ent)); gpu.rel.copy_(gpu.torch.from_numpy(prob.rel))
+    orc._pre = (orc.ent.copy(), orc.rel.copy(), None)
+    _check_step(gpu, orc, 0, orc.sample(0), taps=True)
+    assert gpu.kge.get_status() == 0
+
+
 @pytest.mark.parametrize("score,p,form,tc", [("transe", 1, 0, False), ("distmult", 1, 1, False), ("transh", 2, 0, False),
                                              ("rotate", 1, 1, False), ("complex", 1, 0, True), ("transe", 2, 1, True)])
 def test_l3_regulariser(oracle64, score, p, form, tc):
