@@ -1366,8 +1366,9 @@ __global__ void __launch_bounds__(SCAN_THREADS, 1) tc_scan_kernel(const __grid_c
             turn ^= 1;
             return true;
         });
+        // (after a wait that ran out the call has failed, and `rows` may be in the order of the other tile: nothing of them is handed over)
+        if (ok && cur >= 0) hand_over();
         if (!ok && lane == 0) { *stop = 1; set_status(p.status, KGE_ERR_TIMEOUT); }
-        if (cur >= 0) hand_over();
     }
     tc_fence_before();
     __syncthreads();

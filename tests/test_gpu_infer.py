@@ -320,3 +320,30 @@ def test_tensor_core_queries_outside_the_call_score_infinity(d):
     gpu.kge.bind(gpu.ent, gpu.rel, None, max_queries=most, topk=K, workspace=space[(-space.data_ptr()) % 256:][:need])
     for got, exact in zip(_infer(gpu, qh, qr, tt, K), want):
         assert (got == exact).all()
+
+
+# an odd number of query tiles where two share a CTA, for which the last group has one; as many queries as the workspace holds, so
+# that what lies behind the lists is the workspace's next array
+@pytest.mark.parametrize("nq,d", [(300, 128), (128, 64), (290, 192)])
+def test_tensor_core_scoring_after_waits_that_run_out(nq, d):
+    """Limits so short that a wait runs out anywhere in the scoring: the call reports KGE_ERR_TIMEOUT (or got by), and the next
+    one, which uses the same copy of the table, gives what it gave before."""
+    import kge_synth
+    E, R, K = 60_000, 5, 10
+    prob = Problem(E=E, R=R, T=100, d=d, score="distmult", B=8, N=8, P=1, graph_seed=53, tc=True)
+    qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=53)
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    want = _infer(gpu, qh, qr, tt, K)
+    t = gpu.torch
+    out = [t.empty((nq, K), dtype=t.int32, device=gpu.ent.device), t.empty((nq, K), device=gpu.ent.device), t.empty(nq, dtype=t.int32, device=gpu.ent.device)]
+    ran_out = 0
+    for tries in (1, 1, 1, 1, 2, 4, 8, 16, 64):
+        gpu.kge.debug_set_wait_limit(tries)
+        gpu.kge.score_all_topk(gpu.dev_i32(qh), gpu.dev_i32(qr), K, gpu.dev_i32(tt), *out)
+        status = gpu.kge.get_status()
+        assert status in (0, -11)
+        ran_out += status != 0
+    assert ran_out
+    gpu.kge.debug_set_wait_limit(0)
+    for got, exact in zip(_infer(gpu, qh, qr, tt, K), want):
+        assert (got == exact).all()
