@@ -1430,8 +1430,8 @@ namespace {
 
 // One warp per positive merges the per-piece statistics of its row (and the positive score, which the sampled softmax
 // normalises over too) into the per-positive loss, dL/df+ and the row's factor loss_scale / Z, and multiplies the row of the dT
-// contraction's operand by it.  A row with a piece that left its reference (see tc_loss_chunk) keeps its operand and a factor of
-// one; its (max, 1 / Z) go to the launch that writes its dL/dF.
+// contraction's operand by it.  A row with a piece that left its reference (see tc_loss_chunk), or with no score anywhere near it,
+// keeps its operand and a factor of one; its (max, 1 / Z) go to the launch that writes its dL/dF.
 struct CombineParams {
     const float4* stat_part; int pieces; int B;
     const float* fpos;
@@ -1441,9 +1441,39 @@ struct CombineParams {
     const float4* Q; uint2* Qb; int d4;   // [B, d] query vectors; their bf16 copies
     uint32_t* Xq;                         // norm expansion: [B, 64] bf16, the factor as two terms beside the operand's columns, or NULL
     int32_t* redo;
+    const uint2* Tb; int N;               // [N, d] bf16 copies of the negatives
+    const float *qn2, *tn2;               // squared norms, norm expansion only
+    float k1, k0;                         // base-2 exponent of a score: k1 f + k0
 };
 
-__global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
+// Statistics of a row whose scores all lie so far below its reference that their exponentials are gone: the reference comes from
+// the unrounded rows, and with norms or a temperature far beyond the usual the score block can be 2^126 below it.  The warp
+// goes over the row's scores itself: (base-2 maximum, sum of exponentials, weighted loss sum) over the negatives.
+__device__ __noinline__ float3 row_statistics(const CombineParams& p, int b, int lane) {
+    const bool ce = p.loss == KGE_LOSS_SAMPLED_SOFTMAX;
+    const uint2* q = p.Qb + (int64_t)b * p.d4;
+    const float rn = p.Xq ? p.qn2[b] : 0.f;
+    float m = -INFINITY, z = 0.f, l = 0.f;
+    for (int n = lane; n < p.N; n += 32) {
+        const uint2* t = p.Tb + (int64_t)n * p.d4;
+        float acc = 0.f;
+        auto two = [&](uint32_t x, uint32_t y) {
+            acc = fmaf(__uint_as_float(x << 16), __uint_as_float(y << 16), acc);
+            acc = fmaf(__uint_as_float(x & 0xffff0000u), __uint_as_float(y & 0xffff0000u), acc);
+        };
+        for (int c = 0; c < p.d4; ++c) { const uint2 x = q[c], y = t[c]; two(x.x, y.x); two(x.y, y.y); }
+        const float f = p.Xq ? -sqrtf(fmaxf(rn + p.tn2[n] - 2.f * acc, 0.f)) : acc, y = fmaf(f, p.k1, p.k0);
+        if (y > m) { const float r = exp2f(m - y); z *= r; l *= r; m = y; }
+        const float e = exp2f(y - m);
+        z += e;
+        if (!ce) l += e * softplusf(p.gamma + f);
+    }
+    const float top = warp_max(m), r = m == -INFINITY ? 0.f : exp2f(m - top);
+    return make_float3(top, warp_sum(z * r), warp_sum(l * r));
+}
+
+// (eight CTAs per SM: the call of row_statistics would take 48 registers, 4 us more per step at 4,096 x 16,384 and 8,192 x 8,192)
+__global__ void __launch_bounds__(256, 8) stats_combine_kernel(const __grid_constant__ CombineParams p) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     grid_dependency_wait();
     allow_dependents();
@@ -1466,7 +1496,17 @@ __global__ void __launch_bounds__(256) stats_combine_kernel(CombineParams p) {
     }
     z = warp_sum(z); l = warp_sum(l);
     if (ce) z += exp2f(fp * kLog2e - m);
-    good = good && z >= 1e-30f && z < INFINITY;
+    if (z < 0x1p-40f) {        // (at 2^-40 the weights that matter are still 2^60 above the smallest number)
+        const float3 s = row_statistics(p, b, lane);
+        m = s.x; z = s.y; l = s.z;
+        if (ce) {
+            const float mm = fmaxf(m, fp * kLog2e);
+            z = z * exp2f(m - mm) + exp2f(fp * kLog2e - mm);
+            m = mm;
+        }
+        good = false;
+    }
+    good = good && z < INFINITY;
     const float scale = good ? p.loss_scale / z : 1.f;
     if (good)
         for (int c = lane; c < p.d4; c += 32) {
@@ -1576,7 +1616,8 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
     stage_begin(h, ST_LOSS, s);
     CombineParams cp{p.stat_part, p.row_pieces, p.M, w.fpos, c.loss, c.gamma, c.ce_correction, c.loss_scale,
                      reinterpret_cast<float2*>(w.row_stat), w.Lrow, w.gpos, w.Grow, reinterpret_cast<const float4*>(w.Q),
-                     reinterpret_cast<uint2*>(w.Qb), c.dim / 4, p.l2 ? reinterpret_cast<uint32_t*>(w.Xq) : nullptr, w.status + TC_REDO_FLAG};
+                     reinterpret_cast<uint2*>(w.Qb), c.dim / 4, p.l2 ? reinterpret_cast<uint32_t*>(w.Xq) : nullptr, w.status + TC_REDO_FLAG,
+                     reinterpret_cast<const uint2*>(w.Tb), c.num_neg, w.qn2, w.tn2, ce ? kLog2e : c.adv_temp * kLog2e, ce ? c.ce_correction * kLog2e : 0.f};
     KGE_CUDA_CHECK(h, launch_dependent(stats_combine_kernel, dim3((p.M * 32 + 255) / 256), dim3(256), 0, s, cp));
     KGE_LAUNCH_CHECK(h);
     KGE_CUDA_CHECK(h, launch_redo(p.l2 != 0, ce, h, p, s));

@@ -658,6 +658,34 @@ def test_tensor_core_rows_that_leave_their_reference(oracle64, score, loss, scal
         assert_close(got, exact, atol=1e-2 * np.abs(exact).max(), what=what)
 
 
+# Rows whose reference (fp32) lies far above all scores of their bf16 block.  The rows are exact in bf16 plus what rounding takes
+# away, so that the block's sums are exact and only the norms' fp32 sums (some 1e-5, times the temperature in the exponent) differ.
+# An exponent of 10^5 in base 2 is resolved to 2^-8, so a weight is good to 2^-8 ln 2, and to 2^-9 as a bf16: together below 1e-2 of
+# terms of size `scale`, which cancel in dh against the positive's.
+@pytest.mark.parametrize("score,loss,scale,a,c,atol", [("distmult", "logsigmoid", 1.0, 1000.0, 0.0, 1e-3), ("transe", "logsigmoid", 1.0, 1000.0, 0.0, 1e-3),
+                                                       ("distmult", "softmax", 32.0, 0.0, 300.0, 0.1)])
+@pytest.mark.parametrize("B,N", [(150, 700), (2048, 1100)])
+def test_tensor_core_rows_far_below_their_reference(oracle64, score, loss, scale, a, c, atol, B, N):
+    prob = Problem(E=4000, R=7, T=9000, d=64, score=score, p_norm=2 if score == "transe" else 1, loss=loss, B=B, N=N, P=1, gamma=0.5 if score == "transe" else -64.0,
+                   adv_temp=a, ce_correction=c, lr=1e-6, graph_seed=57, tc=True)
+    rng = np.random.default_rng(57)
+    k = np.zeros((prob.E, 64))
+    k[np.arange(prob.E)[:, None], rng.integers(0, 64, (prob.E, 4))] = rng.integers(-3, 4, (prob.E, 4))
+    prob.ent[:] = scale * (1.0 + k / 128 + 0.002)
+    prob.rel[:] = 0.0 if score == "transe" else 1.0
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    batch = orc.sample(0)
+    want, g = orc.o.batch_loss(orc.cfg, orc.ent, orc.rel, orc.relw, *batch), orc.grads(batch)
+    gpu.kge.train_step(0, prob.lr)
+    assert gpu.kge.get_status() == 0
+    assert_close(gpu.kge.debug_export("LROW"), want["Lrow"], atol=atol, what="losses")
+    ge = gpu.kge.debug_export("GRAD_ENT").reshape(2 * prob.B + prob.N, prob.d)
+    assert np.isfinite(ge).all()
+    if score == "distmult":       # (a distance of the expansion and the exact one, which the oracle differentiates, have little in common here)
+        for got, exact, what in ((ge[:prob.B], g["dh"], "dh"), (ge[2 * prob.B:], g["dtneg"], "dtneg")):
+            assert_close(got, exact, atol=1e-2 * max(np.abs(exact).max(), scale), what=what)
+
+
 # lists of more than 1,024 ids: the last tile one id long, full, and one short; an odd and an even number of tiles; one id everywhere
 @pytest.mark.parametrize("B,N,E", [(500, 25, 400), (600, 848, 5000), (600, 847, 3), (900, 1273, 50000), (1500, 1097, 1), (1024, 2048, 200)])
 def test_touched_ids_over_several_tiles(oracle64, B, N, E):
