@@ -241,6 +241,7 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
 // otherwise ends at once.  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
 // softmax 4,096 x 16,384 x 256 34 + 53 us, TransE-L2 8,192 x 8,192 x 128 67 + 94 us.)
 constexpr float TC_REF_SPAN = 80.f;
+constexpr float TC_EXP_MIN = -126.f;      // below it an exponential is 0
 
 // One chunk of 32 scores.  FULL: all 32 columns lie inside the problem (no per-element masking); otherwise the first `valid`
 // do.  k0: the exponent's constant less the reference; cn: the columns' squared norms (shared memory, norm expansion).  Returns what was
@@ -248,6 +249,7 @@ constexpr float TC_REF_SPAN = 80.f;
 // A1 (distance scores f <= 0, log-sigmoid loss, temperature a = 1): with K = exp(gamma) 2^ref, exp(gamma + f) = K e =: t, so
 // softplus(gamma + f) = log(1 + t) and sigmoid(gamma + f) = t / (1 + t): four special-function instructions per score
 // (distance, exponential, logarithm, reciprocal).
+// K is gone where it is below 2^-126; a chunk whose largest t would not be takes its own maximum too.
 // An L2 score is at most 0, so only a row whose reference is far below (`low`) can exceed it by much, and the chunk's maximum
 // is looked for only in a warp that holds such a row; the other scores' maximum is a tree of three-input maxima.
 template <bool L2, bool CE, bool FULL, bool A1>
@@ -270,15 +272,18 @@ __device__ __forceinline__ float tc_loss_chunk(const TcGemmParams& p, const floa
             vm[j] = max3(max3(x[0], x[1], x[2]), max3(x[3], x[4], x[5]), fmaxf(x[6], x[7]));
         }
         fm = fmaxf(max3(vm[0], vm[1], vm[2]), vm[3]);
-    } else if (__any_sync(0xffffffffu, low)) {
+    } else if (__any_sync(0xffffffffu, low)) {      // the largest score is that of the smallest squared distance
+        float sm = INFINITY;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            float inv;
-            const float f = score(i, inv);
-            if (FULL || i < valid) fm = fmaxf(fm, f);
-        }
+        for (int i = 0; i < 32; ++i) if (FULL || i < valid) sm = fminf(sm, fmaxf(fmaf(-2.f, v[i], rn + cn[i]), 0.f));
+        fm = sm > 0.f ? -sm * fast_rsqrt(sm) : 0.f;
     }
-    const float ym = fmaf(fm, k1, k0), shift = ym > TC_REF_SPAN ? ym : 0.f;      // (k1 >= 0)
+    const float ym = fmaf(fm, k1, k0);      // (k1 >= 0)
+    float shift = ym > TC_REF_SPAN ? ym : 0.f;
+    if (A1) {
+        const float x = fmaf(p.gamma, kLog2e, ref);
+        if (x < TC_EXP_MIN && x + ym >= TC_EXP_MIN) shift = ym;
+    }
     const float kk = k0 - shift;
     const float kexp = A1 ? fast_exp2(fmaf(p.gamma, kLog2e, ref + shift)) : 0.f;
     float zv[4] = {0.f, 0.f, 0.f, 0.f}, lv[4] = {0.f, 0.f, 0.f, 0.f};
@@ -345,7 +350,7 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
     const bool rin = row < p.M;
     const float rn = rs.rn, ref = rs.st.x;
     const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = (CE ? p.ce_c * kLog2e : 0.f) - ref;
-    const bool low = L2 && k0 > TC_REF_SPAN;
+    const bool low = L2 && (k0 > TC_REF_SPAN || (A1 && fmaf(p.gamma, kLog2e, ref) < TC_EXP_MIN));
     const uint32_t rows = __ballot_sync(0xffffffffu, rin);
     const int row0 = row - (int)(threadIdx.x & 31);
     float m = ref, z = 0.f, l = 0.f;

@@ -686,6 +686,64 @@ def test_tensor_core_rows_far_below_their_reference(oracle64, score, loss, scale
             assert_close(got, exact, atol=1e-2 * max(np.abs(exact).max(), scale), what=what)
 
 
+@pytest.mark.parametrize("gamma", [4.0, -30.0])
+@pytest.mark.parametrize("B,N", [(150, 700), (2048, 1100)])
+def test_tensor_core_distances_whose_reference_has_no_sigmoid(oracle64, gamma, B, N):
+    """Log-sigmoid TransE-L2 at temperature 1, queries at the origin: the two negatives that a row takes its reference from lie at
+    130 (sigmoid(gamma - 130) is 0 in fp32), the others at 77 to 86, whose sigmoids are not: dL/dF of some 2^-105 down to 2^-169 at
+    gamma = 4, the former of which fp32 and bf16 hold.  2^-8: dL/dF as bf16; the rest: exponents of 190 in fp32."""
+    prob = Problem(E=400, R=7, T=9000, d=64, score="transe", p_norm=2, B=B, N=N, P=1, gamma=gamma, adv_temp=1.0, lr=1e-6, graph_seed=59, tc=True)
+    rng = np.random.default_rng(59)
+    prob.ent[:] = 0.0
+    prob.ent[100:, 0] = rng.integers(77, 87, 300)
+    prob.ent[399, 0] = 130.0
+    prob.rel[:] = 0.0
+    batch = [rng.integers(0, 100, B), rng.integers(0, 7, B), rng.integers(0, 100, B), rng.integers(100, 399, N)]
+    batch = [a.astype(np.int32) for a in batch]
+    batch[3][[0, N // 2]] = 399
+    batch[3][5] = np.flatnonzero(prob.ent[:, 0] == 77)[0]
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    want, F = orc.grads(batch)["G"], orc.o.batch_loss(orc.cfg, orc.ent, orc.rel, orc.relw, *batch)["F"]
+    gpu.kge.train_step(0, prob.lr, *[gpu.dev_i32(a) for a in batch])
+    assert gpu.kge.get_status() == 0
+    assert (np.abs(want).max(axis=1) > (1e-35 if gamma > 0 else 0.0)).all()
+    assert_close(gpu.kge.debug_export("G").reshape(B, N) * -F, want, rtol=2.0 ** -8 + 1e-3, atol=1e-36, what="dL/dF")
+
+
+# Log-sigmoid TransE-L2: rows whose reference lies far below the rest (temperature 1 and not), in 128- and in 256-column tiles.  The
+# oracle's distances are the exact ones where it differentiates, so the rows' losses and dL/dF are compared.
+@pytest.mark.parametrize("a", [1.0, 0.75])
+@pytest.mark.parametrize("loss", ["logsigmoid", "softmax"])
+@pytest.mark.parametrize("B,N", [(150, 700), (2048, 2500)])
+def test_tensor_core_distance_rows_that_leave_their_reference(oracle64, loss, a, B, N):
+    prob = Problem(E=1000, R=7, T=9000, d=64, score="transe", p_norm=2, loss=loss, B=B, N=N, P=1, gamma=20.0, adv_temp=a, lr=1e-6, graph_seed=61, tc=True)
+    rng = np.random.default_rng(61)
+    prob.ent[:] = 0.0
+    prob.ent[:, 1] = rng.integers(0, 9, 1000)
+    prob.ent[100:500, 0] = rng.integers(10, 41, 400)           # negatives
+    prob.ent[500:, 0] = rng.integers(150, 251, 500)            # some of them, and the references, far away
+    prob.ent[100:, 2] = 1.0                                    # (no distance of 0)
+    prob.rel[:] = 0.0
+    prob.rel[1:, 0] = 200.0                                    # most queries are near those
+    batch = [rng.integers(0, 100, B), rng.integers(0, 7, B), rng.integers(500, 1000, B), rng.integers(100, 1000, N)]
+    batch = [x.astype(np.int32) for x in batch]
+    batch[3][[0, N // 2]] = rng.integers(500, 1000, 2)
+    gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
+    fwd = orc.o.batch_loss(orc.cfg, orc.ent, orc.rel, orc.relw, *batch)
+    want, F = orc.grads(batch)["G"], fwd["F"]
+    k = 1.0 if loss == "softmax" else a
+    ref = np.maximum(F[:, 0], F[:, N // 2])
+    if loss == "softmax":
+        ref = np.maximum(ref, fwd["fpos"])
+    beyond = k * (F.max(axis=1) - ref)
+    assert (beyond > 56).any() and (beyond < 54).any()
+    gpu.kge.train_step(0, prob.lr, *[gpu.dev_i32(x) for x in batch])
+    assert gpu.kge.get_status() == 0
+    # (distances up to 250 in the exponent, each good to some 2^-22)
+    assert_close(gpu.kge.debug_export("LROW"), fwd["Lrow"], rtol=1e-4, atol=1e-3, what="losses")
+    assert_close(gpu.kge.debug_export("G").reshape(B, N) * -F, want, rtol=2.0 ** -8 + 1e-3, atol=1e-30, what="dL/dF")
+
+
 # lists of more than 1,024 ids: the last tile one id long, full, and one short; an odd and an even number of tiles; one id everywhere
 @pytest.mark.parametrize("B,N,E", [(500, 25, 400), (600, 848, 5000), (600, 847, 3), (900, 1273, 50000), (1500, 1097, 1), (1024, 2048, 200)])
 def test_touched_ids_over_several_tiles(oracle64, B, N, E):
