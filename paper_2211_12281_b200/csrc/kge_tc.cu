@@ -38,8 +38,8 @@ constexpr int TC_PIECE = TC_BN / TC_EPI_GROUPS;           // columns of a 128-wi
 // measured against eight, C3 passes 41.5 / 58.0 -> 39.4 / 53.8 us, the special-function-bound C4 passes 98.7 / 154.7 -> 98.9 / 135.8 us,
 // although sixteen warps leave 96 registers per thread and the norm-expansion variants spill a little.
 constexpr int TC_FUSED_WARPS_256 = 16;
-__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 1 = the fused loss epilogue
-    return (epi & 3) == 1 && bn == 256 ? TC_FUSED_WARPS_256 : TC_EPI_WARPS;
+__host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 1, 2 = the fused loss epilogues
+    return ((epi & 3) == 1 || (epi & 3) == 2) && bn == 256 ? TC_FUSED_WARPS_256 : TC_EPI_WARPS;
 }
 __host__ __device__ constexpr int tc_threads(int epi, int bn = 128) { return 32 * (2 + tc_epi_warps(epi, bn)); }
 constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;
@@ -217,7 +217,7 @@ __device__ __forceinline__ float tc_score(const TcGemmParams& p, float acc, floa
 // Per-row inputs of an epilogue, read before the accumulator is waited for.
 struct TcRowState {
     float rn;                 // squared norm of the row (norm expansion)
-    float cn[2];              // EPI_LOSS, norm expansion: squared norms of this lane's column of each of the warp's chunks of 32
+    float cn[2];              // fused loss, norm expansion: squared norms of this lane's column of each of the warp's chunks of 32
     float2 st;                // EPI_LOSS: the row's (base-2 reference, -); EPI_GRAD: (base-2 maximum, 1 / normaliser)
 };
 template <int EPI>
@@ -393,43 +393,46 @@ __device__ __forceinline__ void tc_epilogue_loss(const TcGemmParams& p, const Tc
     if (rin && piece < p.row_pieces) p.stat_part[(int64_t)row * p.row_pieces + piece] = make_float4(m, z, l, 0.f);
 }
 
-// dL/dF of one pair from its accumulator: scale = loss_scale / normaliser, k0 already holds minus
-// the row's base-2 maximum.
-template <bool L2, bool CE>
-__device__ __forceinline__ float tc_grad_one(const TcGemmParams& p, float acc, float rn, int col, float k1, float k0, float scale) {
-    float inv;
-    const float f = tc_score_inv<L2>(p, acc, rn, col, inv);
-    float g = scale * fast_exp2(fmaf(f, k1, k0));
-    if (!CE) g *= tc_sigmoid(p.gamma + f);
-    if (L2) g *= inv;
-    return g;
-}
-
 // The rows that EPI_LOSS could not finish: dL/dF from the recomputed score and the row's final (base-2 max, 1 / normaliser).
-template <bool L2, bool CE>
+// A1: sigmoid(gamma + f) = t / (1 + t) with t = krow e, krow = exp(gamma) 2^max.
+template <bool L2, bool CE, bool A1, class Release>
 __device__ __forceinline__ void tc_epilogue_grad(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr,
-                                                 uint4* stage) {
-    const bool todo = row < p.M && rs.st.y != 0.f;
-    const uint32_t rows = __ballot_sync(0xffffffffu, todo);
-    if (rows == 0u) return;
+                                                 uint4* stage, Release release) {
+    const uint32_t rows = __ballot_sync(0xffffffffu, row < p.M && rs.st.y != 0.f);
+    if (rows == 0u) { release(); return; }
     const float k1 = CE ? kLog2e : p.adv_temp * kLog2e, k0 = (CE ? p.ce_c * kLog2e : 0.f) - rs.st.x;
     const float scale = p.loss_scale * rs.st.y;
+    const float krow = A1 ? fast_exp2(fmaf(p.gamma, kLog2e, rs.st.x)) : 0.f;
+    const float* cn = reinterpret_cast<const float*>(stage);
 #pragma unroll 1
-    for (int c0 = col_off; c0 < col_off + TC_PIECE; c0 += 32) {
+    for (int c = 0; c < TC_PIECE; c += 32) {
         float v[32];
-        tmem_ld32(taddr + (uint32_t)(c0 - col_off), v);
-        const int ncol = it.n0 + c0, valid = min(32, p.N - ncol);
-        if (valid <= 0) return;
+        tmem_ld32(taddr + (uint32_t)c, v);
+        if (c + 32 == TC_PIECE) release();
+        const int ncol = it.n0 + col_off + c, valid = min(32, p.N - ncol);
+        if (valid <= 0) continue;
+        if (L2) { reinterpret_cast<float*>(stage)[threadIdx.x & 31] = c == 0 ? rs.cn[0] : rs.cn[1]; __syncwarp(); }
         uint32_t g2[16];
+        auto one = [&](int i) {                          // (what lies outside the problem, or in a finished row, is not written)
+            float f = v[i], inv = 1.f;
+            if (L2) {
+                const float s2 = fmaxf(fmaf(-2.f, v[i], rs.rn + cn[i]), 0.f);
+                inv = s2 > 0.f ? fast_rsqrt(s2) : 0.f;
+                f = -s2 * inv;
+            }
+            const float e = fast_exp2(fmaf(f, k1, k0));
+            float g = scale * e;
+            if (A1) { const float t = krow * e; g *= t * fast_rcp(1.f + t); }
+            else if (!CE) g *= tc_sigmoid(p.gamma + f);
+            return g * inv;
+        };
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            float g[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                g[j] = todo && 2 * i + j < valid ? tc_grad_one<L2, CE>(p, v[2 * i + j], rs.rn, ncol + 2 * i + j, k1, k0, scale) : 0.f;
-            const __nv_bfloat162 pr = __floats2bfloat162_rn(g[0], g[1]);
+            const float a = one(2 * i), b = one(2 * i + 1);
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(a, b);
             g2[i] = *reinterpret_cast<const uint32_t*>(&pr);
         }
+        if (L2) __syncwarp();
         tc_put_bf16(p, row - (int)(threadIdx.x & 31), ncol, valid, rows, g2, stage);
     }
 }
@@ -453,15 +456,11 @@ __device__ __forceinline__ float float_below(float x) {
 // this thread's tensor-memory lane (taddr points at the first of them).
 template <int EPI, int WIDTH, class Release>
 __device__ __forceinline__ void tc_epilogue(const TcGemmParams& p, const TcItem& it, int row, const TcRowState& rs, int col_off, uint32_t taddr, void* scratch, Release release) {
-    static_assert((EPI & 3) == EPI_STORE || (EPI & 3) == EPI_LOSS ? (EPI & 3) == EPI_STORE || WIDTH == TC_PIECE : WIDTH % TC_PIECE == 0, "the fused loss epilogues work on pieces of TC_PIECE columns");
+    static_assert((EPI & 3) == EPI_STORE || WIDTH == TC_PIECE, "the fused loss epilogues work on pieces of TC_PIECE columns");
     if ((EPI & 3) == EPI_LOSS || (EPI & 3) == EPI_GRAD) {
-#pragma unroll 1
-        for (int c = 0; c < WIDTH; c += TC_PIECE) {
-            uint4* stage = static_cast<uint4*>(scratch);
-            if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage, release);
-            else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0>(p, it, row, rs, col_off + c, taddr + (uint32_t)c, stage);
-        }
-        if ((EPI & 3) == EPI_GRAD) release();
+        uint4* stage = static_cast<uint4*>(scratch);
+        if ((EPI & 3) == EPI_LOSS) tc_epilogue_loss<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off, taddr, stage, release);
+        else tc_epilogue_grad<(EPI & EPI_L2) != 0, (EPI & EPI_CE) != 0, (EPI & EPI_A1) != 0>(p, it, row, rs, col_off, taddr, stage, release);
         return;
     }
     float* const Cout = p.C + (int64_t)it.z * p.split_stride;
@@ -515,6 +514,32 @@ __device__ __forceinline__ void tc_item_next(const TcGemmParams& p, TcItem& it) 
     }
 }
 
+// EPI_GRAD: the row tiles with a row to do, a bit for every `group` of them (in shared memory, every CTA finds them for itself); their items
+// are dealt out to all CTAs in runs, like those of the other epilogues.
+constexpr int TC_TODO_WORDS = 128;
+__device__ __forceinline__ int tc_todo_group(const TcGemmParams& p) { return (p.tiles_m + 32 * TC_TODO_WORDS - 1) / (32 * TC_TODO_WORDS); }
+// First set bit from `bit` on; there is one.
+__device__ __forceinline__ int tc_todo_from(const uint32_t* todo, int bit) {
+    int w = bit >> 5;
+    uint32_t x = todo[w] & (~0u << (bit & 31));
+    while (x == 0u) x = todo[++w];
+    return 32 * w + __ffs(x) - 1;
+}
+__device__ __forceinline__ TcItem tc_todo_item(const TcGemmParams& p, const uint32_t* todo, int item) {
+    const int group = tc_todo_group(p), tn = item % p.tiles_n, r = item / p.tiles_n;
+    int bit = tc_todo_from(todo, 0);
+    for (int k = r / group; k > 0; --k) bit = tc_todo_from(todo, bit + 1);
+    return TcItem{0, (bit * group + r % group) * TC_BM, tn * p.bn};
+}
+// `more`: whether there is a next item.
+__device__ __forceinline__ void tc_todo_next(const TcGemmParams& p, const uint32_t* todo, TcItem& it, bool more) {
+    it.n0 += p.bn;
+    if (it.n0 < p.tiles_n * p.bn || !more) return;
+    const int group = tc_todo_group(p), tile = it.m0 / TC_BM + 1;
+    it.n0 = 0;
+    it.m0 = (tile % group != 0 ? tile : tc_todo_from(todo, tile / group) * group) * TC_BM;
+}
+
 // BN: columns per tile, 128 or 256.
 template <int EPI, int BN = 128>
 __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -535,14 +560,31 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     volatile uint32_t* stop = tmem_slot + 1;     // set by a warp whose wait ran out
     unsigned char* scratch_sm = base + (size_t)TC_STAGES * TC_STAGE_BYTES + 256;
 
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ uint32_t todo[(EPI & 3) == EPI_GRAD ? TC_TODO_WORDS : 1];
+    int items = p.items;
     if ((EPI & 3) == EPI_GRAD) {                        // (nothing in flight writes the flag)
         grid_dependency_wait();
         allow_dependents();
         if (*p.redo == 0) return;
+        for (int i = threadIdx.x; i < TC_TODO_WORDS; i += TC_THREADS) todo[i] = 0u;
+        __syncthreads();
+        const int group = tc_todo_group(p), rows = group * TC_BM;
+        for (int u = warp; u < (p.tiles_m + group - 1) / group; u += TC_THREADS / 32) {
+            bool any = false;
+            for (int64_t r = (int64_t)u * rows + lane, end = min((int64_t)(u + 1) * rows, (int64_t)p.M); r < end; r += 32) any = any || p.row_stat[r].y != 0.f;
+            if (__any_sync(0xffffffffu, any) && lane == 0) atomicOr(&todo[u >> 5], 1u << (u & 31));
+        }
+        __syncthreads();
+        int units = 0;
+        for (int i = lane; i < TC_TODO_WORDS; i += 32) units += __popc(todo[i]);
+        items = __reduce_add_sync(0xffffffffu, units) * group * p.tiles_n;
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int per_cta = (p.items + gridDim.x - 1) / gridDim.x;
+    auto item_at = [&](int item) { return (EPI & 3) == EPI_GRAD ? tc_todo_item(p, todo, item) : tc_item(p, item); };
+    auto item_next = [&](TcItem& it, bool more) { if ((EPI & 3) == EPI_GRAD) tc_todo_next(p, todo, it, more); else tc_item_next(p, it); };
+    const int per_cta = (items + gridDim.x - 1) / gridDim.x;
     const int item_begin = blockIdx.x * per_cta;
+    if ((EPI & 3) == EPI_GRAD && item_begin >= items) return;
     const int kb_total = (p.K + TC_BK - 1) / TC_BK;
 
     if (threadIdx.x == 0) {
@@ -560,7 +602,7 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const int item_end = min(p.items, item_begin + per_cta);
+    const int item_end = min(items, item_begin + per_cta);
     if ((EPI & 3) == EPI_LOSS) grid_dependency_wait();     // (launched while the kernel before it drains)
 
     if (warp == 0) {
@@ -574,8 +616,8 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
             int keep[TC_STAGES];
 #pragma unroll
             for (int s = 0; s < TC_STAGES; ++s) keep[s] = -1;
-            TcItem it = tc_item(p, item_begin);
-            for (int item = item_begin; item < item_end && !*stop; ++item, tc_item_next(p, it)) {
+            TcItem it = item_at(item_begin);
+            for (int item = item_begin; item < item_end && !*stop; ++item, item_next(it, item < item_end)) {
                 const int kb0 = it.z * p.kb_per_split, nkb = min(p.kb_per_split, kb_total - kb0);
                 for (int kb = 0; kb < nkb; ++kb, ++ring) {
                     const int s = ring % TC_STAGES;
@@ -600,8 +642,8 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
             constexpr uint32_t idesc = umma_idesc_bf16(TC_BM, BN, false, false);
             int ring = 0;
             bool ok = true;
-            TcItem it = tc_item(p, item_begin);
-            for (int item = item_begin, local = 0; item < item_end && ok && !*stop; ++item, ++local, tc_item_next(p, it)) {
+            TcItem it = item_at(item_begin);
+            for (int item = item_begin, local = 0; item < item_end && ok && !*stop; ++item, ++local, item_next(it, item < item_end)) {
                 const int nkb = min(p.kb_per_split, kb_total - it.z * p.kb_per_split);
                 const int buf = local % NACC;
                 // the epilogue warps must have drained this buffer (two items ago)
@@ -628,12 +670,12 @@ __global__ void __launch_bounds__(tc_threads(EPI, BN), 1) tc_gemm_kernel(const _
     } else {
         const int quarter = warp & 3;                  // tensor-memory lanes this warp may read
         const int cgrp = (warp - 2) >> 2;              // which group of the tile's columns
-        TcItem it = tc_item(p, item_begin);
+        TcItem it = item_at(item_begin);
         for (int item = item_begin, local = 0; item < item_end; ++item, ++local) {
-            if (local != 0) tc_item_next(p, it);
+            if (local != 0) item_next(it, true);
             // what the epilogue needs of its row does not depend on the accumulator: fetched before the wait
             TcRowState rs = tc_row_state<EPI>(p, it.m0 + quarter * 32 + lane);
-            if ((EPI & EPI_L2) != 0 && (EPI & 3) == EPI_LOSS) {
+            if ((EPI & EPI_L2) != 0 && (EPI & 3) != EPI_STORE) {
 #pragma unroll
                 for (int i = 0; i < GCOLS / 32; ++i) {
                     const int col = it.n0 + cgrp * GCOLS + 32 * i + lane;
@@ -1570,14 +1612,15 @@ cudaError_t launch_loss_bn(bool l2, bool ce, kge_handle* h, const TcGemmParams& 
         default: return launch_gemm_inst<EPI_LOSS | EPI_L2 | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
     }
 }
-// The rows that launch could not finish (in tiles of 128 columns: hardly ever more than a look at the flag).
-cudaError_t launch_redo(bool l2, bool ce, kge_handle* h, TcGemmParams p, cudaStream_t s) {
-    p.bn = TC_BN; p.tiles_n = (p.N + TC_BN - 1) / TC_BN; p.items = p.tiles_m * p.tiles_n;
+// The rows that launch could not finish: hardly ever more than a look at the flag.
+template <int BN>
+cudaError_t launch_redo_bn(bool l2, bool ce, kge_handle* h, const TcGemmParams& p, cudaStream_t s) {
+    if (l2 && !ce && p.adv_temp == 1.f && p.gamma <= 80.f) return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_A1, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
     switch ((l2 ? 2 : 0) | (ce ? 1 : 0)) {
-        case 0: return launch_gemm_inst<EPI_GRAD>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 1: return launch_gemm_inst<EPI_GRAD | EPI_CE>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        case 2: return launch_gemm_inst<EPI_GRAD | EPI_L2>(h->tm_q, h->tm_t, p, h->num_sms, s);
-        default: return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_CE>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 0: return launch_gemm_inst<EPI_GRAD, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 1: return launch_gemm_inst<EPI_GRAD | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        case 2: return launch_gemm_inst<EPI_GRAD | EPI_L2, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
+        default: return launch_gemm_inst<EPI_GRAD | EPI_L2 | EPI_CE, BN>(h->tm_q, h->tm_t, p, h->num_sms, s);
     }
 }
 }  // namespace
@@ -1625,7 +1668,7 @@ int launch_tc_forward(kge_handle* h, cudaStream_t s) {
                      reinterpret_cast<const uint2*>(w.Tb), c.num_neg, w.qn2, w.tn2, ce ? kLog2e : c.adv_temp * kLog2e, ce ? c.ce_correction * kLog2e : 0.f};
     KGE_CUDA_CHECK(h, launch_dependent(stats_combine_kernel, dim3((p.M * 32 + 255) / 256), dim3(256), 0, s, cp));
     KGE_LAUNCH_CHECK(h);
-    KGE_CUDA_CHECK(h, launch_redo(p.l2 != 0, ce, h, p, s));
+    KGE_CUDA_CHECK(h, p.bn == 256 ? launch_redo_bn<256>(p.l2 != 0, ce, h, p, s) : launch_redo_bn<128>(p.l2 != 0, ce, h, p, s));
     KGE_LAUNCH_CHECK(h);
     stage_end(h, ST_LOSS, s);
     return KGE_OK;

@@ -716,6 +716,17 @@ def test_tensor_core_distances_whose_reference_has_no_sigmoid(oracle64, gamma, B
 @pytest.mark.parametrize("loss", ["logsigmoid", "softmax"])
 @pytest.mark.parametrize("B,N", [(150, 700), (2048, 2500)])
 def test_tensor_core_distance_rows_that_leave_their_reference(oracle64, loss, a, B, N):
+    _rows_that_leave(oracle64, loss, a, B, N, None)
+
+
+# such rows in a few tiles of 128 rows only: first and last, neighbours, a last one that is not whole; more tiles than bits (the second
+# round then keeps a bit for two)
+@pytest.mark.parametrize("B,N,tiles", [(2048, 2500, [0]), (2048, 2500, [3, 4, 15]), (1000, 700, [7]), (530_000, 20, [1, 2000, 2003, 4140])])
+def test_tensor_core_few_row_tiles_that_leave_their_reference(oracle64, B, N, tiles):
+    _rows_that_leave(oracle64, "logsigmoid", 1.0, B, N, tiles)
+
+
+def _rows_that_leave(oracle64, loss, a, B, N, tiles):
     prob = Problem(E=1000, R=7, T=9000, d=64, score="transe", p_norm=2, loss=loss, B=B, N=N, P=1, gamma=20.0, adv_temp=a, lr=1e-6, graph_seed=61, tc=True)
     rng = np.random.default_rng(61)
     prob.ent[:] = 0.0
@@ -728,6 +739,8 @@ def test_tensor_core_distance_rows_that_leave_their_reference(oracle64, loss, a,
     batch = [rng.integers(0, 100, B), rng.integers(0, 7, B), rng.integers(500, 1000, B), rng.integers(100, 1000, N)]
     batch = [x.astype(np.int32) for x in batch]
     batch[3][[0, N // 2]] = rng.integers(500, 1000, 2)
+    if tiles is not None:
+        batch[1] = np.where(np.isin(np.arange(B) // 128, tiles) & (rng.random(B) < 0.1), 0, 1 + batch[1] % 6).astype(np.int32)
     gpu, orc = GpuSide(prob), OracleSide(prob, oracle64)
     fwd = orc.o.batch_loss(orc.cfg, orc.ent, orc.rel, orc.relw, *batch)
     want, F = orc.grads(batch)["G"], fwd["F"]
