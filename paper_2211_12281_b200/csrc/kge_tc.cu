@@ -1851,7 +1851,9 @@ int launch_tc_infer_chunk(kge_handle* h, int nq, int64_t e_lo, int64_t e_hi, con
     p.M = nq; p.N = (int)(e_hi - e_lo);
     p.slices = (h->cfg.dim + TC_BK - 1) / TC_BK;
     p.tiles_m = (nq + TC_BM - 1) / TC_BM; p.tiles_n = (p.N + SCAN_BN - 1) / SCAN_BN;
-    const int mt = p.slices <= 2 && p.tiles_m > 1 ? 2 : 1;
+    // two query tiles per CTA where that still gives every SM a pair (500 queries x 10,000 x 128: 103.7 us with two, 92.7 with one;
+    // 257 x 1,000 57.1 and 49.7, which 128 x 256 tiles with the entities kept took 48.1 for; 700 x 150,000 189 and 184)
+    const int mt = p.slices <= 2 && p.tiles_m > 1 && (int64_t)((p.tiles_m + 1) / 2) * p.tiles_n >= h->num_sms ? 2 : 1;
     p.groups = (p.tiles_m + mt - 1) / mt;
     const size_t fixed = 1024 + 256 + (size_t)mt * p.slices * TC_A_BYTES;
     p.ring = (int)std::min<size_t>(SCAN_RING_MAX, (SCAN_SMEM_MAX - fixed) / SCAN_SLICE_BYTES);
