@@ -219,30 +219,29 @@ __device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64
 // are in flight together; what a lane has left over of its four is probed one step at a time by the whole warp, so that a
 // warp's rounds are those of its unluckiest lane's four and not of its unluckiest lane four times.  The table is sparse
 // (2,048 slots for 768 entities) for the same reason.  The sums stay in registers: entity i of the order of arrival belongs
-// to thread i mod threads, which adds its rank scores model by model.  The rank scores lie in ENS_COPIES copies side by side,
+// to thread i mod threads, which adds its rank scores model by model.  The rank scores lie in COPIES copies side by side,
 // a lane reads its own: a random look-up in one copy would meet three others in its bank.  An entity twice in one list
 // loses one of its two bytes (position + 1), so that the bytes read add up to less than the bytes written.
 // ------------------------------------------------------------------------------------------
-constexpr int ENS_COPIES = 16, ENS_CAND = 64, ENS_CUT_TOP = 16;
-template <int MB>
-constexpr size_t ens_union_smem(int slots, int K) {
-    return (size_t)(K + 1) * ENS_COPIES * sizeof(double) + (size_t)slots * (sizeof(int32_t) + MB) + (size_t)slots * sizeof(uint16_t);
+constexpr int ENS_CAND = 64, ENS_CUT_TOP = 16;
+constexpr size_t ens_union_smem(int models, int copies, int slots, int K) {
+    return (size_t)(K + 1) * copies * sizeof(double) + (size_t)slots * (sizeof(int32_t) + models) + (size_t)slots * sizeof(uint16_t);
 }
 
 // V: places of a list that lie on one boundary of a load (4, 2 or 1).  Returns 0, or (all threads) why the table was given up.
-template <int MB, int V, int R>
+template <int MB, int V, int R, int COPIES>
 __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_slots, const int limit, unsigned char* smem) {
     constexpr int WORDS = MB / 4;
     const int slots = 1 << log2_slots, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, K = p.K;
     double* tab = reinterpret_cast<double*>(smem);                              // [K + 1][copies] absent score, then positions 1 .. K
-    int32_t* key = reinterpret_cast<int32_t*>(tab + (size_t)(K + 1) * ENS_COPIES);   // [slots] entity id or -1
+    int32_t* key = reinterpret_cast<int32_t*>(tab + (size_t)(K + 1) * COPIES);   // [slots] entity id or -1
     uint32_t* cell = reinterpret_cast<uint32_t*>(key + slots);                  // [MB / 4][slots] bytes: position + 1 in the block's models
     uint16_t* used = reinterpret_cast<uint16_t*>(cell + (size_t)WORDS * slots);      // [slots] occupied slots, in order of arrival
     __shared__ int n_used, lost;
     for (int i = tid; i < slots / 4; i += nthr) reinterpret_cast<int4*>(key)[i] = make_int4(-1, -1, -1, -1);
     for (int i = tid; i < slots * WORDS / 4; i += nthr) reinterpret_cast<int4*>(cell)[i] = make_int4(0, 0, 0, 0);
-    for (int i = tid; i < (K + 1) * (ENS_COPIES / 2); i += nthr) {
-        const int j = i / (ENS_COPIES / 2);
+    for (int i = tid; i < (K + 1) * (COPIES / 2); i += nthr) {
+        const int j = i / (COPIES / 2);
         const double x = p.table[j == 0 ? K : j - 1];
         reinterpret_cast<double2*>(tab)[i] = make_double2(x, x);
     }
@@ -271,7 +270,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
     int32_t next[4];
     fetch(0, next);
     __syncthreads();
-    const double* mytab = tab + (lane & (ENS_COPIES - 1));
+    const double* mytab = tab + (lane & (COPIES - 1));
     const double absent = tab[0];
     double before = 0.0, sum[R];     // before: an entity's sum over the models ahead of the block it first appears in
     int slot[R];
@@ -337,7 +336,7 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
                 bytes -= __dp4a(c, 0x01010101u, 0u);
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (4 * w + j < mb) s += mytab[(c >> (8 * j) & 0xffu) * ENS_COPIES];
+                    if (4 * w + j < mb) s += mytab[(c >> (8 * j) & 0xffu) * COPIES];
             }
             sum[r] = s;
         }
@@ -578,27 +577,28 @@ __global__ void __launch_bounds__(512) ensemble_sort_left_kernel(EnsParams p) {
 }
 
 // Lists so short that a table of 1.5 slots per entry fits (M K <= 682): one launch, no table overflows, and a query with an
-// entity twice in one list is sorted where it stands (the sort needs no more memory than the table).
-// T threads (fewer where the lists need fewer).
-constexpr int ENS_SMALL_MB = 16, ENS_SMALL_LOG2 = 10, ENS_ENTITIES = 768;
-template <int V, int T>
-__global__ void __launch_bounds__(T) ensemble_small_kernel(EnsParams p) {
+// entity twice in one list is sorted where it stands (the sort needs no more memory than the table).  64 threads where they hold the
+// entries, six each, and (nearly) a block of models at once, else 128 with three or six; two copies of the rank scores: with so few
+// look-ups, filling sixteen takes longer than their conflicts (6 x 33 x 15,000: 219 us on 256 threads with sixteen, 65 so; 4 x 80 174 and
+// 94; 2 x 254 295 and 150).
+constexpr int ENS_SMALL_MB = 16, ENS_SMALL_COPIES = 2, ENS_SMALL_LOG2 = 10, ENS_ENTITIES = 768;
+template <int V, int R>
+__global__ void __launch_bounds__(128) ensemble_small_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
-    if (!ens_union_query<ENS_SMALL_MB, V, ENS_ENTITIES / T>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
+    if (!ens_union_query<ENS_SMALL_MB, V, R, ENS_SMALL_COPIES>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
     __syncthreads();
     ens_sort_call<0>(p, blockIdx.x, ens_smem);
 }
 
-// Longer lists, first launch: one CTA of T threads per query.  A block of models is at most T quads, 1,024 places, so that with
-// ENS_ENTITIES entities before it a slot is always free.  Lists of more than 64 places fill 256 threads with eight models, shorter
-// ones with sixteen, those of up to 32 places 128 threads.
+// Longer lists, first launch: one CTA of T threads per query, MB models in a block.  A block of models is at most T quads, 1,024
+// places, so that with ENS_ENTITIES entities before it a slot is always free.  Which T, MB and COPIES: see the launch.
 constexpr int ENS_LOG2 = 11;
 static_assert(ENS_ENTITIES + 1024 < 1 << ENS_LOG2, "a probe ends");
-template <int MB, int V, int T>
+template <int MB, int V, int T, int COPIES>
 __global__ void __launch_bounds__(T) ensemble_hash_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
     allow_dependents();
-    const int bad = ens_union_query<MB, V, ENS_ENTITIES / T>(p, blockIdx.x, ENS_LOG2, ENS_ENTITIES, ens_smem);
+    const int bad = ens_union_query<MB, V, ENS_ENTITIES / T, COPIES>(p, blockIdx.x, ENS_LOG2, ENS_ENTITIES, ens_smem);
     if (bad && threadIdx.x == 0) p.out_ids[(int64_t)blockIdx.x * p.top_n] = bad == ENS_BAD_TWICE ? ENS_SORT : ENS_LEFT;
 }
 
@@ -655,6 +655,57 @@ __global__ void __launch_bounds__(NT, 2048 / NT) ensemble_left_kernel(EnsParams 
 }  // namespace
 }  // namespace kge
 
+namespace kge {
+namespace {
+
+// The widest load that every quad of a list allows.
+int ens_places_per_load(const int32_t* lists, int k) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(lists);
+    return k % 4 == 0 && at % 16 == 0 ? 4 : (k % 2 == 0 && at % 8 == 0 ? 2 : 1);
+}
+
+using EnsKernel = void (*)(EnsParams);
+struct EnsUnion { EnsKernel kernel; int models, threads, copies; };
+template <int MB, int T, int COPIES>
+EnsUnion ens_union_of(int v) {
+    return EnsUnion{v == 4 ? ensemble_hash_kernel<MB, 4, T, COPIES> : (v == 2 ? ensemble_hash_kernel<MB, 2, T, COPIES> : ensemble_hash_kernel<MB, 1, T, COPIES>), MB, T, COPIES};
+}
+template <int V>
+EnsKernel ens_small_of(int each) { return each == 1 ? ensemble_small_kernel<V, 1> : (each == 3 ? ensemble_small_kernel<V, 3> : ensemble_small_kernel<V, 6>); }
+EnsKernel ens_small_kernel(int v, int each) { return v == 4 ? ens_small_of<4>(each) : (v == 2 ? ens_small_of<2>(each) : ens_small_of<1>(each)); }
+
+// Models per block, threads and copies of the rank scores by the lists' length and number: a block of models should fill the
+// threads, and few models should not have to fill a large table (15,000 queries, us; the present choice against 256 threads with
+// sixteen models, or eight beyond 64 places, and sixteen copies):
+//   up to 24 places     8 models on 128 threads     60 x 20: 208 / 247 (16 on 128)   163 x 10: 345 / 384
+//   up to 48            12 on 128                   40 x 33: 212 / 284               85 x 40: 329 / 388
+//   up to 100           8 on 128 up to 40 models    10 x 80: 159 / 212               30 x 65: 259 / 310    40 x 100: 413 / 413
+//     beyond            16 on 256 to 64 places, 12 on 256 from there   60 x 65: 388 / 458   60 x 80: 398 / 472   (6,000 queries) 120 x 100: 364 / 380
+//   up to 128           8 on 128 up to 12 models    10 x 101: 196 / 228              12 x 128: 237 / 249
+//     beyond            8 on 256;  more than 223 places: sixteen copies take a resident CTA, eight do not, 10 x 254: 398 / 484
+EnsUnion ens_union_choice(int models, int k, int v) {
+    if (k <= 24) return ens_union_of<8, 128, 8>(v);
+    if (k <= 48) return ens_union_of<12, 128, 8>(v);
+    if (models <= (k <= 100 ? 40 : 12) && k <= 128) return ens_union_of<8, 128, 8>(v);
+    if (k <= 64) return ens_union_of<16, 256, 16>(v);
+    if (k <= 100) return ens_union_of<12, 256, 16>(v);
+    return k <= 223 ? ens_union_of<8, 256, 16>(v) : ens_union_of<8, 256, 8>(v);
+}
+// Every kernel of the two above with the most shared memory it is launched with.
+template <class F>
+void ens_each_union(F f) {
+    constexpr size_t sort = 1024 * (sizeof(uint64_t) + sizeof(int32_t));        // (M K <= 682)
+    for (int v : {1, 2, 4}) {
+        for (int each : {1, 3, 6}) f(ens_small_kernel(v, each), std::max(ens_union_smem(ENS_SMALL_MB, ENS_SMALL_COPIES, 1 << ENS_SMALL_LOG2, ENS_MAX_K), sort));
+        for (const EnsUnion& u : {ens_union_of<8, 128, 8>(v), ens_union_of<12, 128, 8>(v), ens_union_of<16, 256, 16>(v), ens_union_of<12, 256, 16>(v),
+                                  ens_union_of<8, 256, 16>(v), ens_union_of<8, 256, 8>(v)})
+            f(u.kernel, ens_union_smem(u.models, u.copies, 1 << ENS_LOG2, ENS_MAX_K));
+    }
+}
+
+}  // namespace
+}  // namespace kge
+
 extern "C" {
 
 int kge_ensemble_rank_scores(double power, int32_t k_list, double* table) {
@@ -686,14 +737,7 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
         constexpr int sort_max = (int)(ENS_MAX_ENTRIES * (sizeof(uint64_t) + sizeof(int32_t)));
         static_assert(parts_smem <= sort_max, "the larger table fits where the sort does");
         cudaError_t e0 = cudaSuccess;
-        constexpr int union_max = (int)std::max(std::max(ens_union_smem<8>(1 << ENS_LOG2, ENS_MAX_K), ens_union_smem<16>(1 << ENS_LOG2, 64)),
-                                                ens_union_smem<ENS_SMALL_MB>(1 << ENS_SMALL_LOG2, ENS_MAX_K));
-        for (void (*k)(EnsParams) : {ensemble_small_kernel<1, 128>, ensemble_small_kernel<2, 128>, ensemble_small_kernel<4, 128>,
-                                     ensemble_small_kernel<1, 256>, ensemble_small_kernel<2, 256>, ensemble_small_kernel<4, 256>,
-                                     ensemble_hash_kernel<8, 1, 256>, ensemble_hash_kernel<8, 2, 256>, ensemble_hash_kernel<8, 4, 256>,
-                                     ensemble_hash_kernel<16, 1, 256>, ensemble_hash_kernel<16, 2, 256>, ensemble_hash_kernel<16, 4, 256>,
-                                     ensemble_hash_kernel<16, 1, 128>, ensemble_hash_kernel<16, 2, 128>, ensemble_hash_kernel<16, 4, 128>})
-            if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, union_max);
+        ens_each_union([&](void (*k)(EnsParams), size_t smem) { if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
         for (void (*k)(EnsParams) : {ensemble_sort_kernel<256>, ensemble_sort_kernel<512>, ensemble_sort_kernel<ENS_THREADS>, ensemble_sort_left_kernel,
                                      ensemble_left_kernel<256>, ensemble_left_kernel<512>, ensemble_left_kernel<ENS_THREADS>})
             if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sort_max);
@@ -709,22 +753,19 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
     p.inv_k = (uint32_t)((((uint64_t)1 << 32) + k_list - 1) / k_list);
     const int quads = (k_list + 3) / 4;
     p.inv_quads = quads == 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + quads - 1) / quads);
-    auto pick = [&](void (*k4)(EnsParams), void (*k2)(EnsParams), void (*k1)(EnsParams)) {    // the widest load that every quad's address allows
-        const uintptr_t at = reinterpret_cast<uintptr_t>(lists);
-        return k_list % 4 == 0 && at % 16 == 0 ? k4 : (k_list % 2 == 0 && at % 8 == 0 ? k2 : k1);
-    };
+    const int v = ens_places_per_load(lists, k_list);
     p.log2_slots = 5;
     while (2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
     if (p.log2_slots <= ENS_SMALL_LOG2) {
-        const int threads = p.log2_slots >= 9 ? (k_list <= 32 ? 128 : 256) : (p.log2_slots >= 7 && k_list > 32 ? 128 : 64);
-        const size_t smem = std::max(ens_union_smem<ENS_SMALL_MB>(1 << p.log2_slots, k_list), sort_smem);
-        if (threads <= 128) pick(ensemble_small_kernel<4, 128>, ensemble_small_kernel<2, 128>, ensemble_small_kernel<1, 128>)<<<nq, threads, smem, s>>>(p);
-        else pick(ensemble_small_kernel<4, 256>, ensemble_small_kernel<2, 256>, ensemble_small_kernel<1, 256>)<<<nq, threads, smem, s>>>(p);
+        const int entries = num_models * k_list, block = std::min(num_models, ENS_SMALL_MB) * quads;
+        const int threads = entries <= 384 && (block <= 64 || (block <= 80 && k_list <= 64)) ? 64 : 128;
+        const int each = entries <= threads ? 1 : (entries <= 3 * threads ? 3 : 6);
+        const size_t smem = std::max(ens_union_smem(ENS_SMALL_MB, ENS_SMALL_COPIES, 1 << p.log2_slots, k_list), sort_smem);
+        ens_small_kernel(v, each)<<<nq, threads, smem, s>>>(p);
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
-    if (k_list > 64) pick(ensemble_hash_kernel<8, 4, 256>, ensemble_hash_kernel<8, 2, 256>, ensemble_hash_kernel<8, 1, 256>)<<<nq, 256, ens_union_smem<8>(1 << ENS_LOG2, k_list), s>>>(p);
-    else if (k_list > 32) pick(ensemble_hash_kernel<16, 4, 256>, ensemble_hash_kernel<16, 2, 256>, ensemble_hash_kernel<16, 1, 256>)<<<nq, 256, ens_union_smem<16>(1 << ENS_LOG2, k_list), s>>>(p);
-    else pick(ensemble_hash_kernel<16, 4, 128>, ensemble_hash_kernel<16, 2, 128>, ensemble_hash_kernel<16, 1, 128>)<<<nq, 128, ens_union_smem<16>(1 << ENS_LOG2, k_list), s>>>(p);
+    const EnsUnion u = ens_union_choice(num_models, k_list, v);
+    u.kernel<<<nq, u.threads, ens_union_smem(u.models, u.copies, 1 << ENS_LOG2, k_list), s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return KGE_ERR_CUDA;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;

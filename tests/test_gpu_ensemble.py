@@ -188,3 +188,13 @@ def test_ensemble_places_per_load(oracle64, M, K, shift, power, top_n):
     assert lib.ensemble_topk(view, table, top_n, ids, sc) == 0
     o_ids, o_sc = oracle64.ensemble_topk(lists, power, top_n)
     assert (ids.cpu().numpy() == o_ids).all() and (sc.cpu().numpy() == o_sc).all()
+
+
+# both sides of every line that the choice of kernel draws: entries per thread and threads of the single launch; list length and
+# number of models of the first launch for longer lists
+@pytest.mark.parametrize("M,K", [(4, 16), (5, 13), (12, 16), (13, 15), (12, 32), (11, 35), (10, 32), (9, 36), (8, 40), (4, 80), (2, 64), (2, 65), (1, 254), (2, 254),
+                                 (29, 24), (28, 25), (15, 48), (14, 49), (41, 49), (40, 64), (41, 64), (41, 65), (40, 100), (41, 100), (12, 101), (13, 101),
+                                 (12, 128), (13, 128), (12, 129), (4, 223), (4, 224), (3, 254)])
+@pytest.mark.parametrize("power,top_n", [(-0.5, 10), (0.5, 17)])
+def test_ensemble_kernel_choice(oracle64, M, K, power, top_n):
+    test_ensemble_places_per_load(oracle64, M, K, 0, power, top_n)
