@@ -82,10 +82,9 @@ def test_tensor_core_topk_against_bf16_operand_oracle(oracle64, score, E, d):
     """Full-entity scoring on tensor cores (bf16 operands, fp32 accumulation) against the oracle
     with bf16-rounded operands.  The accumulation order differs, so the lists are compared as
     sets with a near-tie audit (2e-2 relative is the stated bound of this path; 1e-4 is used),
-    ranks within 2, MRR within 1e-3.  E = 5000 leaves ragged 128-wide tiles, nq = 200 two row tiles.
-    d = 64 and 128 keep the entity tile in a buffer of its own (one and two slices); at E = 70,000 the
-    later chunks give every thread block runs of items that cross from one entity tile to the
-    next.  d = 256 takes the plain ring of whole stages."""
+    ranks within 2, MRR within 1e-3.  E = 5000 leaves ragged 256-entity tiles, nq = 200 two query tiles, one per
+    CTA until a chunk has 148 entity tiles: the later chunks at E = 70,000 pass two by one entity tile at d = 128 (two
+    slices of the ring), those at d = 256 one (four)."""
     import kge_synth
     R, K, nq = 9, 10, 200
     prob = Problem(E=E, R=R, T=100, d=d, score=score, p_norm=1, B=8, N=8, P=1, graph_seed=12, tc=True)
@@ -264,8 +263,8 @@ def test_a_rise_after_a_restart(oracle32, score, tc, d):
     assert (ids == o_ids).all() and (ranks == o_ranks).all() and (sc == o_sc).all()
 
 
-# tensor cores: one, two and three tiles of 128 queries (two side by side for rows of up to 128 coordinates, else one), a table that ends
-# inside and at the end of a 256-entity tile, CTAs of their own for every query group and shared ones, lists that take many candidates
+# tensor cores: one, two and three tiles of 128 queries, a table that ends inside and at the end of a 256-entity tile, CTAs of their own
+# for every query group, lists that take many candidates
 @pytest.mark.parametrize("nq,E,d,K", [(1, 3001, 64, 10), (128, 4352, 128, 40), (129, 6000, 128, 1), (257, 9000, 64, 100), (385, 6001, 192, 10), (130, 20000, 384, 40),
                                       (2900, 5000, 64, 10), (300, 1500, 512, 5)])
 def test_tensor_core_query_groups(oracle64, nq, E, d, K):
@@ -301,13 +300,13 @@ def test_tensor_core_lists_of_equal_scores(oracle64):
     assert (ids == np.arange(K)).all()
 
 
-@pytest.mark.parametrize("d", [64, 192])
-def test_tensor_core_queries_outside_the_call_score_infinity(d):
+@pytest.mark.parametrize("d,E", [(64, 9000), (64, 120_000), (192, 9000)])        # (120,000: two query tiles per CTA)
+def test_tensor_core_queries_outside_the_call_score_infinity(d, E):
     """A call with fewer queries than the workspace holds, where the rest of the query vectors' memory makes every score +inf and the
     rest of the thresholds' ids lie beyond the table: nothing of it reaches the call, which ends and gives what a call with as
     many queries as the workspace holds gives."""
     import kge_synth
-    E, R, K, nq, most = 9000, 5, 10, 130, 400
+    R, K, nq, most = 5, 10, 130, 400
     prob = Problem(E=E, R=R, T=100, d=d, score="distmult", B=8, N=8, P=1, graph_seed=51, tc=True)
     prob.ent = np.abs(prob.ent)                                # (no +inf - inf among the sums)
     qh, qr, tt = kge_synth.make_queries(E, R, nq, seed=51)
@@ -347,3 +346,35 @@ def test_tensor_core_scoring_after_waits_that_run_out(nq, d):
     gpu.kge.debug_set_wait_limit(0)
     for got, exact in zip(_infer(gpu, qh, qr, tt, K), want):
         assert (got == exact).all()
+
+
+def _shared_groups():
+    """The fewest query groups (from nine on) that leave so many SMs idle with CTAs of their own that all CTAs share them."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return next(g for g in range(9, sms) if sms // g * g * 16 < sms * 15)
+
+
+# tensor cores, groups of queries that share the CTAs: a CTA crosses from one group to the next, loads its queries and hands the ones
+# before over; one query tile per group (d = 192, 256, and short chunks) and two (the last group has one, not whole); several
+# superblocks in the last chunk (of at least 32 pairs per CTA and 32 MB: 316 entity tiles of 400 at d = 256, 512 of 1,063 at d = 128).
+# Lists and ranks of a sample of the queries against the oracle.
+@pytest.mark.parametrize("tiles,E,d,K", [(2, 6000, 64, 10), (2, 400_000, 128, 10), (1, 6000, 192, 3), (1, 130_000, 256, 10)])
+def test_tensor_core_query_groups_share_ctas(oracle64, tiles, E, d, K):
+    import kge_synth
+    nq = (_shared_groups() - 1) * tiles * 128 + 70
+    prob = Problem(E=E, R=9, T=100, d=d, score="distmult", B=8, N=8, P=1, graph_seed=63, tc=True)
+    qh, qr, tt = kge_synth.make_queries(E, 9, nq, seed=63)
+    gpu = GpuSide(prob, max_queries=nq, topk=K, load_graph=False)
+    ids, sc, ranks = _infer(gpu, qh, qr, tt, K)
+    some = np.unique(np.concatenate([np.arange(0, nq, 97), np.arange(127, nq, 640), [nq - 1]]))
+    r_ids, r_sc, r_ranks = oracle64.score_all_topk(prob.oracle_cfg(), prob.ent, prob.rel, prob.relw, qh[some], qr[some], K + 5, true_tails=tt[some])
+    for i, q in enumerate(some):
+        assert len(set(ids[q])) == K
+        for e in set(ids[q]) - set(r_ids[i, :K]):          # (near ties only: the sums' order differs)
+            assert e in set(r_ids[i])
+            f = r_sc[i][list(r_ids[i]).index(e)]
+            assert abs(f - r_sc[i, K - 1]) <= 1e-4 * abs(f) + 1e-6
+    assert_close(sc[some], r_sc[:, :K], atol=1e-5, what="scores")
+    # (a rank moves by the entities within 2^-20 of the true tail's score: some three of 400,000)
+    assert np.abs(ranks[some] - r_ranks).max() <= 2 + E // 100_000
