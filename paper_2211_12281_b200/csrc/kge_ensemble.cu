@@ -223,7 +223,7 @@ __device__ __forceinline__ void ens_put(const EnsParams& p, int q, int r, uint64
 // a lane reads its own: a random look-up in one copy would meet three others in its bank.  An entity twice in one list
 // loses one of its two bytes (position + 1), so that the bytes read add up to less than the bytes written.
 // ------------------------------------------------------------------------------------------
-constexpr int ENS_CAND = 64, ENS_CUT_TOP = 16;
+constexpr int ENS_CUT_TOP = 16;
 constexpr size_t ens_union_smem(int models, int copies, int slots, int K) {
     return (size_t)(K + 1) * copies * sizeof(double) + (size_t)slots * (sizeof(int32_t) + models) + (size_t)slots * sizeof(uint16_t);
 }
@@ -347,9 +347,10 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
     bytes = __reduce_add_sync(0xffffffffu, bytes);
     if (lane == 0 && bytes) atomicAdd(&lost, (int)bytes);
 
-    // The best top_n.  Up to ENS_CUT_TOP: the top_n-th best of 32 groups' best scores (upper halves) is a bound that at least top_n
-    // entities reach; those that do, hardly more, are ranked against one another.  Otherwise, and where too many reach it: a round per place.
-    uint64_t os[R];                  // ordered scores, 0: none or taken
+    // The best top_n: those that reach a bound which at least top_n entities reach, hardly more, are ranked against one another.  Up to
+    // ENS_CUT_TOP the bound is the top_n-th best of 32 groups' best scores (upper halves), beyond of up to as many groups as threads,
+    // twice top_n where there are.  (A CTA-wide round per place, each with a barrier: 10 x 100 x 4,000, all 100 places, 294 us.)
+    uint64_t os[R];                  // ordered scores, 0: none
     int32_t id[R];
     uint32_t top_hi = 0;
 #pragma unroll
@@ -359,17 +360,17 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
         id[r] = in ? key[slot[r]] : INT32_MAX;
         top_hi = max(top_hi, (uint32_t)(os[r] >> 32));
     }
-    __shared__ uint64_t cand_s[ENS_CAND];
-    __shared__ int32_t cand_i[ENS_CAND];
-    __shared__ uint32_t group_hi[32];
+    uint64_t* cand_s = reinterpret_cast<uint64_t*>(cell);                       // (the positions are done with; 12 bytes per entity fit: see ens_union_smem's callers)
+    int32_t* cand_i = reinterpret_cast<int32_t*>(cand_s + seen);
+    __shared__ __align__(16) uint32_t group_hi[256];
     __shared__ uint32_t cut;
     __shared__ int n_cand;
-    if (p.top_n <= ENS_CUT_TOP) {
-        const int per_group = nthr >> 5;                                        // 2, 4 or 8 lanes
-        for (int o = per_group >> 1; o > 0; o >>= 1) top_hi = max(top_hi, __shfl_xor_sync(0xffffffffu, top_hi, o));
-        if ((tid & (per_group - 1)) == 0) group_hi[tid / per_group] = top_hi;
-        if (tid == 0) n_cand = 0;
-    }
+    int groups = 32;
+    if (p.top_n > ENS_CUT_TOP) while (groups < nthr && groups < 2 * p.top_n) groups <<= 1;
+    const int per_group = nthr / groups;                                        // 1, 2, 4 or 8 lanes
+    for (int o = per_group >> 1; o > 0; o >>= 1) top_hi = max(top_hi, __shfl_xor_sync(0xffffffffu, top_hi, o));
+    if ((tid & (per_group - 1)) == 0) group_hi[tid / per_group] = top_hi;
+    if (tid == 0) { n_cand = 0; cut = 0u; }
     __syncthreads();
     if (lost) return ENS_BAD_TWICE;
     if (p.top_n <= ENS_CUT_TOP) {
@@ -384,56 +385,36 @@ __device__ int ens_union_query(const EnsParams& p, const int q, const int log2_s
             }
             if (tid == 0) cut = c;
         }
-        __syncthreads();
-        const uint32_t c = cut;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (os[r] != 0ull && (uint32_t)(os[r] >> 32) >= c) {
-                const int at = atomicAdd(&n_cand, 1);
-                if (at < ENS_CAND) { cand_s[at] = os[r]; cand_i[at] = id[r]; }
-            }
-        __syncthreads();
-        const int n = n_cand;
-        if (n <= ENS_CAND) {
-            if (tid < max(n, p.top_n)) {
-                int rank = tid;
-                if (tid < n) {
-                    const uint64_t s = cand_s[tid];
-                    const int32_t e = cand_i[tid];
-                    rank = 0;
-                    for (int j = 0; j < n; ++j) rank += cand_s[j] > s || (cand_s[j] == s && cand_i[j] < e);
-                    if (rank < p.top_n) ens_put(p, q, rank, s, e);
-                } else {
-                    ens_put(p, q, rank, 0ull, 0);
-                }
-            }
-            return 0;
+    } else if (p.top_n <= groups && tid < groups) {
+        const uint32_t mine = group_hi[tid];
+        int ahead = 0;
+#pragma unroll 4
+        for (int j = 0; j < groups; j += 4) {
+            const uint4 o = *reinterpret_cast<const uint4*>(&group_hi[j]);
+            ahead += (o.x > mine || (o.x == mine && j < tid)) + (o.y > mine || (o.y == mine && j + 1 < tid)) +
+                     (o.z > mine || (o.z == mine && j + 2 < tid)) + (o.w > mine || (o.w == mine && j + 3 < tid));
         }
+        if (ahead == p.top_n - 1) cut = mine;
     }
-    __shared__ uint64_t red_s[2][32];
-    __shared__ int32_t red_i[2][32];
-    const int warp = tid >> 5, nwarps = nthr >> 5;
-    uint64_t ws; int32_t wi;                // the warp's best
-    auto warp_best = [&] {
-        uint64_t bs = 0; int32_t bi = INT32_MAX;
+    __syncthreads();
+    const uint32_t c = cut;
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (os[r] > bs || (os[r] == bs && id[r] < bi)) { bs = os[r]; bi = id[r]; }
-        ens_warp_best(bs, bi, ws, wi);
-    };
-    warp_best();
-    for (int r = 0; r < p.top_n; ++r) {
-        if (lane == 0) { red_s[r & 1][warp] = ws; red_i[r & 1][warp] = wi; }
-        __syncthreads();
-        uint64_t s; int32_t e;
-        ens_warp_best(lane < nwarps ? red_s[r & 1][lane] : 0ull, lane < nwarps ? red_i[r & 1][lane] : INT32_MAX, s, e);   // (every warp for itself)
-        if (tid == 0) ens_put(p, q, r, s, e);
-        if (s != 0ull && s == ws && e == wi) {                                  // taken (ids are distinct: one warp, one thread)
-#pragma unroll
-            for (int u = 0; u < R; ++u) if (id[u] == e) { os[u] = 0ull; id[u] = INT32_MAX; }
-            warp_best();
+    for (int r = 0; r < R; ++r)
+        if (os[r] != 0ull && (uint32_t)(os[r] >> 32) >= c) {
+            const int at = atomicAdd(&n_cand, 1);
+            cand_s[at] = os[r]; cand_i[at] = id[r];
         }
+    __syncthreads();
+    const int n = n_cand;
+    for (int i = tid; i < n; i += nthr) {
+        const uint64_t s = cand_s[i];
+        const int32_t e = cand_i[i];
+        int rank = 0;
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) rank += cand_s[j] > s || (cand_s[j] == s && cand_i[j] < e);
+        if (rank < p.top_n) ens_put(p, q, rank, s, e);
     }
+    for (int i = n + tid; i < p.top_n; i += nthr) ens_put(p, q, i, 0ull, 0);
     return 0;
 }
 
@@ -594,6 +575,7 @@ __global__ void __launch_bounds__(128) ensemble_small_kernel(EnsParams p) {
 // places, so that with ENS_ENTITIES entities before it a slot is always free.  Which T, MB and COPIES: see the launch.
 constexpr int ENS_LOG2 = 11;
 static_assert(ENS_ENTITIES + 1024 < 1 << ENS_LOG2, "a probe ends");
+static_assert(ENS_ENTITIES * 12 <= (1 << ENS_LOG2) * 8, "the positions' memory holds all entities' scores and ids (eight or more models; sixteen and 1.5 slots per entity in the single launch)");
 template <int MB, int V, int T, int COPIES>
 __global__ void __launch_bounds__(T) ensemble_hash_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
@@ -682,14 +664,14 @@ EnsKernel ens_small_kernel(int v, int each) { return v == 4 ? ens_small_of<4>(ea
 //   up to 100           8 on 128 up to 40 models    10 x 80: 159 / 212               30 x 65: 259 / 310    40 x 100: 413 / 413
 //     beyond            16 on 256 to 64 places, 12 on 256 from there   60 x 65: 388 / 458   60 x 80: 398 / 472   (6,000 queries) 120 x 100: 364 / 380
 //   up to 128           8 on 128 up to 12 models    10 x 101: 196 / 228              12 x 128: 237 / 249
-//     beyond            8 on 256;  more than 223 places: sixteen copies take a resident CTA, eight do not, 10 x 254: 398 / 484
+//     beyond            8 on 256;  more than 214 places: sixteen copies take a resident CTA, eight do not, 10 x 254: 398 / 484
 EnsUnion ens_union_choice(int models, int k, int v) {
     if (k <= 24) return ens_union_of<8, 128, 8>(v);
     if (k <= 48) return ens_union_of<12, 128, 8>(v);
     if (models <= (k <= 100 ? 40 : 12) && k <= 128) return ens_union_of<8, 128, 8>(v);
     if (k <= 64) return ens_union_of<16, 256, 16>(v);
     if (k <= 100) return ens_union_of<12, 256, 16>(v);
-    return k <= 223 ? ens_union_of<8, 256, 16>(v) : ens_union_of<8, 256, 8>(v);
+    return k <= 214 ? ens_union_of<8, 256, 16>(v) : ens_union_of<8, 256, 8>(v);
 }
 // Every kernel of the two above with the most shared memory it is launched with.
 template <class F>

@@ -194,7 +194,25 @@ def test_ensemble_places_per_load(oracle64, M, K, shift, power, top_n):
 # number of models of the first launch for longer lists
 @pytest.mark.parametrize("M,K", [(4, 16), (5, 13), (12, 16), (13, 15), (12, 32), (11, 35), (10, 32), (9, 36), (8, 40), (4, 80), (2, 64), (2, 65), (1, 254), (2, 254),
                                  (29, 24), (28, 25), (15, 48), (14, 49), (41, 49), (40, 64), (41, 64), (41, 65), (40, 100), (41, 100), (12, 101), (13, 101),
-                                 (12, 128), (13, 128), (12, 129), (4, 223), (4, 224), (3, 254)])
+                                 (12, 128), (13, 128), (12, 129), (4, 214), (4, 215), (3, 254)])
 @pytest.mark.parametrize("power,top_n", [(-0.5, 10), (0.5, 17)])
 def test_ensemble_kernel_choice(oracle64, M, K, power, top_n):
     test_ensemble_places_per_load(oracle64, M, K, 0, power, top_n)
+
+
+# lists of places: the last cut by groups and the first by threads (16, 17), as many as threads and one more (64, 128, 256), more than entities
+@pytest.mark.parametrize("M,K,top_n", [(6, 40, 40), (6, 40, 64), (6, 40, 65), (10, 64, 128), (10, 64, 129), (10, 100, 100), (60, 70, 128), (60, 70, 256), (60, 70, 257),
+                                       (3, 254, 254), (3, 254, 900), (2, 3, 17)])
+@pytest.mark.parametrize("power", [-0.5, 1.0])
+def test_ensemble_long_results(oracle64, M, K, top_n, power):
+    rng = np.random.default_rng(M + top_n)
+    nq, E = 21, 3 * K
+    lists = np.stack([np.stack([rng.permutation(E)[:K] for _ in range(nq)]) for _ in range(M)]).astype(np.int32)
+    lists[:, 3] = np.arange(K)                               # the same list everywhere
+    lists[:, 4] = np.roll(np.arange(K), 1)
+    lists[:M // 2, 4] = np.roll(np.arange(K), 2)             # ties, decided by the id
+    if M > 2:
+        lists[M - 1, 5, 0] = lists[M - 1, 5, 1]              # an entity twice, behind the first block of models where there are several
+    ids, sc = _gpu_ensemble(lists, power, top_n)
+    o_ids, o_sc = oracle64.ensemble_topk(lists, power, top_n)
+    assert (ids == o_ids).all() and (sc == o_sc).all()
