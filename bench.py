@@ -589,7 +589,7 @@ def bench_training(ctx, name, w, cpu_seconds):
             src = ctx.peaks["source"] + " (sustained cuBLAS bf16)"
         roofline = {"bound": bound, "kernel": dominant, "achieved": achieved, "peak": peak, "unit": unit,
                     "frac": t_roof / us, "traffic": ncu_traffic(name, dominant), "peak_source": src, "us_per_launch": us}
-        if w.get("tc"):      # tensor pipe activity of the four passes under ncu (tracked capture of the same kernels)
+        if w.get("tc"):      # tensor pipe activity of the passes under ncu (tracked capture of the same kernels)
             roofline["tensor_pipe_active_ncu_pct"] = {st: ncu_tensor_active(name, st) for st in ("block", "loss", "accum")}
         roofline.update({k: v for k, v in detail.items() if k != "mix"})
     stage_frac = {s: roofs[s][0] / per_stage_us[s] for s in roofs}
@@ -673,7 +673,7 @@ def bench_inference(ctx, name, w, cpu_seconds):
     t_hbm = E * d * 4 / (ctx.peaks["hbm_gbs"] * 1e9)
     if w.get("tc"):
         t_c = 2.0 * pairs * d / (ctx.peaks["bf16_tflops"] * 1e12)
-        roof = {"bound": "tensor", "kernel": "tc_gemm<topk>", "achieved": 2.0 * pairs * d / (ms * 1e-3) / 1e12,
+        roof = {"bound": "tensor", "kernel": "tc_scan", "achieved": 2.0 * pairs * d / (ms * 1e-3) / 1e12,
                 "peak": ctx.peaks["bf16_tflops"], "unit": "TFLOP/s", "peak_source": ctx.peaks["source"] + " (sustained cuBLAS bf16)"}
     else:
         o = {"transe": [(2, MIX_SUB_ABS)], "distmult": [(1, MIX_FMA)]}[w["score"]]

@@ -5,15 +5,15 @@
 //
 // Persistent CTAs (one per SM) each walk a run of 128 x 128 output tiles.  Warp 0 feeds a ring of
 // shared-memory stages with TMA (one elected lane), warp 1 issues the MMAs (one elected lane)
-// into one of two accumulators in tensor memory and owns the allocation, warps 2-17 drain the
-// other accumulator meanwhile (a warp may only touch the 32 lanes of its own quarter; four warps
-// share a quarter, a quarter of the columns each) and apply the epilogue:
+// into one of the accumulators in tensor memory and owns the allocation, eight or sixteen more drain
+// another accumulator meanwhile (a warp may only touch the 32 lanes of its own quarter; two or four warps
+// share a quarter, 64 columns each) and apply the epilogue:
 //   EPI_STORE   C = acc (the score block as a test reads it)
 //   EPI_LOSS    no score leaves the chip: dL/dF up to a factor of the row as bf16, for the two backward contractions, and per row
 //               and 64-column piece the sum of exponentials and the weighted loss sum of Section 3.1 "Loss Functions"; the
 //               score is the contraction (DistMult, ComplEx) or, for TransE with p = 2, the
 //               norm expansion -sqrt(max(|q|^2 + |t|^2 - 2 acc, 0))
-//   EPI_GRAD    dL/dF of the few rows, if any, whose scores lie too far from what EPI_LOSS took as their reference
+//   EPI_GRAD    dL/dF of the rows, if any, whose scores lie too far from what EPI_LOSS took as their reference
 // Every wait on a barrier is bounded; a wait that runs out records KGE_ERR_TIMEOUT, tells the
 // other warps to stop, and the CTA still releases its tensor memory before it returns.
 #include <cuda.h>
@@ -34,9 +34,8 @@ constexpr int TC_EPI_GROUPS = TC_EPI_WARPS / 4;
 constexpr int TC_GRAD_STAGE_BYTES = 2048;                 // per epilogue warp: 32 rows x 32 bf16 columns on their way to memory
 constexpr int TC_STORE_STAGE_BYTES = 4096;                // the same for EPI_STORE's 32 rows x 32 fp32 columns
 constexpr int TC_PIECE = TC_BN / TC_EPI_GROUPS;           // columns of a 128-wide tile per piece of loss statistics
-// The fused loss epilogues on 256-column tiles run on sixteen warps as well (64 columns = one piece of statistics per warp):
-// measured against eight, C3 passes 41.5 / 58.0 -> 39.4 / 53.8 us, the special-function-bound C4 passes 98.7 / 154.7 -> 98.9 / 135.8 us,
-// although sixteen warps leave 96 registers per thread and the norm-expansion variants spill a little.
+// The fused loss epilogues on 256-column tiles run on sixteen warps: 64 columns, one piece of statistics, per warp, as on 128-column tiles.
+// Sixteen leave 96 registers per thread; the distance variants spill up to 20 bytes outside their loops.
 constexpr int TC_FUSED_WARPS_256 = 16;
 __host__ __device__ constexpr int tc_epi_warps(int epi, int bn = 128) {   // 1, 2 = the fused loss epilogues
     return ((epi & 3) == 1 || (epi & 3) == 2) && bn == 256 ? TC_FUSED_WARPS_256 : TC_EPI_WARPS;
@@ -238,7 +237,7 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
 // negatives (the gather kernel computes them), a lower bound of the maximum up to rounding and a constant.  A chunk of 32 scores that exceeds it
 // by more than 2^TC_REF_SPAN takes its own maximum instead, which keeps the statistics in range, and the row is found by
 // stats_combine_kernel and its E written again, over the true maximum and with the factor, by an EPI_GRAD launch that
-// otherwise ends at once.  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
+// otherwise ends at once; so is a row whose scores all lie below it (row_statistics).  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
 // softmax 4,096 x 16,384 x 256 34 + 53 us, TransE-L2 8,192 x 8,192 x 128 67 + 94 us.)
 constexpr float TC_REF_SPAN = 80.f;
 constexpr float TC_EXP_MIN = -126.f;      // below it an exponential is 0
@@ -1788,8 +1787,8 @@ int launch_tc_backward(kge_handle* h, cudaStream_t s, cudaStream_t side) {
         KGE_CUDA_CHECK(h, bn > 64 ? (launch_gemm_dual<256, false, DUAL_STEP, true>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s, h->tm_x64))
                                   : (launch_gemm_dual<128, false, DUAL_STEP, true>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s, h->tm_x64)));
     else
-    KGE_CUDA_CHECK(h, bn == 256 ? launch_gemm_dual<256>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s)
-                                : launch_gemm_dual<128>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s));
+        KGE_CUDA_CHECK(h, bn == 256 ? launch_gemm_dual<256>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s)
+                                    : launch_gemm_dual<128>(h, h->tm_g, h->tm_t64, h->tm_g64, h->tm_q64, q0, q1, s));
     stage_end(h, ST_ACCUM_Q, s);
     KGE_LAUNCH_CHECK(h);
     return KGE_OK;

@@ -1322,7 +1322,7 @@ int launch_forward_backward(kge_handle* h, const int32_t* heads, const int32_t* 
         KGE_CUDA_CHECK(h, cudaEventRecord(h->ev_seg, dedup_side));
     }
     if (c.prec == KGE_PREC_BF16_TC) {
-        // tensor cores: scores, loss and dL/dF in two fused passes, the score block never stored
+        // tensor cores: scores, loss and dL/dF in one fused pass, the score block never stored
         const int rc = launch_tc_forward(h, s);
         if (rc != KGE_OK) return rc;
     } else {
