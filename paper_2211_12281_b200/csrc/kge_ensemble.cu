@@ -562,10 +562,11 @@ __global__ void __launch_bounds__(512) ensemble_sort_left_kernel(EnsParams p) {
 // entity twice in one list is sorted where it stands (the sort needs no more memory than the table).  64 threads where they hold the
 // entries, six each, and (nearly) a block of models at once, else 128 with three or six; two copies of the rank scores: with so few
 // look-ups, filling sixteen takes longer than their conflicts (6 x 33 x 15,000: 219 us on 256 threads with sixteen, 65 so; 4 x 80 174 and
-// 94; 2 x 254 295 and 150).
+// 94; 2 x 254 295 and 150).  Up to four queries per SM a CTA has the SM nearly to itself: threads for a whole block of models then
+// (6 x 100 x 296: 12.4 us on 128, 10.4 on 256; 16 x 20 x 100 10.3 on 64, 9.5 on 128).
 constexpr int ENS_SMALL_MB = 16, ENS_SMALL_COPIES = 2, ENS_SMALL_LOG2 = 10, ENS_ENTITIES = 768;
 template <int V, int R>
-__global__ void __launch_bounds__(128) ensemble_small_kernel(EnsParams p) {
+__global__ void __launch_bounds__(256) ensemble_small_kernel(EnsParams p) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
     if (!ens_union_query<ENS_SMALL_MB, V, R, ENS_SMALL_COPIES>(p, blockIdx.x, p.log2_slots, 1 << p.log2_slots, ens_smem)) return;
     __syncthreads();
@@ -661,16 +662,25 @@ EnsKernel ens_small_kernel(int v, int each) { return v == 4 ? ens_small_of<4>(ea
 // sixteen models, or eight beyond 64 places, and sixteen copies):
 //   up to 24 places     8 models on 128 threads     60 x 20: 208 / 247 (16 on 128)   163 x 10: 345 / 384
 //   up to 48            12 on 128                   40 x 33: 212 / 284               85 x 40: 329 / 388
-//   up to 100           8 on 128 up to 40 models    10 x 80: 159 / 212               30 x 65: 259 / 310    40 x 100: 413 / 413
-//     beyond            16 on 256 to 64 places, 12 on 256 from there   60 x 65: 388 / 458   60 x 80: 398 / 472   (6,000 queries) 120 x 100: 364 / 380
+//   up to 80            8 on 128 up to 40 models    10 x 80: 159 / 212               30 x 65: 259 / 310
+//   up to 100           8 on 128 up to 20 models    10 x 100: 173 / 224              20 x 100: 261 / 294
+//     beyond            16 on 256 to 64 places, 12 on 256 from there   60 x 65: 392 / 458   60 x 80: 404 / 472   85 x 100: 617 / 700
 //   up to 128           8 on 128 up to 12 models    10 x 101: 196 / 228              12 x 128: 237 / 249
 //     beyond            8 on 256;  more than 214 places: sixteen copies take a resident CTA, eight do not, 10 x 254: 398 / 484
-EnsUnion ens_union_choice(int models, int k, int v) {
-    if (k <= 24) return ens_union_of<8, 128, 8>(v);
-    if (k <= 48) return ens_union_of<12, 128, 8>(v);
-    if (models <= (k <= 100 ? 40 : 12) && k <= 128) return ens_union_of<8, 128, 8>(v);
-    if (k <= 64) return ens_union_of<16, 256, 16>(v);
-    if (k <= 100) return ens_union_of<12, 256, 16>(v);
+// Few queries (up to eight per SM) do not fill the SMs with small CTAs, and a query's own time counts: as many models per
+// block and threads as there are (200 queries, against the choice for many: 85 x 10: 16.5 / 20.6, 40 x 20: 12.5 / 14.4, 30 x 50: 12.4 / 14.4,
+// 40 x 100: 20.6 / 28.8; 1,184 queries: 85 x 10: 30.9 / 34.9, 30 x 50: 27.0 / 28.9, 40 x 100: 45.8 / 57.3; 2,368: 51.3 / 47.3, 45.4 / 41.9, 82.0 / 88.3).
+EnsUnion ens_union_choice(int models, int k, int v, bool few) {
+    if (few) {
+        if (k <= 32) return ens_union_of<16, 128, 16>(v);
+        if (k <= 64) return ens_union_of<16, 256, 16>(v);
+    } else {
+        if (k <= 24) return ens_union_of<8, 128, 8>(v);
+        if (k <= 48) return ens_union_of<12, 128, 8>(v);
+        if (models <= (k <= 80 ? 40 : (k <= 100 ? 20 : 12)) && k <= 128) return ens_union_of<8, 128, 8>(v);
+        if (k <= 64) return ens_union_of<16, 256, 16>(v);
+    }
+    if (k <= 100) return ens_union_of<12, 256, 8>(v);
     return k <= 214 ? ens_union_of<8, 256, 16>(v) : ens_union_of<8, 256, 8>(v);
 }
 // Every kernel of the two above with the most shared memory it is launched with.
@@ -679,8 +689,8 @@ void ens_each_union(F f) {
     constexpr size_t sort = 1024 * (sizeof(uint64_t) + sizeof(int32_t));        // (M K <= 682)
     for (int v : {1, 2, 4}) {
         for (int each : {1, 3, 6}) f(ens_small_kernel(v, each), std::max(ens_union_smem(ENS_SMALL_MB, ENS_SMALL_COPIES, 1 << ENS_SMALL_LOG2, ENS_MAX_K), sort));
-        for (const EnsUnion& u : {ens_union_of<8, 128, 8>(v), ens_union_of<12, 128, 8>(v), ens_union_of<16, 256, 16>(v), ens_union_of<12, 256, 16>(v),
-                                  ens_union_of<8, 256, 16>(v), ens_union_of<8, 256, 8>(v)})
+        for (const EnsUnion& u : {ens_union_of<8, 128, 8>(v), ens_union_of<12, 128, 8>(v), ens_union_of<16, 128, 16>(v), ens_union_of<16, 256, 16>(v),
+                                  ens_union_of<12, 256, 8>(v), ens_union_of<8, 256, 16>(v), ens_union_of<8, 256, 8>(v)})
             f(u.kernel, ens_union_smem(u.models, u.copies, 1 << ENS_LOG2, ENS_MAX_K));
     }
 }
@@ -735,22 +745,23 @@ int kge_ensemble_topk(const int32_t* lists, int32_t num_models, int32_t nq, int3
     p.inv_k = (uint32_t)((((uint64_t)1 << 32) + k_list - 1) / k_list);
     const int quads = (k_list + 3) / 4;
     p.inv_quads = quads == 1 ? 0u : (uint32_t)((((uint64_t)1 << 32) + quads - 1) / quads);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;
     const int v = ens_places_per_load(lists, k_list);
     p.log2_slots = 5;
     while (2 << p.log2_slots < 3 * num_models * k_list) ++p.log2_slots;
     if (p.log2_slots <= ENS_SMALL_LOG2) {
         const int entries = num_models * k_list, block = std::min(num_models, ENS_SMALL_MB) * quads;
-        const int threads = entries <= 384 && (block <= 64 || (block <= 80 && k_list <= 64)) ? 64 : 128;
+        int threads = entries <= 384 && (block <= 64 || (block <= 80 && k_list <= 64)) ? 64 : 128;
+        if (nq <= 4 * sms && block > threads) threads = block <= 128 ? 128 : 256;
         const int each = entries <= threads ? 1 : (entries <= 3 * threads ? 3 : 6);
         const size_t smem = std::max(ens_union_smem(ENS_SMALL_MB, ENS_SMALL_COPIES, 1 << p.log2_slots, k_list), sort_smem);
         ens_small_kernel(v, each)<<<nq, threads, smem, s>>>(p);
         return cudaGetLastError() == cudaSuccess ? KGE_OK : KGE_ERR_CUDA;
     }
-    const EnsUnion u = ens_union_choice(num_models, k_list, v);
+    const EnsUnion u = ens_union_choice(num_models, k_list, v, nq <= 8 * sms);
     u.kernel<<<nq, u.threads, ens_union_smem(u.models, u.copies, 1 << ENS_LOG2, k_list), s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return KGE_ERR_CUDA;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return KGE_ERR_CUDA;
     p.log2_parts = 0; p.left_log2 = ENS_LOG2;
     while (p.left_log2 < ENS_BIG_LOG2 && 3 << (p.left_log2 - 2) < num_models * k_list) ++p.left_log2;
     while (num_models * k_list > ENS_BIG_PART << p.log2_parts) ++p.log2_parts;

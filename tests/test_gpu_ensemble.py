@@ -193,7 +193,7 @@ def test_ensemble_places_per_load(oracle64, M, K, shift, power, top_n):
 # both sides of every line that the choice of kernel draws: entries per thread and threads of the single launch; list length and
 # number of models of the first launch for longer lists
 @pytest.mark.parametrize("M,K", [(4, 16), (5, 13), (12, 16), (13, 15), (12, 32), (11, 35), (10, 32), (9, 36), (8, 40), (4, 80), (2, 64), (2, 65), (1, 254), (2, 254),
-                                 (29, 24), (28, 25), (15, 48), (14, 49), (41, 49), (40, 64), (41, 64), (41, 65), (40, 100), (41, 100), (12, 101), (13, 101),
+                                 (29, 24), (28, 25), (15, 48), (14, 49), (41, 49), (40, 64), (41, 64), (41, 65), (40, 80), (41, 80), (20, 100), (21, 100), (12, 101), (13, 101),
                                  (12, 128), (13, 128), (12, 129), (4, 214), (4, 215), (3, 254)])
 @pytest.mark.parametrize("power,top_n", [(-0.5, 10), (0.5, 17)])
 def test_ensemble_kernel_choice(oracle64, M, K, power, top_n):
@@ -216,3 +216,16 @@ def test_ensemble_long_results(oracle64, M, K, top_n, power):
     ids, sc = _gpu_ensemble(lists, power, top_n)
     o_ids, o_sc = oracle64.ensemble_topk(lists, power, top_n)
     assert (ids == o_ids).all() and (sc == o_sc).all()
+
+
+# the same lists for as few queries as take large CTAs and as many as do not (four and eight per SM)
+@pytest.mark.parametrize("M,K", [(6, 100), (16, 20), (13, 50), (3, 10), (85, 10), (40, 20), (25, 32), (30, 50), (40, 100), (10, 101)])
+def test_ensemble_few_and_many_queries(oracle64, M, K):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(M * K)
+    some = np.stack([np.stack([rng.permutation(3 * K)[:K] for _ in range(37)]) for _ in range(M)]).astype(np.int32)
+    o_ids, o_sc = oracle64.ensemble_topk(some, -0.5, 10)
+    for nq in (4 * sms, 4 * sms + 1, 8 * sms, 8 * sms + 1):
+        ids, sc = _gpu_ensemble(some[:, np.arange(nq) % 37], -0.5, 10)
+        assert (ids == o_ids[np.arange(nq) % 37]).all() and (sc == o_sc[np.arange(nq) % 37]).all()
