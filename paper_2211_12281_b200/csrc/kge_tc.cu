@@ -238,7 +238,7 @@ __device__ __forceinline__ TcRowState tc_row_state(const TcGemmParams& p, int ro
 // negatives (the gather kernel computes them), a lower bound of the maximum up to rounding and a constant.  A chunk of 32 scores that exceeds it
 // by more than 2^TC_REF_SPAN takes its own maximum instead, which keeps the statistics in range, and the row is found by
 // stats_combine_kernel and its E written again, over the true maximum and with the factor, by an EPI_GRAD launch that
-// otherwise ends at once; so is a row whose scores all lie below it (row_statistics).  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
+// otherwise ends at once; so is a row whose scores all lie far below it (finish_low_row).  (Until then a pass for the statistics and one for the gradients, the scores recomputed: ComplEx
 // softmax 4,096 x 16,384 x 256 34 + 53 us, TransE-L2 8,192 x 8,192 x 128 67 + 94 us.)
 constexpr float TC_REF_SPAN = 80.f;
 constexpr float TC_EXP_MIN = -126.f;      // below it an exponential is 0
@@ -1523,10 +1523,41 @@ struct CombineParams {
     float k1, k0;                         // base-2 exponent of a score: k1 f + k0
 };
 
-// Statistics of a row whose scores all lie so far below its reference that their exponentials are gone: the reference comes from
-// the unrounded rows, and with norms or a temperature far beyond the usual the score block can be 2^126 below it.  The warp
-// goes over the row's scores itself: (base-2 maximum, sum of exponentials, weighted loss sum) over the negatives.
-__device__ __noinline__ float3 row_statistics(const CombineParams& p, int b, int lane) {
+// What a row leaves behind, from its (base-2 maximum, sum of exponentials, weighted loss sum): the operand's factor, the loss, dL/df+.
+// `good`: its dL/dF stands up to the factor loss_scale / z; otherwise it is left to the second round.
+__device__ __forceinline__ void finish_row(const CombineParams& p, int b, int lane, float fp, float m, float z, float l, bool good) {
+    const float scale = good ? p.loss_scale / z : 1.f;
+    if (good)
+        for (int c = lane; c < p.d4; c += 32) {
+            const float4 q = p.Q[(int64_t)b * p.d4 + c];
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(scale * q.x, scale * q.y), hi = __floats2bfloat162_rn(scale * q.z, scale * q.w);
+            p.Qb[(int64_t)b * p.d4 + c] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        }
+    if (p.Xq) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(scale), lo = __float2bfloat16_rn(scale - __bfloat162float(hi));
+        p.Xq[(int64_t)b * 32 + lane] = lane == 0 ? (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16 : 0u;
+    }
+    if (lane != 0) return;
+    if (p.loss == KGE_LOSS_SAMPLED_SOFTMAX) {
+        const float epos = exp2f(fp * kLog2e - m);
+        p.Lrow[b] = -fp + (m + log2f(z)) * 0.6931471805599453f;
+        p.gpos[b] = p.loss_scale * (epos / z - 1.f);
+    } else {
+        const float zp = -(p.gamma + fp), ep = expf(-fabsf(zp)), rp = 1.f / (1.f + ep);   // once per row: the exact forms
+        const float sp = fmaxf(zp, 0.f) + log1pf(ep), sg = zp >= 0.f ? rp : ep * rp;
+        p.Lrow[b] = sp + l / z;
+        p.gpos[b] = -p.loss_scale * sg;
+    }
+    p.row_scale[b] = scale;
+    p.row_stat[b] = make_float2(m, good ? 0.f : 1.f / z);
+    if (!good) *p.redo = 1;
+}
+
+// A row whose scores all lie so far below its reference that their exponentials are gone: the reference comes from the unrounded
+// rows, and with norms or a temperature far beyond the usual the score block can be 2^126 below it.  The warp goes over the row's
+// scores itself.  (Called last and with nothing to keep, so that the other rows' registers do not pay for it: called from the middle of
+// the kernel, 0.9 to 1.4 us of a step at 4,096 x 16,384 and 8,192 x 8,192.)
+__device__ __noinline__ void finish_low_row(const CombineParams& p, int b, int lane, float fp) {
     const bool ce = p.loss == KGE_LOSS_SAMPLED_SOFTMAX;
     const uint2* q = p.Qb + (int64_t)b * p.d4;
     const float rn = p.Xq ? p.qn2[b] : 0.f;
@@ -1545,11 +1576,17 @@ __device__ __noinline__ float3 row_statistics(const CombineParams& p, int b, int
         z += e;
         if (!ce) l += e * softplusf(p.gamma + f);
     }
-    const float top = warp_max(m), r = m == -INFINITY ? 0.f : exp2f(m - top);
-    return make_float3(top, warp_sum(z * r), warp_sum(l * r));
+    float top = warp_max(m);
+    const float r = m == -INFINITY ? 0.f : exp2f(m - top);
+    z = warp_sum(z * r); l = warp_sum(l * r);
+    if (ce) {                  // the positive score, which the sampled softmax normalises over too
+        const float mm = fmaxf(top, fp * kLog2e);
+        z = z * exp2f(top - mm) + exp2f(fp * kLog2e - mm);
+        top = mm;
+    }
+    finish_row(p, b, lane, fp, top, z, l, false);
 }
 
-// (eight CTAs per SM: the call of row_statistics would take 48 registers, 4 us more per step at 4,096 x 16,384 and 8,192 x 8,192)
 __global__ void __launch_bounds__(256, 8) stats_combine_kernel(const __grid_constant__ CombineParams p) {
     const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     grid_dependency_wait();
@@ -1573,42 +1610,8 @@ __global__ void __launch_bounds__(256, 8) stats_combine_kernel(const __grid_cons
     }
     z = warp_sum(z); l = warp_sum(l);
     if (ce) z += exp2f(fp * kLog2e - m);
-    if (z < 0x1p-40f) {        // (at 2^-40 the weights that matter are still 2^60 above the smallest number)
-        const float3 s = row_statistics(p, b, lane);
-        m = s.x; z = s.y; l = s.z;
-        if (ce) {
-            const float mm = fmaxf(m, fp * kLog2e);
-            z = z * exp2f(m - mm) + exp2f(fp * kLog2e - mm);
-            m = mm;
-        }
-        good = false;
-    }
-    good = good && z < INFINITY;
-    const float scale = good ? p.loss_scale / z : 1.f;
-    if (good)
-        for (int c = lane; c < p.d4; c += 32) {
-            const float4 q = p.Q[(int64_t)b * p.d4 + c];
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(scale * q.x, scale * q.y), hi = __floats2bfloat162_rn(scale * q.z, scale * q.w);
-            p.Qb[(int64_t)b * p.d4 + c] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-        }
-    if (p.Xq) {
-        const __nv_bfloat16 hi = __float2bfloat16_rn(scale), lo = __float2bfloat16_rn(scale - __bfloat162float(hi));
-        p.Xq[(int64_t)b * 32 + lane] = lane == 0 ? (uint32_t)__bfloat16_as_ushort(hi) | (uint32_t)__bfloat16_as_ushort(lo) << 16 : 0u;
-    }
-    if (lane != 0) return;
-    if (ce) {
-        const float epos = exp2f(fp * kLog2e - m);
-        p.Lrow[b] = -fp + (m + log2f(z)) * 0.6931471805599453f;
-        p.gpos[b] = p.loss_scale * (epos / z - 1.f);
-    } else {
-        const float zp = -(p.gamma + fp), ep = expf(-fabsf(zp)), rp = 1.f / (1.f + ep);   // once per row: the exact forms
-        const float sp = fmaxf(zp, 0.f) + log1pf(ep), sg = zp >= 0.f ? rp : ep * rp;
-        p.Lrow[b] = sp + l / z;
-        p.gpos[b] = -p.loss_scale * sg;
-    }
-    p.row_scale[b] = scale;
-    p.row_stat[b] = make_float2(m, good ? 0.f : 1.f / z);
-    if (!good) *p.redo = 1;
+    if (z < 0x1p-40f) finish_low_row(p, b, lane, fp);  // (at 2^-40 the weights that matter are still 2^60 above the smallest number)
+    else finish_row(p, b, lane, fp, m, z, l, good && z < INFINITY);
 }
 
 }  // namespace
