@@ -588,8 +588,8 @@ __global__ void __launch_bounds__(T) ensemble_hash_kernel(EnsParams p) {
 // Second launch: the queries with larger unions.  Up to 8,192 slots (180 KB), eight models at a time.  Up to ENS_BIG_PART
 // entries the table takes whatever the lists hold, in one pass; beyond, the passes are as many as give each at most ENS_BIG_PART
 // entries if their hashes spread evenly (a query whose hashes favour one part that much is sorted), and the best n of the passes
-// so far wait in shared memory.  85 x top-100 lists of 15,000 queries, all left here: unions of 1,000 6.4 ms, 3,600 8.3, 6,500
-// 10.0, where the sort takes 37.8.
+// so far wait in shared memory.  85 x top-100 lists of 15,000 queries, all left here: unions of 1,000 7.2 ms, 3,500 9.0, 6,600
+// 11.0, where the sort takes 37.8.
 constexpr int ENS_BIG_MB = 8, ENS_BIG_LOG2 = 13, ENS_BIG_PART = 5400, ENS_BIG_TOP = ENS_THREADS;
 template <int NT>
 __global__ void __launch_bounds__(NT, 2048 / NT) ensemble_left_kernel(EnsParams p) {
